@@ -96,6 +96,10 @@ ipa_status cuda_fail(cudaError_t e, const char* what);
 bool fault(uint32_t bit);
 // cudaMalloc, or IPA_ERR_OOM without calling it while IPA_FAULT_ALLOC is set.
 ipa_status device_alloc(void** p, size_t bytes, const char* what);
+// Temporary device memory in stream order, from the library's own pool
+// (pool_alloc fails as device_alloc does while IPA_FAULT_ALLOC is set).
+ipa_status pool_alloc(void** p, size_t bytes, cudaStream_t s, const char* what);
+void pool_free(void* p, cudaStream_t s);
 ipa_status check_model(const ipa_model* m);
 ipa_status check_events(const ipa_model* m, const ipa_events* ev);
 
@@ -166,14 +170,9 @@ ipa_status launch_phis_nll(const ModelDev& m, bool grad, const Cols& cols, int64
 ipa_status launch_tag_nll(const ModelDev& m, bool grad, const Cols& cols, int64_t n,
                           const int64_t* seg_begin, const int64_t* seg_end, const int64_t* seg_tiles, int n_seg,
                           const Consts* consts, Scratch* sc, double* out, cudaStream_t s, const LaunchCfg* cfg);
-// toygen.cu / tagged.cu: the tagged model's generator over consts[0]
-ipa_status launch_tag_toygen(const ModelDev& m, const Consts* consts, uint64_t seed, int n_toys,
-                             const int64_t* n_sig, const int64_t* n_bkg, const int64_t* offsets,
-                             const ipa_event_buffers* out, cudaStream_t s);
 // phis.cu: the phi_s model's generator (a PhisConsts record in consts[0])
-ipa_status launch_phis_toygen(const ModelDev& m, const Consts* consts, uint64_t seed, int n_toys,
-                              const int64_t* n_sig, const int64_t* n_bkg, const int64_t* offsets,
-                              const ipa_event_buffers* out, cudaStream_t s);
+struct GenArgs;
+ipa_status launch_phis_toygen(const GenArgs& a, cudaStream_t s);
 // nll.cu: seg_tiles[s] = sum_{r<s} ceil(size_r / kTile), s = 0..n_seg, with the
 // ranges clamped to [0, n]; segments with active[r] == 0 get no tiles (active may
 // be NULL).

@@ -25,8 +25,10 @@
 // (z sigma + tau/sigma) G, dg/dtau = -z g + G).  With Q = sum r: 47 sums.
 #include <math.h>
 
+#include "accept_reject.cuh"
 #include "angular.cuh"
 #include "consts.cuh"
+#include "conv32.cuh"
 #include "faddeeva.cuh"
 #include "fp64_math.cuh"
 #include "int_math.cuh"
@@ -516,24 +518,22 @@ constexpr int kGenBins = 64;    // decay-time bins of the generator's envelope
 // bilinear is at most |b_k| (gL + gH + 2 |gc|) and a convolved exponential
 // g(tau; x) decreases in tau and is at most min(1, e^{-x tau + x^2 sigma^2 /
 // 2}), taken at the left edge: B_i = (m(Gamma_L) + m(Gamma_H) + 2 m(Gamma))
-// sum_k max|f_k| |b_k| r_k (r_k = |C_SP| for the S-P terms).  C: running sums of
-// B in order (C_0 = 0), the proposal's cumulative weights.  One thread.
-__device__ void phis_envelope_bins(const PhisConsts& c, const ModelDev& m, double w, double* B, double* C) {
-    using namespace cdetail;
+// sum_k max|f_k| |b_k| r_k (r_k = |C_SP| for the S-P terms).
+__device__ inline double phis_envelope_ang(const PhisConsts& c) {
     const double sF = 1.0 - c.F, rFs = c.rF * c.rs;
     const double mag[10] = {sF * c.x0, sF * c.xa, sF * c.xe, sF * c.ra * c.re, sF * c.r0 * c.ra, sF * c.r0 * c.re,
                             c.F, rFs * c.ra, rFs * c.re, rFs * c.r0};
     double ang = 0.0;
-    for (int k = 0; k < 10; ++k) ang += basis_max(k) * mag[k] * (k >= 7 ? fabs(c.csp) : 1.0);
-    C[0] = 0.0;
-    for (int i = 0; i < kGenBins; ++i) {
-        const double e = __dadd_rn(m.t_lo, __dmul_rn((double)i, w)) - c.mu;
-        const double ML = fmin(1.0, exp(-c.GL * e + 0.5 * c.GL * c.GL * c.s2));
-        const double MH = fmin(1.0, exp(-c.GH * e + 0.5 * c.GH * c.GH * c.s2));
-        const double MG = fmin(1.0, exp(-c.Gamma * e + 0.5 * c.Gamma * c.Gamma * c.s2));
-        B[i] = (ML + MH + 2.0 * MG) * ang;
-        C[i + 1] = __dadd_rn(C[i], B[i]);
-    }
+#pragma unroll
+    for (int k = 0; k < 10; ++k) ang += cdetail::basis_max(k) * mag[k] * (k >= 7 ? fabs(c.csp) : 1.0);
+    return ang;
+}
+__device__ inline double phis_envelope_bin(const PhisConsts& c, const ModelDev& m, double w, double ang, int i) {
+    const double e = __dadd_rn(m.t_lo, __dmul_rn((double)i, w)) - c.mu;
+    const double ML = fmin(1.0, exp(-c.GL * e + 0.5 * c.GL * c.GL * c.s2));
+    const double MH = fmin(1.0, exp(-c.GH * e + 0.5 * c.GH * c.GH * c.s2));
+    const double MG = fmin(1.0, exp(-c.Gamma * e + 0.5 * c.Gamma * c.Gamma * c.s2));
+    return (ML + MH + 2.0 * MG) * ang;
 }
 
 // rate(t, Omega, q) = sum_k f_k r_k sum_j C_kj G_j, G = (gL, gH, q Re gc, q Im gc),
@@ -557,133 +557,250 @@ __device__ double phis_rate_exact(const PhisConsts& c, const MathTables* mt, dou
     return r;
 }
 
-constexpr int kGenPerThread = 16;              // candidates per thread per chunk (bits of a mask)
-constexpr int kGenChunk = kBlock * kGenPerThread;
-
 // Signal candidate j of toy k: Philox calls (j, k, 0): u_bin, u_acc; (j, k, 1):
 // ck, cl; (j, k, 2): phi, u_pos; (j, k, 3): u_q.  Its bin is the first i with
-// u_bin C_64 <= C_{i+1} (the proposal is piecewise uniform with weights B_i),
-// t = min(e_i + u_pos w, t_hi); the tag is the selected one (Q = +-1) or +1 for
-// u_q <= 1/2, else -1; kept iff u_acc B_i < rate.  The toy takes the first
-// n_sig kept candidates in increasing j.  Background event i: (i, k, 4): t,
-// ck; (i, k, 5): cl, phi; (i, k, 6): u_q.  One block per toy.
-__global__ void __launch_bounds__(kBlock)
-phis_toygen_kernel(ModelDev m, const Consts* __restrict__ consts, uint32_t k0, uint32_t k1, int n_toys,
-                   const int64_t* __restrict__ n_sig, const int64_t* __restrict__ n_bkg,
-                   const int64_t* __restrict__ offsets, int64_t capacity, double* __restrict__ ot,
-                   double* __restrict__ ock, double* __restrict__ ocl, double* __restrict__ ophi,
-                   double* __restrict__ oq) {
-    __shared__ __align__(16) PhisConsts c;
-    __shared__ MathTables mt;
-    __shared__ int warp_sums[kBlock / 32];
-    __shared__ double B[kGenBins], C[kGenBins + 1];
-    {
-        const double* src = reinterpret_cast<const double*>(consts);
-        double* dst = reinterpret_cast<double*>(&c);
+// u_bin C_64 <= C_{i+1} (C the running sums of B in order: the proposal is
+// piecewise uniform with weights B_i), t = min(e_i + u_pos w, t_hi); the tag is
+// the selected one (Q = +-1) or +1 for u_q <= 1/2 (the top bit of its first
+// word clear), else -1; kept iff u_acc B_i < rate.  Background event i: (i, k,
+// 4): t, ck; (i, k, 5): cl, phi; (i, k, 6): u_q.
+//
+// FP32: the ten terms' coefficients have only four distinct time functions (a
+// term whose two amplitudes have the same CP eigenvalue takes T+ or T-, a mixed
+// term U and V),
+//   T+- = (gL + gH)/2 +- [cos phi_s (gL - gH)/2 + D sin phi_s q Im gc],
+//   U = sin phi_s (gL - gH)/2 - D cos phi_s q Im gc,   V = D q Re gc,
+// so rate = F+ T+ + F- T- + FU U + FV V with four angular sums of fourteen
+// products.  quick() decides candidates above the resolution peak; those near
+// it (about a seventh) are packed and take the FP32 erfc and Faddeeva
+// function (conv32.cuh).  Every convolution carries the relative bound of
+// conv32.cuh, every f'_k an error below 8e-5 where both sin^2 >= 1e-4
+// (cosines within 2.5e-7, so sines within 2.6e-5; the sine and cosine of phi
+// within 1e-6), and sum_k |b_k| r_k <= 3 sum_k max|f_k| |b_k| r_k = 3 ang:
+// |rate32 - rate| <= ang (gL + gH + 2 C) (rel + 2.5e-4), doubled to spare.
+struct PhisGen {
+    static constexpr bool kQuickKeeps = true;
+    static constexpr int kBlocksPerSm = 3;
+    struct Shared {
+        PhisConsts c;
+        MathTables mt;
+        double B[kGenBins], C[kGenBins + 1];
+        double t_lo, t_hi, w, total;
+        Conv32 v;
+        float Bf[kGenBins], Cf[kGenBins + 1], ef[kGenBins];   // B, C, e_i - mu
+        float wf, totalf, ang;
+        float p[10];           // coefficient of f'_k in F+ or F- (equal eigenvalues)
+        float u[4], x[4];      // coefficients of f'_3, f'_5, f'_7, f'_9 in FU and FV
+        float cph, sph, D, C2;  // C2 = 2 max(1, |D|)
+    };
+
+    __device__ static void setup(Shared& S, const GenArgs& A) {
+        const double* src = reinterpret_cast<const double*>(A.consts);
+        double* dst = reinterpret_cast<double*>(&S.c);
         for (int i = threadIdx.x; i < kPhisDoubles; i += blockDim.x) dst[i] = src[i];
+        load_math_tables(&S.mt);
+        __syncthreads();
+        const PhisConsts& c = S.c;
+        const double span = __dsub_rn(A.m.t_hi, A.m.t_lo);
+        const double w = __ddiv_rn(span, (double)kGenBins);
+        if (threadIdx.x < kGenBins) {
+            const int i = threadIdx.x;
+            S.B[i] = phis_envelope_bin(c, A.m, w, phis_envelope_ang(c), i);
+            S.Bf[i] = (float)S.B[i];
+            S.ef[i] = (float)(__dadd_rn(A.m.t_lo, __dmul_rn((double)i, w)) - c.mu);
+        } else if (threadIdx.x == 96) {
+            S.t_lo = A.m.t_lo;
+            S.t_hi = A.m.t_hi;
+            S.w = w;
+            S.wf = (float)w;
+            S.ang = (float)phis_envelope_ang(c);
+            S.v = conv32_of(c, A.m.t_lo - c.mu, span);
+            S.cph = (float)c.c;
+            S.sph = (float)c.s;
+            S.D = (float)c.D;
+            S.C2 = 2.0f * fmaxf(1.0f, fabsf(S.D));
+        } else if (threadIdx.x >= 128 && threadIdx.x < 138) {
+            const int k = threadIdx.x - 128;
+            const double sc = kBasisScale[k] * row_scale(c, k);
+            const double ej = kEta[kPairJ[k]];
+            S.p[k] = (float)(sc * (kPairIm[k] ? c.bi[k] : c.br[k]));
+            if (kEta[kPairI[k]] != ej) {
+                const int i = (k - 3) >> 1;          // 3, 5, 7, 9
+                S.u[i] = (float)(sc * (kPairIm[k] ? -ej * c.br[k] : ej * c.bi[k]));
+                S.x[i] = (float)(sc * (kPairIm[k] ? c.bi[k] : c.br[k]));
+            }
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double s = 0.0;
+            S.C[0] = 0.0;
+            S.Cf[0] = 0.0f;
+            for (int i = 0; i < kGenBins; ++i) {
+                s = __dadd_rn(s, S.B[i]);
+                S.C[i + 1] = s;
+                S.Cf[i + 1] = (float)s;
+            }
+            S.total = s;
+            S.totalf = (float)s;
+        }
     }
-    load_math_tables(&mt);
-    const double span = __dsub_rn(m.t_hi, m.t_lo);
-    const double w = __ddiv_rn(span, (double)kGenBins);
-    __syncthreads();
-    if (threadIdx.x == 0) phis_envelope_bins(c, m, w, B, C);
-    __syncthreads();
-    const double total = C[kGenBins];
-    // the first bin i with target <= C[i + 1] (C non-decreasing: binary search)
-    auto bin_of = [&](double u) {
-        const double target = __dmul_rn(u, total);
+
+    __device__ static bool usable(const Shared& S) {
+        return isfinite(S.total) && S.total > 0.0 && isfinite(S.c.N) && S.c.N > 0.0;
+    }
+
+    // N is the integral over both tags (each drawn half of the time) or over the selected one
+    __device__ static void acceptance(const GenArgs& A, float* acc) {
+        __shared__ float sum;
+        if (threadIdx.x == 0) sum = 0.0f;
+        __syncthreads();
+        const PhisConsts& c = *reinterpret_cast<const PhisConsts*>(A.consts);
+        const double w = (A.m.t_hi - A.m.t_lo) / kGenBins;
+        if (threadIdx.x < kGenBins)
+            atomicAdd(&sum, (float)phis_envelope_bin(c, A.m, w, phis_envelope_ang(c), threadIdx.x));
+        __syncthreads();
+        if (threadIdx.x == 0)
+            *acc = (c.qsel != 0.0 ? 1.0f : 0.5f) * (float)c.N / (8.0f * (float)cdetail::kPi * (float)w * sum);
+    }
+
+    // the first bin i with u C_64 <= C[i + 1]
+    __device__ __forceinline__ static int bin_of(const Shared& S, double u) {
+        const double target = __dmul_rn(u, S.total);
         int lo = 0, hi = kGenBins - 1;
         while (lo < hi) {
             const int mid = (lo + hi) >> 1;
-            if (target <= C[mid + 1]) hi = mid; else lo = mid + 1;
+            if (target <= S.C[mid + 1]) hi = mid; else lo = mid + 1;
         }
         return lo;
-    };
-    auto t_of = [&](int b, double u) {
-        return fmin(__dadd_rn(__dadd_rn(m.t_lo, __dmul_rn((double)b, w)), __dmul_rn(u, w)), m.t_hi);
-    };
-    const double nan = __longlong_as_double(0x7ff8000000000000ll);
-    const double Q = c.qsel;
-    auto tag = [&](double u) { return Q != 0.0 ? Q : (u <= 0.5 ? 1.0 : -1.0); };
-    auto angles = [&](const U4& b, const U4& d, double* ck, double* cl, double* ph) {
-        *ck = __dsub_rn(__dmul_rn(2.0, u01(b.x, b.y)), 1.0);
-        *cl = __dsub_rn(__dmul_rn(2.0, u01(b.z, b.w)), 1.0);
-        *ph = __dmul_rn(cdetail::kPi, __dsub_rn(__dmul_rn(2.0, u01(d.x, d.y)), 1.0));
-    };
-    for (int toy = blockIdx.x; toy < n_toys; toy += gridDim.x) {
-        const int64_t ns = n_sig[toy], nb = n_bkg[toy], off = offsets[toy];
-        if (ns < 0 || nb < 0 || off < 0 || off + ns + nb > capacity) continue;   // skipped
-        const bool usable = isfinite(total) && total > 0.0 && isfinite(c.N) && c.N > 0.0;
-        const uint64_t budget = usable ? (uint64_t)ns * 65536ull + (1ull << 22) : 0ull;
-        int64_t got = 0;
-        for (uint64_t j0 = 0; got < ns && j0 < budget; j0 += kGenChunk) {
-            const uint64_t jt = j0 + (uint64_t)threadIdx.x * kGenPerThread;
-            unsigned mask = 0;
-#pragma unroll 1
-            for (int i = 0; i < kGenPerThread; ++i) {
-                const uint64_t j = jt + i;
-                const U4 a = draw(j, (uint32_t)toy, 0u, k0, k1);
-                const U4 b = draw(j, (uint32_t)toy, 1u, k0, k1);
-                const U4 d = draw(j, (uint32_t)toy, 2u, k0, k1);
-                const double uq = Q != 0.0 ? 0.0 : u01(draw(j, (uint32_t)toy, 3u, k0, k1).x,
-                                                       draw(j, (uint32_t)toy, 3u, k0, k1).y);
-                const int bin = bin_of(u01(a.x, a.y));
-                const double t = t_of(bin, u01(d.z, d.w));
-                double ck, cl, ph;
-                angles(b, d, &ck, &cl, &ph);
-                if (__dmul_rn(u01(a.z, a.w), B[bin]) < phis_rate_exact(c, &mt, t, ck, cl, ph, tag(uq)))
-                    mask |= 1u << i;
-            }
-            int total;
-            const int before = block_exclusive_scan(__popc(mask), warp_sums, &total);
-            int rank = 0;
-            while (mask) {
-                const int i = __ffs(mask) - 1;
-                mask &= mask - 1u;
-                const int64_t pos = got + before + rank;
-                ++rank;
-                if (pos >= ns) break;
-                const uint64_t j = jt + i;
-                const U4 a = draw(j, (uint32_t)toy, 0u, k0, k1);
-                const U4 b = draw(j, (uint32_t)toy, 1u, k0, k1);
-                const U4 d = draw(j, (uint32_t)toy, 2u, k0, k1);
-                const U4 e = draw(j, (uint32_t)toy, 3u, k0, k1);
-                double ck, cl, ph;
-                angles(b, d, &ck, &cl, &ph);
-                ot[off + pos] = t_of(bin_of(u01(a.x, a.y)), u01(d.z, d.w));
-                ock[off + pos] = ck;
-                ocl[off + pos] = cl;
-                ophi[off + pos] = ph;
-                oq[off + pos] = tag(u01(e.x, e.y));
-            }
-            got += total;
-        }
-        for (int64_t pos = got + threadIdx.x; pos < ns; pos += blockDim.x)
-            ot[off + pos] = ock[off + pos] = ocl[off + pos] = ophi[off + pos] = oq[off + pos] = nan;
-        for (int64_t i = threadIdx.x; i < nb; i += blockDim.x) {
-            const U4 a = draw((uint64_t)i, (uint32_t)toy, 4u, k0, k1);
-            const U4 b = draw((uint64_t)i, (uint32_t)toy, 5u, k0, k1);
-            const U4 e = draw((uint64_t)i, (uint32_t)toy, 6u, k0, k1);
-            const int64_t pos = off + ns + i;
-            ot[pos] = __dadd_rn(m.t_lo, __dmul_rn(u01(a.x, a.y), span));
-            ock[pos] = __dsub_rn(__dmul_rn(2.0, u01(a.z, a.w)), 1.0);
-            ocl[pos] = __dsub_rn(__dmul_rn(2.0, u01(b.x, b.y)), 1.0);
-            ophi[pos] = __dmul_rn(cdetail::kPi, __dsub_rn(__dmul_rn(2.0, u01(b.z, b.w)), 1.0));
-            oq[pos] = tag(u01(e.x, e.y));
-        }
     }
-}
+    // the same in FP32, or -1 where the uniform lies too near an edge of its bin
+    // (u C_64 and C are off by less than 2.4e-7 C_64 together)
+    __device__ __forceinline__ static int bin32(const Shared& S, uint32_t hi_word) {
+        const float target = u32of(hi_word) * S.totalf;
+        int lo = 0;
+#pragma unroll
+        for (int d = kGenBins / 2; d > 0; d >>= 1) lo += target > S.Cf[lo + d] ? d : 0;
+        const float band = 1.0e-6f * S.totalf;
+        return target - S.Cf[lo] > band && S.Cf[lo + 1] - target > band ? lo : -1;
+    }
+    __device__ __forceinline__ static double t_of(const Shared& S, int b, double u) {
+        return fmin(__dadd_rn(__dadd_rn(S.t_lo, __dmul_rn((double)b, S.w)), __dmul_rn(u, S.w)), S.t_hi);
+    }
+
+    // F+, F-, FU, FV from the words of calls 1 and 2; false outside the bound's range
+    __device__ __forceinline__ static bool sums32(const Shared& S, const U4& b, const U4& d, float* F) {
+        const float ck = fmaf(2.0f, u32of(b.x), -1.0f), cl = fmaf(2.0f, u32of(b.z), -1.0f);
+        const float cl2 = cl * cl;
+        const float sk2 = fmaf(-ck, ck, 1.0f), sl2 = fmaf(-cl, cl, 1.0f);
+        float sp, cp;
+        sincospif(fmaf(2.0f, u32of(d.x), -1.0f), &sp, &cp);
+        const float sksl2 = sk2 * sl2;
+        const float q = sqrtf(fmaxf(sksl2, 0.0f));
+        const float cp2 = cp * cp;
+        const float qc = q * cl, a = qc * ck;
+        F[0] = fmaf(S.p[0], ck * ck * sl2, fmaf(S.p[1], sk2 * fmaf(-sl2, cp2, 1.0f), S.p[4] * (a * cp)));
+        F[1] = fmaf(S.p[2], sk2 * fmaf(sl2, cp2, cl2), fmaf(S.p[6], sl2, S.p[8] * (qc * sp)));
+        const float f3 = sksl2 * (sp * cp), f5 = a * sp, f7 = qc * cp, f9 = ck * sl2;
+        F[2] = fmaf(S.u[0], f3, fmaf(S.u[1], f5, fmaf(S.u[2], f7, S.u[3] * f9)));
+        F[3] = fmaf(S.x[0], f3, fmaf(S.x[1], f5, fmaf(S.x[2], f7, S.x[3] * f9)));
+        return sk2 >= 1.0e-4f && sl2 >= 1.0e-4f;
+    }
+
+    __device__ __forceinline__ static GenCode decide(const Shared& S, float u, int bin, const float* F, const Time32& g,
+                                                     float q) {
+        const float half = 0.5f * (g.L + g.H), diff = 0.5f * (g.L - g.H);
+        const float ci = q * S.D * g.Ci;
+        const float mix = S.cph * diff + S.sph * ci;
+        const float rate = F[0] * (half + mix) + F[1] * (half - mix) + F[2] * (S.sph * diff - S.cph * ci) +
+                           F[3] * (q * S.D * g.Cr);
+        const float err = S.ang * (g.L + g.H + S.C2 * g.C) * (2.0f * g.err + 5.0e-4f);
+        return decide32(u * S.Bf[bin], S.Bf[bin] * 1.5e-6f, rate, err);
+    }
+
+    __device__ __forceinline__ static float tag32(const Shared& S, uint64_t j, uint32_t toy, uint32_t k0, uint32_t k1) {
+        return (float)tag_of(S, S.c.qsel != 0.0 ? 0u : draw(j, toy, 3u, k0, k1).x);
+    }
+    __device__ __forceinline__ static double tag_of(const Shared& S, uint32_t hi) {
+        return S.c.qsel != 0.0 ? S.c.qsel : ((hi >> 31) ? -1.0 : 1.0);
+    }
+
+    __device__ __forceinline__ static GenCode quick(const Shared& S, uint64_t j, uint32_t toy, uint32_t k0, uint32_t k1) {
+        const U4 a = draw(j, toy, 0u, k0, k1);
+        const U4 d = draw(j, toy, 2u, k0, k1);
+        const int bin = bin32(S, a.x);
+        if (bin < 0) return kTest64;
+        const float tau = fmaf(u32of(d.z), S.wf, S.ef[bin]);
+        if (!(tau > S.v.near)) return kTest32;
+        const U4 b = draw(j, toy, 1u, k0, k1);
+        float F[4];
+        if (!sums32(S, b, d, F)) return kTest64;
+        const Far32 f = conv32_far(S.v, tau);
+        if (!f.ok) return kTest64;
+        // what the oscillation can add at most, before its phase and the tag
+        const float half = 0.5f * (f.L + f.H), diff = 0.5f * (f.L - f.H);
+        const float still = F[0] * (half + S.cph * diff) + F[1] * (half - S.cph * diff) + F[2] * S.sph * diff;
+        const float X = S.sph * (F[0] - F[1]) - S.cph * F[2];
+        const float osc = fabsf(S.D) * f.C * (fabsf(X) + fabsf(F[3]));
+        const float lhs = u32of(a.z) * S.Bf[bin];
+        const float err = S.ang * (f.L + f.H + S.C2 * f.C) * (2.0f * S.v.err + 5.0e-4f);
+        if (lhs - S.Bf[bin] * 1.5e-6f > still + osc + err) return kDrop;
+        return decide(S, u32of(a.z), bin, F, conv32(S.v, tau), tag32(S, j, toy, k0, k1));
+    }
+
+    // near the peak
+    __device__ __forceinline__ static GenCode test32(const Shared& S, uint64_t j, uint32_t toy, uint32_t k0, uint32_t k1) {
+        const U4 a = draw(j, toy, 0u, k0, k1);
+        const U4 d = draw(j, toy, 2u, k0, k1);
+        const int bin = bin32(S, a.x);
+        const U4 b = draw(j, toy, 1u, k0, k1);
+        float F[4];
+        if (bin < 0 || !sums32(S, b, d, F)) return kTest64;
+        const float tau = fmaf(u32of(d.z), S.wf, S.ef[bin]);
+        return decide(S, u32of(a.z), bin, F, conv32(S.v, tau), tag32(S, j, toy, k0, k1));
+    }
+
+    __device__ __noinline__ static bool test64(const Shared& S, uint64_t j, uint32_t toy, uint32_t k0, uint32_t k1) {
+        const U4 a = draw(j, toy, 0u, k0, k1);
+        const U4 b = draw(j, toy, 1u, k0, k1);
+        const U4 d = draw(j, toy, 2u, k0, k1);
+        const U4 e = draw(j, toy, 3u, k0, k1);
+        const int bin = bin_of(S, u01_int(a.x, a.y));
+        return __dmul_rn(u01_int(a.z, a.w), S.B[bin]) <
+               phis_rate_exact(S.c, &S.mt, t_of(S, bin, u01_int(d.z, d.w)), sym_int(b.x, b.y), sym_int(b.z, b.w),
+                               __dmul_rn(cdetail::kPi, sym_int(d.x, d.y)), tag_of(S, e.x));
+    }
+
+    __device__ __forceinline__ static void signal(const Shared& S, const GenArgs& A, uint64_t j, uint32_t toy, int64_t pos) {
+        const U4 a = draw(j, toy, 0u, A.k0, A.k1);
+        const U4 b = draw(j, toy, 1u, A.k0, A.k1);
+        const U4 d = draw(j, toy, 2u, A.k0, A.k1);
+        const U4 e = draw(j, toy, 3u, A.k0, A.k1);
+        A.t[pos] = t_of(S, bin_of(S, u01_int(a.x, a.y)), u01_int(d.z, d.w));
+        A.ck[pos] = sym_int(b.x, b.y);
+        A.cl[pos] = sym_int(b.z, b.w);
+        A.phi[pos] = __dmul_rn(cdetail::kPi, sym_int(d.x, d.y));
+        A.q[pos] = tag_of(S, e.x);
+    }
+
+    __device__ __forceinline__ static void background(const Shared& S, const GenArgs& A, uint64_t i, uint32_t toy, int64_t pos) {
+        const U4 a = draw(i, toy, 4u, A.k0, A.k1);
+        const U4 b = draw(i, toy, 5u, A.k0, A.k1);
+        const U4 e = draw(i, toy, 6u, A.k0, A.k1);
+        A.t[pos] = __dadd_rn(S.t_lo, __dmul_rn(u01_int(a.x, a.y), __dsub_rn(S.t_hi, S.t_lo)));
+        A.ck[pos] = sym_int(a.z, a.w);
+        A.cl[pos] = sym_int(b.x, b.y);
+        A.phi[pos] = __dmul_rn(cdetail::kPi, sym_int(b.z, b.w));
+        A.q[pos] = tag_of(S, e.x);
+    }
+
+    __device__ __forceinline__ static void fill_nan(const GenArgs& A, int64_t pos) {
+        A.t[pos] = A.ck[pos] = A.cl[pos] = A.phi[pos] = A.q[pos] = __longlong_as_double(0x7ff8000000000000ll);
+    }
+};
 
 }  // namespace
 
-ipa_status launch_phis_toygen(const ModelDev& m, const Consts* consts, uint64_t seed, int n_toys,
-                              const int64_t* n_sig, const int64_t* n_bkg, const int64_t* offsets,
-                              const ipa_event_buffers* out, cudaStream_t s) {
-    phis_toygen_kernel<<<n_toys, kBlock, 0, s>>>(m, consts, (uint32_t)seed, (uint32_t)(seed >> 32), n_toys, n_sig,
-                                                 n_bkg, offsets, out->capacity, out->t, out->ck, out->cl, out->phi,
-                                                 out->q);
-    return cuda_fail(cudaGetLastError(), "phi_s toygen kernel launch");
-}
+ipa_status launch_phis_toygen(const GenArgs& a, cudaStream_t s) { return launch_generator<PhisGen>(a, s); }
 
 
 namespace {

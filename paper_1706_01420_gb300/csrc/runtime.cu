@@ -63,6 +63,54 @@ ipa_status device_alloc(void** p, size_t bytes, const char* what) {
     return cuda_fail(cudaMalloc(p, bytes), what);
 }
 
+// Stream-ordered temporary memory from a pool of the library's own, one per
+// device: calls that need a workspace of their own size (generators, binned
+// toys) get it without a device synchronisation, on any stream and under
+// stream capture.  The pool keeps at most kPoolKept bytes between calls and
+// returns what is above it to the driver (the default pool keeps nothing, so
+// that the first allocation after every synchronisation maps memory anew).
+namespace {
+constexpr uint64_t kPoolKept = 64ull << 20;
+
+cudaMemPool_t pool_of_device() {
+    static std::mutex mu;
+    static cudaMemPool_t pools[64] = {};
+    static bool tried[64] = {};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+    std::lock_guard<std::mutex> lk(mu);
+    if (!tried[dev]) {
+        tried[dev] = true;
+        cudaMemPoolProps props = {};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        uint64_t kept = kPoolKept;
+        if (cudaMemPoolCreate(&pools[dev], &props) != cudaSuccess) {
+            cudaGetLastError();
+            pools[dev] = nullptr;
+        } else if (cudaMemPoolSetAttribute(pools[dev], cudaMemPoolAttrReleaseThreshold, &kept) != cudaSuccess) {
+            cudaGetLastError();
+        }
+    }
+    return pools[dev];
+}
+}  // namespace
+
+ipa_status pool_alloc(void** p, size_t bytes, cudaStream_t s, const char* what) {
+    *p = nullptr;
+    if (fault(IPA_FAULT_ALLOC)) {
+        set_error("%s: allocation of %zu bytes failed (injected, IPA_FAULT_ALLOC)", what, bytes);
+        return IPA_ERR_OOM;
+    }
+    cudaMemPool_t pool = pool_of_device();
+    return cuda_fail(pool ? cudaMallocFromPoolAsync(p, bytes, pool, s) : cudaMallocAsync(p, bytes, s), what);
+}
+
+void pool_free(void* p, cudaStream_t s) {
+    if (p) cudaFreeAsync(p, s);
+}
+
 void set_error(const char* fmt, ...) {
     va_list ap;
     va_start(ap, fmt);

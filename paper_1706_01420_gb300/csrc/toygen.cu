@@ -17,12 +17,11 @@
 // 32-bit words, in (0, 1].  Candidates are built with correctly rounded
 // multiplies and adds only (no contraction into FMA), so the event values are
 // reproducible bit for bit on any IEEE machine.  A toy keeps its first n_sig
-// accepted candidates in increasing j: one block per toy walks candidate
-// chunks, and a block-wide exclusive scan orders the accepted ones.
+// accepted candidates in increasing j (accept_reject.cuh).
 //
 // Decisions first run in FP32 (this GPU's FP32 rate is 64 times its FP64
 // rate): each test is evaluated with a per-candidate bound on its FP32 error,
-// built from the documented accuracy of expf, erfcf, sincosf and sqrtf and
+// built from the documented accuracy of expf, exp2f, erfcf, sincospif and sqrtf and
 // the rounding of every input, and is decided in FP32 only when the uniform
 // lies outside that band around the threshold.  Inside the band (about one
 // candidate in 10^4), or wherever the bound is not established (a uniform or
@@ -32,7 +31,9 @@
 // are regenerated from their counters and written with the exact FP64 values.
 #include <math.h>
 
+#include "accept_reject.cuh"
 #include "consts.cuh"
+#include "conv32.cuh"
 #include "ipa_internal.cuh"
 #include "philox.cuh"
 #include "tagged.cuh"
@@ -40,13 +41,10 @@
 namespace ipa {
 namespace {
 
-constexpr int kPerThread = 16;             // candidates per thread per chunk (bits of a mask)
-constexpr int kChunk = kBlock * kPerThread;
 constexpr double kPi = 3.14159265358979323846;
 constexpr double kSqrt2 = 1.41421356237309504880;
 constexpr double k2OverSqrt6 = 0.81649658092772603273;
 constexpr double k2OverSqrt3 = 1.15470053837925152902;
-
 
 // A(Omega) = sum_k h_k f_k, evaluated as the oracle's definition (Sec. 4).
 __device__ __forceinline__ double angular_pdf(const Consts& c, double ck, double cl, double phi) {
@@ -86,11 +84,6 @@ struct Filter32 {
     float h[10];
     float bandA;      // absolute band of the angular test: 3e-4 M_Omega
 };
-
-constexpr float kTwoM32 = 2.3283064365386963e-10f;   // 2^-32
-
-// u ~ a 2^-32 from the high word of a uniform: |u32 - u| <= 2^-24 u + 2^-31.
-__device__ __forceinline__ float u32of(uint32_t hi) { return __uint2float_rn(hi) * kTwoM32; }
 
 // +1: u_t M_T < g(t - mu) for sure; -1: not; 0: undecided (FP64 decides).
 // Error bound per candidate (2^-22 ~ 2.4e-7 covers one float rounding with
@@ -135,9 +128,8 @@ __device__ __forceinline__ int angle_filter(const Filter32& f, const U4& b, cons
     const float cl = fmaf(2.0f, u32of(b.z), -1.0f);
     const float sk2 = fmaf(-ck, ck, 1.0f), sl2 = fmaf(-cl, cl, 1.0f);
     if (!(sk2 >= 1.0e-2f) || !(sl2 >= 1.0e-2f)) return 0;
-    const float phi = 3.14159265358979323846f * fmaf(2.0f, u32of(e.x), -1.0f);
     float sp, cp;
-    sincosf(phi, &sp, &cp);
+    sincospif(fmaf(2.0f, u32of(e.x), -1.0f), &sp, &cp);
     const float sk = sqrtf(sk2), sl = sqrtf(sl2);
     const float fk[10] = {ck * ck * sl2,
                           0.5f * sk2 * (1.0f - sl2 * cp * cp),
@@ -160,191 +152,225 @@ __device__ __forceinline__ int angle_filter(const Filter32& f, const U4& b, cons
 }
 
 
-template <int KIND>
-__global__ void __launch_bounds__(kBlock)
-toygen_kernel(ModelDev m, const Consts* __restrict__ consts, uint32_t k0, uint32_t k1, int n_toys,
-              const int64_t* __restrict__ n_sig, const int64_t* __restrict__ n_bkg,
-              const int64_t* __restrict__ offsets, int64_t capacity, double* __restrict__ ot,
-              double* __restrict__ ock, double* __restrict__ ocl, double* __restrict__ ophi) {
-    __shared__ __align__(16) Consts c;
-    __shared__ Filter32 f32;
-    __shared__ int warp_sums[kBlock / 32];
-    {
-        const double* src = reinterpret_cast<const double*>(consts);
-        double* dst = reinterpret_cast<double*>(&c);
+// The decay-time model (angles = false) and the 4D model.
+template <bool ANGLES>
+struct TimeGen {
+    static constexpr bool kQuickKeeps = !ANGLES;
+    static constexpr int kBlocksPerSm = 4;
+    struct Shared {
+        Consts c;
+        Filter32 f;
+        Exp32 e;
+        float near;       // tau above it: z <= -4.3
+        float err;        // relative error bound of the exponential
+        float dl;         // bound of the error of u M_T
+        double t_lo, span;
+    };
+
+    __device__ static void setup(Shared& S, const GenArgs& A) {
+        const double* src = reinterpret_cast<const double*>(A.consts);
+        double* dst = reinterpret_cast<double*>(&S.c);
         for (int i = threadIdx.x; i < kConstsDoubles; i += blockDim.x) dst[i] = src[i];
+        __syncthreads();
+        if (threadIdx.x != 0) return;
+        const Consts& c = S.c;
+        S.t_lo = A.m.t_lo;
+        S.span = __dsub_rn(A.m.t_hi, A.m.t_lo);
+        Filter32& f = S.f;
+        f.d = (float)(A.m.t_lo - c.mu);
+        f.span = (float)S.span;
+        f.Gamma = (float)c.Gamma;
+        f.c_exp = (float)c.c_exp;
+        f.Gs2 = (float)c.Gs2;
+        f.k_z = (float)c.k_z;
+        f.MT = (float)c.MT;
+        f.MO = (float)c.MO;
+        for (int k = 0; k < 10; ++k) f.h[k] = (float)c.h[k];
+        f.bandA = (float)(3.0e-4 * c.MO);
+        const float dtau = kUlp1 * (2.0f * f.span + 2.0f * fabsf(f.d));
+        S.e = exp32_of(c.Gamma, c.c_exp);
+        S.err = exp32_err(S.e, f.span + fabsf(f.d), dtau);
+        // (a negative sigma has no such region: every candidate takes the full test)
+        S.near = c.k_z > 0.0 ? (float)(c.Gs2 + 4.3 / c.k_z) * 1.000001f + 2.0f * dtau : INFINITY;
+        S.dl = f.MT * 1.5e-6f;
     }
-    __syncthreads();
-    const double span = __dsub_rn(m.t_hi, m.t_lo);
-    if (threadIdx.x == 0) {
-        f32.d = (float)(m.t_lo - c.mu);
-        f32.span = (float)span;
-        f32.Gamma = (float)c.Gamma;
-        f32.c_exp = (float)c.c_exp;
-        f32.Gs2 = (float)c.Gs2;
-        f32.k_z = (float)c.k_z;
-        f32.MT = (float)c.MT;
-        f32.MO = (float)c.MO;
-        for (int k = 0; k < 10; ++k) f32.h[k] = (float)c.h[k];
-        f32.bandA = (float)(3.0e-4 * c.MO);
+
+    __device__ static bool usable(const Shared& S) {
+        const Consts& c = S.c;
+        return isfinite(c.MT) && c.MT > 0.0 && isfinite(c.MO) && c.MO > 0.0 && isfinite(c.IT) && c.IT > 0.0;
     }
-    __syncthreads();
-    for (int toy = blockIdx.x; toy < n_toys; toy += gridDim.x) {
-        const int64_t ns = n_sig[toy], nb = n_bkg[toy], off = offsets[toy];
-        if (ns < 0 || nb < 0 || off < 0 || off + ns + nb > capacity) continue;   // skipped
-        // signal: chunks of kChunk candidates, candidate j = j0 + threadIdx.x * kPerThread + i.
-        // Non-finite or non-positive envelopes (non-physical theta) accept nothing: the
-        // signal slots are then filled with NaN instead of searching forever, and so
-        // is whatever remains when the candidate budget runs out.
-        const bool usable = isfinite(c.MT) && c.MT > 0.0 && isfinite(c.MO) && c.MO > 0.0 &&
-                            isfinite(c.IT) && c.IT > 0.0;
-        const uint64_t budget = usable ? (uint64_t)ns * 65536ull + (1ull << 22) : 0ull;
-        int64_t got = 0;
-        uint64_t j0 = 0;
-        for (; got < ns && j0 < budget; j0 += kChunk) {
-            const uint64_t jt = j0 + (uint64_t)threadIdx.x * kPerThread;
-            unsigned mask = 0;
-#pragma unroll 1
-            for (int i = 0; i < kPerThread; ++i) {
-                const uint64_t j = jt + i;
-                const U4 a = draw(j, (uint32_t)toy, 0u, k0, k1);
-                int d = time_filter(f32, a.x, a.z);
-                if (d == 0) {
-                    const double t = __dadd_rn(m.t_lo, __dmul_rn(u01(a.x, a.y), span));
-                    d = __dmul_rn(u01(a.z, a.w), c.MT) < time_pdf(c, t) ? 1 : -1;
-                }
-                if (KIND == IPA_MODEL_ANGTIME4D && d > 0) {
-                    const U4 b = draw(j, (uint32_t)toy, 1u, k0, k1);
-                    const U4 e = draw(j, (uint32_t)toy, 2u, k0, k1);
-                    d = angle_filter(f32, b, e);
-                    if (d == 0) {
-                        const double ck = __dsub_rn(__dmul_rn(2.0, u01(b.x, b.y)), 1.0);
-                        const double cl = __dsub_rn(__dmul_rn(2.0, u01(b.z, b.w)), 1.0);
-                        const double phi = __dmul_rn(kPi, __dsub_rn(__dmul_rn(2.0, u01(e.x, e.y)), 1.0));
-                        d = __dmul_rn(u01(e.z, e.w), c.MO) < angular_pdf(c, ck, cl, phi) ? 1 : -1;
-                    }
-                }
-                if (d > 0) mask |= 1u << i;
-            }
-            int total;
-            const int before = block_exclusive_scan(__popc(mask), warp_sums, &total);
-            int rank = 0;
-            // accepted candidates are regenerated from their counters (exact FP64 values)
-            while (mask) {
-                const int i = __ffs(mask) - 1;
-                mask &= mask - 1u;
-                const int64_t pos = got + before + rank;
-                ++rank;
-                if (pos >= ns) break;
-                const uint64_t j = jt + i;
-                const U4 a = draw(j, (uint32_t)toy, 0u, k0, k1);
-                ot[off + pos] = __dadd_rn(m.t_lo, __dmul_rn(u01(a.x, a.y), span));
-                if (KIND == IPA_MODEL_ANGTIME4D) {
-                    const U4 b = draw(j, (uint32_t)toy, 1u, k0, k1);
-                    const U4 e = draw(j, (uint32_t)toy, 2u, k0, k1);
-                    ock[off + pos] = __dsub_rn(__dmul_rn(2.0, u01(b.x, b.y)), 1.0);
-                    ocl[off + pos] = __dsub_rn(__dmul_rn(2.0, u01(b.z, b.w)), 1.0);
-                    ophi[off + pos] = __dmul_rn(kPi, __dsub_rn(__dmul_rn(2.0, u01(e.x, e.y)), 1.0));
-                }
-            }
-            got += total;
-        }
-        for (int64_t pos = got + threadIdx.x; pos < ns; pos += blockDim.x) {
-            ot[off + pos] = __longlong_as_double(0x7ff8000000000000ll);
-            if (KIND == IPA_MODEL_ANGTIME4D)
-                ock[off + pos] = ocl[off + pos] = ophi[off + pos] = __longlong_as_double(0x7ff8000000000000ll);
-        }
-        // background: uniform in the box, always kept
-        for (int64_t i = threadIdx.x; i < nb; i += blockDim.x) {
-            const U4 a = draw((uint64_t)i, (uint32_t)toy, 4u, k0, k1);
-            const int64_t pos = off + ns + i;
-            ot[pos] = __dadd_rn(m.t_lo, __dmul_rn(u01(a.x, a.y), span));
-            if (KIND == IPA_MODEL_ANGTIME4D) {
-                const U4 b = draw((uint64_t)i, (uint32_t)toy, 5u, k0, k1);
-                ock[pos] = __dsub_rn(__dmul_rn(2.0, u01(a.z, a.w)), 1.0);
-                ocl[pos] = __dsub_rn(__dmul_rn(2.0, u01(b.x, b.y)), 1.0);
-                ophi[pos] = __dmul_rn(kPi, __dsub_rn(__dmul_rn(2.0, u01(b.z, b.w)), 1.0));
-            }
-        }
+
+    // integral of g A over the box (I_T 16 pi / 9) over the envelope's (M_T M_Omega span 8 pi)
+    __device__ static void acceptance(const GenArgs& A, float* acc) {
+        if (threadIdx.x != 0) return;
+        const Consts& c = *A.consts;
+        float v = (float)c.IT / ((float)c.MT * (float)(A.m.t_hi - A.m.t_lo));
+        if (ANGLES) v *= (2.0f / 9.0f) / (float)c.MO;
+        *acc = v;
     }
-}
+
+    // The decay-time test away from the resolution peak, where g is the exponential alone.
+    __device__ __forceinline__ static GenCode quick(const Shared& S, uint64_t j, uint32_t toy, uint32_t k0, uint32_t k1) {
+        const U4 a = draw(j, toy, 0u, k0, k1);
+        const float tau = fmaf(u32of(a.x), S.f.span, S.f.d);
+        const float arg = fmaf(-S.e.x, tau, S.e.off);
+        const float g = exp2f(arg);
+        const float lhs = u32of(a.z) * S.f.MT;
+        if (!(tau > S.near) || !(fabsf(arg) <= kMaxArg) || !(S.err <= 1.0e-3f)) return kTest32;
+        const GenCode c = decide32(lhs, S.dl, g, g * S.err);
+        return ANGLES ? (c == kDrop ? kDrop : kTest32) : c;
+    }
+
+    __device__ __forceinline__ static GenCode test32(const Shared& S, uint64_t j, uint32_t toy, uint32_t k0, uint32_t k1) {
+        const U4 a = draw(j, toy, 0u, k0, k1);
+        int d = time_filter(S.f, a.x, a.z);
+        if (d < 0) return kDrop;
+        if (!ANGLES) return d > 0 ? kKeep : kTest64;
+        const U4 b = draw(j, toy, 1u, k0, k1);
+        const U4 e = draw(j, toy, 2u, k0, k1);
+        const int f = angle_filter(S.f, b, e);
+        if (f < 0) return kDrop;
+        return d > 0 && f > 0 ? kKeep : kTest64;
+    }
+
+    __device__ __noinline__ static bool test64(const Shared& S, uint64_t j, uint32_t toy, uint32_t k0, uint32_t k1) {
+        const U4 a = draw(j, toy, 0u, k0, k1);
+        const double t = __dadd_rn(S.t_lo, __dmul_rn(u01_int(a.x, a.y), S.span));
+        if (!(__dmul_rn(u01_int(a.z, a.w), S.c.MT) < time_pdf(S.c, t))) return false;
+        if (!ANGLES) return true;
+        const U4 b = draw(j, toy, 1u, k0, k1);
+        const U4 e = draw(j, toy, 2u, k0, k1);
+        return __dmul_rn(u01_int(e.z, e.w), S.c.MO) <
+               angular_pdf(S.c, sym_int(b.x, b.y), sym_int(b.z, b.w), __dmul_rn(kPi, sym_int(e.x, e.y)));
+    }
+
+    __device__ __forceinline__ static void signal(const Shared& S, const GenArgs& A, uint64_t j, uint32_t toy, int64_t pos) {
+        const U4 a = draw(j, toy, 0u, A.k0, A.k1);
+        A.t[pos] = __dadd_rn(S.t_lo, __dmul_rn(u01_int(a.x, a.y), S.span));
+        if (!ANGLES) return;
+        const U4 b = draw(j, toy, 1u, A.k0, A.k1);
+        const U4 e = draw(j, toy, 2u, A.k0, A.k1);
+        A.ck[pos] = sym_int(b.x, b.y);
+        A.cl[pos] = sym_int(b.z, b.w);
+        A.phi[pos] = __dmul_rn(kPi, sym_int(e.x, e.y));
+    }
+
+    // background: uniform in the box, always kept
+    __device__ __forceinline__ static void background(const Shared& S, const GenArgs& A, uint64_t i, uint32_t toy, int64_t pos) {
+        const U4 a = draw(i, toy, 4u, A.k0, A.k1);
+        A.t[pos] = __dadd_rn(S.t_lo, __dmul_rn(u01_int(a.x, a.y), S.span));
+        if (!ANGLES) return;
+        const U4 b = draw(i, toy, 5u, A.k0, A.k1);
+        A.ck[pos] = sym_int(a.z, a.w);
+        A.cl[pos] = sym_int(b.x, b.y);
+        A.phi[pos] = __dmul_rn(kPi, sym_int(b.z, b.w));
+    }
+
+    __device__ __forceinline__ static void fill_nan(const GenArgs& A, int64_t pos) {
+        const double nan = __longlong_as_double(0x7ff8000000000000ll);
+        A.t[pos] = nan;
+        if (ANGLES) A.ck[pos] = A.cl[pos] = A.phi[pos] = nan;
+    }
+};
 
 // The tagged model: candidate j of toy k takes (t, u) from call 0 and the tag
-// from the first uniform of call 1 (q = +1 if u_q <= 1/2, else -1), and is
-// kept iff u M_S < S(t - mu, q), S evaluated in FP64 with the exact forms of
-// tagged.cuh (no filter: the FP64 test runs for every candidate).  Background
-// event i takes t and q from call 4.
-__global__ void __launch_bounds__(kBlock)
-toygen_tag_kernel(ModelDev m, const Consts* __restrict__ consts, uint32_t k0, uint32_t k1, int n_toys,
-                  const int64_t* __restrict__ n_sig, const int64_t* __restrict__ n_bkg,
-                  const int64_t* __restrict__ offsets, int64_t capacity, double* __restrict__ ot,
-                  double* __restrict__ oq) {
-    __shared__ __align__(16) TagConsts c;
-    __shared__ int warp_sums[kBlock / 32];
-    {
-        const double* src = reinterpret_cast<const double*>(consts);
-        double* dst = reinterpret_cast<double*>(&c);
+// from the first uniform of call 1 (q = +1 if u_q <= 1/2, which is the top bit
+// of its first word being clear), and is kept iff u M_S < S(t - mu, q) with S
+// in FP64 with the exact forms of tagged.cuh.  Background event i takes t and q
+// from call 4.
+//
+// FP32: away from the peak the four convolutions are exponentials; quick()
+// drops a candidate that the oscillation's amplitude cannot lift over its
+// threshold (nine in ten) without drawing the tag, test32() evaluates the
+// oscillation, near the peak with FP32 erfc and Faddeeva functions.
+struct TagGen {
+    static constexpr bool kQuickKeeps = false;
+    static constexpr int kBlocksPerSm = 3;
+    struct Shared {
+        TagConsts c;
+        Conv32 v;
+        float aH, aL, Ds, MS, dl;
+        double t_lo, span;
+        float f_span;
+    };
+
+    __device__ static void setup(Shared& S, const GenArgs& A) {
+        const double* src = reinterpret_cast<const double*>(A.consts);
+        double* dst = reinterpret_cast<double*>(&S.c);
         for (int i = threadIdx.x; i < kTagConstsDoubles; i += blockDim.x) dst[i] = src[i];
+        __syncthreads();
+        if (threadIdx.x != 0) return;
+        S.t_lo = A.m.t_lo;
+        S.span = __dsub_rn(A.m.t_hi, A.m.t_lo);
+        S.f_span = (float)S.span;
+        S.v = conv32_of(S.c, A.m.t_lo - S.c.mu, S.span);
+        S.aH = (float)S.c.aH;
+        S.aL = (float)S.c.aL;
+        S.Ds = (float)S.c.Ds;
+        S.MS = (float)S.c.MS;
+        S.dl = S.MS * 1.5e-6f;
     }
-    __syncthreads();
-    const double span = __dsub_rn(m.t_hi, m.t_lo);
-    const double nan = __longlong_as_double(0x7ff8000000000000ll);
-    for (int toy = blockIdx.x; toy < n_toys; toy += gridDim.x) {
-        const int64_t ns = n_sig[toy], nb = n_bkg[toy], off = offsets[toy];
-        if (ns < 0 || nb < 0 || off < 0 || off + ns + nb > capacity) continue;   // skipped
-        const bool usable = isfinite(c.MS) && c.MS > 0.0 && isfinite(c.N) && c.N > 0.0;
-        const uint64_t budget = usable ? (uint64_t)ns * 65536ull + (1ull << 22) : 0ull;
-        int64_t got = 0;
-        uint64_t j0 = 0;
-        for (; got < ns && j0 < budget; j0 += kChunk) {
-            const uint64_t jt = j0 + (uint64_t)threadIdx.x * kPerThread;
-            unsigned mask = 0;
-#pragma unroll 1
-            for (int i = 0; i < kPerThread; ++i) {
-                const uint64_t j = jt + i;
-                const U4 a = draw(j, (uint32_t)toy, 0u, k0, k1);
-                const U4 b = draw(j, (uint32_t)toy, 1u, k0, k1);
-                const double t = __dadd_rn(m.t_lo, __dmul_rn(u01(a.x, a.y), span));
-                const double q = u01(b.x, b.y) <= 0.5 ? 1.0 : -1.0;
-                if (__dmul_rn(u01(a.z, a.w), c.MS) < tag_signal(c, t, q)) mask |= 1u << i;
-            }
-            int total;
-            const int before = block_exclusive_scan(__popc(mask), warp_sums, &total);
-            int rank = 0;
-            while (mask) {
-                const int i = __ffs(mask) - 1;
-                mask &= mask - 1u;
-                const int64_t pos = got + before + rank;
-                ++rank;
-                if (pos >= ns) break;
-                const uint64_t j = jt + i;
-                const U4 a = draw(j, (uint32_t)toy, 0u, k0, k1);
-                const U4 b = draw(j, (uint32_t)toy, 1u, k0, k1);
-                ot[off + pos] = __dadd_rn(m.t_lo, __dmul_rn(u01(a.x, a.y), span));
-                oq[off + pos] = u01(b.x, b.y) <= 0.5 ? 1.0 : -1.0;
-            }
-            got += total;
-        }
-        for (int64_t pos = got + threadIdx.x; pos < ns; pos += blockDim.x) ot[off + pos] = oq[off + pos] = nan;
-        for (int64_t i = threadIdx.x; i < nb; i += blockDim.x) {
-            const U4 a = draw((uint64_t)i, (uint32_t)toy, 4u, k0, k1);
-            const int64_t pos = off + ns + i;
-            ot[pos] = __dadd_rn(m.t_lo, __dmul_rn(u01(a.x, a.y), span));
-            oq[pos] = u01(a.z, a.w) <= 0.5 ? 1.0 : -1.0;
-        }
+
+    __device__ static bool usable(const Shared& S) {
+        return isfinite(S.c.MS) && S.c.MS > 0.0 && isfinite(S.c.N) && S.c.N > 0.0;
     }
-}
+
+    // N is the integral over both tags, each drawn half of the time
+    __device__ static void acceptance(const GenArgs& A, float* acc) {
+        if (threadIdx.x != 0) return;
+        const TagConsts& c = *reinterpret_cast<const TagConsts*>(A.consts);
+        *acc = 0.5f * (float)c.N / ((float)c.MS * (float)(A.m.t_hi - A.m.t_lo));
+    }
+
+    __device__ __forceinline__ static GenCode quick(const Shared& S, uint64_t j, uint32_t toy, uint32_t k0, uint32_t k1) {
+        const U4 a = draw(j, toy, 0u, k0, k1);
+        const float tau = fmaf(u32of(a.x), S.f_span, S.v.d);
+        const float lhs = u32of(a.z) * S.MS;
+        const Far32 g = conv32_far(S.v, tau);
+        if (!g.ok) return kTest32;
+        const float most = S.aH * g.H + S.aL * g.L + fabsf(S.Ds) * g.C;
+        return lhs - S.dl > most * (1.0f + S.v.err) ? kDrop : kTest32;
+    }
+
+    __device__ __forceinline__ static GenCode test32(const Shared& S, uint64_t j, uint32_t toy, uint32_t k0, uint32_t k1) {
+        const U4 a = draw(j, toy, 0u, k0, k1);
+        const U4 b = draw(j, toy, 1u, k0, k1);
+        const float tau = fmaf(u32of(a.x), S.f_span, S.v.d);
+        const float q = (b.x >> 31) ? -1.0f : 1.0f;
+        const Time32 g = conv32(S.v, tau);
+        const float sig = S.aH * g.H + S.aL * g.L + q * S.Ds * g.Ci;
+        const float err = (S.aH * g.H + S.aL * g.L + fabsf(S.Ds) * g.C) * g.err;
+        return decide32(u32of(a.z) * S.MS, S.dl, sig, err);
+    }
+
+    __device__ __noinline__ static bool test64(const Shared& S, uint64_t j, uint32_t toy, uint32_t k0, uint32_t k1) {
+        const U4 a = draw(j, toy, 0u, k0, k1);
+        const U4 b = draw(j, toy, 1u, k0, k1);
+        const double t = __dadd_rn(S.t_lo, __dmul_rn(u01_int(a.x, a.y), S.span));
+        return __dmul_rn(u01_int(a.z, a.w), S.c.MS) < tag_signal(S.c, t, tag_of(b.x));
+    }
+
+    __device__ __forceinline__ static double tag_of(uint32_t hi) { return (hi >> 31) ? -1.0 : 1.0; }
+
+    __device__ __forceinline__ static void signal(const Shared& S, const GenArgs& A, uint64_t j, uint32_t toy, int64_t pos) {
+        const U4 a = draw(j, toy, 0u, A.k0, A.k1);
+        const U4 b = draw(j, toy, 1u, A.k0, A.k1);
+        A.t[pos] = __dadd_rn(S.t_lo, __dmul_rn(u01_int(a.x, a.y), S.span));
+        A.q[pos] = tag_of(b.x);
+    }
+
+    __device__ __forceinline__ static void background(const Shared& S, const GenArgs& A, uint64_t i, uint32_t toy, int64_t pos) {
+        const U4 a = draw(i, toy, 4u, A.k0, A.k1);
+        A.t[pos] = __dadd_rn(S.t_lo, __dmul_rn(u01_int(a.x, a.y), S.span));
+        A.q[pos] = tag_of(a.z);
+    }
+
+    __device__ __forceinline__ static void fill_nan(const GenArgs& A, int64_t pos) {
+        A.t[pos] = A.q[pos] = __longlong_as_double(0x7ff8000000000000ll);
+    }
+};
 
 }  // namespace
-
-ipa_status launch_tag_toygen(const ModelDev& m, const Consts* consts, uint64_t seed, int n_toys,
-                             const int64_t* n_sig, const int64_t* n_bkg, const int64_t* offsets,
-                             const ipa_event_buffers* out, cudaStream_t s) {
-    toygen_tag_kernel<<<n_toys, kBlock, 0, s>>>(m, consts, (uint32_t)seed, (uint32_t)(seed >> 32), n_toys, n_sig,
-                                                n_bkg, offsets, out->capacity, out->t, out->q);
-    return cuda_fail(cudaGetLastError(), "tagged toygen kernel launch");
-}
-
 }  // namespace ipa
 
 extern "C" ipa_status ipa_toygen(const ipa_model* model, const double* theta_dev, uint64_t seed,
@@ -383,17 +409,23 @@ extern "C" ipa_status ipa_toygen(const ipa_model* model, const double* theta_dev
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const ModelDev m{model->kind, model->n_par, model->t_lo, model->t_hi};
     if ((st = launch_consts(m, theta_dev, 1, sc->consts, s)) != IPA_OK) return st;
-    if (tag) return launch_tag_toygen(m, sc->consts, seed, n_toys, n_sig_dev, n_bkg_dev, offsets_dev, out, s);
-    if (phis) return launch_phis_toygen(m, sc->consts, seed, n_toys, n_sig_dev, n_bkg_dev, offsets_dev, out, s);
-    const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
-    const int grid = n_toys;
-    if (four)
-        toygen_kernel<IPA_MODEL_ANGTIME4D><<<grid, kBlock, 0, s>>>(
-            m, sc->consts, k0, k1, n_toys, n_sig_dev, n_bkg_dev, offsets_dev, out->capacity, out->t,
-            out->ck, out->cl, out->phi);
-    else
-        toygen_kernel<IPA_MODEL_TIME1D><<<grid, kBlock, 0, s>>>(
-            m, sc->consts, k0, k1, n_toys, n_sig_dev, n_bkg_dev, offsets_dev, out->capacity, out->t,
-            nullptr, nullptr, nullptr);
-    return cuda_fail(cudaGetLastError(), "toygen kernel launch");
+    GenArgs a{};
+    a.m = m;
+    a.consts = sc->consts;
+    a.k0 = (uint32_t)seed;
+    a.k1 = (uint32_t)(seed >> 32);
+    a.n_toys = n_toys;
+    a.n_sig = n_sig_dev;
+    a.n_bkg = n_bkg_dev;
+    a.offsets = offsets_dev;
+    a.capacity = out->capacity;
+    a.t = out->t;
+    a.ck = out->ck;
+    a.cl = out->cl;
+    a.phi = out->phi;
+    a.q = out->q;
+    if (tag) return launch_generator<TagGen>(a, s);
+    if (phis) return launch_phis_toygen(a, s);
+    if (four) return launch_generator<TimeGen<true>>(a, s);
+    return launch_generator<TimeGen<false>>(a, s);
 }
