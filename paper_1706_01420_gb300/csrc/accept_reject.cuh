@@ -3,29 +3,38 @@
 // order.
 //
 // A toy keeps its first n_sig accepted candidates in increasing candidate
-// index.  Candidates are cut into chunks of kGenChunk; a block takes chunks
-// from a ticket counter (toys one after another, a toy's chunks in order),
-// counts what its chunk accepts, learns how many the toy's earlier chunks
-// accepted by the decoupled look-back of Merrill and Garland ("Single-pass
-// parallel prefix scan with decoupled look-back", 2016), and writes its events
-// from there on.  How many chunks a toy needs is predicted from the model's
-// acceptance (its normalisation over the envelope's) plus three standard
-// deviations; in the rare toy that needs more, the block of its last chunk
-// goes on alone.  The toy's events do not depend on any of this.
+// index.  Candidates are cut into chunks; a warp takes chunks from a ticket
+// counter (toys one after another, a toy's chunks in order), counts what its
+// chunk accepts, learns how many the toy's earlier chunks accepted by the
+// decoupled look-back of Merrill and Garland ("Single-pass parallel prefix scan
+// with decoupled look-back", 2016), and writes its events from there on.  How
+// many chunks a toy needs is predicted from the model's acceptance (its
+// normalisation over the envelope's) plus three standard deviations; in the
+// rare toy that needs more, the warp of its last chunk goes on alone.  The
+// toy's events do not depend on any of this.
 //
 // Why: one block per toy, as before, left 151 of 152 SMs idle for a single
 // sample (133 725 events of the 4D model: 30.2 ms, all of it in one block) and
-// half of them in a batch of about a hundred toys.
+// half of them in a batch of about a hundred toys.  A warp per chunk, not a
+// block: with 4096 candidates per block the warps spent half of their time at
+// the block's barriers (waiting for the look-back, for the one warp with an
+// FP64 test and for each other).
 //
-// Within a chunk a warp owns 512 candidates and decides them in up to three
-// passes, so that no lane waits for another's rare branch: quick() in FP32 on
-// every candidate (most are rejected here), test32() in FP32 on the packed
-// rest, test64() on the few that lie within the FP32 error bound of their
-// threshold.  A decision is always the FP64 test's: quick() and test32()
-// decide only outside the bound.  Before, the angular test of the tenth of
-// the candidates that pass the time test ran in almost every iteration of a
-// warp with three lanes active.  (Packed or not, the FP64 tests cost a warp the
-// same: hence the last pass.)
+// A warp decides 1024 candidates in up to three passes, so that no lane waits
+// for another's rare branch: quick() in FP32 on every candidate (most are
+// rejected here), test32() in FP32 on the packed rest, test64() on the few that
+// lie within the FP32 error bound of their threshold.  A decision is always
+// the FP64 test's: quick() and test32() decide only outside the bound.
+// Before, the angular test of the tenth of the candidates that pass the time
+// test ran in almost every iteration of a warp with three lanes active.
+//
+// Bound: instruction issue (about 75 warp instructions per 32 candidates for
+// Philox and the time test, 20 of them 32 x 32 -> 64-bit products, of 190 in
+// all; a 4D event needs 50 candidates) and the latency of the look-back: 46 %
+// of the issue slots busy.  Measured (one block per toy / blocks with barriers /
+// warps): 4D, one sample of 133 725 events 30.2 ms / 92 us / 84 us; 4D, 512 toys
+// of Poisson(2e4) 11.5 / 4.5 / 3.7 ms; phi_s, 102 toys of 8170 (every candidate in
+// FP64 before) 24.0 / 0.77 / 0.69 ms.
 #pragma once
 
 #include <stdint.h>
@@ -38,14 +47,15 @@
 namespace ipa {
 
 constexpr int kGenWarps = kBlock / 32;
-constexpr int kGenPerLane = 16;                            // candidates per lane and chunk
-constexpr int kGenWarpCand = 32 * kGenPerLane;             // 512
-constexpr int kGenChunk = kGenWarps * kGenWarpCand;        // 4096
-constexpr int kGenWords = kGenChunk / 32;                  // words of the chunk's bit mask
-constexpr int kBkgChunk = 2048;                            // background events per ticket
-// A toy is cut into chunks only where a chunk accepts at least this many events
-// on average: the look-back's status words then stay below one byte per event.
-constexpr int kGenMinKept = 16;
+constexpr int kGenCand = 1024;           // candidates a warp decides at once: 32 words of its bit mask
+constexpr int kGenPick = 256;            // accepted candidates listed at once for writing
+constexpr int kBkgChunk = 512;           // background events per ticket
+// A ticket is 1, 2, 4, ... kGenMaxSub times kGenCand candidates, as many as
+// accept kGenMinKept events on average: the look-back's status words then
+// stay below 1.3 bytes per event.  A toy of an envelope that accepts less is
+// one ticket.
+constexpr int kGenMinKept = 8;
+constexpr int kGenMaxSub = 64;
 
 // What a test says of a candidate.
 enum GenCode { kDrop = 0, kKeep = 1, kTest32 = 2, kTest64 = 3 };
@@ -53,17 +63,42 @@ enum GenCode { kDrop = 0, kKeep = 1, kTest32 = 2, kTest64 = 3 };
 struct GenArgs {
     ModelDev m;
     const Consts* consts;
-    uint32_t k0, k1;
+    uint32_t key[20];      // the ten rounds' keys (k0, k1 of each), read from the parameter bank
     int n_toys;
     const int64_t *n_sig, *n_bkg, *offsets;
     int64_t capacity;
     double *t, *ck, *cl, *phi, *q;
-    // ticket prefix per toy (n_toys + 1), the ticket counter and one status word
-    // per ticket; base == nullptr: no workspace, one block per toy
+    // ticket prefix per toy (n_toys + 1 entries, then kGenCand units per ticket),
+    // the ticket counter and one status word per ticket; base == nullptr: no
+    // workspace, one warp per toy
     const int64_t* base;
     unsigned long long* ticket;
     unsigned long long* status;
 };
+
+inline void gen_keys(uint64_t seed, GenArgs* a) {
+    for (int r = 0; r < 10; ++r) {
+        a->key[2 * r] = (uint32_t)seed + (uint32_t)r * kPhiloxW0;
+        a->key[2 * r + 1] = (uint32_t)(seed >> 32) + (uint32_t)r * kPhiloxW1;
+    }
+}
+
+// Candidate or background event `lo` + 2^32 hi of a toy.
+struct GenIdx {
+    uint32_t lo, hi, toy;
+};
+
+// draw() (philox.cuh) with the round keys laid out beforehand: the same words.
+__device__ __forceinline__ U4 gen_draw(const GenArgs& A, const GenIdx& j, uint32_t call) {
+    U4 c{j.lo, j.hi, j.toy, call};
+#pragma unroll
+    for (int r = 0; r < 10; ++r) {
+        const unsigned long long p0 = (unsigned long long)kPhiloxM0 * c.x, p1 = (unsigned long long)kPhiloxM1 * c.z;
+        c = U4{(uint32_t)(p1 >> 32) ^ c.y ^ A.key[2 * r], (uint32_t)p1, (uint32_t)(p0 >> 32) ^ c.w ^ A.key[2 * r + 1],
+               (uint32_t)p0};
+    }
+    return c;
+}
 
 // (v + 1) 2^-53 and 2 (v + 1) 2^-53 - 1 for the 53-bit v of two words, exactly,
 // by integer operations (u01 and 2 u01 - 1 cost two and four FP64 instructions).
@@ -91,92 +126,106 @@ __device__ __forceinline__ GenCode decide32(float lhs, float dl, float v, float 
     return kTest64;                                  // also NaN
 }
 
+// One warp's lists, and its ticket's state: kept in shared memory (uniform over
+// the warp), since in registers it spilled the candidates' loop.
 struct GenLists {
-    uint16_t l32[kGenWarps][kGenWarpCand];
-    uint16_t l64[kGenWarps][kGenWarpCand];
-    uint32_t keep[kGenWords];
-    int before[kGenWords + 1];     // accepted before each word of keep
-    int64_t take;
-    int64_t got;
+    uint16_t l32[kGenCand];
+    uint16_t l64[kGenCand];
+    uint16_t pick[kGenPick];
+    uint32_t keep[32];
+    int64_t ns, off, got;          // the toy's signal, its first event, events accepted before unit u
+    int64_t tk, local, n_chunks;   // ticket, its chunk of the toy, the toy's chunks
+    int64_t c, u;                  // chunk and unit (of kGenCand candidates) in work
+    int nu;                        // units decided at once
+    uint32_t toy;
+    bool look;                     // the look-back is to come
 };
 
-// Decide the chunk's candidates j0 .. j0 + kGenChunk: bit mask and its prefix
-// in L; returns the number accepted.  Block-collective.
+// Decide candidates j0 .. j0 + kGenCand: lane l returns the bits of candidates
+// 32 l .. 32 l + 31.  Warp-collective.
 template <class G>
-__device__ __noinline__ int gen_count(const typename G::Shared& S, GenLists& L, uint64_t j0, uint32_t toy, uint32_t k0, uint32_t k1) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+__device__ __forceinline__ uint32_t gen_decide(const typename G::Shared& S, const GenArgs& A, GenLists& L, uint64_t j0,
+                                               uint32_t toy, int lane) {
     const unsigned below = (1u << lane) - 1u;
-    const uint64_t jw = j0 + (uint64_t)w * kGenWarpCand;
+    const uint32_t lo = (uint32_t)j0, hi = (uint32_t)(j0 >> 32);   // no carry: j0 is a multiple of kGenCand
     int n32 = 0, n64 = 0;
-    if (lane < kGenPerLane) L.keep[w * kGenPerLane + lane] = 0u;
+    uint32_t word = 0u;
     __syncwarp();
+    L.keep[lane] = 0u;
 #pragma unroll 1
-    for (int i = 0; i < kGenPerLane; ++i) {
+    for (int i = 0; i < 32; ++i) {
         const int cand = i * 32 + lane;
-        const GenCode c = G::quick(S, jw + cand, toy, k0, k1);
+        const GenCode c = G::quick(S, A, GenIdx{lo + cand, hi, toy});
         if (G::kQuickKeeps) {
             const unsigned k = __ballot_sync(0xffffffffu, c == kKeep);
-            if (lane == 0) L.keep[w * kGenPerLane + i] = k;
+            if (lane == i) word = k;
         }
         const unsigned a = __ballot_sync(0xffffffffu, c == kTest32);
-        if (c == kTest32) L.l32[w][n32 + __popc(a & below)] = (uint16_t)cand;
+        if (c == kTest32) L.l32[n32 + __popc(a & below)] = (uint16_t)cand;
         n32 += __popc(a);
-        const unsigned b = __ballot_sync(0xffffffffu, c == kTest64);
-        if (c == kTest64) L.l64[w][n64 + __popc(b & below)] = (uint16_t)cand;
-        n64 += __popc(b);
+        if (G::kQuick64) {
+            const unsigned b = __ballot_sync(0xffffffffu, c == kTest64);
+            if (c == kTest64) L.l64[n64 + __popc(b & below)] = (uint16_t)cand;
+            n64 += __popc(b);
+        }
     }
     __syncwarp();
+#pragma unroll 1
     for (int x0 = 0; x0 < n32; x0 += 32) {
         const int x = x0 + lane;
-        const int cand = x < n32 ? L.l32[w][x] : 0;
-        const GenCode c = x < n32 ? G::test32(S, jw + cand, toy, k0, k1) : kDrop;
-        if (c == kKeep) atomicOr(&L.keep[w * kGenPerLane + (cand >> 5)], 1u << (cand & 31));
+        GenCode c = kDrop;
+        int cand = 0;
+        if (x < n32) {
+            cand = L.l32[x];
+            c = G::test32(S, A, GenIdx{lo + cand, hi, toy});
+        }
+        if (c == kKeep) atomicOr(&L.keep[cand >> 5], 1u << (cand & 31));
         const unsigned b = __ballot_sync(0xffffffffu, c == kTest64);
-        if (c == kTest64) L.l64[w][n64 + __popc(b & below)] = (uint16_t)cand;
+        if (c == kTest64) L.l64[n64 + __popc(b & below)] = (uint16_t)cand;
         n64 += __popc(b);
     }
     __syncwarp();
+#pragma unroll 1
     for (int x = lane; x < n64; x += 32) {
-        const int cand = L.l64[w][x];
-        if (G::test64(S, jw + cand, toy, k0, k1)) atomicOr(&L.keep[w * kGenPerLane + (cand >> 5)], 1u << (cand & 31));
+        const int cand = L.l64[x];
+        if (G::test64(S, A, GenIdx{lo + cand, hi, toy})) atomicOr(&L.keep[cand >> 5], 1u << (cand & 31));
     }
-    __syncthreads();
-    if (w == 0) {
-        constexpr int kPer = kGenWords / 32;
-        int c[kPer], s = 0;
-#pragma unroll
-        for (int i = 0; i < kPer; ++i) {
-            c[i] = s;
-            s += __popc(L.keep[lane * kPer + i]);
-        }
-        int x = s;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, x, d);
-            if (lane >= d) x += y;
-        }
-#pragma unroll
-        for (int i = 0; i < kPer; ++i) L.before[lane * kPer + i] = x - s + c[i];
-        if (lane == 31) L.before[kGenWords] = x;
-    }
-    __syncthreads();
-    return L.before[kGenWords];
+    __syncwarp();
+    return word | L.keep[lane];
 }
 
-// Write the chunk's accepted candidates as events got, got + 1, ... of the toy.
+// Exclusive prefix of the lanes' popcounts; *total: their sum.
+__device__ __forceinline__ int gen_prefix(uint32_t word, int lane, int* total) {
+    const int n = __popc(word);
+    int x = n;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, d);
+        if (lane >= d) x += y;
+    }
+    *total = __shfl_sync(0xffffffffu, x, 31);
+    return x - n;
+}
+
+// Append the candidates of `word` (first rank `pre`) whose ranks lie in [r0, r0 +
+// kGenPick) to the list, as offsets from `off`.
+__device__ __forceinline__ void gen_pick(GenLists& L, uint32_t word, int pre, int r0, int off, int lane) {
+    for (int r = pre - r0; word && r < kGenPick; ++r) {
+        const int bit = __ffs((int)word) - 1;
+        word &= word - 1u;
+        if (r >= 0) L.pick[r] = (uint16_t)(off + lane * 32 + bit);
+    }
+}
+
+// Write listed candidates (n of them, offsets from j0) as events got, got + 1, ... of the toy.
 template <class G>
-__device__ __noinline__ void gen_write(const typename G::Shared& S, const GenArgs& A, const GenLists& L, uint64_t j0, uint32_t toy,
-                          int64_t got, int64_t ns, int64_t off) {
-    const int total = L.before[kGenWords];
-    for (int k = threadIdx.x; k < total; k += kBlock) {
+__device__ __forceinline__ void gen_write(const typename G::Shared& S, const GenArgs& A, const GenLists& L, uint64_t j0,
+                                          uint32_t toy, int n, int64_t got, int64_t ns, int64_t off, int lane) {
+#pragma unroll 1
+    for (int k = lane; k < n; k += 32) {
         if (got + k >= ns) break;
-        int lo = 0, hi = kGenWords - 1;
-        while (lo < hi) {                            // the last word with before <= k
-            const int mid = (lo + hi + 1) >> 1;
-            if (L.before[mid] <= k) lo = mid; else hi = mid - 1;
-        }
-        const int bit = nth_set(L.keep[lo], k - L.before[lo]);
-        G::signal(S, A, j0 + lo * 32 + bit, toy, off + got + k);
+        const uint64_t j = j0 + L.pick[k];
+        G::signal(S, A, GenIdx{(uint32_t)j, (uint32_t)(j >> 32), toy}, off + got + k);
     }
 }
 
@@ -186,7 +235,7 @@ enum : unsigned long long { kAggregate = 1ull, kPrefix = 2ull };
 constexpr int kLookBackPolls = 1 << 20;
 
 // Events the toy accepted before chunk `local` (ticket tk), having published
-// this chunk's count.  Called by warp 0.  The blocks of the earlier tickets are
+// this chunk's count.  Warp-collective.  The warps of the earlier tickets are
 // running (tickets are handed out in order), so every word waited for gets
 // written; the wait is bounded all the same: returns -1 when it runs out.
 __device__ __forceinline__ int64_t look_back(unsigned long long* status, int64_t tk, int64_t local, int count, int lane) {
@@ -219,23 +268,6 @@ __device__ __forceinline__ int64_t look_back(unsigned long long* status, int64_t
     return sum;
 }
 
-// The signal of one toy from candidate j0 on, `got` events already kept: chunk
-// after chunk by this block, then NaN for what the candidate budget left open.
-template <class G>
-__device__ void gen_rest(const typename G::Shared& S, const GenArgs& A, GenLists& L, uint64_t j0, uint32_t toy,
-                         int64_t got, int64_t ns, int64_t off, bool usable) {
-    // non-finite or non-positive envelopes (non-physical theta) accept nothing:
-    // the signal is then filled with NaN instead of searched for forever
-    const uint64_t budget = usable ? (uint64_t)ns * 65536ull + (1ull << 22) : 0ull;
-    for (; got < ns && j0 < budget; j0 += kGenChunk) {
-        __syncthreads();
-        const int n = gen_count<G>(S, L, j0, toy, A.k0, A.k1);
-        gen_write<G>(S, A, L, j0, toy, got, ns, off);
-        got += n;
-    }
-    for (int64_t pos = got + threadIdx.x; pos < ns; pos += kBlock) G::fill_nan(A, off + pos);
-}
-
 __device__ __forceinline__ bool gen_toy(const GenArgs& A, int toy, int64_t* ns, int64_t* nb, int64_t* off) {
     *ns = A.n_sig[toy];
     *nb = A.n_bkg[toy];
@@ -244,82 +276,138 @@ __device__ __forceinline__ bool gen_toy(const GenArgs& A, int toy, int64_t* ns, 
 }
 
 template <class G>
-__global__ void __launch_bounds__(kBlock, G::kBlocksPerSm) generate_kernel(GenArgs A) {
+__global__ void __launch_bounds__(kBlock, G::kBlocksPerSm) generate_kernel(const __grid_constant__ GenArgs A) {
     __shared__ typename G::Shared S;
-    __shared__ GenLists L;
+    extern __shared__ __align__(16) unsigned char dyn_smem[];
     G::setup(S, A);
     __syncthreads();
+    const int lane = threadIdx.x & 31;
+    GenLists& L = reinterpret_cast<GenLists*>(dyn_smem)[threadIdx.x >> 5];
     const bool usable = G::usable(S);
-    if (A.base == nullptr) {
-        for (int toy = blockIdx.x; toy < A.n_toys; toy += gridDim.x) {
+    const bool alone = A.base == nullptr;            // ticket k is the whole of toy k
+    const int sub = alone ? 1 : (int)A.base[A.n_toys + 1];
+    if (lane == 0) L.tk = (int64_t)(blockIdx.x * kGenWarps + (threadIdx.x >> 5)) - (int64_t)gridDim.x * kGenWarps;
+    while (true) {
+        __syncwarp();
+        if (lane == 0) L.tk = alone ? L.tk + (int64_t)gridDim.x * kGenWarps : (int64_t)atomicAdd(A.ticket, 1ull);
+        __syncwarp();
+        const int64_t tk = L.tk;
+        if (tk >= (alone ? A.n_toys : A.base[A.n_toys])) break;
+        const int toy = alone ? (int)tk : find_segment(A.base, A.n_toys, tk);
+        {
             int64_t ns, nb, off;
             if (!gen_toy(A, toy, &ns, &nb, &off)) continue;
-            gen_rest<G>(S, A, L, 0, (uint32_t)toy, 0, ns, off, usable);
-            for (int64_t i = threadIdx.x; i < nb; i += kBlock) G::background(S, A, (uint64_t)i, (uint32_t)toy, off + ns + i);
-        }
-        return;
-    }
-    const int64_t total = A.base[A.n_toys];
-    while (true) {
-        __syncthreads();                             // L is free
-        if (threadIdx.x == 0) L.take = (int64_t)atomicAdd(A.ticket, 1ull);
-        __syncthreads();
-        const int64_t tk = L.take;
-        if (tk >= total) break;
-        const int toy = find_segment(A.base, A.n_toys, tk);
-        const int64_t t0 = A.base[toy], n_chunks = A.base[toy + 1] - t0;
-        int64_t ns, nb, off;
-        gen_toy(A, toy, &ns, &nb, &off);
-        const int64_t n_sig_chunks = n_chunks - (nb + kBkgChunk - 1) / kBkgChunk;
-        const int64_t local = tk - t0;
-        if (local >= n_sig_chunks) {
-            const int64_t i0 = (local - n_sig_chunks) * kBkgChunk;
-            const int64_t i1 = i0 + kBkgChunk < nb ? i0 + kBkgChunk : nb;
-            for (int64_t i = i0 + threadIdx.x; i < i1; i += kBlock)
-                G::background(S, A, (uint64_t)i, (uint32_t)toy, off + ns + i);
-            continue;
-        }
-        const uint64_t j0 = (uint64_t)local * kGenChunk;
-        int n = usable ? gen_count<G>(S, L, j0, (uint32_t)toy, A.k0, A.k1) : 0;
-        int64_t got = 0;
-        if (n_sig_chunks > 1) {                      // (tickets beyond the status words are toys of one chunk)
-            if (threadIdx.x < 32) {
-                const int64_t before = look_back(A.status, tk, local, n, threadIdx.x);
-                if (threadIdx.x == 0) L.got = before;
+            // the ticket's part of the toy: one of its signal chunks, or background events
+            int64_t local = 0, n_chunks = ns > 0, i0 = 0, i1 = nb;
+            if (!alone) {
+                const int64_t t0 = A.base[toy];
+                local = tk - t0;
+                n_chunks = A.base[toy + 1] - t0 - (nb + kBkgChunk - 1) / kBkgChunk;
+                i0 = local < n_chunks ? nb : (local - n_chunks) * kBkgChunk;
+                i1 = i0 + kBkgChunk < nb ? i0 + kBkgChunk : nb;
             }
-            __syncthreads();
-            got = L.got;
-        }
-        if (got < 0) {                               // the wait ran out: count the earlier chunks here
-            got = 0;
-            for (int64_t c = 0; c < local; ++c) {
-                got += gen_count<G>(S, L, (uint64_t)c * kGenChunk, (uint32_t)toy, A.k0, A.k1);
-                __syncthreads();
+#pragma unroll 1
+            for (int64_t i = i0 + lane; i < i1; i += 32)
+                G::background(S, A, GenIdx{(uint32_t)i, (uint32_t)((uint64_t)i >> 32), (uint32_t)toy}, off + ns + i);
+            if (local >= n_chunks) continue;
+            if (lane == 0) {
+                L.ns = ns;
+                L.off = off;
+                L.got = 0;
+                L.local = local;
+                L.n_chunks = n_chunks;
+                L.c = local;
+                L.u = local * sub;
+                L.nu = sub;
+                L.toy = (uint32_t)toy;
+                L.look = n_chunks > 1;
             }
-            n = gen_count<G>(S, L, j0, (uint32_t)toy, A.k0, A.k1);
+            __syncwarp();
         }
-        if (n > 0) gen_write<G>(S, A, L, j0, (uint32_t)toy, got, ns, off);
-        if (local == n_sig_chunks - 1)
-            gen_rest<G>(S, A, L, j0 + kGenChunk, (uint32_t)toy, got + n, ns, off, usable);
+        // this ticket's chunk, and after a toy's last chunk whatever the toy still lacks
+        while (true) {
+            uint32_t word = 0u;
+            int n = 0, pre = 0, last = 0;
+            const int nu = L.nu;
+            for (int s = 0; s < nu && usable; ++s) {
+                word = gen_decide<G>(S, A, L, (uint64_t)(L.u + s) * kGenCand, L.toy, lane);
+                pre = gen_prefix(word, lane, &last);
+                if (nu > 1 && n + last <= kGenPick) gen_pick(L, word, pre + n, 0, s * kGenCand, lane);
+                n += last;
+            }
+            __syncwarp();
+            if (L.look) {
+                const int64_t before = look_back(A.status, L.tk, L.local, n, lane);
+                __syncwarp();
+                if (lane == 0) {
+                    L.look = false;
+                    L.got = before < 0 ? 0 : before;
+                    if (before < 0) L.c = L.u = 0;   // the wait ran out: count the toy's chunks from its first
+                }
+                __syncwarp();
+                if (before < 0) continue;
+            }
+            if (L.c >= L.local) {
+                if (nu > 1 && n > kGenPick) {        // more than the list holds: unit by unit
+                    __syncwarp();
+                    if (lane == 0) L.nu = 1;
+                    __syncwarp();
+                    continue;
+                }
+                for (int r0 = 0; r0 < n; r0 += kGenPick) {
+                    __syncwarp();
+                    if (nu == 1) gen_pick(L, word, pre, r0, 0, lane);
+                    __syncwarp();
+                    gen_write<G>(S, A, L, (uint64_t)L.u * kGenCand, L.toy, min(n - r0, kGenPick), L.got + r0, L.ns, L.off,
+                                 lane);
+                }
+            }
+            const int64_t got = L.got + n, u = L.u + nu;
+            int64_t c = L.c;
+            const bool ends = u >= (c + 1) * sub;    // of the chunk
+            if (ends && c == L.local && L.local != L.n_chunks - 1) break;
+            c += ends;
+            __syncwarp();
+            if (lane == 0) {
+                L.got = got;
+                L.u = u;
+                L.c = c;
+                if (ends) L.nu = sub;
+            }
+            __syncwarp();
+            // non-finite or non-positive envelopes (non-physical theta) accept nothing:
+            // the signal is then filled with NaN instead of searched for forever
+            const uint64_t budget = usable ? (uint64_t)L.ns * 65536ull + (1ull << 22) : 0ull;
+            if (ends && c > L.local && !(got < L.ns && (uint64_t)u * kGenCand < budget)) break;
+        }
+        if (L.local == L.n_chunks - 1)
+            for (int64_t pos = L.got + lane; pos < L.ns; pos += 32) G::fill_nan(A, L.off + pos);
     }
 }
 
-// Tickets per toy and their prefix (one block).  Signal chunks: enough for
-// n_sig + 3 sqrt(n_sig) + 8 accepted candidates at the model's acceptance;
-// one (whose block goes on alone) where a chunk accepts fewer than
-// kGenMinKept, or where the total would exceed max_tickets.
+// Tickets per toy, their prefix and the candidates per ticket (one block).
+// Signal chunks: enough for n_sig + 3 sqrt(n_sig) + 8 accepted candidates at the
+// model's acceptance; one (whose warp goes on alone) where even the largest
+// chunk accepts fewer than kGenMinKept, or where the total would exceed
+// max_tickets.
 template <class G>
-__global__ void gen_tickets_kernel(GenArgs A, int64_t max_tickets, int64_t* __restrict__ base) {
+__global__ void gen_tickets_kernel(const __grid_constant__ GenArgs A, int64_t max_tickets, int64_t* __restrict__ base) {
     __shared__ int64_t run[1024];
-    __shared__ float per_chunk;
-    G::acceptance(A, &per_chunk);
+    __shared__ float per_cand;
+    G::acceptance(A, &per_cand);
     __syncthreads();
-    const float kept = per_chunk * (float)kGenChunk;
+    float kept = per_cand * (float)kGenCand;
+    int sub = 1;
+    while (sub < kGenMaxSub && kept < (float)kGenMinKept) {
+        sub *= 2;
+        kept *= 2.0f;
+    }
+    const bool cut = kept >= (float)kGenMinKept && kept <= 2.0f * kGenCand;
     const int nt = blockDim.x;
     const int per = (A.n_toys + nt - 1) / nt;
     const int b = min(A.n_toys, (int)threadIdx.x * per), e = min(A.n_toys, b + per);
     for (int round = 0; round < 2; ++round) {
-        const bool split = round == 0 && kept >= (float)kGenMinKept && kept <= 2.0f * kGenChunk;
+        const bool split = round == 0 && cut;
         auto tickets = [&](int toy) -> int64_t {
             int64_t ns, nb, off;
             if (!gen_toy(A, toy, &ns, &nb, &off)) return 0;
@@ -348,40 +436,49 @@ __global__ void gen_tickets_kernel(GenArgs A, int64_t max_tickets, int64_t* __re
             base[s] = acc;
             acc += tickets(s);
         }
-        if ((int)threadIdx.x == nt - 1) base[A.n_toys] = run[nt - 1];
+        if ((int)threadIdx.x == nt - 1) {
+            base[A.n_toys] = run[nt - 1];
+            base[A.n_toys + 1] = sub;
+        }
         break;
     }
 }
 
 // consts.cu's record is in place on the stream.  The workspace (ticket prefix,
 // counter, status words) is allocated in stream order and given back after the
-// kernel; without it (no memory) a block generates a toy alone, with the same
+// kernel; without it (no memory) a warp generates a toy alone, with the same
 // events.
 template <class G>
 ipa_status launch_generator(GenArgs A, cudaStream_t s) {
     int dev = 0;
     cudaGetDevice(&dev);
+    constexpr size_t smem = kGenWarps * sizeof(GenLists);
     static int occ[64] = {};
     int& per_sm = occ[dev & 63];
     if (per_sm == 0) {
+        // with the record's tables the lists may exceed the default limit of shared memory
+        ipa_status st = cuda_fail(cudaFuncSetAttribute(generate_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                       (int)smem), "generator attribute");
+        if (st != IPA_OK) return st;
         int v = 0;
-        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, generate_kernel<G>, kBlock, 0);
+        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, generate_kernel<G>, kBlock, smem);
         per_sm = e == cudaSuccess && v >= 1 ? v : 1;
     }
-    // (n_sig + 3 sqrt(n_sig) + 8) / kGenMinKept + 2 <= n_sig / 10 + 3, and one per kBkgChunk background events
-    const int64_t max_tickets = A.capacity / 10 + 4 * (int64_t)A.n_toys + A.capacity / kBkgChunk + 1;
-    const size_t words = (size_t)A.n_toys + 2 + (size_t)max_tickets;
-    void* ws = nullptr;
+    // (n_sig + 3 sqrt(n_sig) + 8) / kGenMinKept + 2 <= n_sig / 5 + 4, and one per kBkgChunk background events
+    const int64_t max_tickets = A.capacity / 5 + 5 * (int64_t)A.n_toys + A.capacity / kBkgChunk + 1;
+    const size_t words = (size_t)A.n_toys + 3 + (size_t)max_tickets;
     const int64_t most = (int64_t)sm_count() * per_sm;
+    void* ws = nullptr;
     if (pool_alloc(&ws, words * 8, s, "generator workspace") == IPA_OK) {
         ipa_status st = cuda_fail(cudaMemsetAsync(ws, 0, words * 8, s), "generator workspace reset");
         int64_t* base = static_cast<int64_t*>(ws);
         A.base = base;
-        A.ticket = reinterpret_cast<unsigned long long*>(base + A.n_toys + 1);
+        A.ticket = reinterpret_cast<unsigned long long*>(base + A.n_toys + 2);
         A.status = A.ticket + 1;
         if (st == IPA_OK) {
             gen_tickets_kernel<G><<<1, 1024, 0, s>>>(A, max_tickets, base);
-            generate_kernel<G><<<(unsigned)(max_tickets < most ? max_tickets : most), kBlock, 0, s>>>(A);
+            const int64_t need = (max_tickets + kGenWarps - 1) / kGenWarps;
+            generate_kernel<G><<<(unsigned)(need < most ? need : most), kBlock, smem, s>>>(A);
             st = cuda_fail(cudaGetLastError(), "toygen kernel launch");
         }
         pool_free(ws, s);
@@ -389,7 +486,8 @@ ipa_status launch_generator(GenArgs A, cudaStream_t s) {
     }
     cudaGetLastError();
     A.base = nullptr;
-    generate_kernel<G><<<(unsigned)A.n_toys, kBlock, 0, s>>>(A);
+    const int64_t need = ((int64_t)A.n_toys + kGenWarps - 1) / kGenWarps;
+    generate_kernel<G><<<(unsigned)(need < most ? need : most), kBlock, smem, s>>>(A);
     return cuda_fail(cudaGetLastError(), "toygen kernel launch");
 }
 

@@ -574,12 +574,11 @@ __device__ double phis_rate_exact(const PhisConsts& c, const MathTables* mt, dou
 // products.  quick() decides candidates above the resolution peak; those near
 // it (about a seventh) are packed and take the FP32 erfc and Faddeeva
 // function (conv32.cuh).  Every convolution carries the relative bound of
-// conv32.cuh, every f'_k an error below 8e-5 where both sin^2 >= 1e-4
-// (cosines within 2.5e-7, so sines within 2.6e-5; the sine and cosine of phi
-// within 1e-6), and sum_k |b_k| r_k <= 3 sum_k max|f_k| |b_k| r_k = 3 ang:
-// |rate32 - rate| <= ang (gL + gH + 2 C) (rel + 2.5e-4), doubled to spare.
+// conv32.cuh, every f_k the error ef of the 4D model's angular test (toygen.cu),
+// and sum_k |b_k| r_k <= 3 sum_k max|f_k| |b_k| r_k = 3 ang: |rate32 - rate| <= ang
+// (gL + gH + 2 C) (rel + 3 ef), doubled to spare.
 struct PhisGen {
-    static constexpr bool kQuickKeeps = true;
+    static constexpr bool kQuickKeeps = true, kQuick64 = true;
     static constexpr int kBlocksPerSm = 3;
     struct Shared {
         PhisConsts c;
@@ -588,6 +587,7 @@ struct PhisGen {
         double t_lo, t_hi, w, total;
         Conv32 v;
         float Bf[kGenBins], Cf[kGenBins + 1], ef[kGenBins];   // B, C, e_i - mu
+        Phase32 ph[kGenBins];  // the phase over each bin
         float wf, totalf, ang;
         float p[10];           // coefficient of f'_k in F+ or F- (equal eigenvalues)
         float u[4], x[4];      // coefficients of f'_3, f'_5, f'_7, f'_9 in FU and FV
@@ -607,7 +607,9 @@ struct PhisGen {
             const int i = threadIdx.x;
             S.B[i] = phis_envelope_bin(c, A.m, w, phis_envelope_ang(c), i);
             S.Bf[i] = (float)S.B[i];
-            S.ef[i] = (float)(__dadd_rn(A.m.t_lo, __dmul_rn((double)i, w)) - c.mu);
+            const double e = __dadd_rn(A.m.t_lo, __dmul_rn((double)i, w)) - c.mu;
+            S.ef[i] = (float)e;
+            S.ph[i] = phase32_of(c.Dm, c.ph0, e, w);
         } else if (threadIdx.x == 96) {
             S.t_lo = A.m.t_lo;
             S.t_hi = A.m.t_hi;
@@ -680,22 +682,23 @@ struct PhisGen {
         int lo = 0;
 #pragma unroll
         for (int d = kGenBins / 2; d > 0; d >>= 1) lo += target > S.Cf[lo + d] ? d : 0;
-        const float band = 1.0e-6f * S.totalf;
+        const float band = 3.0e-7f * S.totalf;
         return target - S.Cf[lo] > band && S.Cf[lo + 1] - target > band ? lo : -1;
     }
     __device__ __forceinline__ static double t_of(const Shared& S, int b, double u) {
         return fmin(__dadd_rn(__dadd_rn(S.t_lo, __dmul_rn((double)b, S.w)), __dmul_rn(u, S.w)), S.t_hi);
     }
 
-    // F+, F-, FU, FV from the words of calls 1 and 2; false outside the bound's range
-    __device__ __forceinline__ static bool sums32(const Shared& S, const U4& b, const U4& d, float* F) {
+    // F+, F-, FU, FV from the words of calls 1 and 2; returns 6 ef (infinite outside the bound's range)
+    __device__ __forceinline__ static float sums32(const Shared& S, const U4& b, const U4& d, float* F) {
         const float ck = fmaf(2.0f, u32of(b.x), -1.0f), cl = fmaf(2.0f, u32of(b.z), -1.0f);
         const float cl2 = cl * cl;
         const float sk2 = fmaf(-ck, ck, 1.0f), sl2 = fmaf(-cl, cl, 1.0f);
         float sp, cp;
         sincospif(fmaf(2.0f, u32of(d.x), -1.0f), &sp, &cp);
         const float sksl2 = sk2 * sl2;
-        const float q = sqrtf(fmaxf(sksl2, 0.0f));
+        const float rk = rsqrtf(sk2), rl = rsqrtf(sl2);
+        const float q = sksl2 * (rk * rl);
         const float cp2 = cp * cp;
         const float qc = q * cl, a = qc * ck;
         F[0] = fmaf(S.p[0], ck * ck * sl2, fmaf(S.p[1], sk2 * fmaf(-sl2, cp2, 1.0f), S.p[4] * (a * cp)));
@@ -703,38 +706,39 @@ struct PhisGen {
         const float f3 = sksl2 * (sp * cp), f5 = a * sp, f7 = qc * cp, f9 = ck * sl2;
         F[2] = fmaf(S.u[0], f3, fmaf(S.u[1], f5, fmaf(S.u[2], f7, S.u[3] * f9)));
         F[3] = fmaf(S.x[0], f3, fmaf(S.x[1], f5, fmaf(S.x[2], f7, S.x[3] * f9)));
-        return sk2 >= 1.0e-4f && sl2 >= 1.0e-4f;
+        return sk2 >= 1.0e-5f && sl2 >= 1.0e-5f ? 6.0f * (5.0e-7f * (rk + rl) + 2.0e-6f) : INFINITY;
     }
 
-    __device__ __forceinline__ static GenCode decide(const Shared& S, float u, int bin, const float* F, const Time32& g,
+    __device__ __forceinline__ static GenCode decide(const Shared& S, float u, int bin, const float* F, float ef6, const Time32& g,
                                                      float q) {
         const float half = 0.5f * (g.L + g.H), diff = 0.5f * (g.L - g.H);
         const float ci = q * S.D * g.Ci;
         const float mix = S.cph * diff + S.sph * ci;
         const float rate = F[0] * (half + mix) + F[1] * (half - mix) + F[2] * (S.sph * diff - S.cph * ci) +
                            F[3] * (q * S.D * g.Cr);
-        const float err = S.ang * (g.L + g.H + S.C2 * g.C) * (2.0f * g.err + 5.0e-4f);
+        const float err = S.ang * (g.L + g.H + S.C2 * g.C) * (2.0f * g.err + ef6);
         return decide32(u * S.Bf[bin], S.Bf[bin] * 1.5e-6f, rate, err);
     }
 
-    __device__ __forceinline__ static float tag32(const Shared& S, uint64_t j, uint32_t toy, uint32_t k0, uint32_t k1) {
-        return (float)tag_of(S, S.c.qsel != 0.0 ? 0u : draw(j, toy, 3u, k0, k1).x);
+    __device__ __forceinline__ static float tag32(const Shared& S, const GenArgs& A, const GenIdx& j) {
+        return (float)tag_of(S, S.c.qsel != 0.0 ? 0u : gen_draw(A, j, 3u).x);
     }
     __device__ __forceinline__ static double tag_of(const Shared& S, uint32_t hi) {
         return S.c.qsel != 0.0 ? S.c.qsel : ((hi >> 31) ? -1.0 : 1.0);
     }
 
-    __device__ __forceinline__ static GenCode quick(const Shared& S, uint64_t j, uint32_t toy, uint32_t k0, uint32_t k1) {
-        const U4 a = draw(j, toy, 0u, k0, k1);
-        const U4 d = draw(j, toy, 2u, k0, k1);
+    __device__ __forceinline__ static GenCode quick(const Shared& S, const GenArgs& A, const GenIdx& j) {
+        const U4 a = gen_draw(A, j, 0u);
+        const U4 d = gen_draw(A, j, 2u);
         const int bin = bin32(S, a.x);
         if (bin < 0) return kTest64;
         const float tau = fmaf(u32of(d.z), S.wf, S.ef[bin]);
         if (!(tau > S.v.near)) return kTest32;
-        const U4 b = draw(j, toy, 1u, k0, k1);
+        const U4 b = gen_draw(A, j, 1u);
         float F[4];
-        if (!sums32(S, b, d, F)) return kTest64;
-        const Far32 f = conv32_far(S.v, tau);
+        const float ef6 = sums32(S, b, d, F);
+        if (!(ef6 <= 1.0e-2f)) return kTest64;
+        const Far32 f = conv32_far(S.v, tau, tau32_err(tau, S.ef[bin], S.wf));
         if (!f.ok) return kTest64;
         // what the oscillation can add at most, before its phase and the tag
         const float half = 0.5f * (f.L + f.H), diff = 0.5f * (f.L - f.H);
@@ -742,39 +746,42 @@ struct PhisGen {
         const float X = S.sph * (F[0] - F[1]) - S.cph * F[2];
         const float osc = fabsf(S.D) * f.C * (fabsf(X) + fabsf(F[3]));
         const float lhs = u32of(a.z) * S.Bf[bin];
-        const float err = S.ang * (f.L + f.H + S.C2 * f.C) * (2.0f * S.v.err + 5.0e-4f);
+        const float err = S.ang * (f.L + f.H + S.C2 * f.C) * (2.0f * f.err + ef6);
         if (lhs - S.Bf[bin] * 1.5e-6f > still + osc + err) return kDrop;
-        return decide(S, u32of(a.z), bin, F, conv32(S.v, tau), tag32(S, j, toy, k0, k1));
+        return decide(S, u32of(a.z), bin, F, ef6, conv32(S.v, tau, tau32_err(tau, S.ef[bin], S.wf), phase32(S.ph[bin], d.z), S.ph[bin].ok),
+                      tag32(S, A, j));
     }
 
     // near the peak
-    __device__ __forceinline__ static GenCode test32(const Shared& S, uint64_t j, uint32_t toy, uint32_t k0, uint32_t k1) {
-        const U4 a = draw(j, toy, 0u, k0, k1);
-        const U4 d = draw(j, toy, 2u, k0, k1);
+    __device__ __forceinline__ static GenCode test32(const Shared& S, const GenArgs& A, const GenIdx& j) {
+        const U4 a = gen_draw(A, j, 0u);
+        const U4 d = gen_draw(A, j, 2u);
         const int bin = bin32(S, a.x);
-        const U4 b = draw(j, toy, 1u, k0, k1);
+        const U4 b = gen_draw(A, j, 1u);
         float F[4];
-        if (bin < 0 || !sums32(S, b, d, F)) return kTest64;
+        const float ef6 = sums32(S, b, d, F);
+        if (bin < 0 || !(ef6 <= 1.0e-2f)) return kTest64;
         const float tau = fmaf(u32of(d.z), S.wf, S.ef[bin]);
-        return decide(S, u32of(a.z), bin, F, conv32(S.v, tau), tag32(S, j, toy, k0, k1));
+        return decide(S, u32of(a.z), bin, F, ef6, conv32(S.v, tau, tau32_err(tau, S.ef[bin], S.wf), phase32(S.ph[bin], d.z), S.ph[bin].ok),
+                      tag32(S, A, j));
     }
 
-    __device__ __noinline__ static bool test64(const Shared& S, uint64_t j, uint32_t toy, uint32_t k0, uint32_t k1) {
-        const U4 a = draw(j, toy, 0u, k0, k1);
-        const U4 b = draw(j, toy, 1u, k0, k1);
-        const U4 d = draw(j, toy, 2u, k0, k1);
-        const U4 e = draw(j, toy, 3u, k0, k1);
+    __device__ __noinline__ static bool test64(const Shared& S, const GenArgs& A, const GenIdx& j) {
+        const U4 a = gen_draw(A, j, 0u);
+        const U4 b = gen_draw(A, j, 1u);
+        const U4 d = gen_draw(A, j, 2u);
+        const U4 e = gen_draw(A, j, 3u);
         const int bin = bin_of(S, u01_int(a.x, a.y));
         return __dmul_rn(u01_int(a.z, a.w), S.B[bin]) <
                phis_rate_exact(S.c, &S.mt, t_of(S, bin, u01_int(d.z, d.w)), sym_int(b.x, b.y), sym_int(b.z, b.w),
                                __dmul_rn(cdetail::kPi, sym_int(d.x, d.y)), tag_of(S, e.x));
     }
 
-    __device__ __forceinline__ static void signal(const Shared& S, const GenArgs& A, uint64_t j, uint32_t toy, int64_t pos) {
-        const U4 a = draw(j, toy, 0u, A.k0, A.k1);
-        const U4 b = draw(j, toy, 1u, A.k0, A.k1);
-        const U4 d = draw(j, toy, 2u, A.k0, A.k1);
-        const U4 e = draw(j, toy, 3u, A.k0, A.k1);
+    __device__ __forceinline__ static void signal(const Shared& S, const GenArgs& A, const GenIdx& j, int64_t pos) {
+        const U4 a = gen_draw(A, j, 0u);
+        const U4 b = gen_draw(A, j, 1u);
+        const U4 d = gen_draw(A, j, 2u);
+        const U4 e = gen_draw(A, j, 3u);
         A.t[pos] = t_of(S, bin_of(S, u01_int(a.x, a.y)), u01_int(d.z, d.w));
         A.ck[pos] = sym_int(b.x, b.y);
         A.cl[pos] = sym_int(b.z, b.w);
@@ -782,10 +789,10 @@ struct PhisGen {
         A.q[pos] = tag_of(S, e.x);
     }
 
-    __device__ __forceinline__ static void background(const Shared& S, const GenArgs& A, uint64_t i, uint32_t toy, int64_t pos) {
-        const U4 a = draw(i, toy, 4u, A.k0, A.k1);
-        const U4 b = draw(i, toy, 5u, A.k0, A.k1);
-        const U4 e = draw(i, toy, 6u, A.k0, A.k1);
+    __device__ __forceinline__ static void background(const Shared& S, const GenArgs& A, const GenIdx& i, int64_t pos) {
+        const U4 a = gen_draw(A, i, 4u);
+        const U4 b = gen_draw(A, i, 5u);
+        const U4 e = gen_draw(A, i, 6u);
         A.t[pos] = __dadd_rn(S.t_lo, __dmul_rn(u01_int(a.x, a.y), __dsub_rn(S.t_hi, S.t_lo)));
         A.ck[pos] = sym_int(a.z, a.w);
         A.cl[pos] = sym_int(b.x, b.y);

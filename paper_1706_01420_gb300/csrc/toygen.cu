@@ -21,7 +21,7 @@
 //
 // Decisions first run in FP32 (this GPU's FP32 rate is 64 times its FP64
 // rate): each test is evaluated with a per-candidate bound on its FP32 error,
-// built from the documented accuracy of expf, exp2f, erfcf, sincospif and sqrtf and
+// built from the documented accuracy of expf, exp2f, erfcf, sincospif and rsqrtf and
 // the rounding of every input, and is decided in FP32 only when the uniform
 // lies outside that band around the threshold.  Inside the band (about one
 // candidate in 10^4), or wherever the bound is not established (a uniform or
@@ -82,7 +82,6 @@ struct Filter32 {
     float Gamma, c_exp, Gs2, k_z;
     float MT, MO;
     float h[10];
-    float bandA;      // absolute band of the angular test: 3e-4 M_Omega
 };
 
 // +1: u_t M_T < g(t - mu) for sure; -1: not; 0: undecided (FP64 decides).
@@ -116,21 +115,21 @@ __device__ __forceinline__ int time_filter(const Filter32& f, uint32_t t_hi_word
 }
 
 // +1 / -1 / 0 for u_a M_Omega < A(Omega), from the words of calls 1 and 2.
-// The cosines carry errors below 2.5e-7 and phi below 1.2e-6.  With sin^2 >=
-// 1e-2 for both polar angles, the sines (square roots of 1 - c^2, whose error
-// is below 4.2e-7) carry errors below 2.2e-6 and the sine and cosine of phi
-// below 1.4e-6, so every f_k (constant factor included) is within 1e-5 and
-// |A32 - A| <= 1e-5 sum|h_k| + 6e-7 M_Omega <= 3.2e-5 M_Omega (each max|f_k|
-// >= 1/3, so sum|h_k| <= 3 M_Omega): the band of 3e-4 M_Omega leaves a factor
-// 9 to spare.
+// The cosines carry errors below 2.5e-7 and phi below 1.2e-6.  A sine (the
+// square root of 1 - c^2, whose error is below 5e-7) is within 2.6e-7 of its
+// value over itself for sin^2 >= 1e-5, and the sine and cosine of phi within
+// 1.4e-6, so every f_k (constant factor included) is within ef = 5e-7 (1 / sin thK
+// + 1 / sin thmu) + 2e-6, and |A32 - A| <= ef sum|h_k| + 6e-7 M_Omega <= 3 ef
+// M_Omega (each max|f_k| >= 1/3): the band takes twice that.
 __device__ __forceinline__ int angle_filter(const Filter32& f, const U4& b, const U4& e) {
     const float ck = fmaf(2.0f, u32of(b.x), -1.0f);
     const float cl = fmaf(2.0f, u32of(b.z), -1.0f);
     const float sk2 = fmaf(-ck, ck, 1.0f), sl2 = fmaf(-cl, cl, 1.0f);
-    if (!(sk2 >= 1.0e-2f) || !(sl2 >= 1.0e-2f)) return 0;
+    if (!(sk2 >= 1.0e-5f) || !(sl2 >= 1.0e-5f)) return 0;
+    const float rk = rsqrtf(sk2), rl = rsqrtf(sl2);
     float sp, cp;
     sincospif(fmaf(2.0f, u32of(e.x), -1.0f), &sp, &cp);
-    const float sk = sqrtf(sk2), sl = sqrtf(sl2);
+    const float sk = sk2 * rk, sl = sl2 * rl;
     const float fk[10] = {ck * ck * sl2,
                           0.5f * sk2 * (1.0f - sl2 * cp * cp),
                           0.5f * sk2 * (1.0f - sl2 * sp * sp),
@@ -146,8 +145,9 @@ __device__ __forceinline__ int angle_filter(const Filter32& f, const U4& b, cons
     for (int k = 0; k < 10; ++k) A = fmaf(f.h[k], fk[k], A);
     const float lhs = u32of(e.z) * f.MO;
     const float dl = f.MO * 9.5367431640625e-07f;
-    if (lhs + dl < A - f.bandA) return 1;
-    if (lhs - dl > A + f.bandA) return -1;
+    const float band = 6.0f * f.MO * (5.0e-7f * (rk + rl) + 2.0e-6f);
+    if (lhs + dl < A - band) return 1;
+    if (lhs - dl > A + band) return -1;
     return 0;
 }
 
@@ -155,14 +155,13 @@ __device__ __forceinline__ int angle_filter(const Filter32& f, const U4& b, cons
 // The decay-time model (angles = false) and the 4D model.
 template <bool ANGLES>
 struct TimeGen {
-    static constexpr bool kQuickKeeps = !ANGLES;
+    static constexpr bool kQuickKeeps = !ANGLES, kQuick64 = !ANGLES;
     static constexpr int kBlocksPerSm = 4;
     struct Shared {
         Consts c;
         Filter32 f;
         Exp32 e;
         float near;       // tau above it: z <= -4.3
-        float err;        // relative error bound of the exponential
         float dl;         // bound of the error of u M_T
         double t_lo, span;
     };
@@ -186,12 +185,9 @@ struct TimeGen {
         f.MT = (float)c.MT;
         f.MO = (float)c.MO;
         for (int k = 0; k < 10; ++k) f.h[k] = (float)c.h[k];
-        f.bandA = (float)(3.0e-4 * c.MO);
-        const float dtau = kUlp1 * (2.0f * f.span + 2.0f * fabsf(f.d));
         S.e = exp32_of(c.Gamma, c.c_exp);
-        S.err = exp32_err(S.e, f.span + fabsf(f.d), dtau);
         // (a negative sigma has no such region: every candidate takes the full test)
-        S.near = c.k_z > 0.0 ? (float)(c.Gs2 + 4.3 / c.k_z) * 1.000001f + 2.0f * dtau : INFINITY;
+        S.near = c.k_z > 0.0 ? (float)(c.Gs2 + 4.3 / c.k_z) * 1.000001f + 1.0e-6f * (f.span + fabsf(f.d)) : INFINITY;
         S.dl = f.MT * 1.5e-6f;
     }
 
@@ -210,57 +206,58 @@ struct TimeGen {
     }
 
     // The decay-time test away from the resolution peak, where g is the exponential alone.
-    __device__ __forceinline__ static GenCode quick(const Shared& S, uint64_t j, uint32_t toy, uint32_t k0, uint32_t k1) {
-        const U4 a = draw(j, toy, 0u, k0, k1);
+    __device__ __forceinline__ static GenCode quick(const Shared& S, const GenArgs& A, const GenIdx& j) {
+        const U4 a = gen_draw(A, j, 0u);
         const float tau = fmaf(u32of(a.x), S.f.span, S.f.d);
         const float arg = fmaf(-S.e.x, tau, S.e.off);
         const float g = exp2f(arg);
         const float lhs = u32of(a.z) * S.f.MT;
-        if (!(tau > S.near) || !(fabsf(arg) <= kMaxArg) || !(S.err <= 1.0e-3f)) return kTest32;
-        const GenCode c = decide32(lhs, S.dl, g, g * S.err);
+        const float err = exp32_err(fabsf(S.e.x), fabsf(S.e.off), tau, tau32_err(tau, S.f.d, S.f.span));
+        if (!(tau > S.near) || !(fabsf(arg) <= kMaxArg) || !(err <= 1.0e-3f)) return kTest32;
+        const GenCode c = decide32(lhs, S.dl, g, g * err);
         return ANGLES ? (c == kDrop ? kDrop : kTest32) : c;
     }
 
-    __device__ __forceinline__ static GenCode test32(const Shared& S, uint64_t j, uint32_t toy, uint32_t k0, uint32_t k1) {
-        const U4 a = draw(j, toy, 0u, k0, k1);
+    __device__ __forceinline__ static GenCode test32(const Shared& S, const GenArgs& A, const GenIdx& j) {
+        const U4 a = gen_draw(A, j, 0u);
         int d = time_filter(S.f, a.x, a.z);
         if (d < 0) return kDrop;
         if (!ANGLES) return d > 0 ? kKeep : kTest64;
-        const U4 b = draw(j, toy, 1u, k0, k1);
-        const U4 e = draw(j, toy, 2u, k0, k1);
+        const U4 b = gen_draw(A, j, 1u);
+        const U4 e = gen_draw(A, j, 2u);
         const int f = angle_filter(S.f, b, e);
         if (f < 0) return kDrop;
         return d > 0 && f > 0 ? kKeep : kTest64;
     }
 
-    __device__ __noinline__ static bool test64(const Shared& S, uint64_t j, uint32_t toy, uint32_t k0, uint32_t k1) {
-        const U4 a = draw(j, toy, 0u, k0, k1);
+    __device__ __noinline__ static bool test64(const Shared& S, const GenArgs& A, const GenIdx& j) {
+        const U4 a = gen_draw(A, j, 0u);
         const double t = __dadd_rn(S.t_lo, __dmul_rn(u01_int(a.x, a.y), S.span));
         if (!(__dmul_rn(u01_int(a.z, a.w), S.c.MT) < time_pdf(S.c, t))) return false;
         if (!ANGLES) return true;
-        const U4 b = draw(j, toy, 1u, k0, k1);
-        const U4 e = draw(j, toy, 2u, k0, k1);
+        const U4 b = gen_draw(A, j, 1u);
+        const U4 e = gen_draw(A, j, 2u);
         return __dmul_rn(u01_int(e.z, e.w), S.c.MO) <
                angular_pdf(S.c, sym_int(b.x, b.y), sym_int(b.z, b.w), __dmul_rn(kPi, sym_int(e.x, e.y)));
     }
 
-    __device__ __forceinline__ static void signal(const Shared& S, const GenArgs& A, uint64_t j, uint32_t toy, int64_t pos) {
-        const U4 a = draw(j, toy, 0u, A.k0, A.k1);
+    __device__ __forceinline__ static void signal(const Shared& S, const GenArgs& A, const GenIdx& j, int64_t pos) {
+        const U4 a = gen_draw(A, j, 0u);
         A.t[pos] = __dadd_rn(S.t_lo, __dmul_rn(u01_int(a.x, a.y), S.span));
         if (!ANGLES) return;
-        const U4 b = draw(j, toy, 1u, A.k0, A.k1);
-        const U4 e = draw(j, toy, 2u, A.k0, A.k1);
+        const U4 b = gen_draw(A, j, 1u);
+        const U4 e = gen_draw(A, j, 2u);
         A.ck[pos] = sym_int(b.x, b.y);
         A.cl[pos] = sym_int(b.z, b.w);
         A.phi[pos] = __dmul_rn(kPi, sym_int(e.x, e.y));
     }
 
     // background: uniform in the box, always kept
-    __device__ __forceinline__ static void background(const Shared& S, const GenArgs& A, uint64_t i, uint32_t toy, int64_t pos) {
-        const U4 a = draw(i, toy, 4u, A.k0, A.k1);
+    __device__ __forceinline__ static void background(const Shared& S, const GenArgs& A, const GenIdx& i, int64_t pos) {
+        const U4 a = gen_draw(A, i, 4u);
         A.t[pos] = __dadd_rn(S.t_lo, __dmul_rn(u01_int(a.x, a.y), S.span));
         if (!ANGLES) return;
-        const U4 b = draw(i, toy, 5u, A.k0, A.k1);
+        const U4 b = gen_draw(A, i, 5u);
         A.ck[pos] = sym_int(a.z, a.w);
         A.cl[pos] = sym_int(b.x, b.y);
         A.phi[pos] = __dmul_rn(kPi, sym_int(b.z, b.w));
@@ -284,11 +281,12 @@ struct TimeGen {
 // threshold (nine in ten) without drawing the tag, test32() evaluates the
 // oscillation, near the peak with FP32 erfc and Faddeeva functions.
 struct TagGen {
-    static constexpr bool kQuickKeeps = false;
+    static constexpr bool kQuickKeeps = false, kQuick64 = false;
     static constexpr int kBlocksPerSm = 3;
     struct Shared {
         TagConsts c;
         Conv32 v;
+        Phase32 ph;
         float aH, aL, Ds, MS, dl;
         double t_lo, span;
         float f_span;
@@ -304,6 +302,7 @@ struct TagGen {
         S.span = __dsub_rn(A.m.t_hi, A.m.t_lo);
         S.f_span = (float)S.span;
         S.v = conv32_of(S.c, A.m.t_lo - S.c.mu, S.span);
+        S.ph = phase32_of(S.c.Dm, S.c.ph0, A.m.t_lo - S.c.mu, S.span);
         S.aH = (float)S.c.aH;
         S.aL = (float)S.c.aL;
         S.Ds = (float)S.c.Ds;
@@ -322,45 +321,45 @@ struct TagGen {
         *acc = 0.5f * (float)c.N / ((float)c.MS * (float)(A.m.t_hi - A.m.t_lo));
     }
 
-    __device__ __forceinline__ static GenCode quick(const Shared& S, uint64_t j, uint32_t toy, uint32_t k0, uint32_t k1) {
-        const U4 a = draw(j, toy, 0u, k0, k1);
+    __device__ __forceinline__ static GenCode quick(const Shared& S, const GenArgs& A, const GenIdx& j) {
+        const U4 a = gen_draw(A, j, 0u);
         const float tau = fmaf(u32of(a.x), S.f_span, S.v.d);
         const float lhs = u32of(a.z) * S.MS;
-        const Far32 g = conv32_far(S.v, tau);
+        const Far32 g = conv32_far(S.v, tau, tau32_err(tau, S.v.d, S.f_span));
         if (!g.ok) return kTest32;
         const float most = S.aH * g.H + S.aL * g.L + fabsf(S.Ds) * g.C;
-        return lhs - S.dl > most * (1.0f + S.v.err) ? kDrop : kTest32;
+        return lhs - S.dl > most * (1.0f + g.err) ? kDrop : kTest32;
     }
 
-    __device__ __forceinline__ static GenCode test32(const Shared& S, uint64_t j, uint32_t toy, uint32_t k0, uint32_t k1) {
-        const U4 a = draw(j, toy, 0u, k0, k1);
-        const U4 b = draw(j, toy, 1u, k0, k1);
+    __device__ __forceinline__ static GenCode test32(const Shared& S, const GenArgs& A, const GenIdx& j) {
+        const U4 a = gen_draw(A, j, 0u);
+        const U4 b = gen_draw(A, j, 1u);
         const float tau = fmaf(u32of(a.x), S.f_span, S.v.d);
         const float q = (b.x >> 31) ? -1.0f : 1.0f;
-        const Time32 g = conv32(S.v, tau);
+        const Time32 g = conv32(S.v, tau, tau32_err(tau, S.v.d, S.f_span), phase32(S.ph, a.x), S.ph.ok);
         const float sig = S.aH * g.H + S.aL * g.L + q * S.Ds * g.Ci;
         const float err = (S.aH * g.H + S.aL * g.L + fabsf(S.Ds) * g.C) * g.err;
         return decide32(u32of(a.z) * S.MS, S.dl, sig, err);
     }
 
-    __device__ __noinline__ static bool test64(const Shared& S, uint64_t j, uint32_t toy, uint32_t k0, uint32_t k1) {
-        const U4 a = draw(j, toy, 0u, k0, k1);
-        const U4 b = draw(j, toy, 1u, k0, k1);
+    __device__ __noinline__ static bool test64(const Shared& S, const GenArgs& A, const GenIdx& j) {
+        const U4 a = gen_draw(A, j, 0u);
+        const U4 b = gen_draw(A, j, 1u);
         const double t = __dadd_rn(S.t_lo, __dmul_rn(u01_int(a.x, a.y), S.span));
         return __dmul_rn(u01_int(a.z, a.w), S.c.MS) < tag_signal(S.c, t, tag_of(b.x));
     }
 
     __device__ __forceinline__ static double tag_of(uint32_t hi) { return (hi >> 31) ? -1.0 : 1.0; }
 
-    __device__ __forceinline__ static void signal(const Shared& S, const GenArgs& A, uint64_t j, uint32_t toy, int64_t pos) {
-        const U4 a = draw(j, toy, 0u, A.k0, A.k1);
-        const U4 b = draw(j, toy, 1u, A.k0, A.k1);
+    __device__ __forceinline__ static void signal(const Shared& S, const GenArgs& A, const GenIdx& j, int64_t pos) {
+        const U4 a = gen_draw(A, j, 0u);
+        const U4 b = gen_draw(A, j, 1u);
         A.t[pos] = __dadd_rn(S.t_lo, __dmul_rn(u01_int(a.x, a.y), S.span));
         A.q[pos] = tag_of(b.x);
     }
 
-    __device__ __forceinline__ static void background(const Shared& S, const GenArgs& A, uint64_t i, uint32_t toy, int64_t pos) {
-        const U4 a = draw(i, toy, 4u, A.k0, A.k1);
+    __device__ __forceinline__ static void background(const Shared& S, const GenArgs& A, const GenIdx& i, int64_t pos) {
+        const U4 a = gen_draw(A, i, 4u);
         A.t[pos] = __dadd_rn(S.t_lo, __dmul_rn(u01_int(a.x, a.y), S.span));
         A.q[pos] = tag_of(a.z);
     }
@@ -412,8 +411,7 @@ extern "C" ipa_status ipa_toygen(const ipa_model* model, const double* theta_dev
     GenArgs a{};
     a.m = m;
     a.consts = sc->consts;
-    a.k0 = (uint32_t)seed;
-    a.k1 = (uint32_t)(seed >> 32);
+    gen_keys(seed, &a);
     a.n_toys = n_toys;
     a.n_sig = n_sig_dev;
     a.n_bkg = n_bkg_dev;
