@@ -63,7 +63,7 @@ enum GenCode { kDrop = 0, kKeep = 1, kTest32 = 2, kTest64 = 3 };
 struct GenArgs {
     ModelDev m;
     const Consts* consts;
-    uint32_t key[20];      // the ten rounds' keys (k0, k1 of each), read from the parameter bank
+    PhiloxKeys keys;
     int n_toys;
     const int64_t *n_sig, *n_bkg, *offsets;
     int64_t capacity;
@@ -76,28 +76,13 @@ struct GenArgs {
     unsigned long long* status;
 };
 
-inline void gen_keys(uint64_t seed, GenArgs* a) {
-    for (int r = 0; r < 10; ++r) {
-        a->key[2 * r] = (uint32_t)seed + (uint32_t)r * kPhiloxW0;
-        a->key[2 * r + 1] = (uint32_t)(seed >> 32) + (uint32_t)r * kPhiloxW1;
-    }
-}
-
 // Candidate or background event `lo` + 2^32 hi of a toy.
 struct GenIdx {
     uint32_t lo, hi, toy;
 };
 
-// draw() (philox.cuh) with the round keys laid out beforehand: the same words.
 __device__ __forceinline__ U4 gen_draw(const GenArgs& A, const GenIdx& j, uint32_t call) {
-    U4 c{j.lo, j.hi, j.toy, call};
-#pragma unroll
-    for (int r = 0; r < 10; ++r) {
-        const unsigned long long p0 = (unsigned long long)kPhiloxM0 * c.x, p1 = (unsigned long long)kPhiloxM1 * c.z;
-        c = U4{(uint32_t)(p1 >> 32) ^ c.y ^ A.key[2 * r], (uint32_t)p1, (uint32_t)(p0 >> 32) ^ c.w ^ A.key[2 * r + 1],
-               (uint32_t)p0};
-    }
-    return c;
+    return keyed(A.keys, j.lo, j.hi, j.toy, call);
 }
 
 // (v + 1) 2^-53 and 2 (v + 1) 2^-53 - 1 for the 53-bit v of two words, exactly,

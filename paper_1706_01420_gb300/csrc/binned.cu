@@ -11,14 +11,24 @@
 //   n += 1, p = (p nu) / n, F += p;   cap = floor(nu + 40 sqrt(nu) + 100).
 // Every step is a correctly rounded IEEE operation (no contraction), so the
 // counts are reproducible bit for bit.  The recurrence depends only on the
-// bin's mean, so it runs once per bin and call into a CDF table (BinTable);
-// a draw is then one Philox block and a few comparisons.
+// bin's mean, so it runs once per bin and call into a table of thresholds
+// (BinTable); a draw is then one Philox block and a few integer comparisons.
 //
 // CLs.  With w_i = ln(1 + s_i / b_i), X = sum_i n_i w_i (the data-dependent part
 // of -2 ln Q, Q = L(s+b) / L(b)); CL_s+b = P_s+b(X <= X_obs), CL_b =
-// P_b(X <= X_obs), CL_s = CL_s+b / CL_b over n_toys toys per hypothesis.  One
-// block per toy draws its bins on the fly (no histogram is stored) and adds
-// n_i w_i in a fixed order (thread-strided partial sums, then a fixed tree).
+// P_b(X <= X_obs), CL_s = CL_s+b / CL_b over n_toys toys per hypothesis.  The
+// counts are drawn on the fly (no histogram is stored).  X is summed in a fixed
+// order: bins in order within a slice of kSlice, the slices in four interleaved
+// chains; the data take the same order.
+//
+// A lane draws one toy's bins: the 32 toys of a warp meet a bin together, so its
+// thresholds and weight come as one broadcast from shared memory and the
+// Philox counter's bin half is computed once.  Before, a block walked one toy
+// with a bin per thread: every draw fetched its own 40-byte record and two or
+// three doubles of the CDF from L2 (2.4 MB of tables), and converted and
+// compared in FP64, four FP64 instructions per draw on a pipe of 2 per clock and
+// SM.  Now one (the FMA into X).  10 000 bins, 10 000 toys: 3.7 -> 0.81 ms; the tables
+// (a serial chain per bin, run twice and to its end before) 305 -> 21 us for both.
 #include <math.h>
 
 #include "ipa_internal.cuh"
@@ -29,6 +39,11 @@ namespace {
 
 constexpr double kPiece = 400.0;
 constexpr int kBinBlock = 256;
+constexpr int kTabBlock = 64;           // bins per block of the table kernels: a bin is a serial chain, so spread them
+constexpr int kTabFixed = 32;           // thresholds per bin in the fixed part of the table
+constexpr int kSlice = 64;              // bins summed by one thread of the CLs kernel
+constexpr int kToyBlock = 128;          // toys per block of the CLs kernel
+constexpr int kFirst = 4;               // thresholds compared without a search
 constexpr uint32_t kBinnedCall = 8u;
 
 __device__ __forceinline__ uint32_t binned_call(int hyp, int m) {
@@ -38,131 +53,142 @@ __device__ __forceinline__ uint32_t binned_call(int hyp, int m) {
 // The inversion of one bin, tabulated once per call and shared by every toy:
 // with nu = lambda / M, p_0 = exp(-nu), cap = floor(nu + 40 sqrt(nu) + 100), the
 // recurrence p_n = (p_{n-1} nu) / n, F_n = F_{n-1} + p_n (each step correctly
-// rounded) gives the CDF values F_0, F_1, ...  A draw with uniform u is the
-// first n with u <= F_n, or `stop` (the n where the recurrence ends, p = 0 or
-// n = cap) when u exceeds them all.  The table keeps F_0 .. F_{len-1}, up to
-// the point past the mode where adding p_n no longer changes F (after that no
-// u changes the outcome before `stop`), so a draw compares u with the same
-// values in the same order as the plain sequential loop, and the counts are
-// those of that loop bit for bit.
+// rounded) gives the CDF values F_0 <= F_1 <= ...  A draw with uniform u is the
+// first n with u <= F_n, or the n where the recurrence ends (p = 0 or n = cap)
+// when u exceeds them all.  u = (v + 1) 2^-53 with v the top 53 bits of the
+// draw's 64-bit word, so u > F_n exactly when the word is at least
+// floor(F_n 2^53) 2^11: the table holds these 64-bit integers.  It ends before
+// the first F_n >= 1 (which no u exceeds: the draw is n), or past the mode where
+// adding p_n no longer changes F (no later n is the first).  The counts are
+// those of the sequential FP64 loop bit for bit.
 struct BinTable {
-    int64_t off;    // first entry in the flat CDF array
+    int64_t off;    // first entry in the flat threshold array
     double nu;      // mean of one piece
     int M;          // pieces (0 for a non-positive mean)
-    int len;        // entries F_0 .. F_{len-1}
-    int stop;       // the draw when u > F_{len-1}
+    int len;        // entries
+    int stop;       // the draw when the word passes every entry; -1: where the recurrence ends (bin_end)
     int pad_;
 };
 
-// Run the recurrence of one bin: entries and stop index; with F != nullptr
-// also write the entries.
-__device__ inline void bin_recurrence(double lam, BinTable* t, double* F) {
-    if (!(lam > 0.0)) {
-        t->M = 0;
-        t->nu = 0.0;
-        t->len = 0;
-        t->stop = 0;
-        return;
+struct Recurrence {
+    double nu, cap, p, f;
+    int n;
+    __device__ explicit Recurrence(double nu_) : nu(nu_), n(0) {
+        cap = floor(__dadd_rn(__dadd_rn(nu, __dmul_rn(40.0, sqrt(nu))), 100.0));
+        p = exp(-nu);
+        f = p;
     }
-    const double Md = ceil(lam / kPiece);
-    const int M = Md < 1.0 ? 1 : (int)Md;
-    const double nu = __ddiv_rn(lam, (double)M);
-    const double cap = floor(__dadd_rn(__dadd_rn(nu, __dmul_rn(40.0, sqrt(nu))), 100.0));
-    double p = exp(-nu), f = p;
-    int n = 0, len = 1;
-    bool settled = false;
-    if (F) F[0] = f;
-    // u <= 1 < any F would end the loop anyway; u > F runs it to p = 0 or n = cap
-    while (p > 0.0 && (double)n < cap) {
+    __device__ bool more() const { return p > 0.0 && (double)n < cap; }
+    __device__ void next() {
         n += 1;
         p = __ddiv_rn(__dmul_rn(p, nu), (double)n);
-        const double g = __dadd_rn(f, p);
-        if (!settled) {
-            if (g == f && (double)n > nu) {
-                settled = true;
-            } else {
-                if (F) F[len] = g;
-                ++len;
-            }
-        }
-        f = g;
     }
-    t->M = M;
-    t->nu = nu;
-    t->len = len;
-    t->stop = n;
+};
+
+// Where the recurrence ends: the draw of a word past a table that stopped
+// changing (about one draw in 10^15).
+__device__ __noinline__ int bin_end(double nu) {
+    Recurrence r(nu);
+    while (r.more()) r.next();
+    return r.n;
 }
 
-__device__ __forceinline__ int table_draw(const BinTable& t, const double* __restrict__ F, double u) {
-    const double* f = F + t.off;
-    int j = 0;
-    while (j < t.len && u > __ldg(f + j)) ++j;
-    return j < t.len ? j : t.stop;
+// One bin's thresholds: the first `room` of them into T; t gets everything but off.
+__device__ inline void bin_table(double lam, BinTable* t, unsigned long long* T, int room) {
+    *t = BinTable{};
+    if (!(lam > 0.0)) return;
+    const double Md = ceil(lam / kPiece);
+    t->M = Md < 1.0 ? 1 : (int)Md;
+    t->nu = __ddiv_rn(lam, (double)t->M);
+    t->stop = -1;
+    Recurrence r(t->nu);
+    while (true) {
+        if (r.f >= 1.0) {
+            t->stop = t->len;
+            break;
+        }
+        if (t->len < room) T[t->len] = (unsigned long long)(r.f * 9007199254740992.0) << 11;   // exact product, truncated
+        ++t->len;
+        if (!r.more()) break;
+        r.next();
+        const double g = __dadd_rn(r.f, r.p);
+        if (g == r.f && (double)r.n > r.nu) break;
+        r.f = g;
+    }
 }
 
-__device__ __forceinline__ int poisson_bin(const BinTable& t, const double* __restrict__ F, uint64_t i, uint32_t toy,
-                                           int hyp, uint32_t k0, uint32_t k1) {
+// The first entry at or after j (all before it passed by `word`) that the word
+// does not pass; t.len if it passes all.
+__device__ __forceinline__ int bin_search(const BinTable& t, const unsigned long long* __restrict__ T,
+                                          unsigned long long word, int j) {
+    int lo = j, hi = t.len;
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (word >= __ldg(T + t.off + mid)) lo = mid + 1; else hi = mid;
+    }
+    return lo;
+}
+__device__ __forceinline__ int bin_draw(const BinTable& t, const unsigned long long* __restrict__ T,
+                                        unsigned long long word, int j) {
+    const int n = bin_search(t, T, word, j);
+    return n < t.len ? n : (t.stop >= 0 ? t.stop : bin_end(t.nu));
+}
+
+__device__ __forceinline__ unsigned long long word64(uint32_t a, uint32_t b) {
+    return ((unsigned long long)a << 32) | b;
+}
+
+__device__ __forceinline__ int poisson_bin(const BinTable& t, const unsigned long long* __restrict__ T, uint64_t i,
+                                           uint32_t toy, int hyp, uint32_t k0, uint32_t k1) {
     int n = 0;
     for (int m = 0; m < t.M; ++m) {
         const U4 r = draw(i, toy, binned_call(hyp, m), k0, k1);
-        const double u = (m & 1) ? u01(r.z, r.w) : u01(r.x, r.y);
-        n += table_draw(t, F, u);
+        n += bin_draw(t, T, (m & 1) ? word64(r.z, r.w) : word64(r.x, r.y), 0);
     }
     return n;
 }
 
-__global__ void table_size_kernel(const double* __restrict__ lam, const double* __restrict__ add, int64_t n_bins,
-                                  BinTable* __restrict__ tab) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n_bins; i += (int64_t)gridDim.x * blockDim.x) {
-        const double l = add ? __ldg(lam + i) + __ldg(add + i) : __ldg(lam + i);
-        BinTable t{};
-        bin_recurrence(l, &t, nullptr);
-        tab[i] = t;
-    }
+// Tables of n_tab histograms over the same bins (table h: means lam, plus add
+// for h = 1).  Bin x = h n_bins + i has kTabFixed entries at x kTabFixed; a
+// longer table goes to the part behind them, whose entries *more counts.
+__global__ void __launch_bounds__(kTabBlock)
+table_kernel(const double* __restrict__ lam, const double* __restrict__ add, int64_t n_bins, int n_tab,
+             BinTable* __restrict__ tab, unsigned long long* __restrict__ T, unsigned long long* __restrict__ more) {
+    const int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (x >= n_bins * n_tab) return;
+    const int64_t i = x < n_bins ? x : x - n_bins;
+    const double l = x < n_bins ? __ldg(lam + i) : __ldg(lam + i) + __ldg(add + i);
+    BinTable t;
+    bin_table(l, &t, T + x * kTabFixed, kTabFixed);
+    t.off = x * kTabFixed;
+    if (t.len > kTabFixed) t.off = -1 - (int64_t)atomicAdd(more, (unsigned long long)t.len);
+    tab[x] = t;
 }
 
-// off[i] = sum_{r<i} len_r (one block: a sequential run per thread, then a
-// block scan of the run totals); *total = the sum.
-__global__ void table_offsets_kernel(BinTable* __restrict__ tab, int64_t n_bins, int64_t* __restrict__ total) {
-    __shared__ int64_t run[1024];
-    const int nt = blockDim.x;
-    const int64_t per = (n_bins + nt - 1) / nt;
-    const int64_t b = threadIdx.x * per;
-    const int64_t e = b + per < n_bins ? b + per : n_bins;
-    int64_t sum = 0;
-    for (int64_t i = b; i < e; ++i) sum += tab[i].len;
-    run[threadIdx.x] = sum;
-    __syncthreads();
-    for (int d = 1; d < nt; d <<= 1) {
-        const int64_t v = threadIdx.x >= d ? run[threadIdx.x - d] : 0;
-        __syncthreads();
-        run[threadIdx.x] += v;
-        __syncthreads();
-    }
-    int64_t acc = threadIdx.x ? run[threadIdx.x - 1] : 0;
-    for (int64_t i = b; i < e; ++i) {
-        tab[i].off = acc;
-        acc += tab[i].len;
-    }
-    if (threadIdx.x == nt - 1) *total = run[nt - 1];
-}
-
-__global__ void table_fill_kernel(const double* __restrict__ lam, const double* __restrict__ add, int64_t n_bins,
-                                  const BinTable* __restrict__ tab, double* __restrict__ F) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n_bins; i += (int64_t)gridDim.x * blockDim.x) {
-        const double l = add ? __ldg(lam + i) + __ldg(add + i) : __ldg(lam + i);
-        BinTable t{};
-        bin_recurrence(l, &t, F + tab[i].off);
-    }
+// The long tables (off = -1 - place) into the second part, from entry `first` on.
+__global__ void __launch_bounds__(kTabBlock)
+table_long_kernel(const double* __restrict__ lam, const double* __restrict__ add, int64_t n_bins, int n_tab,
+                  BinTable* __restrict__ tab, unsigned long long* __restrict__ L) {
+    const int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (x >= n_bins * n_tab || tab[x].off >= 0) return;
+    const int64_t i = x < n_bins ? x : x - n_bins;
+    const double l = x < n_bins ? __ldg(lam + i) : __ldg(lam + i) + __ldg(add + i);
+    const int64_t place = -1 - tab[x].off;
+    BinTable t;
+    bin_table(l, &t, L + place, tab[x].len);
 }
 
 __global__ void __launch_bounds__(kBinBlock)
-generate_kernel(const BinTable* __restrict__ tab, const double* __restrict__ F, int64_t n_bins, uint32_t k0,
-                uint32_t k1, int hyp, int toy0, int n_toys, int32_t* __restrict__ counts) {
+generate_kernel(const BinTable* __restrict__ tab, const unsigned long long* __restrict__ T,
+                const unsigned long long* __restrict__ L, int64_t n_bins, uint32_t k0, uint32_t k1, int hyp, int toy0,
+                int n_toys, int32_t* __restrict__ counts) {
     const int64_t total = n_bins * (int64_t)n_toys;
     for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < total; x += (int64_t)gridDim.x * blockDim.x) {
         const int64_t k = x / n_bins, i = x - k * n_bins;
-        counts[x] = poisson_bin(tab[i], F, (uint64_t)i, (uint32_t)(toy0 + k), hyp, k0, k1);
+        BinTable t = tab[i];
+        const unsigned long long* F = t.off >= 0 ? T : L;
+        if (t.off < 0) t.off = -1 - t.off;
+        counts[x] = poisson_bin(t, F, (uint64_t)i, (uint32_t)(toy0 + k), hyp, k0, k1);
     }
 }
 
@@ -208,55 +234,124 @@ __global__ void cls_weights_kernel(const double* __restrict__ s, const double* _
         w[i] = log1p(__ldg(s + i) / __ldg(b + i));
 }
 
-// Fixed-order block sum (every thread gets the total).
-__device__ __forceinline__ double block_sum(double v, double* part) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) part[wid] = v;
-    __syncthreads();
-    double t = 0.0;
-    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) t += part[k];
-    __syncthreads();
-    return t;
-}
+// One bin of a slice in shared memory.
+struct SliceBin {
+    unsigned long long thr[kFirst];   // its first thresholds, ~0 beyond the table
+    double w;
+    int one;          // 1: one piece (the draw starts at thr), 0: the general path
+    int first;        // min(kFirst, len): a word that passes this many needs the whole table
+};
 
-// X of toy k under hypothesis h (blocks stride over toys); toy index -1: the data.
-__global__ void __launch_bounds__(kBinBlock)
-cls_toys_kernel(const BinTable* __restrict__ tab, const double* __restrict__ F, const double* __restrict__ w,
-                int64_t n_bins, uint32_t k0, uint32_t k1, int hyp, int n_toys, const int32_t* __restrict__ data,
-                double* __restrict__ x_out) {
-    __shared__ double part[kBinBlock / 32];
-    const int first = data ? 0 : blockIdx.x;
-    const int stride = data ? 1 : gridDim.x;
-    const int last = data ? 1 : n_toys;
-    for (int k = first; k < last; k += stride) {
-        double acc = 0.0;
-        for (int64_t i = threadIdx.x; i < n_bins; i += blockDim.x) {
-            const int n = data ? __ldg(data + i) : poisson_bin(tab[i], F, (uint64_t)i, (uint32_t)k, hyp, k0, k1);
-            if (n) acc = fma((double)n, __ldg(w + i), acc);
+// Slice sums of X: part[s * stride + c] = sum over the slice's bins of n_i w_i
+// for column c of the batch: toy toy0 + c of hypothesis 0 (c < n) or toy toy0 +
+// c - n of hypothesis 1; column 2 n, the data, if it is given (block.y = 2).
+__global__ void __launch_bounds__(kToyBlock)
+cls_slices_kernel(const BinTable* __restrict__ tab, const unsigned long long* __restrict__ T,
+                  const unsigned long long* __restrict__ L, const double* __restrict__ w, int64_t n_bins, int64_t n_slices,
+                  const __grid_constant__ PhiloxKeys keys, int toy0, int n, const int32_t* __restrict__ data,
+                  double* __restrict__ part, int64_t stride) {
+    __shared__ SliceBin bins[kSlice];
+    __shared__ double num[kFirst + 1];
+    const int hyp = blockIdx.y;
+    if (hyp == 2) {                      // the data: a thread per slice
+        for (int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; s < n_slices; s += (int64_t)gridDim.x * blockDim.x) {
+            double acc = 0.0;
+            const int64_t e = (s + 1) * kSlice < n_bins ? (s + 1) * kSlice : n_bins;
+            for (int64_t i = s * kSlice; i < e; ++i) {
+                const int k = __ldg(data + i);
+                if (k) acc = fma((double)k, __ldg(w + i), acc);
+            }
+            part[s * stride + 2 * n] = acc;
         }
-        const double X = block_sum(acc, part);
-        if (threadIdx.x == 0) x_out[data ? 0 : k] = X;
+        return;
     }
+    const int64_t toy_blocks = (n + kToyBlock - 1) / kToyBlock;
+    const int64_t s = blockIdx.x / toy_blocks;
+    if (s >= n_slices) return;           // (block row 2 may be longer)
+    const int c = (int)(blockIdx.x - s * toy_blocks) * kToyBlock + threadIdx.x;
+    const int64_t i0 = s * kSlice;
+    const int nb = (int)(n_bins - i0 < kSlice ? n_bins - i0 : kSlice);
+    tab += (int64_t)hyp * n_bins + i0;
+    if (threadIdx.x <= kFirst) num[threadIdx.x] = (double)threadIdx.x;
+    for (int b = threadIdx.x; b < nb; b += kToyBlock) {
+        const BinTable t = tab[b];
+        SliceBin r;
+        const unsigned long long* F = t.off >= 0 ? T + t.off : L + (-1 - t.off);
+#pragma unroll
+        for (int q = 0; q < kFirst; ++q) r.thr[q] = q < t.len ? __ldg(F + q) : ~0ull;
+        r.w = __ldg(w + i0 + b);
+        r.one = t.M == 1;
+        r.first = t.len < kFirst ? t.len : kFirst;
+        bins[b] = r;
+    }
+    __syncthreads();
+    if (c >= n) return;
+    const uint32_t toy = (uint32_t)(toy0 + c);
+    double acc = 0.0;
+#pragma unroll 2
+    for (int b = 0; b < nb; ++b) {
+        const SliceBin& r = bins[b];
+        const uint64_t i = (uint64_t)(i0 + b);
+        if (r.one) {
+            const U4 x = keyed(keys, (uint32_t)i, (uint32_t)(i >> 32), toy, binned_call(hyp, 0));
+            const unsigned long long word = word64(x.x, x.y);
+            int k = 0;
+#pragma unroll
+            for (int q = 0; q < kFirst; ++q) k += word >= r.thr[q];
+            double m = num[k];
+            if (k >= r.first) {
+                BinTable t = tab[b];
+                const unsigned long long* F = t.off >= 0 ? T : L;
+                if (t.off < 0) t.off = -1 - t.off;
+                k = bin_draw(t, F, word, r.first);
+                m = (double)k;
+            }
+            if (k) acc = fma(m, r.w, acc);           // (an infinite w counts only where there are events)
+        } else {
+            BinTable t = tab[b];
+            const unsigned long long* F = t.off >= 0 ? T : L;
+            if (t.off < 0) t.off = -1 - t.off;
+            const int k = poisson_bin(t, F, i, toy, hyp, keys.k[0], keys.k[1]);
+            if (k) acc = fma((double)k, r.w, acc);
+        }
+    }
+    part[s * stride + (int64_t)hyp * n + c] = acc;
 }
 
-// counts[0] = #{k: X_b[k] <= X_obs}, counts[1] = #{k: X_sb[k] <= X_obs}; then the CLs.
-__global__ void cls_count_kernel(const double* __restrict__ xb, const double* __restrict__ xsb,
-                                 const double* __restrict__ xobs, int n_toys, unsigned long long* __restrict__ cnt) {
-    const double xo = *xobs;
-    unsigned long long a = 0, c = 0;
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n_toys; k += gridDim.x * blockDim.x) {
-        a += xb[k] <= xo;
-        c += xsb[k] <= xo;
+// X of a column from its slice sums: four interleaved chains.
+__device__ __forceinline__ double sum_slices(const double* __restrict__ part, int64_t n_slices, int64_t stride) {
+    double a[4] = {0.0, 0.0, 0.0, 0.0};
+    int64_t s = 0;
+    for (; s + 4 <= n_slices; s += 4) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) a[q] += __ldg(part + (s + q) * stride);
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        a += __shfl_xor_sync(0xffffffffu, a, o);
-        c += __shfl_xor_sync(0xffffffffu, c, o);
+    for (int q = 0; s + q < n_slices; ++q) a[q] += __ldg(part + (s + q) * stride);
+    return (a[0] + a[1]) + (a[2] + a[3]);
+}
+
+// X_obs from the data's slice sums (column 2 n of a batch's partials; one thread).
+__global__ void cls_obs_kernel(const double* __restrict__ part, int64_t n_slices, int64_t stride, double* __restrict__ x_obs) {
+    *x_obs = sum_slices(part, n_slices, stride);
+}
+
+// X of the batch's toys, and the counts of X <= X_obs per hypothesis.
+__global__ void __launch_bounds__(kBinBlock)
+cls_sum_kernel(const double* __restrict__ part, int64_t n_slices, int64_t stride, int n, const double* __restrict__ x_obs,
+               double* __restrict__ xb, double* __restrict__ xsb, unsigned long long* __restrict__ cnt) {
+    const double xo = *x_obs;
+    const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const bool in = c < 2 * (int64_t)n, sb = c >= n;
+    double X = 0.0;
+    if (in) {
+        X = sum_slices(part + c, n_slices, stride);
+        if (xb) (sb ? xsb + (c - n) : xb + c)[0] = X;
     }
+    const unsigned mb = __ballot_sync(0xffffffffu, in && !sb && X <= xo);
+    const unsigned ms = __ballot_sync(0xffffffffu, in && sb && X <= xo);
     if ((threadIdx.x & 31) == 0) {
-        atomicAdd(cnt, a);
-        atomicAdd(cnt + 1, c);
+        if (mb) atomicAdd(cnt, (unsigned long long)__popc(mb));
+        if (ms) atomicAdd(cnt + 1, (unsigned long long)__popc(ms));
     }
 }
 
@@ -273,36 +368,46 @@ __global__ void cls_final_kernel(const unsigned long long* __restrict__ cnt, int
     }
 }
 
-// The CDF tables of the bin means lam (+ add, if given), in stream-ordered
-// allocations the caller frees with cudaFreeAsync.  Synchronises the stream
-// once (the size of the flat table).
-ipa_status build_tables(const double* lam, const double* add, int64_t n_bins, cudaStream_t s, BinTable** tab,
-                        double** F, int64_t* scratch_total, int64_t* host_total);
-
 int grid_for(int64_t work) {
     const int64_t g = (work + kBinBlock - 1) / kBinBlock;
     const int64_t cap = (int64_t)sm_count() * 16;
     return (int)(g < 1 ? 1 : (g > cap ? cap : g));
 }
 
-ipa_status build_tables(const double* lam, const double* add, int64_t n_bins, cudaStream_t s, BinTable** tab,
-                        double** F, int64_t* scratch_total, int64_t* host_total) {
-    *tab = nullptr;
-    *F = nullptr;
-    ipa_status st = cuda_fail(cudaMallocAsync((void**)tab, sizeof(BinTable) * (size_t)n_bins, s), "binned tables");
-    if (st != IPA_OK) return st;
-    table_size_kernel<<<grid_for(n_bins), kBinBlock, 0, s>>>(lam, add, n_bins, *tab);
-    table_offsets_kernel<<<1, 1024, 0, s>>>(*tab, n_bins, scratch_total);
-    if ((st = cuda_fail(cudaMemcpyAsync(host_total, scratch_total, sizeof(int64_t), cudaMemcpyDeviceToHost, s),
-                        "binned table size")) != IPA_OK)
-        return st;
-    if ((st = cuda_fail(cudaStreamSynchronize(s), "binned table size")) != IPA_OK) return st;
-    if ((st = cuda_fail(cudaMallocAsync((void**)F, sizeof(double) * (size_t)(*host_total > 0 ? *host_total : 1), s),
-                        "binned tables")) != IPA_OK)
-        return st;
-    table_fill_kernel<<<grid_for(n_bins), kBinBlock, 0, s>>>(lam, add, n_bins, *tab, *F);
-    return cuda_fail(cudaGetLastError(), "binned table launch");
-}
+// The tables of one histogram (add == nullptr) or of lam and lam + add, in
+// stream-ordered memory.  Synchronises the stream once (the size of the second
+// part; nothing of it is needed where every table fits kTabFixed entries).
+struct Tables {
+    BinTable* tab = nullptr;
+    unsigned long long *T = nullptr, *L = nullptr, *more = nullptr;
+    cudaStream_t s;
+    explicit Tables(cudaStream_t s_) : s(s_) {}
+    ~Tables() {
+        pool_free(tab, s);
+        pool_free(T, s);
+        pool_free(L, s);
+    }
+    ipa_status build(const double* lam, const double* add, int64_t n_bins) {
+        const int n_tab = add ? 2 : 1;
+        const size_t n = (size_t)n_bins * n_tab;
+        ipa_status st = pool_alloc((void**)&tab, sizeof(BinTable) * n, s, "binned tables");
+        if (st == IPA_OK) st = pool_alloc((void**)&T, 8 * (n * kTabFixed + 1), s, "binned tables");
+        if (st != IPA_OK) return st;
+        more = T + n * kTabFixed;
+        if ((st = cuda_fail(cudaMemsetAsync(more, 0, 8, s), "binned table size")) != IPA_OK) return st;
+        const unsigned grid = (unsigned)((n + kTabBlock - 1) / kTabBlock);
+        table_kernel<<<grid, kTabBlock, 0, s>>>(lam, add, n_bins, n_tab, tab, T, more);
+        unsigned long long h = 0;
+        if ((st = cuda_fail(cudaMemcpyAsync(&h, more, 8, cudaMemcpyDeviceToHost, s), "binned table size")) != IPA_OK)
+            return st;
+        if ((st = cuda_fail(cudaStreamSynchronize(s), "binned table size")) != IPA_OK) return st;
+        if (h) {
+            if ((st = pool_alloc((void**)&L, 8 * (size_t)h, s, "binned tables")) != IPA_OK) return st;
+            table_long_kernel<<<grid, kTabBlock, 0, s>>>(lam, add, n_bins, n_tab, tab, L);
+        }
+        return cuda_fail(cudaGetLastError(), "binned table launch");
+    }
+};
 
 }  // namespace
 }  // namespace ipa
@@ -317,23 +422,13 @@ extern "C" ipa_status ipa_binned_generate(const double* lambda_dev, int64_t n_bi
     }
     if (n_bins == 0 || n_toys == 0) return IPA_OK;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    int64_t* total = nullptr;
-    ipa_status st = cuda_fail(cudaMallocAsync((void**)&total, sizeof(int64_t), s), "binned scratch");
+    Tables t(s);
+    ipa_status st = t.build(lambda_dev, nullptr, n_bins);
     if (st != IPA_OK) return st;
-    BinTable* tab = nullptr;
-    double* F = nullptr;
-    int64_t h_total = 0;
-    st = build_tables(lambda_dev, nullptr, n_bins, s, &tab, &F, total, &h_total);
-    if (st == IPA_OK) {
-        generate_kernel<<<grid_for(n_bins * n_toys), kBinBlock, 0, s>>>(tab, F, n_bins, (uint32_t)seed,
-                                                                        (uint32_t)(seed >> 32), hypothesis, toy0,
-                                                                        n_toys, counts_out_dev);
-        st = cuda_fail(cudaGetLastError(), "binned generator launch");
-    }
-    if (F) cudaFreeAsync(F, s);
-    if (tab) cudaFreeAsync(tab, s);
-    cudaFreeAsync(total, s);
-    return st;
+    generate_kernel<<<grid_for(n_bins * n_toys), kBinBlock, 0, s>>>(t.tab, t.T, t.L, n_bins, (uint32_t)seed,
+                                                                    (uint32_t)(seed >> 32), hypothesis, toy0, n_toys,
+                                                                    counts_out_dev);
+    return cuda_fail(cudaGetLastError(), "binned generator launch");
 }
 
 extern "C" ipa_status ipa_binned_smear(const double* hist_dev, int64_t n_bins, double bin_width, double sigma,
@@ -371,37 +466,41 @@ extern "C" ipa_status ipa_cls(const double* s_dev, const double* b_dev, int64_t 
         return IPA_ERR_ARG;
     }
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    const size_t nb = (size_t)n_bins, nt = (size_t)n_toys;
-    // two counters, the table size, w per bin, X per toy (unless the caller keeps them)
-    const size_t bytes = 32 + nb * sizeof(double) + (x_out_dev ? 0 : (2 * nt + 1) * sizeof(double));
-    unsigned char* buf = nullptr;
-    ipa_status st = cuda_fail(cudaMallocAsync((void**)&buf, bytes, s), "cls scratch alloc");
+    Tables t(s);
+    ipa_status st = t.build(b_dev, s_dev, n_bins);
     if (st != IPA_OK) return st;
+    // the toys go in batches whose slice sums take at most kPartBytes
+    constexpr size_t kPartBytes = 48u << 20;
+    const int64_t n_slices = (n_bins + kSlice - 1) / kSlice;
+    int64_t batch = (int64_t)(kPartBytes / (2 * sizeof(double)) / (size_t)n_slices) / kToyBlock * kToyBlock;
+    if (batch < kToyBlock) batch = kToyBlock;
+    if (batch > n_toys) batch = n_toys;
+    const int64_t stride = 2 * batch + 1;
+    // two counters, X_obs, w per bin, the slice sums
+    const size_t bytes = 32 + sizeof(double) * ((size_t)n_bins + (size_t)(n_slices * stride));
+    unsigned char* buf = nullptr;
+    if ((st = pool_alloc((void**)&buf, bytes, s, "cls scratch")) != IPA_OK) return st;
     unsigned long long* cnt = reinterpret_cast<unsigned long long*>(buf);
-    int64_t* total = reinterpret_cast<int64_t*>(buf + 16);
+    double* obs = x_out_dev ? x_out_dev + 2 * (size_t)n_toys : reinterpret_cast<double*>(buf + 16);
     double* w = reinterpret_cast<double*>(buf + 32);
-    double* x = x_out_dev ? x_out_dev : w + nb;
-    const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
-    BinTable *tb = nullptr, *tsb = nullptr;
-    double *Fb = nullptr, *Fsb = nullptr;
-    int64_t h_total = 0;
-    st = build_tables(b_dev, nullptr, n_bins, s, &tb, &Fb, total, &h_total);
-    if (st == IPA_OK) st = build_tables(s_dev, b_dev, n_bins, s, &tsb, &Fsb, total, &h_total);
-    if (st == IPA_OK) {
-        cudaMemsetAsync(cnt, 0, 2 * sizeof(unsigned long long), s);
-        cls_weights_kernel<<<grid_for(n_bins), kBinBlock, 0, s>>>(s_dev, b_dev, n_bins, w);
-        const int gt = n_toys < sm_count() * 8 ? n_toys : sm_count() * 8;
-        cls_toys_kernel<<<gt, kBinBlock, 0, s>>>(tb, Fb, w, n_bins, k0, k1, 0, n_toys, nullptr, x);
-        cls_toys_kernel<<<gt, kBinBlock, 0, s>>>(tsb, Fsb, w, n_bins, k0, k1, 1, n_toys, nullptr, x + nt);
-        cls_toys_kernel<<<1, kBinBlock, 0, s>>>(tb, Fb, w, n_bins, k0, k1, 0, 1, data_dev, x + 2 * nt);
-        cls_count_kernel<<<grid_for(n_toys), kBinBlock, 0, s>>>(x, x + nt, x + 2 * nt, n_toys, cnt);
-        cls_final_kernel<<<1, 1, 0, s>>>(cnt, n_toys, cl_out_dev, counts_out_dev);
-        st = cuda_fail(cudaGetLastError(), "cls launch");
+    double* part = w + n_bins;
+    PhiloxKeys keys(seed);
+    cudaMemsetAsync(cnt, 0, 2 * sizeof(unsigned long long), s);
+    cls_weights_kernel<<<grid_for(n_bins), kBinBlock, 0, s>>>(s_dev, b_dev, n_bins, w);
+    const int64_t data_blocks = (n_slices + kToyBlock - 1) / kToyBlock;
+    for (int64_t k = 0; k < n_toys; k += batch) {
+        const int n = (int)(n_toys - k < batch ? n_toys - k : batch);
+        const int64_t blocks = n_slices * ((n + kToyBlock - 1) / kToyBlock);
+        const int64_t x = k == 0 && data_blocks > blocks ? data_blocks : blocks;
+        cls_slices_kernel<<<dim3((unsigned)x, k == 0 ? 3 : 2), kToyBlock, 0, s>>>(
+            t.tab, t.T, t.L, w, n_bins, n_slices, keys, (int)k, n, data_dev, part, stride);
+        if (k == 0) cls_obs_kernel<<<1, 1, 0, s>>>(part + 2 * n, n_slices, stride, obs);
+        cls_sum_kernel<<<(unsigned)((2 * (int64_t)n + kBinBlock - 1) / kBinBlock), kBinBlock, 0, s>>>(
+            part, n_slices, stride, n, obs, x_out_dev ? x_out_dev + k : nullptr,
+            x_out_dev ? x_out_dev + n_toys + k : nullptr, cnt);
     }
-    if (Fb) cudaFreeAsync(Fb, s);
-    if (tb) cudaFreeAsync(tb, s);
-    if (Fsb) cudaFreeAsync(Fsb, s);
-    if (tsb) cudaFreeAsync(tsb, s);
-    cudaFreeAsync(buf, s);
+    cls_final_kernel<<<1, 1, 0, s>>>(cnt, n_toys, cl_out_dev, counts_out_dev);
+    st = cuda_fail(cudaGetLastError(), "cls launch");
+    pool_free(buf, s);
     return st;
 }

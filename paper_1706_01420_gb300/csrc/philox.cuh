@@ -34,6 +34,30 @@ __device__ __forceinline__ U4 philox(U4 c, uint32_t k0, uint32_t k1) {
     return c;
 }
 
+// The ten rounds' keys laid out beforehand, for kernels that take them as a
+// parameter and read them from the parameter bank (an operand of the rounds'
+// exclusive-ors instead of two additions per round).
+struct PhiloxKeys {
+    uint32_t k[20];
+    PhiloxKeys() = default;
+    explicit PhiloxKeys(uint64_t seed) {
+        for (int r = 0; r < 10; ++r) {
+            k[2 * r] = (uint32_t)seed + (uint32_t)r * kPhiloxW0;
+            k[2 * r + 1] = (uint32_t)(seed >> 32) + (uint32_t)r * kPhiloxW1;
+        }
+    }
+};
+__device__ __forceinline__ U4 keyed(const PhiloxKeys& keys, uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3) {
+    U4 c{c0, c1, c2, c3};
+#pragma unroll
+    for (int r = 0; r < 10; ++r) {
+        const unsigned long long p0 = (unsigned long long)kPhiloxM0 * c.x, p1 = (unsigned long long)kPhiloxM1 * c.z;
+        c = U4{(uint32_t)(p1 >> 32) ^ c.y ^ keys.k[2 * r], (uint32_t)p1,
+               (uint32_t)(p0 >> 32) ^ c.w ^ keys.k[2 * r + 1], (uint32_t)p0};
+    }
+    return c;
+}
+
 // u = ((((a << 32) | b) >> 11) + 1) 2^-53, in (0, 1] (exact).
 __device__ __forceinline__ double u01(uint32_t a, uint32_t b) {
     const unsigned long long v = ((((unsigned long long)a) << 32) | b) >> 11;

@@ -411,7 +411,7 @@ extern "C" ipa_status ipa_toygen(const ipa_model* model, const double* theta_dev
     GenArgs a{};
     a.m = m;
     a.consts = sc->consts;
-    gen_keys(seed, &a);
+    a.keys = PhiloxKeys(seed);
     a.n_toys = n_toys;
     a.n_sig = n_sig_dev;
     a.n_bkg = n_bkg_dev;
