@@ -14,15 +14,30 @@
 //   imaginary part:
 //       -eta s Re b / 2, eta s Re b / 2, D Im b, D eta c Re b
 // (part = Re or Im as the term takes; the products of g+- are written out
-// in ipanema.h).  Per event: the ten f'_k (integer pipe), the four time
-// functions (as in tagged.cu), F_j = sum_k Cq_kj f'_k, P = sum_j F_j G_j + cb.
+// in ipanema.h).
 //
-// Gradient.  Amplitude, phase and mistag parameters act only through C: the
-// pass accumulates S_kj = sum_e r f'_k G_j (40 sums) and the segment's finalise
-// contracts them with dC/dtheta.  The five time parameters act through the G_j:
-// each event adds r sum_j F_j dG_j/dtheta (5 sums, the derivatives written out
-// from dg/dz = (z sigma^2 - tau) g - sigma^2 G, dg/dsigma = z^2 sigma g -
-// (z sigma + tau/sigma) G, dg/dtau = -z g + G).  With Q = sum r: 47 sums.
+// The kernel does not evaluate the 40 entries of C: the terms share four time
+// functions.  A term whose amplitudes have the same CP eigenvalue takes
+// T+ or T-, a mixed one U and V,
+//   T+- = (gL + gH)/2 +- [c (gL - gH)/2 + D s q Im g_c],
+//   U = s (gL - gH)/2 - D c q Im g_c,   V = D q Re g_c:
+//   equal: part(b) T_eta;  real mixed: eta Im b U + Re b V;  imaginary mixed: -eta Re b U + Im b V.
+// Per event: the ten f'_k (integer pipe), the four convolutions (as in
+// tagged.cu), four angular sums F+, F-, FU, FV (14 products instead of 40), and
+// P = F+ T+ + F- T- + FU U + FV V + cb regrouped by convolution.
+//
+// Gradient.  The amplitude and C_SP parameters need the 14 sums of r f'_k times
+// its time functions (40 before).  phi_s: dT+- = -+U, dU = (T+ - T-)/2, one
+// sum of (F- - F+) U + FU dU.  The mistag needs the tag-odd part of the rate, a
+// sum the time parameters need anyway.  These are linear in 14 sums (r times
+// the rate's part of each convolution, plain and times tau, and the Gaussian's):
+// dg/dz = (z sigma^2 - tau) g - sigma^2 G, dg/dsigma = z^2 sigma g - (z sigma +
+// tau/sigma) G, dg/dtau = -z g + G.  With the log and Q = sum r: 31 sums, one per
+// lane once reduced (47 before).
+//
+// Bound: the FP64 pipe.  Fewer operations per event and registers for three
+// blocks per SM in place of two are the gain over the 40-product form; figures at
+// phis_kernel.
 #include <math.h>
 
 #include "accept_reject.cuh"
@@ -45,10 +60,22 @@ constexpr int kPerLane = kTile / 32;
 constexpr int kSub = 4;
 constexpr int kMaxWarps = 8;
 constexpr int kTeam = kPerLane / kSub;   // warps that share a tile: each takes kSub of a lane's events
-constexpr int kNA = 47;          // accumulators with the gradient (n_acc of the phi_s model)
-static_assert(kNA == n_acc(IPA_MODEL_PHIS, true) && kNA <= kMaxAcc, "the scratch must hold the accumulators");
-constexpr int kS = 2;            // first S_kj
-constexpr int kT = 42;           // first time-parameter sum (Gamma, sigma, mu, DG, Dm)
+constexpr int kRow = n_acc(IPA_MODEL_PHIS, true);   // doubles per tile or group partial (the width of a shard's rows)
+constexpr int kNA = 31;          // accumulators with the gradient; the row's other entries are zero
+static_assert(kNA <= 32 && kNA <= kRow && kRow <= kMaxAcc, "one accumulator per lane, rows in the scratch");
+// Accumulators: the log, Q = sum r, the equal terms' sums (order kEq), the mixed
+// terms' sums with U and with V / D (order kMix), phi_s, then the time sums.
+enum {
+    kLog, kQ, kE, kMU = kE + 6, kMV = kMU + 4, kPhi = kMV + 4,
+    kL0, kL1, kH0, kH1,          // r FwL gL, times tau; H likewise
+    kY10, kY11, kY20, kY21,      // r Y1, r Y2 (the tag-odd part and its quadrature), times tau
+    kGa, kGb, kGc, kGd,          // r Gx times FwL, FwH, q FV, q X
+    kGt1, kGt2,                  // r tau Gx times FwL + FwH, q FV
+    kEnd
+};
+static_assert(kEnd == kNA, "accumulator list");
+__device__ const int kEq[6] = {0, 1, 4, 2, 6, 8};    // eta = +1 (three), eta = -1 (three)
+__device__ const int kMix[4] = {3, 5, 7, 9};
 __device__ const double kEta[4] = {1.0, 1.0, -1.0, -1.0};
 
 // (i, j, imaginary part?) of the ten bilinears conj(A_i) A_j (0, para, perp, S)
@@ -86,74 +113,50 @@ __device__ inline void c_row(int k, double pr, double pi, double one, double c, 
     }
 }
 
-// d b_k / d(A0sq, Apesq, delta_pa, delta_pe, F_S, delta_S), parameter a: b_k =
-// m e^{i psi} with the magnitude m a product of square roots and the phase psi
-// a difference of strong phases.
-__device__ inline void b_deriv(const PhisConsts& c, int k, int a, double* dr, double* di) {
-    const double sF = c.rs * c.rs;
-    double dm = 0.0, dpsi = 0.0, m = 0.0, cp = 1.0, sp = 0.0;
-    const double r0 = c.r0, ra = c.ra, re = c.re, rF = c.rF, rs = c.rs;
-    const double rFs = rF * rs, dFs = (1.0 - 2.0 * c.F) / (2.0 * rFs);
-    switch (k) {
-    case 0: m = sF * c.x0; dm = a == 0 ? sF : (a == 4 ? -c.x0 : 0.0); break;
-    case 1: m = sF * c.xa; dm = (a == 0 || a == 1) ? -sF : (a == 4 ? -c.xa : 0.0); break;
-    case 2: m = sF * c.xe; dm = a == 1 ? sF : (a == 4 ? -c.xe : 0.0); break;
-    case 3:   // para, perp: psi = dpe - dpa
-        m = sF * ra * re;
-        dm = a == 0 ? sF * (-c.xe) / (2.0 * ra * re)
-           : a == 1 ? sF * (c.xa - c.xe) / (2.0 * ra * re)
-           : a == 4 ? -ra * re : 0.0;
-        dpsi = a == 2 ? -1.0 : (a == 3 ? 1.0 : 0.0);
-        cp = c.cw[0]; sp = c.sw[0];
-        break;
-    case 4:   // 0, para: psi = dpa
-        m = sF * r0 * ra;
-        dm = a == 0 ? sF * (c.xa - c.x0) / (2.0 * r0 * ra)
-           : a == 1 ? sF * (-c.x0) / (2.0 * r0 * ra)
-           : a == 4 ? -r0 * ra : 0.0;
-        dpsi = a == 2 ? 1.0 : 0.0;
-        cp = c.cw[1]; sp = c.sw[1];
-        break;
-    case 5:   // 0, perp: psi = dpe
-        m = sF * r0 * re;
-        dm = a == 0 ? sF * c.xe / (2.0 * r0 * re)
-           : a == 1 ? sF * c.x0 / (2.0 * r0 * re)
-           : a == 4 ? -r0 * re : 0.0;
-        dpsi = a == 3 ? 1.0 : 0.0;
-        cp = c.cw[2]; sp = c.sw[2];
-        break;
-    case 6: m = c.F; dm = a == 4 ? 1.0 : 0.0; break;
-    case 7:   // S, para: psi = dpa - dS
-        m = rFs * ra;
-        dm = (a == 0 || a == 1) ? -rFs / (2.0 * ra) : (a == 4 ? dFs * ra : 0.0);
-        dpsi = a == 2 ? 1.0 : (a == 5 ? -1.0 : 0.0);
-        cp = c.cw[3]; sp = c.sw[3];
-        break;
-    case 8:   // S, perp: psi = dpe - dS
-        m = rFs * re;
-        dm = a == 1 ? rFs / (2.0 * re) : (a == 4 ? dFs * re : 0.0);
-        dpsi = a == 3 ? 1.0 : (a == 5 ? -1.0 : 0.0);
-        cp = c.cw[4]; sp = c.sw[4];
-        break;
-    default:  // S, 0: psi = -dS
-        m = rFs * r0;
-        dm = a == 0 ? rFs / (2.0 * r0) : (a == 4 ? dFs * r0 : 0.0);
-        dpsi = a == 5 ? -1.0 : 0.0;
-        cp = c.cw[5]; sp = -c.sw[5];
-        break;
+// The ten f'_k on the integer pipe, rounded once to double (as in the 4D kernel:
+// 35 FP64 instructions less per event; worth 2 % here), in FP64 near |cos| = 1.
+__device__ __forceinline__ void phis_basis(double ck, double cl, double phi, const MathTables* mt, double f[10]) {
+    if (basis_q62_ok(ck, cl, phi)) {
+        long long F[10];
+        basis_q62(ck, cl, phi, mt, F);
+#pragma unroll
+        for (int k = 0; k < 10; ++k) f[k] = q62_to_double_nb(F[k], 0);
+    } else {
+        basis_unscaled(ck, cl, phi, mt, f);
     }
-    *dr = dm * cp - m * dpsi * sp;
-    *di = dm * sp + m * dpsi * cp;
 }
 
-// Per-warp copy: the record and Cq_kj = (cs / 2) C_kj c_k (the basis factor c_k
-// for the unscaled f'_k, 1 for a cached basis; 1/2 for the doubled G).
+// Per-warp copy: the record and the coefficients of the angular sums, with cs / 4
+// (P from the doubled convolutions, and the halves of T and U), the basis factor
+// c_k (1 for a cached basis) and C_SP folded in.
 struct PhisWarp {
     PhisConsts c;
-    double cq[40];
+    double eq[6], mu[4], mv[4];
+    double D2, D2s, D2c;      // 2 D, 2 D s, 2 D c
 };
 
-// One event: log term and, with GRAD, the 45 sums.  G2 = 2 G (doubled as in tagged.cu).
+__device__ __forceinline__ void phis_coefficients(PhisWarp& pw, bool cached, int lane) {
+    const PhisConsts& c = pw.c;
+    if (lane < 10) {
+        const int k = lane < 6 ? kEq[lane] : kMix[lane - 6];
+        const double sc = 0.25 * c.cs * row_scale(c, k) * (cached ? 1.0 : kBasisScale[k]);
+        const double re = kPairIm[k] ? c.bi[k] : c.br[k];
+        if (lane < 6) {
+            pw.eq[lane] = sc * re;
+        } else {
+            const double ej = kEta[kPairJ[k]];
+            pw.mu[lane - 6] = sc * (kPairIm[k] ? -ej * c.br[k] : ej * c.bi[k]);
+            pw.mv[lane - 6] = sc * re;
+        }
+    } else if (lane == 10) {
+        pw.D2 = 2.0 * c.D;
+        pw.D2s = 2.0 * c.D * c.s;
+        pw.D2c = 2.0 * c.D * c.c;
+    }
+}
+
+// One event: log term and, with GRAD, the sums.  The convolutions are doubled
+// (as in tagged.cu).
 template <bool GRAD, bool WEIGHTED>
 __device__ __forceinline__ void phis_event(const PhisWarp& pw, const MathTables* mt, double t, double q, double w,
                                            const double* f, const TagSlow& sl, double* acc, double* prod,
@@ -167,133 +170,165 @@ __device__ __forceinline__ void phis_event(const PhisWarp& pw, const MathTables*
     sincos_int_wide(fma(c.Dm, tau, -c.ph0), mt, &sn, &cn);
     const long long bH = __double_as_longlong(sl.xH), bL = __double_as_longlong(sl.xL);
     const long long bG = __double_as_longlong(sl.gx);
-    const double T2H = bH < 0 ? -sl.xH : E2H - sl.xH;
-    const double T2L = bL < 0 ? -sl.xL : E2L - sl.xL;
-    const double Cr = bG < 0 ? sl.wr : fma(E2C, cn, -sl.wr);
-    const double Ci = bG < 0 ? sl.wi : fma(E2C, sn, -sl.wi);
-    const double gx = __longlong_as_double(bG & 0x7FFFFFFFFFFFFFFFll);
-    const double G2[4] = {T2L, T2H, q * Cr, q * Ci};
-    double Fw[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        double v = pw.cq[j] * f[0];
-#pragma unroll
-        for (int k = 1; k < 10; ++k) v = fma(pw.cq[4 * k + j], f[k], v);
-        Fw[j] = v;
-    }
-    const double P = fma(Fw[0], G2[0], fma(Fw[1], G2[1], fma(Fw[2], G2[2], fma(Fw[3], G2[3], c.cb))));
+    const double H = bH < 0 ? -sl.xH : E2H - sl.xH;
+    const double L = bL < 0 ? -sl.xL : E2L - sl.xL;
+    const double Cr = q * (bG < 0 ? sl.wr : fma(E2C, cn, -sl.wr));
+    const double Ci = q * (bG < 0 ? sl.wi : fma(E2C, sn, -sl.wi));
+    // F+, F-, FU, FV; the rate's coefficients of L and H, and of D2 Ci (X)
+    const double Fp = fma(pw.eq[2], f[4], fma(pw.eq[1], f[1], pw.eq[0] * f[0]));
+    const double Fm = fma(pw.eq[5], f[8], fma(pw.eq[4], f[6], pw.eq[3] * f[2]));
+    const double FU = fma(pw.mu[3], f[9], fma(pw.mu[2], f[7], fma(pw.mu[1], f[5], pw.mu[0] * f[3])));
+    const double FV = fma(pw.mv[3], f[9], fma(pw.mv[2], f[7], fma(pw.mv[1], f[5], pw.mv[0] * f[3])));
+    const double Fs = Fp + Fm, Fd = Fp - Fm;
+    const double hd = fma(c.c, Fd, c.s * FU);
+    const double FL = Fs + hd, FH = Fs - hd;
+    const double X = fma(c.s, Fd, -(c.c * FU));
+    const double Y1 = fma(Cr, FV, Ci * X);
+    const double P = fma(FL, L, fma(FH, H, fma(pw.D2, Y1, c.cb)));
     if (WEIGHTED && __double_as_longlong(w) != 0x3FF0000000000000ll)
-        acc[0] = fma(w, log_fast(P, mt), acc[0]);
+        acc[kLog] = fma(w, log_fast(P, mt), acc[kLog]);
     else
         log_mul(P, prod, esum);
     if (!GRAD) return;
     const double r = WEIGHTED ? w * rcp_newton(P) : rcp_newton(P);
-    acc[1] += r;
-    double rG[4];
+    acc[kQ] += r;
+    const double sG = L + H, dG = L - H;
+    const double m = fma(c.c, dG, pw.D2s * Ci);       // (T+ - T-)/2 and dU/dphi_s, four times
+    const double rp = r * (sG + m), rm = r * (sG - m);
+    const double u = fma(c.s, dG, -(pw.D2c * Ci));    // U, four times
+    const double ru = r * u, rv = r * Cr;
+    acc[kE + 0] = fma(rp, f[0], acc[kE + 0]);
+    acc[kE + 1] = fma(rp, f[1], acc[kE + 1]);
+    acc[kE + 2] = fma(rp, f[4], acc[kE + 2]);
+    acc[kE + 3] = fma(rm, f[2], acc[kE + 3]);
+    acc[kE + 4] = fma(rm, f[6], acc[kE + 4]);
+    acc[kE + 5] = fma(rm, f[8], acc[kE + 5]);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) rG[j] = r * G2[j];
-#pragma unroll
-    for (int k = 0; k < 10; ++k)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[kS + 4 * k + j] = fma(f[k], rG[j], acc[kS + 4 * k + j]);
-    // derivatives of the doubled time functions; G2g = 2 G (the Gaussian density)
-    const double G2g = 2.0 * c.cG * gx;
-    const double s2 = c.s2, sg = c.sigma, its = tau * c.inv_s;
-    const double dL_G = fma(c.GL * s2 - tau, T2L, -s2 * G2g);
-    const double dH_G = fma(c.GH * s2 - tau, T2H, -s2 * G2g);
-    const double dL_s = fma(c.GL * c.GL * sg, T2L, -(c.GL * sg + its) * G2g);
-    const double dH_s = fma(c.GH * c.GH * sg, T2H, -(c.GH * sg + its) * G2g);
-    const double dL_t = fma(-c.GL, T2L, G2g);
-    const double dH_t = fma(-c.GH, T2H, G2g);
-    // complex: z = Gamma - i Dm
-    const double a0 = c.Gamma * s2 - tau, dms2 = c.Dm * s2;
-    const double zr = fma(a0, Cr, fma(dms2, Ci, -s2 * G2g));       // Re d(2g_c)/dz
-    const double zi = fma(a0, Ci, -dms2 * Cr);                      // Im d(2g_c)/dz
-    const double g2 = (c.Gamma - c.Dm) * (c.Gamma + c.Dm), gd2 = 2.0 * c.Gamma * c.Dm;
-    const double sr = fma(sg, fma(g2, Cr, gd2 * Ci), -(c.Gamma * sg + its) * G2g);   // Re d/dsigma
-    const double si = fma(sg, fma(g2, Ci, -gd2 * Cr), c.Dm * sg * G2g);               // Im d/dsigma
-    const double tr = -fma(c.Gamma, Cr, c.Dm * Ci) + G2g;                               // Re d/dtau
-    const double ti = -fma(c.Gamma, Ci, -c.Dm * Cr);                                    // Im d/dtau
-    const double qF2 = q * Fw[2], qF3 = q * Fw[3];
-    const double dG = fma(Fw[0], dL_G, fma(Fw[1], dH_G, fma(qF2, zr, qF3 * zi)));
-    const double dS = fma(Fw[0], dL_s, fma(Fw[1], dH_s, fma(qF2, sr, qF3 * si)));
-    const double dT = -fma(Fw[0], dL_t, fma(Fw[1], dH_t, fma(qF2, tr, qF3 * ti)));
-    const double dDG = 0.5 * fma(Fw[0], dL_G, -Fw[1] * dH_G);
-    const double dDm = fma(qF2, zi, -qF3 * zr);                     // d/dDm = -i d/dz
-    acc[kT + 0] = fma(r, dG, acc[kT + 0]);
-    acc[kT + 1] = fma(r, dS, acc[kT + 1]);
-    acc[kT + 2] = fma(r, dT, acc[kT + 2]);
-    acc[kT + 3] = fma(r, dDG, acc[kT + 3]);
-    acc[kT + 4] = fma(r, dDm, acc[kT + 4]);
+    for (int i = 0; i < 4; ++i) {
+        acc[kMU + i] = fma(ru, f[3 + 2 * i], acc[kMU + i]);
+        acc[kMV + i] = fma(rv, f[3 + 2 * i], acc[kMV + i]);
+    }
+    acc[kPhi] = fma(r * m, FU, fma(-ru, Fd, acc[kPhi]));
+    const double hL = (r * FL) * L, hH = (r * FH) * H;
+    acc[kL0] += hL;
+    acc[kL1] = fma(hL, tau, acc[kL1]);
+    acc[kH0] += hH;
+    acc[kH1] = fma(hH, tau, acc[kH1]);
+    const double y1 = r * Y1, y2 = r * fma(Ci, FV, -(Cr * X));
+    acc[kY10] += y1;
+    acc[kY11] = fma(y1, tau, acc[kY11]);
+    acc[kY20] += y2;
+    acc[kY21] = fma(y2, tau, acc[kY21]);
+    const double g = r * __longlong_as_double(bG & 0x7FFFFFFFFFFFFFFFll), gq = g * q, gt = g * tau;
+    acc[kGa] = fma(g, FL, acc[kGa]);
+    acc[kGb] = fma(g, FH, acc[kGb]);
+    acc[kGc] = fma(gq, FV, acc[kGc]);
+    acc[kGd] = fma(gq, X, acc[kGd]);
+    acc[kGt1] = fma(gt, Fs, acc[kGt1]);               // (FL + FH) / 2
+    acc[kGt2] = fma(gq * tau, FV, acc[kGt2]);
 }
 
-// NLL and gradient of one segment (every lane holds acc; lane j writes
-// component j).  With S2_kj = c_k S_kj (the scaled basis), SR = sum r rate =
-// (1/2) sum_kj C_kj S2_kj, the time sums D_t = cs sum r d rate / d theta_t:
-//   time parameters:            -D_t + cs dlnN_t SR,
-//   f_b:                        SR / N - Q / V,
-//   amplitudes, phi_s, omega, C_SP:  -(cs/2) sum_kj dC_kj/dtheta S2_kj + cs dlnN SR
-// (C rows 7, 8, 9 carry C_SP).
+// NLL and gradient of one segment; lane a holds accumulator a in v, lane j writes
+// component j.  Term k's share of the rate's sum, R_k = sum r f_k (its time
+// function times its part of b_k), and R'_k, the same with i b_k for b_k, come
+// from the 14 sums, one per lane.  With |A_i|^2 = X_i (X = (1 - F_S) x_i for the P
+// wave, F_S for the S wave) every term is sqrt(X_i X_j) e^{i psi} times functions
+// of other parameters: with Z_i the sum of R_k over the amplitudes i of the terms
+// (twice for |A_i|^2),
+//   dR/dA0sq = (Z_0 / x_0 - Z_pa / x_pa) / 2,  dR/dApesq = (Z_pe / x_pe - Z_pa / x_pa) / 2,
+//   dR/dF_S = (Z_S / F_S - (Z_0 + Z_pa + Z_pe) / (1 - F_S)) / 2,
+// and the phases' derivatives are sums of +-R'_k.  Then
+//   dNLL/dtheta = -cs dR/dtheta + cs dlnN/dtheta SR,  SR = sum_k R_k,
+//   dNLL/df_b = SR / N - Q / V.
 template <bool GRAD, bool CACHED>
-__device__ __forceinline__ void phis_finalize(const PhisConsts& c, const double* acc, int n_par, double* out, int lane) {
-    if (lane == 0) out[0] = -acc[0];
+__device__ __forceinline__ void phis_finalize(const PhisConsts& c, double v, int n_par, double* out, int lane) {
+    if (lane == 0) out[0] = -v;
     if (!GRAD) return;
-    // (loops unrolled: acc stays in registers)
-    double SR = 0.0;
-#pragma unroll
-    for (int k = 0; k < 10; ++k) {
-        double row[4];
-        c_row(k, c.br[k], c.bi[k], 1.0, c.c, c.s, 1.0, c.D, row);
-        const double sc = row_scale(c, k) * (CACHED ? 1.0 : kBasisScale[k]);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) SR = fma(row[j], sc * acc[kS + 4 * k + j], SR);
+    constexpr unsigned kAll = 0xffffffffu;
+    auto A = [&](int i) { return __shfl_sync(kAll, v, i); };
+    const double D2 = 2.0 * c.D;
+    // lanes 0-9: R_k; 10-15: R'_k of k = 3, 4, 5, 7, 8, 9; 16-18: R_k / C_SP of k = 7, 8, 9
+    double R;
+    {
+        const int pk = lane - 10;
+        const int k = lane < 10 ? lane : (lane < 16 ? (pk < 3 ? 3 + pk : 4 + pk) : (lane < 19 ? lane - 9 : 0));
+        const bool prime = lane >= 10 && lane < 16;
+        const double re = prime ? -c.bi[k] : c.br[k], im = prime ? c.br[k] : c.bi[k];
+        const double ej = kEta[kPairJ[k]];
+        const bool equal = kEta[kPairI[k]] == ej;
+        const int e = k == 0 ? 0 : (k == 1 ? 1 : (k == 4 ? 2 : (k == 2 ? 3 : (k == 6 ? 4 : 5))));
+        const double S1 = __shfl_sync(kAll, v, equal ? kE + e : kMU + ((k - 3) >> 1));
+        const double S2 = __shfl_sync(kAll, v, equal ? kE : kMV + ((k - 3) >> 1));
+        const double part = kPairIm[k] ? im : re;
+        const double a1 = equal ? part : (kPairIm[k] ? -ej * re : ej * im);
+        const double sc = 0.25 * (lane >= 16 ? 1.0 : row_scale(c, k)) * (CACHED ? 1.0 : kBasisScale[k]);
+        R = sc * (equal ? a1 * S1 : fma(a1, S1, (part * D2) * S2));
     }
-    SR *= 0.5;
+    double Rk[10];
+#pragma unroll
+    for (int k = 0; k < 10; ++k) Rk[k] = __shfl_sync(kAll, R, k);
+    const double SR = (((Rk[0] + Rk[1]) + (Rk[2] + Rk[3])) + ((Rk[4] + Rk[5]) + (Rk[6] + Rk[7]))) + (Rk[8] + Rk[9]);
     const double csSR = c.cs * SR;
-    if (lane >= IPA_NPAR_PHIS) {
-        for (int j = lane; j < n_par; j += 32) out[1 + j] = 0.0;
-        return;
+    const double p3 = __shfl_sync(kAll, R, 10), p4 = __shfl_sync(kAll, R, 11), p5 = __shfl_sync(kAll, R, 12);
+    const double p7 = __shfl_sync(kAll, R, 13), p8 = __shfl_sync(kAll, R, 14), p9 = __shfl_sync(kAll, R, 15);
+    const double csp = __shfl_sync(kAll, R, 16) + __shfl_sync(kAll, R, 17) + __shfl_sync(kAll, R, 18);
+    const double inv = 1.0 / (lane == 0 ? c.x0 : (lane == 1 ? c.xa : (lane == 2 ? c.xe : (lane == 3 ? c.F : 1.0 - c.F))));
+    const double i0 = __shfl_sync(kAll, inv, 0), ia = __shfl_sync(kAll, inv, 1), ie = __shfl_sync(kAll, inv, 2);
+    const double iF = __shfl_sync(kAll, inv, 3), iP = __shfl_sync(kAll, inv, 4);
+    const double Z0 = fma(2.0, Rk[0], (Rk[4] + Rk[5]) + Rk[9]), Za = fma(2.0, Rk[1], (Rk[3] + Rk[4]) + Rk[7]);
+    const double Ze = fma(2.0, Rk[2], (Rk[3] + Rk[5]) + Rk[8]), ZS = fma(2.0, Rk[6], (Rk[7] + Rk[8]) + Rk[9]);
+    const double Q = A(kQ), phi = A(kPhi);
+    const double L0 = A(kL0), L1 = A(kL1), H0 = A(kH0), H1 = A(kH1);
+    const double y10 = A(kY10);
+    const double Y10 = D2 * y10, Y11 = D2 * A(kY11), Y20 = D2 * A(kY20), Y21 = D2 * A(kY21);
+    const double kk = 2.0 * c.cG;
+    const double ga = kk * A(kGa), gb = kk * A(kGb), gc = (kk * D2) * A(kGc), gd = (kk * D2) * A(kGd);
+    const double gt = kk * fma(2.0, A(kGt1), D2 * A(kGt2));
+    double d = 0.0;      // cs sum r dR/dtheta of the lane's parameter
+    if (lane == IPA_GAMMA) {
+        d = c.s2 * ((c.GL * L0 + c.GH * H0) + (c.Gamma * Y10 + c.Dm * Y20) - ((ga + gb) + gc)) - ((L1 + H1) + Y11);
+    } else if (lane == IPA_SIGMA) {
+        const double g2 = (c.Gamma - c.Dm) * (c.Gamma + c.Dm), gd2 = 2.0 * c.Gamma * c.Dm;
+        d = c.sigma * ((c.GL * (c.GL * L0 - ga) + c.GH * (c.GH * H0 - gb)) + (g2 * Y10 + gd2 * Y20) -
+                       (c.Gamma * gc - c.Dm * gd)) - c.inv_s * gt;
+    } else if (lane == IPA_MU) {
+        d = (c.GL * L0 + c.GH * H0) + (c.Gamma * Y10 + c.Dm * Y20) - ((ga + gb) + gc);
+    } else if (lane == IPA_PHIS_DG) {
+        d = 0.5 * (c.s2 * ((c.GL * L0 - c.GH * H0) - (ga - gb)) - (L1 - H1));
+    } else if (lane == IPA_PHIS_DM) {
+        d = c.s2 * ((c.Gamma * Y20 - c.Dm * Y10) + gd) - Y21;
+    } else if (lane == IPA_A0SQ) {
+        d = 0.5 * c.cs * (Z0 * i0 - Za * ia);
+    } else if (lane == IPA_APESQ) {
+        d = 0.5 * c.cs * (Ze * ie - Za * ia);
+    } else if (lane == IPA_DPA) {
+        d = c.cs * ((p4 + p7) - p3);
+    } else if (lane == IPA_DPE) {
+        d = c.cs * ((p3 + p5) + p8);
+    } else if (lane == IPA_FS) {
+        d = 0.5 * c.cs * (ZS * iF - ((Z0 + Za) + Ze) * iP);
+    } else if (lane == IPA_DS) {
+        d = c.cs * (-((p7 + p8) + p9));
+    } else if (lane == IPA_PHIS_PHIS) {
+        d = phi;
+    } else if (lane == IPA_PHIS_OMEGA) {
+        d = -4.0 * y10;
+    } else if (lane == IPA_PHIS_CSP) {
+        d = c.cs * (csp);
     }
-    double v;
-    if (lane == IPA_FB) {
-        v = fma(SR, c.inv_N, -acc[1] * c.inv_V);
-    } else if (lane == IPA_PHIS_QNORM) {
-        v = 0.0;
-    } else if (lane < 3 || lane == IPA_PHIS_DG || lane == IPA_PHIS_DM) {
-        // register operands only (an index computed from the lane would put acc in local memory)
-        const double Dt = lane == 0 ? acc[kT] : lane == 1 ? acc[kT + 1] : lane == 2 ? acc[kT + 2]
-                        : lane == IPA_PHIS_DG ? acc[kT + 3] : acc[kT + 4];
-        v = fma(c.dlnN[lane], csSR, -Dt);
-    } else {
-        double dsum = 0.0;
-#pragma unroll
-        for (int k = 0; k < 10; ++k) {
-            double row[4];
-            double rs = row_scale(c, k);
-            if (lane == IPA_PHIS_PHIS) {
-                c_row(k, c.br[k], c.bi[k], 0.0, -c.s, c.c, 1.0, c.D, row);
-            } else if (lane == IPA_PHIS_OMEGA) {
-                c_row(k, c.br[k], c.bi[k], 1.0, c.c, c.s, 0.0, -2.0, row);
-            } else if (lane == IPA_PHIS_CSP) {
-                c_row(k, c.br[k], c.bi[k], 1.0, c.c, c.s, 1.0, c.D, row);
-                rs = k >= 7 ? 1.0 : 0.0;
-            } else {
-                double dr, di;
-                b_deriv(c, k, lane - IPA_A0SQ, &dr, &di);
-                c_row(k, dr, di, 1.0, c.c, c.s, 1.0, c.D, row);
-            }
-            const double sc = rs * (CACHED ? 1.0 : kBasisScale[k]);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) dsum = fma(row[j], sc * acc[kS + 4 * k + j], dsum);
-        }
-        v = fma(c.dlnN[lane], csSR, -0.5 * c.cs * dsum);
-    }
-    out[1 + lane] = v;
+    if (lane < IPA_NPAR_PHIS)
+        out[1 + lane] = lane == IPA_FB ? fma(SR, c.inv_N, -Q * c.inv_V)
+                        : (lane == IPA_PHIS_QNORM ? 0.0 : fma(c.dlnN[lane], csSR, -d));
     for (int j = IPA_NPAR_PHIS + lane; j < n_par; j += 32) out[1 + j] = 0.0;
 }
 
+// Three blocks per SM (164 registers, no spills) over two (200): 404 -> 367 us for
+// 1e6 events, and four (128 registers, spills) 392 us.  The 40-product form with
+// its 47 sums took 623 us at two blocks (237 registers).  A tile's team is the
+// block's four warps (each takes 4 of every lane's 16 events), so that a small
+// fit's tiles run four FP64 instruction streams at once.
 template <bool GRAD, bool WEIGHTED, bool CACHED>
-__global__ void __launch_bounds__(32 * kTeam, 1)
+__global__ void __launch_bounds__(32 * kTeam, 3)
 phis_kernel(Cols cols, int64_t n, const int64_t* __restrict__ seg_begin, const int64_t* __restrict__ seg_end,
             const int64_t* __restrict__ seg_tiles, int n_seg, const Consts* __restrict__ consts,
             double* __restrict__ partials, unsigned* __restrict__ counters, unsigned* __restrict__ gcount,
@@ -301,15 +336,13 @@ phis_kernel(Cols cols, int64_t n, const int64_t* __restrict__ seg_begin, const i
     constexpr int NA = GRAD ? kNA : 1;
     const int out_stride = GRAD ? 1 + n_par : 1;
     __shared__ MathTables mt;
-    __shared__ int64_t s_take;
+    __shared__ int64_t s_take[2];
+    __shared__ double xbuf[2][kTeam][32];
     extern __shared__ __align__(16) unsigned char dyn_smem[];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int n_wib = kTeam;
     TagSlow* const sbuf = reinterpret_cast<TagSlow*>(dyn_smem) + wib * (kSub * 32);
     PhisWarp& pw = reinterpret_cast<PhisWarp*>(dyn_smem + (size_t)n_wib * kSub * 32 * sizeof(TagSlow))[wib];
-    double* const xbuf = reinterpret_cast<double*>(dyn_smem + (size_t)n_wib * (kSub * 32 * sizeof(TagSlow) +
-                                                                               sizeof(PhisWarp)));
-    double* const xtot = xbuf + (size_t)kTeam * NA * 32;
 
     load_math_tables(&mt);
     __syncthreads();
@@ -325,13 +358,15 @@ phis_kernel(Cols cols, int64_t n, const int64_t* __restrict__ seg_begin, const i
         }
     }
 
-    int cur = -1;
-    while (true) {
-        // the team (the block's four warps) takes tiles together
-        if (threadIdx.x == 0) s_take = (int64_t)atomicAdd(work, 1u) * per_take;
-        __syncthreads();
-        const int64_t first = s_take;
-        __syncthreads();
+    // The team (the block's four warps) takes tiles together; the next take is
+    // fetched while the last tile of one is in work.  s_take and xbuf are used in
+    // turns, so that one barrier per tile orders their writes after the reads of
+    // the turn before.
+    int cur = -1, turn = 0, par = 0;
+    if (threadIdx.x == 0) s_take[0] = (int64_t)atomicAdd(work, 1u) * per_take;
+    __syncthreads();
+    for (;; turn ^= 1) {
+        const int64_t first = s_take[turn];
         if (first >= total) break;
         const int64_t stop = first + per_take < total ? first + per_take : total;
         for (int64_t tile = first; tile < stop; ++tile) {
@@ -351,12 +386,7 @@ phis_kernel(Cols cols, int64_t n, const int64_t* __restrict__ seg_begin, const i
                 double* dst = reinterpret_cast<double*>(&pw.c);
                 for (int i = lane; i < kPhisDoubles; i += 32) dst[i] = __ldg(src + i);
                 __syncwarp();
-                if (lane < 10) {
-                    double row[4];
-                    c_row(lane, pw.c.br[lane], pw.c.bi[lane], 1.0, pw.c.c, pw.c.s, 1.0, pw.c.D, row);
-                    const double sc = 0.5 * pw.c.cs * row_scale(pw.c, lane) * (CACHED ? 1.0 : kBasisScale[lane]);
-                    for (int j = 0; j < 4; ++j) pw.cq[4 * lane + j] = sc * row[j];
-                }
+                phis_coefficients(pw, CACHED, lane);
                 __syncwarp();
                 cur = seg;
             }
@@ -409,7 +439,7 @@ phis_kernel(Cols cols, int64_t n, const int64_t* __restrict__ seg_begin, const i
 #pragma unroll
                             for (int kk = 0; kk < 10; ++kk) f[kk] = __ldg(cols.fk + kk * cols.fk_stride + e);
                         } else {
-                            basis_unscaled(__ldg(cols.ck + e), __ldg(cols.cl + e), __ldg(cols.phi + e), &mt, f);
+                            phis_basis(__ldg(cols.ck + e), __ldg(cols.cl + e), __ldg(cols.phi + e), &mt, f);
                         }
                         phis_event<GRAD, WEIGHTED>(pw, &mt, __ldg(cols.t + e), __ldg(cols.q + e), w, f, sl, acc,
                                                    &prod, &esum);
@@ -418,30 +448,20 @@ phis_kernel(Cols cols, int64_t n, const int64_t* __restrict__ seg_begin, const i
                 __syncwarp();
             }
             acc[0] += log_of(prod, esum, &mt);
-            // every warp's sums to shared memory; warp w then reduces accumulators
-            // w, w + 4, ...: the team's four values lane by lane in warp order, then
-            // the xor butterfly over the lanes (the reduction work spread over the
-            // four sub-partitions); warp 0 commits the tile
-#pragma unroll
-            for (int a = 0; a < NA; ++a) xbuf[(wib * NA + a) * 32 + lane] = acc[a];
-            __syncthreads();
-            for (int a = wib; a < NA; a += kTeam) {
-                double v = xbuf[a * 32 + lane];
-                for (int w = 1; w < kTeam; ++w) v += xbuf[(w * NA + a) * 32 + lane];
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-                if (lane == 0) xtot[a] = v;
-            }
+            // each warp reduces its lanes (lane a ends with accumulator a), and warp 0
+            // adds the team's four in warp order and commits the tile
+            xbuf[par][wib][lane] = warp_butterfly<NA>(acc, lane);
+            if (threadIdx.x == 32 * (kTeam - 1) && tile + 1 == stop)
+                s_take[turn ^ 1] = (int64_t)atomicAdd(work, 1u) * per_take;
             __syncthreads();
             if (wib == 0) {
-#pragma unroll
-                for (int a = 0; a < NA; ++a) acc[a] = xtot[a];
-                if (tile_commit_wide<NA>(lane, tile, t0, t1, seg, partials, gcount, counters, acc)) {
-                    phis_finalize<GRAD, CACHED>(pw.c, acc, n_par, out + (size_t)seg * out_stride, lane);
+                double v = ((xbuf[par][0][lane] + xbuf[par][1][lane]) + xbuf[par][2][lane]) + xbuf[par][3][lane];
+                if (row_commit<NA, GRAD ? kRow : 1>(lane, tile, t0, t1, seg, partials, gcount, counters, &v)) {
+                    phis_finalize<GRAD, CACHED>(pw.c, v, n_par, out + (size_t)seg * out_stride, lane);
                     if (lane == 0) counters[seg] = 0u;
                 }
             }
-            __syncthreads();
+            par ^= 1;
         }
     }
     work_done(work, lane);
@@ -453,7 +473,7 @@ ipa_status launch_phis_t(const Cols& cols, int64_t n, const int64_t* seg_begin, 
                          int n_par, cudaStream_t st, const LaunchCfg* force) {
     const bool single = seg_begin == nullptr;
     const int64_t tiles = tile_estimate(n, n_seg);
-    if (GRAD && single && sc->partials_cap < (size_t)((n + kTile - 1) / kTile) * kNA) {
+    if (GRAD && single && sc->partials_cap < (size_t)((n + kTile - 1) / kTile) * kRow) {
         set_error("phi_s likelihood: the scratch holds too few accumulators per tile");
         return IPA_ERR_ARG;
     }
@@ -463,8 +483,7 @@ ipa_status launch_phis_t(const Cols& cols, int64_t n, const int64_t* seg_begin, 
     const int W = kTeam;
     const int K = cfg.tiles_per_take >= 1 ? cfg.tiles_per_take : 1;
     const size_t per_warp = sizeof(PhisWarp) + kSub * 32 * sizeof(TagSlow);
-    constexpr int NA = GRAD ? kNA : 1;
-    const size_t smem = (size_t)W * per_warp + ((size_t)kTeam * NA * 32 + NA) * sizeof(double);
+    const size_t smem = (size_t)W * per_warp;
     auto kern = phis_kernel<GRAD, WEIGHTED, CACHED>;
     static bool attr[64] = {};
     static int occ[64][kMaxWarps + 1] = {};
@@ -812,19 +831,17 @@ ipa_status launch_phis_toygen(const GenArgs& a, cudaStream_t s) { return launch_
 
 namespace {
 // ipa_nll_grad_combine for the phi_s model: the kernel's last reduction level
-// (the wide form) over gathered group partials, then phis_finalize (one warp).
+// over gathered group partials, then phis_finalize (one warp).
 template <bool CACHED>
 __global__ void phis_combine_kernel(const double* __restrict__ groups, int64_t n_groups,
                                     const Consts* __restrict__ consts, int n_par, double* __restrict__ out) {
-    constexpr int NA = n_acc(IPA_MODEL_PHIS, true);
     const int lane = threadIdx.x & 31;
     if (n_groups == 0) {
         for (int j = lane; j < 1 + n_par; j += 32) out[j] = 0.0;
         return;
     }
-    double acc[NA];
-    reduce_partials_wide<NA>(groups, 0, n_groups, 1, acc);
-    phis_finalize<true, CACHED>(*reinterpret_cast<const PhisConsts*>(consts), acc, n_par, out, lane);
+    const double v = sum_rows<kNA, kRow>(groups, 0, n_groups, 1, lane);
+    phis_finalize<true, CACHED>(*reinterpret_cast<const PhisConsts*>(consts), v, n_par, out, lane);
 }
 }  // namespace
 
