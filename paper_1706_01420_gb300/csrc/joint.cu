@@ -35,13 +35,18 @@ __global__ void joint_scatter_kernel(JointDev j, int n_fits, const double* __res
     j.theta_seg[s * j.n_model + p] = q >= 0 ? theta_joint[i * j.n_joint + q] : j.value[c * j.n_model + p];
 }
 
-// One thread per (fit, output): output 0 is the NLL, sum over c of NLL_c;
+// One warp per (fit, output): output 0 is the NLL, sum over c of NLL_c;
 // output 1 + q the sum over (c, p) with map[c][p] = q of dNLL_c/dtheta_c[p],
 // both in the order c ascending, then p ascending.  Without the gradient, one
-// thread per fit.
-__global__ void joint_gather_kernel(JointDev j, int n_fits, const int* __restrict__ active,
-                                    double* __restrict__ res_joint) {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+// warp per fit.  The lanes load 32 entries of the map at once and their matches'
+// results, and the matches are added one after another by shuffles: with a
+// thread per output that walked the map entry by entry, twelve categories of 16
+// parameters were 192 dependent loads (21 us of Example 2's pass, cold; now 5.7).
+constexpr int kGatherBlock = 128;
+__global__ void __launch_bounds__(kGatherBlock)
+joint_gather_kernel(JointDev j, int n_fits, const int* __restrict__ active, double* __restrict__ res_joint) {
+    const int lane = threadIdx.x & 31;
+    const int64_t idx = ((int64_t)blockIdx.x * kGatherBlock + threadIdx.x) >> 5;
     const int n_out = j.grad ? 1 + j.n_joint : 1;
     if (idx >= (int64_t)n_fits * n_out) return;
     const int64_t i = idx / n_out;
@@ -49,16 +54,24 @@ __global__ void joint_gather_kernel(JointDev j, int n_fits, const int* __restric
     if (active && !active[i]) return;
     const int stride = j.grad ? 1 + j.n_model : 1;
     const double* r = j.res_seg + i * j.n_cat * stride;
+    // entries of output 0: the categories' NLLs; else the map's
+    const int n = o == 0 ? j.n_cat : j.n_cat * j.n_model;
     double v = 0.0;
-    if (o == 0) {
-        for (int c = 0; c < j.n_cat; ++c) v += r[c * stride];
-    } else {
-        const int q = o - 1;
-        for (int c = 0; c < j.n_cat; ++c)
-            for (int p = 0; p < j.n_model; ++p)
-                if (j.map[c * j.n_model + p] == q) v += r[c * stride + 1 + p];
+#pragma unroll 4
+    for (int e0 = 0; e0 < n; e0 += 32) {
+        const int e = e0 + lane;
+        bool hit = e < n;
+        int64_t at = (int64_t)e * stride;
+        if (o > 0 && hit) {
+            hit = j.map[e] == o - 1;
+            const int c = e / j.n_model;
+            at = (int64_t)c * stride + 1 + (e - c * j.n_model);
+        }
+        const double x = hit ? r[at] : 0.0;
+        for (unsigned m = __ballot_sync(0xffffffffu, hit); m; m &= m - 1u)
+            v += __shfl_sync(0xffffffffu, x, __ffs((int)m) - 1);
     }
-    res_joint[i * n_out + o] = v;
+    if (lane == 0) res_joint[i * n_out + o] = v;
 }
 
 // fit i: the event range of its categories (decides IPA_FIT_EMPTY)
@@ -214,9 +227,9 @@ ipa_status launch_joint_scatter(const JointDev& j, int n_fits, const double* the
 
 ipa_status launch_joint_gather(const JointDev& j, int n_fits, const int* active, double* res_joint,
                                cudaStream_t s) {
-    const int b = 128;
-    const int64_t n = (int64_t)n_fits * (j.grad ? 1 + j.n_joint : 1);
-    joint_gather_kernel<<<(unsigned)((n + b - 1) / b), b, 0, s>>>(j, n_fits, active, res_joint);
+    const int64_t n = 32 * (int64_t)n_fits * (j.grad ? 1 + j.n_joint : 1);
+    joint_gather_kernel<<<(unsigned)((n + kGatherBlock - 1) / kGatherBlock), kGatherBlock, 0, s>>>(j, n_fits, active,
+                                                                                                   res_joint);
     return cuda_fail(cudaGetLastError(), "joint gather");
 }
 
