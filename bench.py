@@ -188,7 +188,8 @@ COUNT_METRICS = ("smsp__inst_executed.sum,smsp__inst_executed_pipe_fp64.sum,"
                  "sm__sass_thread_inst_executed_op_dfma_pred_on.sum,sm__sass_thread_inst_executed_op_dmul_pred_on.sum,"
                  "sm__sass_thread_inst_executed_op_dadd_pred_on.sum,dram__bytes_read.sum,dram__bytes_write.sum,"
                  "gpu__time_duration.sum,smsp__cycles_active.sum,smsp__issue_active.sum")
-COUNT_COMMON = ["tile_reduce.cuh", "fp64_math.cuh", "fp64_tables.cuh", "int_math.cuh", "ipa_internal.cuh"]
+COUNT_COMMON = ["tile_reduce.cuh", "fp64_math.cuh", "fp64_tables.cuh", "int_math.cuh", "fast_fixed.cuh",
+                "ipa_internal.cuh"]
 COUNT_CAPTURES = {
     "nll_kernel<4D, grad>": ("counts_4d.csv", "bench.py --profile-case", 8_000_000,
                              ["nll.cu", "angular.cuh"] + COUNT_COMMON),

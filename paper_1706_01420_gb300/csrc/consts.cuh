@@ -30,6 +30,7 @@
 #include <math.h>
 
 #include "fp64_math.cuh"
+#include "fast_fixed.cuh"
 #include "ipa_internal.cuh"
 
 namespace ipa {
@@ -363,6 +364,54 @@ __device__ inline double mo_sum(const double* h) {
     return ((a[0] + a[1]) + (a[2] + a[3])) + a[4];
 }
 
+// The factors of the angular functions (kBasisScale of angular.cuh).
+__device__ inline double basis_factor(int k) {
+    return k == 1 || k == 2 ? 0.5 : (k == 4 ? 1.41421356237309504880 : (k == 5 ? -1.41421356237309504880
+         : (k == 6 ? 1.0 / 3.0 : (k == 7 ? 0.81649658092772603273 : (k == 8 ? -0.81649658092772603273
+         : (k == 9 ? 1.15470053837925152902 : 1.0))))));
+}
+__device__ inline double coef_hq(const Consts& c, int k) { return (c.h[k] * basis_factor(k)) * (0.5 * c.cs); }
+__device__ inline double coef_hc(const Consts& c, int k) { return c.h[k] * (0.5 * c.cs); }
+
+// Coefficient k of A' in the basis of fx_basis (fast_fixed.cuh) from hq.
+__device__ inline double coef_g(const double* hq, int k) {
+    if (k == 0) return hq[0] + hq[6];
+    if (k == 1) return hq[1] + hq[2];
+    if (k == 2) return neg_bits(hq[0] + hq[2]);
+    if (k == 3) return hq[2] - hq[1];
+    return hq[k < 7 ? k - 1 : k];                        // f'_3, f'_4, f'_5, f'_7, f'_8, f'_9
+}
+// 2^(s + 1) max|g| in [1, 2) from the bits of max|g|: s, or 9999 where the fixed-point
+// path cannot take the coefficients (all zero, non-finite, or s outside [-64, 900]).
+__device__ inline int coef_scale(long long amax) {
+    const int sc = 1022 - (int)(amax >> 52);
+    return amax < 0x7FF0000000000000ll && sc >= -64 && sc <= 900 ? sc : 9999;
+}
+__device__ inline int2 coef_ga(double g, int sc) {
+    const Fx v = fx(sc == 9999 ? 0 : to_q62(g * __longlong_as_double((long long)(sc + 1023) << 52)));
+    return make_int2(v.h, v.l);
+}
+__device__ inline double coef_tcut(const Consts& c) {
+    const double tc = c.mu + (c.Gs2 + 6.25 * (c.sigma * kSqrt2));
+    return tc == tc ? tc : INFINITY;                     // NaN constants: every event takes the full path
+}
+__device__ inline FxExp coef_exp(const ModelDev& m, const Consts& c) {
+    const double a = abs_bits(m.t_lo), b = abs_bits(m.t_hi);
+    return fx_exp_setup(c.Gamma, c.mu, c.c_exp, a > b ? a : b);
+}
+__device__ inline void coef_flags(Consts* c, int sc) {
+    c->k.hexp = 2 - (sc == 9999 ? 0 : sc);
+    c->k.fixed = sc != 9999 && abs_below(c->cs, 1e300) && c->k.ex.ok;
+    // A typical r T = T2 / (A' T2 + cb) is near 1 / max(max|g| / 4, cb / 2): the scale follows
+    // it, so that the sums' relative precision depends neither on the unit of time
+    // nor on f_b, with 2^12 of headroom for events where A' is small.
+    const int ea = sc == 9999 ? -1023 : -sc - 3;
+    const int eb = (int)((__double_as_longlong(c->cb) >> 52) & 0x7FF) - 1024;
+    const int e = ea > eb ? ea : eb;
+    c->k.rtop = 15 + (e < -900 ? 900 : -e);
+    c->k.pad[0] = c->k.pad[1] = c->k.pad[2] = 0;
+}
+
 // The tables of exp_fast, sincos_fast and erfcx_fast into shared memory
 // (block-cooperative; the caller syncs).
 __device__ inline void load_consts_tables(MathTables* t) {
@@ -428,6 +477,22 @@ __device__ inline void compute_consts_thread(const ModelDev& m, const double* th
         for (int i = 0; i < kRowEntries; ++i) hd[i] = i == 0 ? 1.0 : 0.0;
         c->MO = 1.0;
     }
+    long long amax = 0;
+    for (int k = 0; k < 10; ++k) {
+        c->k.hq[k] = coef_hq(*c, k);
+        c->k.hc[k] = coef_hc(*c, k);
+    }
+    for (int k = 0; k < 10; ++k) {
+        const long long a = __double_as_longlong(abs_bits(coef_g(c->k.hq, k)));
+        amax = a > amax ? a : amax;
+    }
+    const int sc = coef_scale(amax);
+    for (int k = 0; k < 10; ++k) c->k.ga[k] = coef_ga(coef_g(c->k.hq, k), sc);
+    c->k.aq = 0.5 * c->cs;
+    c->k.c2 = c->c_exp + fp64tab::kLn2Hi;
+    c->k.tcut = coef_tcut(*c);
+    c->k.ex = coef_exp(m, *c);
+    coef_flags(c, sc);
 }
 
 // Exchange buffer of compute_consts_block.
@@ -439,6 +504,7 @@ struct ConstsBlockScratch {
     double rG;
     double F[2], dF[2][3];
     int ok;                        // theta in the domain
+    int sc;                        // scale of the fixed-point coefficients
     Consts c;                      // the record, copied out at the end
 };
 constexpr int kConstsBlock = 192;
@@ -455,8 +521,9 @@ constexpr int kConstsBlock = 192;
 //            scalars that need theta only;
 //   phase 2  warp 0: g, Phi, G, F and its derivatives at both edges, M_T;
 //            warps 1-3: the 70 entries of h and dh, one per lane;
-//   phase 3  warp 0: I_T and the five divisions by it; warp 1: M_Omega
-//            (shuffle tree);
+//   phase 3  warp 0: I_T and the five divisions by it, then the likelihood's
+//            coefficients (NllCoef); warp 1: M_Omega (shuffle tree); warp 2: the
+//            parameters of the fixed-point exponential and the near-peak cut;
 // then every thread copies part of the record out.  Every value comes from the
 // same expression as in compute_consts_thread, so both give the same bits
 // (this file is compiled without FMA contraction).
@@ -552,6 +619,24 @@ __device__ inline void compute_consts_block(const ModelDev& m, const double* th,
             else S->c.inv_ITIO = v;
             if (lane == 0) S->c.IT = IT;
         }
+        __syncwarp();
+        if (lane < 10) S->c.k.hq[lane] = coef_hq(S->c, lane);
+        else if (lane < 20) S->c.k.hc[lane - 10] = coef_hc(S->c, lane - 10);
+        __syncwarp();
+        const double g = lane < 10 ? coef_g(S->c.k.hq, lane) : 0.0;
+        long long amax = __double_as_longlong(abs_bits(g));
+        for (int o = 16; o > 0; o >>= 1) {
+            const long long v = __shfl_xor_sync(0xffffffffu, amax, o);
+            amax = v > amax ? v : amax;
+        }
+        const int sc = coef_scale(amax);
+        if (lane < 10) S->c.k.ga[lane] = coef_ga(g, sc);
+        if (lane == 10) S->c.k.aq = 0.5 * S->c.cs;
+        if (lane == 0) S->sc = sc;
+    } else if (w == 2) {
+        if (lane == 0) S->c.k.ex = coef_exp(m, S->c);
+        else if (lane == 1) S->c.k.tcut = coef_tcut(S->c);
+        else if (lane == 2) S->c.k.c2 = S->c.c_exp + fp64tab::kLn2Hi;
     } else if (w == 1) {
         // a_i = p_2i + p_2i+1 in lane 2i, then ((a_0 + a_1) + (a_2 + a_3)) + a_4 as in mo_sum
         const double p = four && lane < 10 ? abs_bits(hd[lane]) * basis_max(lane) : 0.0;
@@ -561,6 +646,8 @@ __device__ inline void compute_consts_block(const ModelDev& m, const double* th,
         const double a4 = __shfl_sync(0xffffffffu, a, 8);
         if (lane == 0) S->c.MO = four ? q + a4 : 1.0;
     }
+    __syncthreads();
+    if (threadIdx.x == 0) coef_flags(&S->c, S->sc);
     __syncthreads();
     const double* src = reinterpret_cast<const double*>(&S->c);
     double* dst = reinterpret_cast<double*>(c);

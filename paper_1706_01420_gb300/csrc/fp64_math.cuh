@@ -40,6 +40,7 @@ struct MathTables {
     long long exq[fp64tab::kErfcxPieces * fp64tab::kErfcxCoeffs];   // the same pieces in Q62 (int_math.cuh)
     long long sq[65], cq[65];   // sin, cos (j pi/32) in Q62 (int_math.cuh)
     long long eq[64];           // 2^(j/64) in Q62 (int_math.cuh)
+    long long lq[128];          // -log(c_j) in Q56 (fast_fixed.cuh)
 };
 
 // Block-cooperative copy of the tables into shared memory (caller syncs).
@@ -53,6 +54,7 @@ __device__ __forceinline__ void load_math_tables(MathTables* t) {
     for (int i = threadIdx.x; i < 128; i += blockDim.x) {
         t->linv[i] = kLogInv[i];
         t->ltab[i] = kLogTab[i];
+        t->lq[i] = kLogQ56[i];
     }
     for (int i = threadIdx.x; i < kErfcxPieces * kErfcxCoeffs; i += blockDim.x) {
         t->ex[i] = kErfcxTab[i];

@@ -32,6 +32,7 @@ the fixed-point tables and constants of the integer-pipe functions
           2/pi and pi/32 in Q64; 32/pi in Q59 and pi/32 in Q128 as two
           64-bit words (the wide-range reduction); the Taylor coefficients 1/3!, .., 1/9! of sin
           and 1/2!, .., 1/8! of cos in Q64
+  log:    round(L_j 2^56) and ln2 in Q56 (fast_fixed.cuh)
   exp:    round(2^(j/64) 2^62), j = 0..63; 64/ln2 in Q56; ln2/64 in Q128 as
           two 64-bit words; 1/2!, .., 1/6! in Q63
 
@@ -127,6 +128,7 @@ def main():
     ln2_64_hi, ln2_64_lo = split(ln2 / 64)
     log_c = [d(1 / (1 + (mp.mpf(j) + mp.mpf(1) / 2) / 128)) for j in range(128)]
     log_l = [d(-mp.log(mp.mpf(c))) for c in log_c]
+    log_q56 = [q(-mp.log(mp.mpf(c)), 56) for c in log_c]
     sin_tab = [d(mp.sin(j * mp.pi / 32)) for j in range(64)]
     cos_tab = [d(mp.cos(j * mp.pi / 32)) for j in range(64)]
     inv_pi_32 = d(32 / mp.pi)
@@ -232,6 +234,12 @@ __device__ const long long kCosQ62[65] = {{
 __device__ const long long kExp2Q62[64] = {{
 {fmt_int(exp2_q62)}
 }};
+
+// round(-log(c_j) 2^56) of the rounded c_j, and ln 2 in Q56 (fast_fixed.cuh)
+__device__ const long long kLogQ56[128] = {{
+{fmt_int(log_q56)}
+}};
+constexpr long long kLn2Q56 = {q(ln2, 56)}ll;
 
 // erfcx piece k (centre k/2): coefficients of u^0 .. u^{ERFCX_DEG}, as doubles
 // and in Q62

@@ -45,6 +45,33 @@ __host__ __device__ constexpr int n_acc(int kind, bool grad) {
 constexpr int kMaxAcc = 47;
 constexpr int kSmallAcc = 15;
 
+// Parameters of the fixed-point decay exponential (fast_fixed.cuh).
+struct FxExp {
+    long long c;
+    int gh, gl;
+    int top, ysh, ok, pad_;
+};
+
+// What the 1D and 4D likelihood kernels multiply by, with the factors of the event
+// loop folded in (coef_* in consts.cuh):
+//   A' = sum_k hq_k f'_k = (cs / 2) A, so that P = T2 A' + cb with T2 = 2 T;
+//   hq_k = h_k c_k cs / 2 for the unscaled products f'_k, hc_k = h_k cs / 2 for a
+//   cached basis, aq = cs / 2 (the 1D model's A' for A = 1),
+//   c2 = Gamma^2 sigma^2 / 2 + ln 2, so that exp(-Gamma tau + c2) = 2 E,
+//   ga: the coefficients of A' in the basis of fx_basis, times the power of two
+//   that brings the largest into [1/2, 1), in Q62 split as fast_fixed.cuh does.
+struct NllCoef {
+    double hq[10], hc[10];
+    double aq, c2;
+    double tcut;     // t above it: z < -6.25, the Gaussian-erfcx term is below 1e-17 of T
+    int2 ga[10];
+    int hexp;        // A' = (sum_k ga_k g_k in Q60) 2^(hexp - 2)
+    int fixed;       // coefficients and exponential in range: the fixed-point path may be used
+    int rtop;        // scale of r T at unit weight in fixed point (tile_fast): below 2^(rtop - 3)
+    int pad[3];
+    FxExp ex;
+};
+
 // Parameter-derived constants of one fit (step a1 of the hot path), computed
 // once per call on the device from theta and read by every event tile.
 struct Consts {
@@ -69,6 +96,7 @@ struct Consts {
     double MO;        // angular envelope: sum |h_k| max|f_k|
     double IT;        // I_T
     double pad_;
+    NllCoef k;
 };
 constexpr int kConstsDoubles = sizeof(Consts) / sizeof(double);
 static_assert(sizeof(Consts) % 16 == 0, "Consts must be a multiple of 16 bytes");

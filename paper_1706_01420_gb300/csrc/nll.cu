@@ -20,11 +20,10 @@
 //     erfc(z) = exp(-z^2) erfcx(z) for z >= 0, with exp(-Gamma tau + Gamma^2
 //     sigma^2/2) exp(-z^2) = exp(-tau^2/(2 sigma^2)): the Gaussian factor that
 //     the gradient needs anyway replaces the exponential inside erfc;
-//   * sin/cos, the whole angular basis and the Gaussian's exp run on the
-//     integer pipe in 64-bit fixed point and are rounded once to double
-//     (int_math.cuh); the decay exponential, log and erfcx are table-driven
-//     FP64 (fp64_math.cuh): the split between the FP64 and the integer pipes
-//     is the measured fastest one;
+//   * sin/cos, the whole angular basis, A and the ten angular sums, the decay
+//     exponential, the Gaussian and erfcx run on the integer pipe in 64-bit
+//     fixed point at four to six instructions per product (fast_fixed.cuh); the
+//     rows that allow it (rows_fast) leave about 15 FP64 instructions per event;
 //   * sin(theta_K) sin(theta_mu) is one square root; the constant factors of
 //     the ten angular functions are folded into the amplitude coefficients.
 //
@@ -42,6 +41,7 @@
 #include "fp64_math.cuh"
 #include "int_math.cuh"
 #include "angular.cuh"
+#include "fast_fixed.cuh"
 #include "ipa_internal.cuh"
 #include "tile_reduce.cuh"
 
@@ -51,40 +51,8 @@ namespace {
 constexpr int kNllBlock = 128;                       // threads per block of the basis kernel
 constexpr int kPerLane = kTile / 32;                 // events per lane per tile
 
-// Per-warp copy of a segment's constants in shared memory, with the factors
-// the event loop multiplies by folded in:
-//   A' = sum_k hq_k f_k = (cs / 2) A, so that P = T2 A' + cb with T2 = 2 T,
-//   hq_k = h_k c_k cs / 2 for the unscaled products f'_k (h_k cs / 2 for a
-//   cached basis), aq = cs / 2 (the 1D model's A' for A = 1),
-//   c2 = Gamma^2 sigma^2 / 2 + ln 2, so that exp(-Gamma tau + c2) = 2 E,
-//   hcq_k = h_k c_k (cs / 2) times the power of two 2^s that brings the largest
-//   into [1, 2), in Q62, so that the fixed-point sum gives A' directly.
-struct WarpConsts {
-    Consts c;
-    double hq[10];
-    double aq;
-    double c2;
-    double tcut;     // t above it: z < -6.25, the Gaussian-erfcx term is below 1e-17 of T
-    long long hcq[10];   // h_k c_k (cs / 2) 2^s in Q62 (the fixed-point amplitude sum), with
-    int hexp;            // 2 - s: A' = (sum_k hcq_k F_k in Q60) 2^-s, s making max|hcq| lie in [1, 2)
-    int fixed;           // coefficients finite and s in range: the fixed-point path may be used
-};
-
-// The largest of a non-negative 64-bit value over the warp.
-__device__ __forceinline__ long long max_abs_bits(long long v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const long long w = __shfl_xor_sync(0xffffffffu, v, o);
-        v = w > v ? w : v;
-    }
-    return v;
-}
-
-// 2^e as a double for -1022 <= e <= 1023 (built from its bit pattern).
-__device__ __forceinline__ double exp2_int(int e) {
-    return __longlong_as_double((long long)(e + 1023) << 52);
-}
-
+// A warp keeps a copy of its segment's record (Consts, with the factors the event
+// loop multiplies by in its part k: NllCoef) in shared memory.
 // Decay-time events per compaction round of one lane (see nll_kernel).
 constexpr int kSub = 4;
 static_assert(kSub == 4, "a compaction round keeps four ballot masks");
@@ -101,11 +69,11 @@ __device__ __forceinline__ double2 gauss_erfcx(const Consts& c, double tau, cons
     // than 37 sigma before mu), where the Gaussian, below 1e-306, is nothing
     // against the exponential term of 2 g(tau)
     const double gr = -(tau * tau) * c.k_g;
-    const double g = exp_int_nb(below_neg(gr, -705.0) ? -705.0 : gr, mt);
+    const double g = fx_exp_neg(below_neg(gr, -705.0) ? -705.0 : gr, mt);
     const double z = (c.Gs2 - tau) * c.k_z;
     const double x = fabs(z);
     const bool zneg = negative(z);
-    double X = erfcx_poly(x, mt);
+    double X = fx_erfcx(x, mt);
     if (above(x, 6.25)) {
         // z < 0: the erfcx term is below 1e-17 of E; z >= 0 (tau far below the
         // resolution peak, outside the usual range): exact library erfcx
@@ -125,18 +93,17 @@ __device__ __forceinline__ double amplitude_sum(const double* hq, const double* 
 // One event: the log term (w log P added to acc[0], or for w = 1 exactly, P
 // folded into the lane's product) and the adjoint sums.  For the 4D model f
 // holds either the unscaled products f'_k (CACHED = false) or the cached basis
-// f_k (CACHED = true); Ap = (cs/2) A (wc.aq for the 1D model); ge is the
+// f_k (CACHED = true); Ap = (cs/2) A (c.k.aq for the 1D model); ge is the
 // event's gauss_erfcx value or (0, +0).
 // Accumulators (kD = 12 for 4D, 3 for 1D), with r = w / P and A' = (cs/2) A:
 //   acc[1] = sum r,  acc[2 + k] = sum r T2 f_k (4D) or acc[2] = sum r T2 (1D),
 //   acc[kD] = sum r A' tau T2,  acc[kD + 1] = sum r A' Gx,  acc[kD + 2] = sum r A' tau Gx;
 // the derivatives in Gamma, sigma and mu are linear in these (finalize).
 template <int KIND, bool GRAD, bool CACHED, bool WEIGHTED>
-__device__ __forceinline__ void event(const WarpConsts& wc, const MathTables* mt, double t, const double* f,
+__device__ __forceinline__ void event(const Consts& c, const MathTables* mt, double t, const double* f,
                                       double Ap, double w, double2 ge, double* acc, double* prod, int* esum) {
-    const Consts& c = wc.c;
     const double tau = t - c.mu;
-    const double E2 = exp_int(fma(-c.Gamma, tau, wc.c2), mt);
+    const double E2 = exp_int(fma(-c.Gamma, tau, c.k.c2), mt);
     const long long gb = __double_as_longlong(ge.y);
     const double T2 = gb >= 0 ? E2 - ge.x : ge.x;
     const double Gx = __longlong_as_double(gb & 0x7FFFFFFFFFFFFFFFll);
@@ -168,78 +135,84 @@ __device__ __forceinline__ void event(const WarpConsts& wc, const MathTables* mt
     }
 }
 
-// ---- the fast tile (4D model, angles on the integer pipe) ----
-// A whole tile of the 4D model's NLL + gradient takes this path; the last,
-// partial tile of a segment and the other variants take the plain loop of
-// nll_kernel.
+// ---- the fast rows (4D model, fixed point on the integer pipe) ----
+// The rows of 32 events that are complete (lane l: events tbase + l + 32 i of a
+// tile) of the 4D model's NLL + gradient take this path; the last, partial row of
+// a segment and the other variants take the plain loop of tile_plain.
 //
 // On this GPU a warp FP64 instruction occupies the sub-partition's FP64 unit
-// for about 64 cycles (2 FP64 operations per clock per SM).  A few FP64
-// instructions spread among a warp's integer work overlap with it, but a burst
-// of them does not (measured: removing the ten back-to-back DFMA of the
-// angular adjoint sums saved far more time than removing isolated DMUL or DADD
-// instructions, which cost about nothing).  So the ten sums S_k = sum r T f'_k
-// are accumulated here on the integer pipe: r T is converted once per event to
-// signed 64-bit fixed point with 40 fraction bits (rounded to nearest, for
-// |r T| < 2^19), and each product with the Q62 angular product f'_k is the
-// high 64 bits of the 128-bit product (Q38: the floor, corrected on average
-// by half a unit per product at the end of the tile).  A lane adds its 16
-// events exactly in 64-bit integers (no overflow: |r T f'_k| < 2^19) and
-// converts each sum to a double once per tile, so these sums do not depend on
-// the order of the events within a lane.  Error of a sum: about 2^-39 per
-// event, of random sign (a sum over 1e6 events is off by ~1e-9 absolute,
-// while the sums themselves are ~1e5 and the gradient tolerance is 1e-9 of
-// them).  The remaining accumulators are FP64 as in the plain loop.  The
-// integer work runs with the branch-free functions of int_math.cuh; lanes
-// outside their ranges are fixed up with the FP64 paths of the plain loop.  A
-// tile in which some P lies outside the Newton reciprocal's range (zero,
-// subnormal, negative, huge, infinite or NaN) or some |r T| >= 2^19 is redone
-// by the plain loop.  Either way the tile's sums depend only on its events,
-// never on the launch geometry.
+// for about 64 cycles (2 FP64 operations per clock per SM), so everything with
+// a known range runs in 64-bit fixed point (fast_fixed.cuh): the decay
+// exponential, the angular basis, A' and the ten angular sums.  What stays FP64:
+// P, 1/P, the log (or the product of the P's) and the four sums with r, tau and
+// the Gaussian.
+//
+// The sums: r T is converted once per event to signed fixed point, in units of
+// 2^(top - 63), each product with a basis function (Q62) is the high part of the
+// 128-bit product (units of 2^(top - 61)), and a lane adds its events exactly in
+// 64-bit integers and converts each sum to a double once per tile (sums of f'_k
+// are differences of sums of basis functions, taken in integers).  top follows
+// the segment's typical r T (NllCoef::rtop) and the largest weight of the tile,
+// so a unit is 2^-46 of a typical term; error of a sum: 0.41 units rms per
+// event, of random sign, below that of the reciprocal r (6e-14 relative), and the
+// mean of the truncation is put back.  Lanes outside the ranges are fixed up in
+// FP64.  A tile in which some P lies outside the Newton reciprocal's range (zero,
+// subnormal, negative, huge, infinite or NaN) or some |r T| >= 2^(top - 3) is redone
+// by the plain loop.  Either way the tile's sums depend only on its events, never
+// on the launch geometry.
+//
+// Measured (one pass of the public call, 512 toys of 2000 events, then 1e7
+// weighted events): the angular products, A and the exponential in FP64 and
+// 14-instruction 64-bit products, an FP64 multiply-add per angular sum: 1060 and
+// 1073 us; this path: 643 and 685.  About 1150 warp instructions per row now
+// occupy the FP64 unit 60 %, the two 32-bit multiplier and adder pipes 50 % each
+// and the issue slots 50 %; 128 registers leave 16 warps per SM, and launch
+// bounds for 20 or 24 cost more in spills than they hide (728 and 760 us).
 
 // The integer-pipe results of one event that its FP64 work needs.
 struct RowIn {
     double tau, w, E2, Ap;
-    long long F[10];   // f'_k in Q62
+    long long g[10];   // fx_basis
 };
 
-// tau, E2 = 2 e^{-Gamma tau + Gamma^2 sigma^2 / 2}, the ten f'_k and A' =
-// (cs / 2) A of event e: the angular basis and A' with the branch-free
-// fixed-point functions, E2 with the table-driven FP64 exp (measured 7 % faster
-// here than the integer-pipe exp, whose long dependent chain sat in front of
-// the event's FP64 work; the FP64 pipe has room since the adjoint sums moved to
-// fixed point); false if the lane needs fix_int_phase.
-template <bool WEIGHTED>
-__device__ __forceinline__ bool int_phase(const WarpConsts& wc, const MathTables* mt, const Cols& cols, int64_t e,
-                                          RowIn& v) {
-    const double t = __ldg(cols.t + e);
-    const double ck = __ldg(cols.ck + e), cl = __ldg(cols.cl + e), phi = __ldg(cols.phi + e);
-    v.w = WEIGHTED ? __ldg(cols.w + e) : 1.0;
-    v.tau = t - wc.c.mu;
-    v.E2 = exp_fast(fma(-wc.c.Gamma, v.tau, wc.c2), mt);
-    basis_q62_nb(ck, cl, phi, mt, v.F);
-    long long Af = 0;
-#pragma unroll
-    for (int k = 0; k < 10; ++k) Af += __mul64hi(wc.hcq[k], v.F[k]);
-    v.Ap = q62_to_double_nb(Af, wc.hexp);
-    return wc.fixed && basis_q62_ok(ck, cl, phi);
-}
-
-// The FP64 basis of the plain loop for a lane that int_phase could not serve
-// (the FP64 products, in [-1, 1] for valid angles, go to Q62).
-__device__ __forceinline__ void fix_int_phase(const WarpConsts& wc, const MathTables* mt, const Cols& cols,
-                                              int64_t e, RowIn& v) {
-    const double ck = __ldg(cols.ck + e), cl = __ldg(cols.cl + e), phi = __ldg(cols.phi + e);
-    if (!(wc.fixed && basis_q62_ok(ck, cl, phi))) {
+// The FP64 values for a lane outside the fixed-point ranges (rare): the basis, A'
+// (with the f'_k in the plain loop's order) and the exponential.
+__device__ __noinline__ void fix_row(const Consts& c, const MathTables* mt, double t, double ck, double cl, double phi,
+                                     bool ok_exp, RowIn& v) {
+    if (!ok_exp) v.E2 = exp_fast(fma(-c.Gamma, v.tau, c.k.c2), mt);
+    if (!fx_angles_ok(ck, cl, phi)) {
         double f[10];
         basis_unscaled(ck, cl, phi, mt, f);
-        v.Ap = amplitude_sum(wc.hq, f);
+        v.Ap = amplitude_sum(c.k.hq, f);
+        const double sk2 = fma(-ck, ck, 1.0), G = sk2 * f[6], gcc = sk2 - f[1];
+        const double g[10] = {f[6], sk2, G, gcc, f[3], f[4], f[5], f[7], f[8], f[9]};
 #pragma unroll
-        for (int k = 0; k < 10; ++k) v.F[k] = to_q62_nb(f[k]);
+        for (int k = 0; k < 10; ++k) v.g[k] = to_q62_nb(g[k]);
     }
 }
 
-// rcp_newton and log_fast without their range branches (P in [2^-125, 2^126)).
+template <bool WEIGHTED>
+__device__ __forceinline__ void load_row(const Consts& c, const MathTables* mt, const Cols& cols, int64_t e, RowIn& v) {
+    const double t = __ldg(cols.t + e);
+    const double ck = __ldg(cols.ck + e), cl = __ldg(cols.cl + e), phi = __ldg(cols.phi + e);
+    v.w = WEIGHTED ? __ldg(cols.w + e) : 1.0;
+    v.tau = t - c.mu;
+    bool ok_exp = true;
+    v.E2 = fx_exp(t, c.k.ex, mt, &ok_exp);
+    fx_basis(ck, cl, phi, mt, v.g);
+    long long A = 0;
+#pragma unroll
+    for (int k = 0; k < 10; ++k) A = fx_mad(Fx{c.k.ga[k].x, c.k.ga[k].y}, fx(v.g[k]), A);
+    v.Ap = fx_to_double(A, c.k.hexp);
+    const bool ok = ok_exp && fx_angles_ok(ck, cl, phi);
+    if (__any_sync(0xffffffffu, !ok)) {
+        RowIn x = v;                         // (a copy, so that v itself stays in registers)
+        fix_row(c, mt, t, ck, cl, phi, ok_exp, x);
+        v = x;
+    }
+}
+
+// rcp_newton without its range branch (P in [2^-125, 2^126)).
 __device__ __forceinline__ double rcp_newton_nb(double x) {
     const long long b = __double_as_longlong(x);
     const int e = (int)((b >> 52) & 0x7FF);
@@ -252,24 +225,6 @@ __device__ __forceinline__ double rcp_newton_nb(double x) {
     return fma(y, fma(-x, y, 1.0), y);
 }
 
-__device__ __forceinline__ double log_fast_nb(double x, const MathTables* t) {
-    using namespace fp64tab;
-    const long long b = __double_as_longlong(x);
-    const int e = (int)(b >> 52) - 1023;
-    const int j = (int)((b >> 45) & 127);
-    const double m = __longlong_as_double((b & 0x000FFFFFFFFFFFFFll) | 0x3FF0000000000000ll);
-    const double r = fma(m, t->linv[j], -1.0);
-    double q = fma(r, 1.0 / 7.0, -1.0 / 6.0);
-    q = fma(q, r, 0.2);
-    q = fma(q, r, -0.25);
-    q = fma(q, r, 1.0 / 3.0);
-    q = fma(q, r, -0.5);
-    const double l = fma(r * r, q, r);
-    const double ed = __longlong_as_double(0x4330000000000000ll + (long long)(e + 2048)) -
-                      (4503599627370496.0 + 2048.0);
-    return fma(ed, kLn2Hi, fma(ed, kLn2Lo, t->ltab[j] + l));
-}
-
 // log_mul for positive normal P (no branch for zero, subnormal or special P).
 __device__ __forceinline__ void log_mul_nb(double P, double* prod, int* esum) {
     const long long b = __double_as_longlong(P);
@@ -277,72 +232,65 @@ __device__ __forceinline__ void log_mul_nb(double P, double* prod, int* esum) {
     *esum += (int)(b >> 52) - 1023;
 }
 
-// x 2^40 rounded to the nearest signed 64-bit integer (ties away from zero),
-// for |x| < 2^19 (else *bad is set; NaN and infinities included).
-__device__ __forceinline__ long long to_q40(double x, bool* bad) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-    const int E = (int)((b >> 52) & 0x7FFull) - 1023;
-    *bad |= E > 18;
-    const unsigned long long M = (b & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull;
-    const int sh = E - 12;
-    const int s = (-sh) & 63;
-    const unsigned long long dn = (M + (s ? 1ull << (s - 1) : 0ull)) >> s;
-    const long long v = (long long)(sh >= 0 ? M << (sh & 63) : (sh > -64 ? dn : 0ull));
-    return (b >> 63) ? -v : v;
-}
+// A lane's sums over rows on the fast path: FP64 (f: sum r, sum r A' tau T2, sum r A'
+// Gx, sum r A' tau Gx, and with weights sum w log P), the log product, and the fixed-
+// point sums of r T g_k.
+struct FastSums {
+    double f[5];
+    double prod;
+    int esum;
+    int n;             // events with r T != 0 (for the mean of the truncation)
+    bool bad;          // P outside [2^-125, 2^126) or |r T| >= 2^(top - 3)
+    int top;           // scale of r T (set once per tile)
+    long long g[10];
+};
 
-// The FP64 work of one event on the fast path: event() with the exponential
-// and the angular products from int_phase and the ten angular adjoint sums in
-// fixed point (acci, Q38).  ge: the event's gauss_erfcx value or (0, +0).
-// *bad is set when P is outside [2^-125, 2^126) or |r T| >= 2^19.
-template <bool GRAD, bool WEIGHTED>
-__device__ __forceinline__ void event_fast(const WarpConsts& wc, const MathTables* mt, const RowIn& v, double2 ge,
-                                           double* acc, long long* acci, double* prod, int* esum, bool* bad) {
-    const Consts& c = wc.c;
+template <bool WEIGHTED>
+__device__ __forceinline__ void event_fast(const Consts& c, const MathTables* mt, const RowIn& v, double2 ge, FastSums& s) {
     const long long gb = __double_as_longlong(ge.y);
     const double T2 = gb >= 0 ? v.E2 - ge.x : ge.x;
     const double Gx = __longlong_as_double(gb & 0x7FFFFFFFFFFFFFFFll);
     const double P = fma(T2, v.Ap, c.cb);
     const long long pb = __double_as_longlong(P);
-    *bad |= (unsigned long long)(pb - 0x3820000000000000ll) >= 0x0FB0000000000000ull;
+    s.bad |= (unsigned long long)(pb - 0x3820000000000000ll) >= 0x0FB0000000000000ull;
     if (WEIGHTED) {
         // weight exactly 1: P joins the lane's product (as in event)
         const bool one = __double_as_longlong(v.w) == 0x3FF0000000000000ll;
-        acc[0] = fma(one ? 0.0 : v.w, log_fast_nb(P, mt), acc[0]);
-        log_mul_nb(one ? P : 1.0, prod, esum);
+        s.f[4] = fma(one ? 0.0 : v.w, fx_to_double(fx_log(P, mt), 6), s.f[4]);
+        log_mul_nb(one ? P : 1.0, &s.prod, &s.esum);
     } else {
-        log_mul_nb(P, prod, esum);
+        log_mul_nb(P, &s.prod, &s.esum);
     }
-    if (GRAD) {
-        const double r = WEIGHTED ? v.w * rcp_newton_nb(P) : rcp_newton_nb(P);
-        acc[1] += r;
-        const long long rq = to_q40(r * T2, bad);
+    const double r = WEIGHTED ? v.w * rcp_newton_nb(P) : rcp_newton_nb(P);
+    s.f[0] += r;
+    const double rT = r * T2;
+    const int top = WEIGHTED ? s.top : c.k.rtop;
+    s.bad |= (int)((__double_as_longlong(rT) >> 52) & 0x7FF) > 1023 - 4 + top;
+    const long long rq = fx_odd(rT, top);
+    s.n += rq != 0;
+    const Fx R = fx(rq);
 #pragma unroll
-        for (int k = 0; k < 10; ++k) acci[k] += __mul64hi(rq, v.F[k]);
-        const double rA = r * v.Ap;
-        const double u = rA * v.tau;
-        acc[12] = fma(u, T2, acc[12]);
-        acc[13] = fma(rA, Gx, acc[13]);
-        acc[14] = fma(u, Gx, acc[14]);
-    }
+    for (int k = 0; k < 10; ++k) s.g[k] = fx_mad0(R, fx(v.g[k]), s.g[k]);
+    const double rA = r * v.Ap;
+    const double u = rA * v.tau;
+    s.f[1] = fma(u, T2, s.f[1]);
+    s.f[2] = fma(rA, Gx, s.f[2]);
+    s.f[3] = fma(u, Gx, s.f[3]);
 }
 
-// Rows i0 .. i0 + kSub - 1 of a whole tile (lane l: events tbase + l + 32 i) of
-// the 4D model on the fast path: the near-peak events of the kSub rows marked
-// by ballot and their Gaussian/erfcx values evaluated packed into sbuf, then
-// the events row by row into acc (FP64 sums), acci (the fixed-point S_k), the
-// log product and *bad.
+// Rows i0 .. i1 - 1 (at most kSub, complete) of a tile of the 4D model: the near-peak
+// events marked by ballot and their Gaussian/erfcx values evaluated packed into
+// sbuf, then the events row by row into s.
 template <bool WEIGHTED>
-__device__ __forceinline__ void block_fast(const WarpConsts& wc, const MathTables* mt, const Cols& cols,
-                                           int64_t tbase, int i0, double2* sbuf, int lane, double* acc,
-                                           long long* acci, double* prod, int* esum, bool* bad) {
+__device__ __forceinline__ void rows_fast(const Consts& c, const MathTables* mt, const Cols& cols, int64_t tbase, int i0,
+                                          int i1, double2* sbuf, int lane, FastSums& s) {
     const unsigned below = (1u << lane) - 1u;
     unsigned m[kSub];
     int p[kSub];
 #pragma unroll
     for (int q = 0; q < kSub; ++q) {
         const int64_t e = tbase + lane + 32 * (i0 + q);
-        m[q] = __ballot_sync(0xffffffffu, !greater(__ldg(cols.t + e), wc.tcut));
+        m[q] = __ballot_sync(0xffffffffu, i0 + q < i1 && !greater(__ldg(cols.t + (i0 + q < i1 ? e : tbase)), c.k.tcut));
     }
     p[0] = 0;
     p[1] = __popc(m[0]);
@@ -354,44 +302,87 @@ __device__ __forceinline__ void block_fast(const WarpConsts& wc, const MathTable
         const unsigned mq = q == 0 ? m[0] : (q == 1 ? m[1] : (q == 2 ? m[2] : m[3]));
         const int before = q == 0 ? 0 : (q == 1 ? p[1] : (q == 2 ? p[2] : p[3]));
         const int64_t e = tbase + nth_set(mq, j - before) + 32 * (i0 + q);
-        sbuf[j] = gauss_erfcx(wc.c, __ldg(cols.t + e) - wc.c.mu, mt);
+        sbuf[j] = gauss_erfcx(c, __ldg(cols.t + e) - c.mu, mt);
     }
     __syncwarp();
 #pragma unroll 1
-    for (int q = 0; q < kSub; ++q) {
+    for (int q = 0; q < i1 - i0; ++q) {
         const unsigned mq = q == 0 ? m[0] : (q == 1 ? m[1] : (q == 2 ? m[2] : m[3]));
         const int before = q == 0 ? 0 : (q == 1 ? p[1] : (q == 2 ? p[2] : p[3]));
         const double2 gv = sbuf[(before + __popc(mq & below)) & (kSub * 32 - 1)];
         const double2 ge = (mq >> lane) & 1u ? gv : make_double2(0.0, 0.0);
-        const int64_t e = tbase + lane + 32 * (i0 + q);
         RowIn v;
-        const bool ok = int_phase<WEIGHTED>(wc, mt, cols, e, v);
-        if (__any_sync(0xffffffffu, !ok)) fix_int_phase(wc, mt, cols, e, v);
-        event_fast<true, WEIGHTED>(wc, mt, v, ge, acc, acci, prod, esum, bad);
+        load_row<WEIGHTED>(c, mt, cols, tbase + lane + 32 * (i0 + q), v);
+        event_fast<WEIGHTED>(c, mt, v, ge, s);
     }
     __syncwarp();
 }
 
-// One whole tile (kTile events from tbase) of the 4D model's NLL + gradient on
-// the fast path, kSub rows at a time.  Returns false if the tile must be redone
-// by the plain loop (acc, prod and esum are then meaningless).
+__device__ __forceinline__ void clear(FastSums& s) {
+#pragma unroll
+    for (int a = 0; a < 5; ++a) s.f[a] = 0.0;
+    s.prod = 1.0;
+    s.esum = 0;
+    s.n = 0;
+    s.bad = false;
+#pragma unroll
+    for (int k = 0; k < 10; ++k) s.g[k] = 0;
+}
+
+// The lane's sums over a tile's complete rows as the accumulators of the plain
+// loop: each truncated product was a unit low on average.
+__device__ __forceinline__ void fast_accumulators(const FastSums& s, double* acc) {
+    const long long up = s.n;
+    const long long g1 = s.g[1] - s.g[3], g2 = s.g[1] - s.g[2] + s.g[3];
+    const long long S[10] = {s.g[0] - s.g[2], g1, g2 + up, s.g[4] + up, s.g[5] + up,
+                             s.g[6] + up, s.g[0] + up, s.g[7] + up, s.g[8] + up, s.g[9] + up};
+    acc[0] = s.f[4];
+    acc[1] = s.f[0];
+#pragma unroll
+    for (int k = 0; k < 10; ++k) acc[2 + k] = fx_to_double(S[k], s.top + 1);
+    acc[12] = s.f[1];
+    acc[13] = s.f[2];
+    acc[14] = s.f[3];
+}
+
+// The complete rows of one tile of the 4D model's NLL + gradient on the fast
+// path, kSub at a time.  Returns false if the tile must be redone by the plain
+// loop (acc, prod and esum are then meaningless).
 template <bool WEIGHTED>
-__device__ __forceinline__ bool tile_fast(const WarpConsts& wc, const MathTables* mt, const Cols& cols,
-                                          int64_t tbase, double2* sbuf, int lane, double* acc, double* prod,
-                                          int* esum) {
-    bool bad = false;
-    long long acci[10];
-#pragma unroll
-    for (int k = 0; k < 10; ++k) acci[k] = 0;
+__device__ __forceinline__ bool tile_fast(const Consts& c, const MathTables* mt, const Cols& cols, int64_t tbase,
+                                          int rows, double2* sbuf, int lane, double* acc, double* prod, int* esum) {
+    FastSums s;
+    clear(s);
+    s.top = c.k.rtop;
+    if (WEIGHTED) {
+        // the exponent of the tile's largest |w| (0 where all weights are 1, as without weights)
+        unsigned hi = 0;
+#pragma unroll 4
+        for (int i = 0; i < rows; ++i) {
+            const unsigned h = (unsigned)((unsigned long long)__double_as_longlong(__ldg(cols.w + tbase + lane + 32 * i)) >> 32);
+            hi = (h & 0x7FFFFFFFu) > hi ? (h & 0x7FFFFFFFu) : hi;
+        }
+        const int top = s.top + (int)(__reduce_max_sync(0xffffffffu, hi) >> 20) - 1023;
+        s.top = top < -900 ? -900 : (top > 900 ? 900 : top);
+    }
+    double tot[5] = {0.0, 0.0, 0.0, 0.0, 0.0}, tprod = 1.0;
 #pragma unroll 1
-    for (int i0 = 0; i0 < kPerLane; i0 += kSub)
-        block_fast<WEIGHTED>(wc, mt, cols, tbase, i0, sbuf, lane, acc, acci, prod, esum, &bad);
-    // the lane's fixed-point sums (Q38) as doubles; each high product is the
-    // floor of the exact one, half a unit low on average, so the lane's
-    // kPerLane products get kPerLane / 2 units back
+    for (int i0 = 0; i0 < rows; i0 += kSub) {
+        rows_fast<WEIGHTED>(c, mt, cols, tbase, i0, i0 + kSub < rows ? i0 + kSub : rows, sbuf, lane, s);
 #pragma unroll
-    for (int k = 0; k < 10; ++k) acc[2 + k] = q62_to_double_nb(acci[k] + kPerLane / 2, 24);
-    return !__any_sync(0xffffffffu, bad);
+        for (int a = 0; a < (WEIGHTED ? 5 : 4); ++a) {
+            tot[a] += s.f[a];
+            s.f[a] = 0.0;
+        }
+        tprod *= s.prod;
+        s.prod = 1.0;
+    }
+#pragma unroll
+    for (int a = 0; a < 5; ++a) s.f[a] = tot[a];
+    fast_accumulators(s, acc);
+    *prod = tprod;
+    *esum = s.esum;
+    return !__any_sync(0xffffffffu, s.bad);
 }
 
 // Write NLL (and gradient) of one segment from its reduced accumulators.
@@ -443,24 +434,24 @@ __device__ void finalize(const Consts& c, const double* acc, int n_par, double* 
         out[1 + j] = 0.0;
 }
 
-// The plain loop over one tile's events [tbase, min(tbase + kTile, ev1)): lane
-// l adds events l, l + 32, ... in order into acc (and the log product).  Those
+// The plain loop over one tile's rows from `first` on, events below min(tbase +
+// kTile, ev1): lane l adds events l, l + 32, ... in order into acc (and the log product).  Those
 // near the resolution peak are marked by ballot kSub rows at a time and their
 // Gaussian/erfcx values evaluated packed, 32 per pass, into the warp's buffer.
 template <int KIND, bool GRAD, bool CACHED, bool WEIGHTED>
-__device__ __forceinline__ void tile_plain(const WarpConsts& wc, const MathTables* mt, const Cols& cols,
+__device__ __forceinline__ void tile_plain(const Consts& c, const MathTables* mt, const Cols& cols, int first,
                                            int64_t tbase, int64_t ev1, double2* sbuf, int lane, double* acc,
                                            double* prod, int* esum) {
     const unsigned below = (1u << lane) - 1u;
 #pragma unroll 1
-    for (int i0 = 0; i0 < kPerLane; i0 += kSub) {
+    for (int i0 = first; i0 < kPerLane && tbase + 32 * i0 < ev1; i0 += kSub) {
         unsigned m0, m1, m2, m3;
         {
             unsigned mk[kSub];
 #pragma unroll
             for (int q = 0; q < kSub; ++q) {
                 const int64_t e = tbase + lane + 32 * (i0 + q);
-                const bool slow = e < ev1 && !greater(__ldg(cols.t + e), wc.tcut);
+                const bool slow = e < ev1 && !greater(__ldg(cols.t + e), c.k.tcut);
                 mk[q] = __ballot_sync(0xffffffffu, slow);
             }
             m0 = mk[0];
@@ -475,7 +466,7 @@ __device__ __forceinline__ void tile_plain(const WarpConsts& wc, const MathTable
             const unsigned m = q == 0 ? m0 : (q == 1 ? m1 : (q == 2 ? m2 : m3));
             const int before = q == 0 ? 0 : (q == 1 ? p1 : (q == 2 ? p2 : p3));
             const int64_t e = tbase + nth_set(m, j - before) + 32 * (i0 + q);
-            sbuf[j] = gauss_erfcx(wc.c, __ldg(cols.t + e) - wc.c.mu, mt);
+            sbuf[j] = gauss_erfcx(c, __ldg(cols.t + e) - c.mu, mt);
         }
         __syncwarp();
 #pragma unroll 1
@@ -488,32 +479,33 @@ __device__ __forceinline__ void tile_plain(const WarpConsts& wc, const MathTable
                                                     : make_double2(0.0, 0.0);
                 const double w = WEIGHTED ? __ldg(cols.w + e) : 1.0;
                 double f[10];
-                double Ap = wc.aq;
+                double Ap = c.k.aq;
                 if (KIND == IPA_MODEL_ANGTIME4D) {
                     if (CACHED) {
 #pragma unroll
                         for (int k = 0; k < 10; ++k) f[k] = __ldg(cols.fk + k * cols.fk_stride + e);
-                        Ap = amplitude_sum(wc.hq, f);
+                        Ap = amplitude_sum(c.k.hc, f);
                     } else {
                         const double ck = __ldg(cols.ck + e), cl = __ldg(cols.cl + e), phi = __ldg(cols.phi + e);
-                        if (wc.fixed && basis_q62_ok(ck, cl, phi)) {
+                        if (c.k.fixed && fx_angles_ok(ck, cl, phi)) {
                             // the angular products and A on the integer pipe
-                            long long F[10];
-                            basis_q62(ck, cl, phi, mt, F);
-                            long long Af = 0;
+                            long long g[10];
+                            fx_basis(ck, cl, phi, mt, g);
+                            long long A = 0;
 #pragma unroll
-                            for (int k = 0; k < 10; ++k) {
-                                f[k] = q62_to_double(F[k], 0);
-                                Af += __mul64hi(wc.hcq[k], F[k]);
-                            }
-                            Ap = q62_to_double(Af, wc.hexp);        // Af is Q60, times 2^-s
+                            for (int k = 0; k < 10; ++k) A = fx_mad(Fx{c.k.ga[k].x, c.k.ga[k].y}, fx(g[k]), A);
+                            Ap = fx_to_double(A, c.k.hexp);
+                            const long long F[10] = {g[0] - g[2], g[1] - g[3], g[1] - g[2] + g[3], g[4], g[5],
+                                                     g[6], g[0], g[7], g[8], g[9]};
+#pragma unroll
+                            for (int k = 0; k < 10; ++k) f[k] = fx_to_double(F[k], 0);
                         } else {
                             basis_unscaled(ck, cl, phi, mt, f);
-                            Ap = amplitude_sum(wc.hq, f);
+                            Ap = amplitude_sum(c.k.hq, f);
                         }
                     }
                 }
-                event<KIND, GRAD, CACHED, WEIGHTED>(wc, mt, __ldg(cols.t + e), f, Ap, w, ge, acc, prod,
+                event<KIND, GRAD, CACHED, WEIGHTED>(c, mt, __ldg(cols.t + e), f, Ap, w, ge, acc, prod,
                                                     esum);
             }
         }
@@ -521,38 +513,13 @@ __device__ __forceinline__ void tile_plain(const WarpConsts& wc, const MathTable
     }
 }
 
-// A segment's constants into the warp's copy in shared memory, with the
-// factors the event loop uses (warp-collective).
-template <bool CACHED>
-__device__ __forceinline__ void load_warp_consts(WarpConsts& wc, const Consts* src_consts, int lane) {
+// A segment's record into the warp's copy in shared memory (warp-collective).
+__device__ __forceinline__ void load_warp_consts(Consts& c, const Consts* src_consts, int lane) {
     __syncwarp();
     const double* src = reinterpret_cast<const double*>(src_consts);
-    double* dst = reinterpret_cast<double*>(&wc.c);
+    double* dst = reinterpret_cast<double*>(&c);
+#pragma unroll
     for (int i = lane; i < kConstsDoubles; i += 32) dst[i] = __ldg(src + i);
-    __syncwarp();
-    const double half_cs = 0.5 * wc.c.cs;
-    if (lane < 10) wc.hq[lane] = (CACHED ? wc.c.h[lane] : wc.c.h[lane] * kBasisScale[lane]) * half_cs;
-    if (lane == 10) wc.aq = half_cs;
-    if (lane == 11) wc.c2 = wc.c.c_exp + fp64tab::kLn2Hi;
-    if (lane == 12) {
-        const double tc = wc.c.mu + (wc.c.Gs2 + 6.25 / wc.c.k_z);
-        wc.tcut = tc == tc ? tc : INFINITY;    // NaN constants: every event takes the full path
-    }
-    // h_k c_k (cs / 2) scaled by 2^s into Q62 for the fixed-point
-    // amplitude sum (multiplying by a power of two is exact);
-    // non-finite coefficients (non-physical theta) or a scale outside
-    // [-64, 900] keep the FP64 path, which propagates NaN
-    const double hca = lane < 10 ? (wc.c.h[lane] * kBasisScale[lane]) * half_cs : 0.0;
-    const long long amag = __double_as_longlong(hca) & 0x7FFFFFFFFFFFFFFFll;
-    const long long amax = max_abs_bits(amag);
-    const int eb = (int)(amax >> 52);                 // biased exponent of max |hca|
-    const int sc = amax == 0 ? 0 : 1023 - eb;         // max |hca| 2^sc in [1, 2)
-    const bool sc_ok = amax < 0x7FF0000000000000ll && sc >= -64 && sc <= 900;
-    if (lane < 10) wc.hcq[lane] = sc_ok ? to_q62(hca * exp2_int(sc)) : 0;
-    if (lane == 0) {
-        wc.hexp = 2 - sc;
-        wc.fixed = sc_ok && abs_below(wc.c.cs, 1e300) ? 1 : 0;
-    }
     __syncwarp();
 }
 
@@ -574,7 +541,7 @@ nll_kernel(Cols cols, int64_t n, const int64_t* __restrict__ seg_begin,
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int n_wib = blockDim.x >> 5;
     double2* const sbuf = reinterpret_cast<double2*>(dyn_smem) + wib * (kSub * 32);
-    WarpConsts& wc = reinterpret_cast<WarpConsts*>(dyn_smem + (size_t)n_wib * kSub * 32 * sizeof(double2))[wib];
+    Consts& wc = reinterpret_cast<Consts*>(dyn_smem + (size_t)n_wib * kSub * 32 * sizeof(double2))[wib];
 
     load_math_tables(&mt);
     __syncthreads();
@@ -618,7 +585,7 @@ nll_kernel(Cols cols, int64_t n, const int64_t* __restrict__ seg_begin,
                 if (ev1 < ev0) ev1 = ev0;
             }
             if (seg != cur) {
-                load_warp_consts<CACHED>(wc, consts + seg, lane);
+                load_warp_consts(wc, consts + seg, lane);
                 cur = seg;
             }
 
@@ -634,24 +601,27 @@ nll_kernel(Cols cols, int64_t n, const int64_t* __restrict__ seg_begin,
             // into the warp's buffer, so the FP64 pipe does not spend a full warp
             // instruction on lanes that would discard the result.
             const int64_t tbase = ev0 + (tile - t0) * kTile;
-            bool done = false;
-            if (KIND == IPA_MODEL_ANGTIME4D && GRAD && !CACHED && tbase + kTile <= ev1) {
-                done = tile_fast<WEIGHTED>(wc, &mt, cols, tbase, sbuf, lane, acc, &prod, &esum);
-                if (!done) {
+            int first = 0;               // rows left to the plain loop
+            if (KIND == IPA_MODEL_ANGTIME4D && GRAD && !CACHED) {
+                const int64_t left = ev1 - tbase;
+                const int rows = !wc.k.fixed ? 0 : (left >= kTile ? kPerLane : (int)(left >> 5));
+                if (rows > 0 && tile_fast<WEIGHTED>(wc, &mt, cols, tbase, rows, sbuf, lane, acc, &prod, &esum)) {
+                    first = rows;
+                } else if (rows > 0) {
 #pragma unroll
                     for (int a = 0; a < NA; ++a) acc[a] = 0.0;
                     prod = 1.0;
                     esum = 0;
                 }
             }
-            if (!done)
-                tile_plain<KIND, GRAD, CACHED, WEIGHTED>(wc, &mt, cols, tbase, ev1, sbuf, lane, acc, &prod, &esum);
+            if (first < kPerLane)
+                tile_plain<KIND, GRAD, CACHED, WEIGHTED>(wc, &mt, cols, first, tbase, ev1, sbuf, lane, acc, &prod, &esum);
             acc[0] += log_of(prod, esum, &mt);
             const double share = warp_butterfly<NA>(acc, lane);
             // the group and segment levels; the warp that completes the
             // segment writes its NLL and gradient
             if (!tile_commit<NA>(share, lane, tile, t0, t1, seg, partials, gcount, counters, acc)) continue;
-            finalize<KIND, GRAD, CACHED>(wc.c, acc, n_par, out + (size_t)seg * out_stride, lane);
+            finalize<KIND, GRAD, CACHED>(wc, acc, n_par, out + (size_t)seg * out_stride, lane);
             if (lane == 0) counters[seg] = 0u;
         }
     }
@@ -703,7 +673,7 @@ ipa_status launch_t(const Cols& cols, int64_t n, const int64_t* seg_begin, const
     const LaunchCfg cfg = force ? *force : launch_cfg(KIND, GRAD, CACHED, n_seg > 1, tiles);
     const int W = cfg.warps_per_block >= 1 && cfg.warps_per_block <= kMaxWarps ? cfg.warps_per_block : 1;
     const int K = cfg.tiles_per_take >= 1 ? cfg.tiles_per_take : 1;
-    const size_t smem = (size_t)W * (sizeof(WarpConsts) + kSub * 32 * sizeof(double2));
+    const size_t smem = (size_t)W * (sizeof(Consts) + kSub * 32 * sizeof(double2));
     // resident blocks per SM for each block size (cached per device and variant)
     static int occ[64][kMaxWarps + 1] = {};
     int dev = 0;

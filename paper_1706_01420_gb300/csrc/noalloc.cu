@@ -30,7 +30,7 @@ namespace {
 
 constexpr int64_t kNoAllocMaxEvents = IPA_NOALLOC_MAX_EVENTS;
 constexpr int64_t kNoAllocMaxTiles = kNoAllocMaxEvents / kTile + 1;
-constexpr size_t kConstsBytes = 1024;     // one Consts record, padded
+constexpr size_t kConstsBytes = 1280;     // one Consts record, padded
 constexpr size_t kCounterBytes = 256;     // completion counter and the two work counters, padded
 constexpr size_t kGroupBytes = ((size_t)kNoAllocMaxTiles * sizeof(unsigned) + 255) / 256 * 256;  // group counters
 constexpr size_t kPartialsBytes = (size_t)kNoAllocMaxTiles * kSmallAcc * sizeof(double);

@@ -1,0 +1,89 @@
+"""The fixed-point rows of the 4D likelihood (complete rows of 32 events of a
+tile) and their hand-over to the plain loop, against the oracle:
+
+* event counts around a row, a group of four rows, a tile and several tiles;
+* every unit of time and scale of weights (the fixed-point sums follow the
+  segment's typical r T and the tile's largest weight), with and without
+  background, and no signal at all (no fixed-point coefficients);
+* a tile in which some r T exceeds the sums' range (A near zero, no background)
+  and tiles with events beyond the fitted range (their exponential leaves the
+  fixed-point range), both at full accuracy;
+* a column of ones gives the bits of no column at all.
+
+Tolerance: each gradient component within 2e-13 of the sum of the absolute
+values of the pieces it is built from (the reciprocal's 6e-14, E2's |argument|
+2^-53 with arguments up to 50, and the fixed-point units of 2^-46 of a typical
+term), the NLL within 1e-14 of sum |w log P|.
+"""
+import numpy as np
+import pytest
+
+from paper_1706_01420_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+TH4 = np.array([0.66, 0.045, 0.0, 0.1, 0.52, 0.25, 3.2, 3.1, 0.04, 0.3])
+LO, HI = 0.3, 15.0
+
+
+@pytest.fixture(scope="module")
+def env(oracle):
+    from tests import gpu_common as G
+    G.need_gpu()
+    import torch
+    from paper_1706_01420_gb300 import api
+
+    def grad(ev, th, lo, hi):
+        return api.ipa_nll_grad(api.model_4d(lo, hi), G.to_dev(ev), torch.tensor(th, device="cuda")).cpu().numpy()
+    return oracle, G, grad
+
+
+def compare(env, ev, th, ts=1.0):
+    O, G, grad = env
+    m = O.Model("4d", LO * ts, HI * ts)
+    got = grad(ev, th, LO * ts, HI * ts)
+    f, g = O.nll_grad(m, ev, th)
+    logl, _ = O.nll_grad_terms(m, ev, th)
+    assert abs(got[0] - f) <= 1e-14 * np.abs(logl).sum()
+    assert np.all(np.abs(got[1:] - g) <= 2e-13 * G.grad_scale(O, m, ev, th)), (got[1:], g)
+
+
+@pytest.mark.parametrize("weighted", [False, True])
+@pytest.mark.parametrize("n", [31, 32, 33, 127, 128, 129, 160, 511, 512, 513, 545, 16384 + 33])
+def test_event_counts(env, n, weighted):
+    compare(env, synth.events_4d(n, 41, weighted=weighted), TH4)
+
+
+@pytest.mark.parametrize("f_b", [0.0, 0.1, 0.999, 1.0])
+@pytest.mark.parametrize("ws", [None, 1.0, 1e-30, -3e12])
+@pytest.mark.parametrize("ts", [1e-12, 1.0, 1e9])
+def test_units_and_weight_scales(env, ts, ws, f_b):
+    ev = synth.events_4d(700, 43, weighted=ws is not None)
+    ev["t"] = ev["t"] * ts
+    if ws is not None:
+        ev["w"] = ev["w"] * ws
+    th = TH4.copy()
+    th[0] /= ts
+    th[1:3] *= ts
+    th[3] = f_b
+    compare(env, ev, th, ts)
+
+
+def test_handover_to_the_plain_loop(env):
+    ev = synth.events_4d(1100, 47)
+    th = TH4.copy()
+    th[3:6] = 0.0, 1.0 - 2e-6, 1e-6                       # A near cos^2 thK sin^2 thmu, no background
+    ev["ck"] = np.where(np.abs(ev["ck"]) < 0.1, 0.1, ev["ck"])
+    compare(env, ev, th)
+    ev["ck"][700] = 2.0 ** -13                            # r T 2^17 times the typical one: its tile is redone
+    compare(env, ev, th)
+    ev = synth.events_4d(1100, 53)
+    ev["t"][[5, 600]] = 40.0, 16.5                        # beyond t_hi
+    compare(env, ev, TH4)
+
+
+def test_unit_weights_are_no_weights(env):
+    _, _, grad = env
+    ev = synth.events_4d(1500, 59)
+    ev["ck"][77] = 1.0
+    assert np.array_equal(grad(ev, TH4, LO, HI), grad({**ev, "w": np.ones(1500)}, TH4, LO, HI))
