@@ -1,8 +1,8 @@
 // Step a1 of the hot path: theta -> the Consts record read by every event
-// tile (see consts.cuh for the formulas): one six-warp block per fit for a
-// few fits, one thread per fit for many; the same for the tagged model's
-// record (tagged.cuh) and the phi_s model's (phis_consts.cuh).  This file is compiled without FMA contraction, so
-// both layouts of a record give the same bits.
+// tile (see consts.cuh for the formulas): a block per fit up to kBlockSegs fits,
+// one thread per fit beyond; the same for the tagged model's record
+// (tagged.cuh) and the phi_s model's (phis_consts.cuh).  This file is compiled
+// without FMA contraction, so both layouts of a record give the same bits.
 #include "consts.cuh"
 #include "phis_consts.cuh"
 #include "tagged.cuh"
@@ -10,6 +10,13 @@
 namespace ipa {
 
 namespace {
+// A thread's record is one serial chain (about 50, 28 and 45 us for the 4D,
+// tagged and phi_s models however many fits there are); a block's is short
+// (8 to 11 us) and seven blocks per SM overlap.  Measured, block against
+// thread, us: 512 fits 16 / 52, 14 / 29, 16 / 45; 1024 fits 27 / 47, 22 / 25,
+// 27 / 39; 2048 fits 43 / 47, 39 / 25, 48 / 40.
+constexpr int kBlockSegs = 1024;
+
 // One block of six warps per fit (few fits: latency).
 __global__ void __launch_bounds__(kConstsBlock) consts_block_kernel(ModelDev m, const double* __restrict__ theta,
                                                                     Consts* __restrict__ out) {
@@ -70,7 +77,7 @@ __global__ void __launch_bounds__(kPhisConstsBlock) phis_consts_block_kernel(Mod
 
 ipa_status launch_phis_consts(const ModelDev& m, const double* theta, int n_seg, Consts* out, cudaStream_t st) {
     if (n_seg <= 0) return IPA_OK;
-    if (n_seg < 64)
+    if (n_seg <= kBlockSegs)
         phis_consts_block_kernel<<<n_seg, kPhisConstsBlock, 0, st>>>(m, theta, out);
     else
         phis_consts_kernel<<<(n_seg + 63) / 64, 64, 0, st>>>(m, theta, n_seg, out);
@@ -79,7 +86,7 @@ ipa_status launch_phis_consts(const ModelDev& m, const double* theta, int n_seg,
 
 ipa_status launch_tag_consts(const ModelDev& m, const double* theta, int n_seg, Consts* out, cudaStream_t st) {
     if (n_seg <= 0) return IPA_OK;
-    if (n_seg < 64)
+    if (n_seg <= kBlockSegs)
         tag_consts_block_kernel<<<n_seg, kTagConstsBlock, 0, st>>>(m, theta, out);
     else
         tag_consts_kernel<<<(n_seg + 63) / 64, 64, 0, st>>>(m, theta, n_seg, out);
@@ -91,7 +98,7 @@ ipa_status launch_consts(const ModelDev& m, const double* theta, int n_seg, Cons
     if (n_seg <= 0) return IPA_OK;
     if (m.kind == IPA_MODEL_TAGGED1D) return launch_tag_consts(m, theta, n_seg, out, st);
     if (m.kind == IPA_MODEL_PHIS) return launch_phis_consts(m, theta, n_seg, out, st);
-    if (n_seg >= 64) {
+    if (n_seg > kBlockSegs) {
         consts_thread_kernel<<<(n_seg + 63) / 64, 64, 0, st>>>(m, theta, n_seg, out);
         return cuda_fail(cudaGetLastError(), "consts kernel launch");
     }
