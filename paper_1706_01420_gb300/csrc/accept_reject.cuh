@@ -94,7 +94,7 @@ __device__ __forceinline__ double u01_int(uint32_t a, uint32_t b) {
     return q62_to_double_nb((long long)(u53(a, b) << 9), 0);
 }
 __device__ __forceinline__ double sym_int(uint32_t a, uint32_t b) {
-    return q62_to_double_nb((long long)(u53(a, b) << 10) - kOneQ62, 0);
+    return q62_to_double_nb((long long)(u53(a, b) << 10) - (1ll << 62), 0);
 }
 
 constexpr float kTwoM32 = 2.3283064365386963e-10f;   // 2^-32

@@ -412,6 +412,17 @@ __device__ inline void coef_flags(Consts* c, int sc) {
     c->k.pad[0] = c->k.pad[1] = c->k.pad[2] = 0;
 }
 
+// The fixed-point parameters of the tagged and phi_s models' time functions: exponential i of
+// the rates Gamma_H, Gamma_L, Gamma (with Dm), or the phase (i = 3).
+__device__ inline FxExp fx_field(const ModelDev& m, double GH, double GL, double Gamma, double Dm, double sigma,
+                                 double mu, int i) {
+    const double a = abs_bits(m.t_lo), b = abs_bits(m.t_hi), tm = a > b ? a : b;
+    if (i == 3) return fx_phase_setup(Dm, mu, Gamma * Dm * sigma * sigma, tm);
+    const double x = i == 0 ? GH : (i == 1 ? GL : Gamma);
+    const double d = i == 2 ? Dm : 0.0;
+    return fx_exp_setup(x, mu, 0.5 * (x - d) * (x + d) * sigma * sigma, tm);
+}
+
 // The tables of exp_fast, sincos_fast and erfcx_fast into shared memory
 // (block-cooperative; the caller syncs).
 __device__ inline void load_consts_tables(MathTables* t) {

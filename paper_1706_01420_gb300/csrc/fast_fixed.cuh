@@ -67,7 +67,7 @@ __device__ __forceinline__ long long fx_odd(double x, int top) {
 }
 
 // v 2^(e2 - 62) as a double, rounded to nearest (halves away from zero; +0 for 0; the
-// result must be normal).  Half of q62_to_double_nb's instructions.
+// result must be normal).  Half of q62_to_double's instructions.
 __device__ __forceinline__ double fx_to_double(long long v, int e2) {
     const unsigned long long a = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
     const int lz = __clzll((long long)a);
@@ -98,16 +98,11 @@ constexpr int kE5 = 1466040222;                   // 2^70
 constexpr int kE6 = 2646306;                      // 2^70
 }  // namespace fxc
 
-// sin and cos of phi in Q62, |phi| < 4, with an error of a few 2^-60: phi in units
-// of pi/32, nearest table entry, Taylor polynomials of the remainder (their
-// inner terms, which reach the result by powers of a square below 2^-9, in 32
-// bits), the angle-addition formulas.
-__device__ __forceinline__ void fx_sincos(double phi, const MathTables* t, long long* sn, long long* cs) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(phi);
-    const unsigned long long X = fx_magnitude(b, 2);                          // |phi| in Q61
-    const unsigned long long U = __umul64hi(X, fp64tab::kTwoOverPiQ64);       // |phi| 32/pi in Q57
-    const unsigned k = (unsigned)((U + (1ull << 56)) >> 57);
-    const long long f = (long long)((U - ((unsigned long long)k << 57)) << 6);   // Q63, |f| <= 1/2
+// sin and cos of (pi/32) (k + f) in Q62, 0 <= k <= 64 and f in Q63, |f| <= 1/2, with an
+// error of a few 2^-60: Taylor polynomials of the remainder (their inner terms, which
+// reach the result by powers of a square below 2^-9, in 32 bits), the angle-
+// addition formulas.
+__device__ __forceinline__ void fx_sincos_at(unsigned k, long long f, const MathTables* t, long long* sn, long long* cs) {
     const Fx F = fx(f);
     const long long z = fx_mad(F, F, 0);                                      // f^2 in Q62
     const Fx Z = fx(z);
@@ -121,11 +116,21 @@ __device__ __forceinline__ void fx_sincos(double phi, const MathTables* t, long 
     const long long i4 = fxc::kC4 - (((long long)z32 * i6) >> 10);
     const long long i2 = fxc::kC2 - (fx_mad(Z, fx(i4), 0) >> 8);              // Q70
     const Fx nc = fx(-(fx_mad(Z, fx(i2), 0) >> 3));                           // -(1 - cos r) in Q65
-    const unsigned kk = k > 64u ? 64u : k;
-    const long long Sk = t->sq[kk], Ck = t->cq[kk];
+    const long long Sk = t->sq[k], Ck = t->cq[k];
     const Fx S = fx(Sk), C = fx(Ck);
-    const long long sv = Sk + (fx_mad(C, sr, fx_mad(S, nc, 0)) >> 1);         // sums in Q63
+    *sn = Sk + (fx_mad(C, sr, fx_mad(S, nc, 0)) >> 1);                        // sums in Q63
     *cs = Ck + ((fx_mad(C, nc, 0) - fx_mad(S, sr, 0)) >> 1);
+}
+
+// sin and cos of phi in Q62, |phi| < 4: phi in units of pi/32, nearest table entry.
+__device__ __forceinline__ void fx_sincos(double phi, const MathTables* t, long long* sn, long long* cs) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(phi);
+    const unsigned long long X = fx_magnitude(b, 2);                          // |phi| in Q61
+    const unsigned long long U = __umul64hi(X, fp64tab::kTwoOverPiQ64);       // |phi| 32/pi in Q57
+    const unsigned k = (unsigned)((U + (1ull << 56)) >> 57);
+    const long long f = (long long)((U - ((unsigned long long)k << 57)) << 6);   // Q63, |f| <= 1/2
+    long long sv;
+    fx_sincos_at(k > 64u ? 64u : k, f, t, &sv, cs);
     *sn = (long long)b < 0 ? -sv : sv;
 }
 
@@ -154,8 +159,15 @@ __device__ __forceinline__ long long fx_sqrt_product(long long a, long long b, l
     return (long long)((s << 1) >> ((e2 - 1) & 63));
 }
 
-// Whether fx_basis holds its accuracy (the range of basis_q62_ok).
-__device__ __forceinline__ bool fx_angles_ok(double ck, double cl, double phi) { return basis_q62_ok(ck, cl, phi); }
+// Whether fx_basis holds its accuracy for these angles: |phi| < 4 and |cos thK|,
+// |cos thmu| < 1 - 2^-17, so that sin^2 = 1 - cos^2 >= 2^-16 and its fixed-point
+// error (2^-60 absolute) stays below 2^-44 relative.  Outside (about 1.5e-5 of
+// uniformly distributed angles, and invalid |cos| > 1 or NaN) the caller uses the
+// FP64 basis.
+__device__ __forceinline__ bool fx_angles_ok(double ck, double cl, double phi) {
+    constexpr double kMaxCos = 1.0 - 0x1p-17;
+    return abs_below(ck, kMaxCos) && abs_below(cl, kMaxCos) && abs_below(phi, 4.0);
+}
 
 // Ten products of the helicity angles in Q62 (absolute error a few 2^-60), a basis
 // of the f'_k (angular.cuh) that takes one product less each:
@@ -190,15 +202,14 @@ __device__ __forceinline__ void fx_basis(double ck, double cl, double phi, const
     g[9] = fx_q62(CK, SL);
 }
 
-// Parameters of fx_exp, part of a segment's record (ipa_internal.cuh): y = c - t g in units of
-// 1/64 octave at 2^ysh, t in fixed point (top), for
-//   2 e^{-Gamma tau + Gamma^2 sigma^2 / 2} = 2^(y/64),
-//   y = 64 (1 + (Gamma mu + Gamma^2 sigma^2 / 2) / ln2) - t 64 Gamma / ln2,
-// and |t| < 2^(top - 1).  The scale keeps |y| 2^ysh < 2^60.  Compiled without FMA contraction.
-__device__ inline FxExp fx_exp_setup(double Gamma, double mu, double c_exp, double t_most) {
-    constexpr double kInv = 92.332482616893656877;       // 64 / ln2
+// A linear function of t, y = c - t g with g = rate (inv + inv_lo), in fixed point: part of
+// a segment's record (ipa_internal.cuh).  y has ysh fraction bits (|y| 2^ysh < 2^60), t is taken
+// with `top`, |t| < 2^(top - 1); g is carried to 2^-61 of itself, so that the error of y does not
+// grow with t.  ok = 0 where some |y| could reach 65000 (or is NaN).  Compiled without FMA
+// contraction.
+__device__ inline FxExp fx_line_setup(double rate, double inv, double inv_lo, double c, double t_most) {
     FxExp s = {0, 0, 0, 2, 32, 0, 0};
-    const double g = Gamma * kInv, c = 64.0 + (Gamma * mu + c_exp) * kInv;
+    const double g = rate * inv, g_lo = fma(rate, inv, -g) + rate * inv_lo;
     const int e = (int)((__double_as_longlong(t_most) >> 52) & 0x7FF) - 1022;      // t_most < 2^e
     if (!(t_most > 0.0) || e > 60 || e < -60) return s;
     const double ag = abs_bits(g), m = ag * __longlong_as_double((long long)(e + 1023) << 52) + abs_bits(c);
@@ -207,12 +218,21 @@ __device__ inline FxExp fx_exp_setup(double Gamma, double mu, double c_exp, doub
     s.top = e + 1;
     s.ysh = 60 - (ey > 6 ? ey : 6);
     // c 2^ysh and g 2^(ysh + top + 1), both below 2^62
-    const long long cb = fx_signed(c, 63 - s.ysh), gb = fx_signed(g, 62 - s.ysh - s.top);
-    s.c = cb;
-    s.gh = fx(gb).h;
-    s.gl = fx(gb).l;
+    s.c = fx_signed(c, 63 - s.ysh);
+    const Fx gf = fx(fx_signed(g, 62 - s.ysh - s.top) + fx_signed(g_lo, 62 - s.ysh - s.top));
+    s.gh = gf.h;
+    s.gl = gf.l;
     s.ok = 1;
     return s;
+}
+
+// For fx_exp: 2 e^{-Gamma tau + c_exp} = 2^(y/64), y = 64 (1 + (Gamma mu + c_exp) / ln2) - t 64 Gamma / ln2.
+__device__ inline FxExp fx_exp_setup(double Gamma, double mu, double c_exp, double t_most) {
+    return fx_line_setup(Gamma, 92.33248261689366, 1.3027375194195861e-15, 64.0 + (Gamma * mu + c_exp) * 92.33248261689366, t_most);
+}
+// For fx_phase: Dm tau - ph0 in units of pi/32.
+__device__ inline FxExp fx_phase_setup(double Dm, double mu, double ph0, double t_most) {
+    return fx_line_setup(neg_bits(Dm), 10.185916357881302, -6.297176536058395e-16, neg_bits(Dm * mu + ph0) * 10.185916357881302, t_most);
 }
 
 // 2^(y / 64) for y in fixed point with ysh fraction bits, as a double: table and Taylor
@@ -236,16 +256,25 @@ __device__ __forceinline__ double fx_exp2(long long y, int ysh, const MathTables
                                             ((unsigned long long)(unsigned)(*x + 1023) << 52)));
 }
 
-// 2 e^{-Gamma tau + Gamma^2 sigma^2 / 2} at t (relative error below 2^-54, most of it from
-// y's last place); *ok is cleared where t or the result lies outside its range.
-__device__ __forceinline__ double fx_exp(double t, const FxExp& s, const MathTables* mt, bool* ok) {
-    const long long T = fx_signed(t, s.top);
+// 2 e^{-Gamma tau + Gamma^2 sigma^2 / 2} (fx_exp_setup) at t, T = fx(fx_signed(t, s.top)); relative
+// error below 2^-54, most of it from y's last place.  *ok is cleared where the result lies
+// outside its range (the caller checks fx_in_range).
+__device__ __forceinline__ double fx_exp(Fx T, const FxExp& s, const MathTables* mt, bool* ok) {
     int x;
-    const double v = fx_exp2(s.c - fx_mad(fx(T), Fx{s.gh, s.gl}, 0), s.ysh, mt, &x);
-    // |t| within the range, and a normal result
-    const unsigned th = (unsigned)((unsigned long long)__double_as_longlong(t) >> 52) & 0x7FFu;
-    *ok = *ok && (int)th - 1022 < s.top && (unsigned)(x + 1015) < 2030u;
+    const double v = fx_exp2(s.c - fx_mad(T, Fx{s.gh, s.gl}, 0), s.ysh, mt, &x);
+    *ok = *ok && (unsigned)(x + 1015) < 2030u;
     return v;
+}
+__device__ __forceinline__ bool fx_in_range(double t, int top) {
+    return (int)((unsigned)((unsigned long long)__double_as_longlong(t) >> 52) & 0x7FFu) - 1022 < top;
+}
+
+// sin and cos (Q62) of the phase of fx_phase_setup at t.
+__device__ __forceinline__ void fx_phase(Fx T, const FxExp& s, const MathTables* mt, long long* sn, long long* cs) {
+    const unsigned long long y = (unsigned long long)(s.c - fx_mad(T, Fx{s.gh, s.gl}, 0));
+    const unsigned long long up = y + (1ull << ((s.ysh - 1) & 63));
+    const unsigned k = (unsigned)((long long)up >> (s.ysh & 63));
+    fx_sincos_at(k & 63u, (long long)((up << ((64 - s.ysh) & 63)) ^ (1ull << 63)) >> 1, mt, sn, cs);
 }
 
 // e^a for -705 <= a <= 0: |a| in units of ln2/64, its fixed point following its
@@ -260,7 +289,7 @@ __device__ __forceinline__ double fx_exp_neg(double a, const MathTables* mt) {
     return fx_exp2(-fx_mad(fx(T), kInv, 0), (54 - top) & 63, mt, &x);
 }
 
-// erfcx(x) = exp(x^2) erfc(x) for 0 <= x <= 6.25 (the pieces of erfcx_poly_q); larger x,
+// erfcx(x) = exp(x^2) erfc(x) for 0 <= x <= 6.25 (the pieces of erfcx_poly); larger x,
 // infinities and NaN are evaluated as 6.25.
 __device__ __forceinline__ double fx_erfcx(double x, const MathTables* t) {
     using namespace fp64tab;

@@ -19,7 +19,7 @@
 //   erfcx_poly(x)    exp(x^2) erfc(x) for 0 <= x <= 6.25: 13 pieces of width 1/2
 //                    centred at k/2, degree-13 Chebyshev interpolants (relative
 //                    error ~2e-16); erfcx_fast falls back to erfcx() above 6.25.
-//                    (erfcx_poly_q in int_math.cuh evaluates the same pieces in
+//                    (fx_erfcx in fast_fixed.cuh evaluates the same pieces in
 //                    fixed point on the integer pipe.)
 #pragma once
 

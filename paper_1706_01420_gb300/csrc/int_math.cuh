@@ -21,16 +21,10 @@
 //               2^(j/64) (Q62, j = k mod 64) and 2^floor(k/64).  Relative error
 //               before the final rounding: about 2^-53 from the input
 //               quantisation for |a| < 1/2, a few 2^-62 otherwise.
-//   erfcx_poly_q  0 <= x <= 6.25: x in Q60, k = nearest multiple of 1/2 (piece
-//               centre), u = x - k/2 in Q63 (|u| <= 1/4), the degree-13
-//               Chebyshev interpolant of the piece (monomials in u, Q62) by
-//               Horner's rule with 64 x 64 -> 128-bit products.  Absolute error
-//               before the final rounding below 2^-61 (the values are above
-//               0.088, so below 2e-17 relative, plus the interpolant's own
-//               ~1e-16).
 //
 // Outside these ranges sincos_int and exp_int fall back to the table-driven
-// FP64 functions; erfcx_fast_q falls back to the library erfcx.
+// FP64 functions.  fast_fixed.cuh has cheaper, branch-free forms of narrower ranges
+// for the event loops; these serve what lies outside those.
 #pragma once
 
 #include "fp64_math.cuh"
@@ -181,88 +175,9 @@ __device__ __forceinline__ long long to_q62(double x) {
     return (b >> 63) ? -v : v;
 }
 
-// (a b) in Q62 for a, b in signed Q62 with |a b| < 2: the high product shifted
-// left by 2 (the two lowest bits are lost: error below 2^-60).
-__device__ __forceinline__ long long mul_q62(long long a, long long b) { return __mul64hi(a, b) << 2; }
-
-constexpr long long kOneQ62 = 1ll << 62;
-
-// sqrt(x) in Q62 for x in [0, 1] given in Q124 (a product of two Q62 values,
-// so that small x keep their relative precision): an FP32 seed refined by two
-// Newton steps on the exact 128-bit residual (relative error about 2^-60, plus
-// 2^-62 absolute from the final shift).
-__device__ __forceinline__ long long sqrt_q124(unsigned __int128 X) {
-    if (X == 0) return 0;
-    const unsigned long long xh = (unsigned long long)(X >> 64), xl = (unsigned long long)X;
-    const int lz = xh ? __clzll((long long)xh) : 64 + __clzll((long long)xl);
-    const int d = 124 - (127 - lz);                    // >= 0: x <= 1
-    const int s = d & ~1;                              // even shift: xn = Xn 2^-124 in [1/2, 2)
-    const unsigned __int128 Xn = X << s;
-    const int top = 127 - lz + s;                      // 123 or 124
-    const unsigned fb = ((unsigned)(top - 124 + 127) << 23) | ((unsigned)(Xn >> (top - 23)) & 0x7FFFFFu);
-    const float y0f = rsqrtf(__uint_as_float(fb));     // ~1/sqrt(xn) in (0.7, 1.42)
-    const unsigned yb = __float_as_uint(y0f);
-    const int ye = (int)((yb >> 23) & 0xFF) - 127;     // -1 or 0
-    const long long Y0 = (long long)(((unsigned long long)((yb & 0x7FFFFF) | 0x800000)) << (39 + ye));
-    long long Q = mul_q62((long long)(Xn >> 62), Y0);  // ~sqrt(xn) in Q62
-#pragma unroll
-    for (int it = 0; it < 2; ++it) {
-        const __int128 R = (__int128)Xn - (__int128)Q * Q;               // residual in Q124
-        Q += __mul64hi((long long)(R >> 62), Y0) << 1;                    // + R y0 / 2
-    }
-    return Q >> (s >> 1);
-}
-
-// 1 - x^2 in Q62 for x in signed Q62, |x| <= 1, from the exact square
-// (error below 2^-62).
-__device__ __forceinline__ long long one_minus_sq_q62(long long x) {
-    return (long long)((((unsigned __int128)1 << 124) - (unsigned __int128)((__int128)x * x)) >> 62);
-}
-
-// Whether basis_q62 keeps its accuracy for these angles: |phi| < 4 and
-// |cos thK|, |cos thmu| < 1 - 2^-17, so that sin^2 = 1 - cos^2 >= 2^-16 and its
-// fixed-point error (2^-60 absolute) stays below 2^-44 relative.  Outside (about
-// 1.5e-5 of uniformly distributed angles, and invalid |cos| > 1 or NaN) the
-// caller uses the FP64 basis.
-__device__ __forceinline__ bool basis_q62_ok(double ck, double cl, double phi) {
-    constexpr double kMaxCos = 1.0 - 0x1p-17;
-    return abs_below(ck, kMaxCos) && abs_below(cl, kMaxCos) && abs_below(phi, 4.0);
-}
-
-// The ten unscaled angular products f'_k (sec. 4 helicity basis, without their
-// constant factors) in signed Q62 (absolute error a few 2^-60), for angles
-// that pass basis_q62_ok.  sin thK sin thmu = sqrt((1 - cos^2 thK)(1 - cos^2 thmu)).
-__device__ __forceinline__ void basis_q62(double ck, double cl, double phi, const MathTables* t, long long F[10]) {
-    const unsigned long long pb = (unsigned long long)__double_as_longlong(phi);
-    long long sp, cp;
-    sincos_q62(pb, t, &sp, &cp);
-    if (pb >> 63) sp = -sp;
-    const long long CK = to_q62(ck), CL = to_q62(cl);
-    const long long sk2 = one_minus_sq_q62(CK), sl2 = one_minus_sq_q62(CL);
-    const long long ck2 = kOneQ62 - sk2, cl2 = kOneQ62 - sl2;
-    const long long cp2 = mul_q62(cp, cp);
-    const unsigned __int128 sksl2_124 = (unsigned __int128)((__int128)sk2 * sl2);
-    const long long sksl2 = (long long)(sksl2_124 >> 62);
-    const long long q = sqrt_q124(sksl2_124);
-    const long long slcp2 = mul_q62(sl2, cp2);
-    F[0] = mul_q62(ck2, sl2);
-    F[1] = mul_q62(sk2, kOneQ62 - slcp2);
-    F[2] = mul_q62(sk2, slcp2 + cl2);
-    F[3] = mul_q62(sksl2, mul_q62(sp, cp));
-    const long long a = mul_q62(q, mul_q62(CK, CL));
-    F[4] = mul_q62(a, cp);
-    F[5] = mul_q62(a, sp);
-    F[6] = sl2;
-    const long long bq = mul_q62(q, CL);
-    F[7] = mul_q62(bq, cp);
-    F[8] = mul_q62(bq, sp);
-    F[9] = mul_q62(CK, sl2);
-}
-
 // ---- branch-free forms ----
 // The same values as above for inputs in the functions' ranges; outside them the
-// values are unspecified, every shift stays below 64 and every table index
-// inside its table.  fast_fixed.cuh has cheaper forms of the same functions.
+// values are unspecified and every shift stays below 64.
 
 // q62_to_double, also for v = 0 (which gives +0).
 __device__ __forceinline__ double q62_to_double_nb(long long v, int e2) {
@@ -286,65 +201,12 @@ __device__ __forceinline__ unsigned long long shift_nb(unsigned long long M, int
     return sh >= 0 ? up : (sh > -64 ? dn : 0ull);
 }
 
-// exp_int without its range test (-705 < a < 709, the caller checks).
-__device__ __forceinline__ double exp_int_nb(double a, const MathTables* t) {
-    using namespace fp64tab;
-    const unsigned long long b = (unsigned long long)__double_as_longlong(a);
-    const int E = (int)((b >> 52) & 0x7FFull) - 1023;
-    const bool neg = (b >> 63) != 0;
-    const unsigned long long M = (b & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull;
-    const unsigned long long A = shift_nb(M, E + 1);       // |a| in Q53
-    const unsigned long long P = __umul64hi(A, kInvLn2x64Q56);
-    const unsigned long long k = (P + (1ull << 44)) >> 45;
-    const unsigned __int128 kl = (unsigned __int128)k * kLn2d64Q128Hi +
-                                 (((unsigned __int128)k * kLn2d64Q128Lo) >> 64);
-    const long long r = (long long)(((__int128)A << 11) - (__int128)kl);
-    const long long rs = neg ? -r : r;
-    const long long ks = neg ? -(long long)k : (long long)k;
-    long long v = kExpC6Q63;
-    v = kExpC5Q63 + __mul64hi(rs, v);
-    v = kExpC4Q63 + __mul64hi(rs, v);
-    v = kExpC3Q63 + __mul64hi(rs, v);
-    v = kExpC2Q63 + __mul64hi(rs, v);
-    const long long pm = rs + (__mul64hi(__mul64hi(rs, v), rs) << 1);
-    const long long T = t->eq[ks & 63];
-    const long long y = T + __mul64hi(T, pm);
-    return q62_to_double_nb(y, (int)(ks >> 6));
-}
-
 // to_q62 for any double (unspecified outside |x| <= 1).
 __device__ __forceinline__ long long to_q62_nb(double x) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(x);
     const unsigned long long M = (b & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull;
     const long long v = (long long)shift_nb(M, (int)((b >> 52) & 0x7FFull) - 1023 + 10);
     return (b >> 63) ? -v : v;
-}
-
-// erfcx(x) = exp(x^2) erfc(x) for 0 <= x <= 6.25 from the piecewise
-// polynomial of fp64_tables.cuh (erfcx_poly's pieces), on the integer pipe.  x
-// above 6.25, infinite or NaN is evaluated as 6.25 and a negative x as |x|: the
-// value is then meaningless and callers select it away (erfcx_fast_q).  The
-// Horner loop is not unrolled: unrolled, the 64-bit products of the kernels
-// that call this twice per event overflowed the instruction cache.
-__device__ __forceinline__ double erfcx_poly_q(double x, const MathTables* t) {
-    using namespace fp64tab;
-    long long b = __double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFll;
-    b = b > 0x4019000000000000ll ? 0x4019000000000000ll : b;      // 6.25
-    const unsigned long long M = ((unsigned long long)b & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull;
-    const unsigned long long X = shift_nb(M, (int)(b >> 52) - 1023 + 8);   // x in Q60, < 2^63
-    int k = (int)((X + (1ull << 58)) >> 59);                      // nearest piece centre k/2
-    k = k > kErfcxPieces - 1 ? kErfcxPieces - 1 : k;
-    const long long u = (long long)((X - ((unsigned long long)k << 59)) << 3);   // Q63, |u| <= 2^61
-    const long long* c = t->exq + k * kErfcxCoeffs;
-    long long v = c[kErfcxCoeffs - 1];
-#pragma unroll 1
-    for (int i = kErfcxCoeffs - 2; i >= 0; --i)
-        v = c[i] + (long long)((unsigned long long)__mul64hi(v, u) << 1);   // |v| < 1.5 in Q62
-    return q62_to_double_nb(v, 0);
-}
-
-__device__ __forceinline__ double erfcx_fast_q(double x, const MathTables* t) {
-    return above(x, 6.25) ? erfcx(x) : erfcx_poly_q(x, t);
 }
 
 }  // namespace ipa

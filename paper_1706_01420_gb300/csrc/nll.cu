@@ -82,7 +82,7 @@ __device__ __forceinline__ double2 gauss_erfcx(const Consts& c, double tau, cons
     return make_double2(g * X, zneg ? g : -g);
 }
 
-// A' = sum_k hq_k f_k in FP64 (cached basis, or angles outside basis_q62_ok).
+// A' = sum_k hq_k f_k in FP64 (cached basis, or angles outside fx_angles_ok).
 __device__ __forceinline__ double amplitude_sum(const double* hq, const double* f) {
     double Ap = hq[0] * f[0];
 #pragma unroll
@@ -161,7 +161,7 @@ __device__ __forceinline__ void event(const Consts& c, const MathTables* mt, dou
 // by the plain loop.  Either way the tile's sums depend only on its events, never
 // on the launch geometry.
 //
-// Measured (one pass of the public call, 512 toys of 2000 events, then 1e7
+// Measured (one pass of the public call, 512 toys of 20 000 events, then 1e7
 // weighted events): the angular products, A and the exponential in FP64 and
 // 14-instruction 64-bit products, an FP64 multiply-add per angular sum: 1060 and
 // 1073 us; this path: 643 and 685.  About 1150 warp instructions per row now
@@ -198,7 +198,8 @@ __device__ __forceinline__ void load_row(const Consts& c, const MathTables* mt, 
     v.w = WEIGHTED ? __ldg(cols.w + e) : 1.0;
     v.tau = t - c.mu;
     bool ok_exp = true;
-    v.E2 = fx_exp(t, c.k.ex, mt, &ok_exp);
+    v.E2 = fx_exp(fx(fx_signed(t, c.k.ex.top)), c.k.ex, mt, &ok_exp);
+    ok_exp = ok_exp && fx_in_range(t, c.k.ex.top);
     fx_basis(ck, cl, phi, mt, v.g);
     long long A = 0;
 #pragma unroll

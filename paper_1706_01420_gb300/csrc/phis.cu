@@ -113,14 +113,17 @@ __device__ inline void c_row(int k, double pr, double pi, double one, double c, 
     }
 }
 
-// The ten f'_k on the integer pipe, rounded once to double (as in the 4D kernel:
-// 35 FP64 instructions less per event; worth 2 % here), in FP64 near |cos| = 1.
+// The ten f'_k on the integer pipe, rounded once to double (1e6 events: 313 us with
+// 14-instruction 64-bit products, 300 us with those of fast_fixed.cuh), in FP64 near
+// |cos| = 1.
 __device__ __forceinline__ void phis_basis(double ck, double cl, double phi, const MathTables* mt, double f[10]) {
-    if (basis_q62_ok(ck, cl, phi)) {
-        long long F[10];
-        basis_q62(ck, cl, phi, mt, F);
+    if (fx_angles_ok(ck, cl, phi)) {
+        long long g[10];
+        fx_basis(ck, cl, phi, mt, g);
+        const long long F[10] = {g[0] - g[2], g[1] - g[3], g[1] - g[2] + g[3], g[4], g[5],
+                                 g[6], g[0], g[7], g[8], g[9]};
 #pragma unroll
-        for (int k = 0; k < 10; ++k) f[k] = q62_to_double_nb(F[k], 0);
+        for (int k = 0; k < 10; ++k) f[k] = fx_to_double(F[k], 0);
     } else {
         basis_unscaled(ck, cl, phi, mt, f);
     }
@@ -163,17 +166,13 @@ __device__ __forceinline__ void phis_event(const PhisWarp& pw, const MathTables*
                                            int* esum) {
     const PhisConsts& c = pw.c;
     const double tau = t - c.mu;
-    const double E2H = exp_int(fma(-c.GH, tau, c.cH2), mt);
-    const double E2L = exp_int(fma(-c.GL, tau, c.cL2), mt);
-    const double E2C = exp_int(fma(-c.Gamma, tau, c.cC2), mt);
-    double sn, cn;
-    sincos_int_wide(fma(c.Dm, tau, -c.ph0), mt, &sn, &cn);
+    const TimeValues v = time_values(c, t, tau, mt);
     const long long bH = __double_as_longlong(sl.xH), bL = __double_as_longlong(sl.xL);
     const long long bG = __double_as_longlong(sl.gx);
-    const double H = bH < 0 ? -sl.xH : E2H - sl.xH;
-    const double L = bL < 0 ? -sl.xL : E2L - sl.xL;
-    const double Cr = q * (bG < 0 ? sl.wr : fma(E2C, cn, -sl.wr));
-    const double Ci = q * (bG < 0 ? sl.wi : fma(E2C, sn, -sl.wi));
+    const double H = bH < 0 ? -sl.xH : v.H - sl.xH;
+    const double L = bL < 0 ? -sl.xL : v.L - sl.xL;
+    const double Cr = q * (bG < 0 ? sl.wr : fma(v.C, v.cn, -sl.wr));
+    const double Ci = q * (bG < 0 ? sl.wi : fma(v.C, v.sn, -sl.wi));
     // F+, F-, FU, FV; the rate's coefficients of L and H, and of D2 Ci (X)
     const double Fp = fma(pw.eq[2], f[4], fma(pw.eq[1], f[1], pw.eq[0] * f[0]));
     const double Fm = fma(pw.eq[5], f[8], fma(pw.eq[4], f[6], pw.eq[3] * f[2]));
@@ -322,8 +321,9 @@ __device__ __forceinline__ void phis_finalize(const PhisConsts& c, double v, int
     for (int j = IPA_NPAR_PHIS + lane; j < n_par; j += 32) out[1 + j] = 0.0;
 }
 
-// Three blocks per SM (164 registers, no spills) over two (200): 404 -> 367 us for
-// 1e6 events, and four (128 registers, spills) 392 us.  The 40-product form with
+// Three blocks per SM (168 registers, no spills) over two (200): 404 -> 367 us for
+// 1e6 events, and four (128 registers, spills) 392 us; with the time functions and the
+// angles in cheap fixed-point products (fast_fixed.cuh, faddeeva.cuh) 300 us.  The 40-product form with
 // its 47 sums took 623 us at two blocks (237 registers).  A tile's team is the
 // block's four warps (each takes 4 of every lane's 16 events), so that a small
 // fit's tiles run four FP64 instruction streams at once.

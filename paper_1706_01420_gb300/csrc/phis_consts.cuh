@@ -42,7 +42,8 @@ struct PhisConsts {
     double br[10], bi[10];          // Re, Im of b_k
     double csp;                     // C_SP: factor of the S-P interference terms k = 7, 8, 9
     double qsel;                    // normalisation over both tags (0) or over the tag +1 / -1
-    double pad_;
+    long long fx_ok;                // as in TagConsts
+    FxExp fx[4];
 };
 static_assert(sizeof(PhisConsts) <= sizeof(Consts), "PhisConsts must fit a Consts slot");
 static_assert(sizeof(PhisConsts) % 16 == 0, "PhisConsts must be a multiple of 16 bytes");
@@ -194,7 +195,6 @@ __device__ inline void amp_fields(const double* th, const double* r, const doubl
     const double qsel = th[IPA_PHIS_QNORM];
     c->csp = th[IPA_PHIS_CSP];
     c->qsel = qsel > 0.0 ? 1.0 : (qsel < 0.0 ? -1.0 : 0.0);
-    c->pad_ = 0.0;
 }
 
 // b_k = m_k e^{i psi_k} (the P-wave magnitudes carry 1 - F_S): m_k = (f1 f2) f3,
@@ -398,6 +398,9 @@ __device__ inline void phis_consts_thread(const ModelDev& m, const double* th, c
         }
     }
     theta_fields(th, c);
+    for (int i = 0; i < 4; ++i)
+        c->fx[i] = cdetail::fx_field(m, rate_H(th), rate_L(th), th[IPA_GAMMA], th[IPA_PHIS_DM], th[IPA_SIGMA], th[IPA_MU], i);
+    c->fx_ok = c->fx[0].ok & c->fx[1].ok & c->fx[2].ok & c->fx[3].ok;
     scale_fields(th, rc[0], r[5], c);
     amp_fields(th, r, sw, cw, sw[6], cw[6], c);
     for (int k = 0; k < 10; ++k) b_entry(k, th, r, sw, cw, &c->br[k], &c->bi[k]);
@@ -437,7 +440,7 @@ constexpr int kPhisConstsBlock = 256;
 //            theta alone;
 //   phase 2  warp 0: F and its derivatives at the four real edges; warp 1: the
 //            fields of 1/sigma; warp 2: b_k (lane k) and the amplitude fields;
-//            warp 5: the complex edges;
+//            warp 5: the complex edges; warp 6: the fixed-point parameters;
 //   phase 3  warps 0-2: dN/dtheta_j / N (a parameter per lane) and the fields of 1/N;
 // then every thread copies part of the record out.
 __device__ inline void phis_consts_block(const ModelDev& m, const double* th, PhisConsts* c, PhisBlockScratch* S) {
@@ -485,6 +488,9 @@ __device__ inline void phis_consts_block(const ModelDev& m, const double* th, Ph
             else
                 for (int i = 0; i < 8; ++i) S->ec[8 * lane + i] = 0.0;
         }
+    } else if (w == 6) {
+        if (lane < 4)
+            S->c.fx[lane] = cdetail::fx_field(m, rate_H(th), rate_L(th), th[IPA_GAMMA], th[IPA_PHIS_DM], th[IPA_SIGMA], th[IPA_MU], lane);
     }
     __syncthreads();
 
@@ -496,6 +502,8 @@ __device__ inline void phis_consts_block(const ModelDev& m, const double* th, Ph
     else if (w == 2) {
         const int rest[5] = {IPA_FB, IPA_PHIS_DM, IPA_PHIS_OMEGA, IPA_PHIS_CSP, IPA_PHIS_QNORM};
         j = lane < 5 ? rest[lane] : (lane == 5 ? IPA_NPAR_PHIS : -1);
+    } else if (w == 6 && lane == 0) {
+        S->c.fx_ok = S->c.fx[0].ok & S->c.fx[1].ok & S->c.fx[2].ok & S->c.fx[3].ok;
     }
     if (j >= 0) {
         const double N = norm_N(th, S->F, S->ec, S->sw[6], S->cw[6]), inv_N = cdetail::recip(N);

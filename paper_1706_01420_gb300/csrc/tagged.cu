@@ -7,7 +7,8 @@
 // term is below 1e-17 of its exponential and
 //   2 gH = exp(-Gamma_H tau + Gamma_H^2 sigma^2/2 + ln2),  2 gL likewise,
 //   2 g  = exp(-Gamma tau + (Gamma^2 - Dm^2) sigma^2/2 + ln2) e^{i (Dm tau - Gamma Dm sigma^2)}:
-// three exponentials and one sine/cosine pair, all on the integer pipe.  Events
+// three exponentials and one sine/cosine pair, all on the integer pipe (their
+// arguments are linear in t, in fixed point from the start: fast_fixed.cuh).  Events
 // with t <= tcut (up to about six resolution widths past the peak) also need
 // the Gaussian, two erfcx and one Faddeeva function; as in the 4D kernel they
 // are listed by ballot and evaluated 32 to a pass into the warp's buffer, so
@@ -41,17 +42,13 @@ template <bool GRAD, bool WEIGHTED>
 __device__ __forceinline__ void tag_event(const TagConsts& c, const MathTables* mt, double t, double q, double w,
                                           const TagSlow& sl, double* acc, double* prod, int* esum) {
     const double tau = t - c.mu;
-    const double E2H = exp_int(fma(-c.GH, tau, c.cH2), mt);
-    const double E2L = exp_int(fma(-c.GL, tau, c.cL2), mt);
-    const double E2C = exp_int(fma(-c.Gamma, tau, c.cC2), mt);
-    double sn, cn;
-    sincos_int_wide(fma(c.Dm, tau, -c.ph0), mt, &sn, &cn);
+    const TimeValues v = time_values(c, t, tau, mt);
     const long long bH = __double_as_longlong(sl.xH), bL = __double_as_longlong(sl.xL);
     const long long bG = __double_as_longlong(sl.gx);
-    const double T2H = bH < 0 ? -sl.xH : E2H - sl.xH;
-    const double T2L = bL < 0 ? -sl.xL : E2L - sl.xL;
-    const double Cr = bG < 0 ? sl.wr : fma(E2C, cn, -sl.wr);
-    const double Ci = bG < 0 ? sl.wi : fma(E2C, sn, -sl.wi);
+    const double T2H = bH < 0 ? -sl.xH : v.H - sl.xH;
+    const double T2L = bL < 0 ? -sl.xL : v.L - sl.xL;
+    const double Cr = bG < 0 ? sl.wr : fma(v.C, v.cn, -sl.wr);
+    const double Ci = bG < 0 ? sl.wi : fma(v.C, v.sn, -sl.wi);
     const double gx = __longlong_as_double(bG & 0x7FFFFFFFFFFFFFFFll);
     const double P = fma(c.qH, T2H, fma(c.qL, T2L, fma(q * c.qD, Ci, c.cb)));
     if (WEIGHTED && __double_as_longlong(w) != 0x3FF0000000000000ll)

@@ -53,7 +53,8 @@ struct TagConsts {
     double dlnN[8];       // (dN / dtheta_j) / N
     double tcut;          // t above it: every erfc term of the event is below 1e-17 of its exponential
     double MS;            // generator envelope: max of S over the range and both tags (upper bound)
-    double pad_;
+    long long fx_ok;      // all of fx usable
+    FxExp fx[4];          // 2 e^{...} of the three rates (H, L, C) and the phase in fixed point (time_values)
 };
 static_assert(sizeof(TagConsts) <= sizeof(Consts), "TagConsts must fit a Consts slot");
 static_assert(sizeof(TagConsts) % 16 == 0, "TagConsts must be a multiple of 16 bytes");
@@ -176,7 +177,6 @@ __device__ inline void scale_fields(const double* th, double rs, double rV2, Tag
     c->D = 1.0 - 2.0 * th[IPA_OMEGA];
     c->cb = th[IPA_FB] * rV2;
     c->inv_V2 = rV2;
-    c->pad_ = 0.0;
 }
 
 // Record fields from sin/cos phi_s (sn, cn), the cut's root tq and the envelope bounds M.
@@ -247,6 +247,9 @@ __device__ inline void tag_consts_thread(const ModelDev& m, const double* th, co
     double sn, cn;
     sincos_fast(th[IPA_PHIS], mt, &sn, &cn);
     theta_fields(th, c);
+    for (int i = 0; i < 4; ++i)
+        c->fx[i] = cdetail::fx_field(m, rate_H(th), rate_L(th), th[IPA_GAMMA], th[IPA_DM], th[IPA_SIGMA], th[IPA_MU], i);
+    c->fx_ok = c->fx[0].ok & c->fx[1].ok & c->fx[2].ok & c->fx[3].ok;
     scale_fields(th, r[0], r[3], c);
     phase_fields(th, sn, cn, cut_root(th), M, c);
     for (int k = 0; k < 4; ++k)
@@ -275,6 +278,7 @@ constexpr int kTagConstsBlock = 256;
 //   phase 1  warp 0: the six erfcx; warp 1: the six exponentials; warp 2: the
 //            three envelope bounds; warp 3: sin/cos phi_s; warp 4: the four
 //            reciprocals and the cut's root; warp 5: the fields of theta alone;
+//            warp 6: the fixed-point exponentials' and phase's parameters;
 //   phase 2  warp 0: F and its derivatives at the four edges; warp 1: the
 //            phase fields; warp 2: the fields that need 1/sigma;
 //   phase 3  warp 0: N, 1/N, dN/dtheta_j / N (lane j) and the fields of 1/N;
@@ -300,6 +304,9 @@ __device__ inline void tag_consts_block(const ModelDev& m, const double* th, Tag
         else if (lane == 4) S->tq = cut_root(th);
     } else if (w == 5) {
         if (lane == 0) theta_fields(th, &S->c);
+    } else if (w == 6) {
+        if (lane < 4)
+            S->c.fx[lane] = cdetail::fx_field(m, rate_H(th), rate_L(th), th[IPA_GAMMA], th[IPA_DM], th[IPA_SIGMA], th[IPA_MU], lane);
     }
     __syncthreads();
 
@@ -311,6 +318,8 @@ __device__ inline void tag_consts_block(const ModelDev& m, const double* th, Tag
         if (lane == 0) phase_fields(th, S->sn, S->cn, S->tq, S->M, &S->c);
     } else if (w == 2) {
         if (lane == 0) scale_fields(th, S->r[0], S->r[3], &S->c);
+    } else if (w == 6) {
+        if (lane == 0) S->c.fx_ok = S->c.fx[0].ok & S->c.fx[1].ok & S->c.fx[2].ok & S->c.fx[3].ok;
     }
     __syncthreads();
 
@@ -347,9 +356,13 @@ __device__ __forceinline__ TagSlow tag_slow(const C& c, double tau, const MathTa
     // branch-free integer exp, the argument clamped at -705 (the Gaussian is then
     // below 1e-306, nothing against the exponential terms)
     const double gr = -(tau * tau) * c.k_g;
-    const double gx = exp_int_nb(below_neg(gr, -705.0) ? -705.0 : gr, mt);
+    const double gx = fx_exp_neg(below_neg(gr, -705.0) ? -705.0 : gr, mt);
     const double uH = (c.uH0 - tau) * c.k_z, uL = (c.uL0 - tau) * c.k_z, a = (c.uC0 - tau) * c.k_z;
-    const double XH = erfcx_fast_q(abs_bits(uH), mt), XL = erfcx_fast_q(abs_bits(uL), mt);
+    double XH = fx_erfcx(uH, mt), XL = fx_erfcx(uL, mt);
+    if (above(abs_bits(uH), 6.25) || above(abs_bits(uL), 6.25)) {
+        if (above(abs_bits(uH), 6.25)) XH = erfcx(abs_bits(uH));
+        if (above(abs_bits(uL), 6.25)) XL = erfcx(abs_bits(uL));
+    }
     const bool ap = !negative(a);
     double wr, wi;
     faddeeva_uhp(ap ? c.beta : neg_bits(c.beta), abs_bits(a), &wr, &wi);
@@ -360,6 +373,36 @@ __device__ __forceinline__ TagSlow tag_slow(const C& c, double tau, const MathTa
     s.wi = gx * wi;
     s.gx = with_sign(gx, ap);
     return s;
+}
+
+// The doubled exponentials of the three rates and the phase's sine and cosine at t (tau = t -
+// mu), as they enter every event; about 500 integer instructions, no FP64.
+struct TimeValues {
+    double H, L, C, sn, cn;
+};
+template <class C>
+__device__ __noinline__ TimeValues time_values_wide(const C& c, double tau, const MathTables* mt) {
+    TimeValues v;
+    v.H = exp_int(fma(-c.GH, tau, c.cH2), mt);
+    v.L = exp_int(fma(-c.GL, tau, c.cL2), mt);
+    v.C = exp_int(fma(-c.Gamma, tau, c.cC2), mt);
+    sincos_int_wide(fma(c.Dm, tau, -c.ph0), mt, &v.sn, &v.cn);
+    return v;
+}
+template <class C>
+__device__ __forceinline__ TimeValues time_values(const C& c, double t, double tau, const MathTables* mt) {
+    const Fx T = fx(fx_signed(t, c.fx[0].top));           // one scale: all four follow the fitted range
+    bool ok = c.fx_ok && fx_in_range(t, c.fx[0].top);
+    TimeValues v;
+    v.H = fx_exp(T, c.fx[0], mt, &ok);
+    v.L = fx_exp(T, c.fx[1], mt, &ok);
+    v.C = fx_exp(T, c.fx[2], mt, &ok);
+    long long sn, cn;
+    fx_phase(T, c.fx[3], mt, &sn, &cn);
+    v.sn = fx_to_double(sn, 0);
+    v.cn = fx_to_double(cn, 0);
+    if (!ok) v = time_values_wide(c, tau, mt);
+    return v;
 }
 
 // 2 g(tau; x) for real x, exact form (library exp and erfcx).  C: TagConsts or

@@ -87,3 +87,30 @@ def test_unit_weights_are_no_weights(env):
     ev = synth.events_4d(1500, 59)
     ev["ck"][77] = 1.0
     assert np.array_equal(grad(ev, TH4, LO, HI), grad({**ev, "w": np.ones(1500)}, TH4, LO, HI))
+
+
+@pytest.mark.parametrize("ts", [1e-12, 1.0, 1e9])
+@pytest.mark.parametrize("kind", ["tagged", "phis"])
+def test_time_functions_and_their_range(env, kind, ts):
+    """The tagged and phi_s models' exponentials and phase are linear in t in fixed
+    point over the fitted range, in any unit of time; events beyond it take the
+    general functions.  Tolerance: 5e-13 of the sum of |terms| (the terms of one
+    component can cancel among themselves by a factor of a few)."""
+    O, G, _ = env
+    import torch
+    from paper_1706_01420_gb300 import api
+    th = np.array({"tagged": [0.66, 0.045, 0.0, 0.1, 0.085, 17.77, 0.8, 0.3],
+                   "phis": list(TH4) + [0.085, 17.77, 0.8, 0.3, 0.8, 0.0]}[kind])
+    first = 4 if kind == "tagged" else 10                 # DG, Dm
+    ev = {"tagged": synth.events_tagged, "phis": synth.events_phis}[kind](700, 61)
+    ev["t"][[3, 40, 600]] = 17.0, 40.0, 16.0              # beyond t_hi = 15 and beyond 16, the power of two above
+    ev["t"] = ev["t"] * ts
+    th[[0, first, first + 1]] /= ts
+    th[1:3] *= ts
+    got = api.ipa_nll_grad(getattr(api, "model_" + kind)(0.0, HI * ts), G.to_dev(ev),
+                                       torch.tensor(th, device="cuda")).cpu().numpy()
+    m = O.Model("tag" if kind == "tagged" else "phis", 0.0, HI * ts)
+    f, g = O.nll_grad(m, ev, th)
+    logl, terms = O.nll_grad_terms(m, ev, th)
+    assert abs(got[0] - f) <= 1e-14 * np.abs(logl).sum()
+    assert np.all(np.abs(got[1:] - g) <= 5e-13 * np.abs(terms).sum(1)), (got[1:], g)
