@@ -39,6 +39,11 @@ __device__ __forceinline__ long long fx_mad(Fx a, Fx b, long long acc) {
     const int m = __mulhi(a.h, b.l) + (__mulhi(b.h, a.l) + 1);
     return ((long long)a.h * b.h + (long long)m) + acc;
 }
+// acc + a b 2^-64, `one` = (a != 0): centred, and exact for a = 0
+__device__ __forceinline__ long long fx_mad1(Fx a, Fx b, long long acc, int one) {
+    const int m = __mulhi(a.h, b.l) + (__mulhi(b.h, a.l) + one);
+    return ((long long)a.h * b.h + (long long)m) + acc;
+}
 // a b for Q62 operands, in Q62
 __device__ __forceinline__ long long fx_q62(Fx a, Fx b) {
     return (long long)((unsigned long long)fx_mad(a, b, 0) << 2);

@@ -177,6 +177,19 @@ __device__ __forceinline__ double rcp_newton(double x) {
     return fma(y, fma(-x, y, 1.0), y);
 }
 
+// rcp_newton without its range branch (P in [2^-125, 2^126)).
+__device__ __forceinline__ double rcp_newton_nb(double x) {
+    const long long b = __double_as_longlong(x);
+    const int e = (int)((b >> 52) & 0x7FF);
+    const unsigned xf = ((unsigned)((unsigned long long)b >> 32) & 0x80000000u) |
+                        ((unsigned)(e - 1023 + 127) << 23) | ((unsigned)(b >> 29) & 0x7FFFFFu);
+    const unsigned yf = __float_as_uint(__frcp_rn(__uint_as_float(xf)));
+    const long long yb = ((long long)(yf & 0x80000000u) << 32) |
+                         ((long long)(((yf >> 23) & 0xFFu) - 127 + 1023) << 52) | ((long long)(yf & 0x7FFFFFu) << 29);
+    const double y = __longlong_as_double(yb);
+    return fma(y, fma(-x, y, 1.0), y);
+}
+
 // Piecewise polynomial of erfcx on [0, 6.25]; outside, the piece index is
 // clamped and the value is meaningless (callers select it away).
 __device__ __forceinline__ double erfcx_poly(double x, const MathTables* t) {

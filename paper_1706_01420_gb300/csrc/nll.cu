@@ -213,26 +213,6 @@ __device__ __forceinline__ void load_row(const Consts& c, const MathTables* mt, 
     }
 }
 
-// rcp_newton without its range branch (P in [2^-125, 2^126)).
-__device__ __forceinline__ double rcp_newton_nb(double x) {
-    const long long b = __double_as_longlong(x);
-    const int e = (int)((b >> 52) & 0x7FF);
-    const unsigned xf = ((unsigned)((unsigned long long)b >> 32) & 0x80000000u) |
-                        ((unsigned)(e - 1023 + 127) << 23) | ((unsigned)(b >> 29) & 0x7FFFFFu);
-    const unsigned yf = __float_as_uint(__frcp_rn(__uint_as_float(xf)));
-    const long long yb = ((long long)(yf & 0x80000000u) << 32) |
-                         ((long long)(((yf >> 23) & 0xFFu) - 127 + 1023) << 52) | ((long long)(yf & 0x7FFFFFu) << 29);
-    const double y = __longlong_as_double(yb);
-    return fma(y, fma(-x, y, 1.0), y);
-}
-
-// log_mul for positive normal P (no branch for zero, subnormal or special P).
-__device__ __forceinline__ void log_mul_nb(double P, double* prod, int* esum) {
-    const long long b = __double_as_longlong(P);
-    *prod *= __longlong_as_double((b & 0x000FFFFFFFFFFFFFll) | 0x3FF0000000000000ll);
-    *esum += (int)(b >> 52) - 1023;
-}
-
 // A lane's sums over rows on the fast path: FP64 (f: sum r, sum r A' tau T2, sum r A'
 // Gx, sum r A' tau Gx, and with weights sum w log P), the log product, and the fixed-
 // point sums of r T g_k.

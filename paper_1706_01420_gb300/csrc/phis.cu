@@ -39,6 +39,7 @@
 // blocks per SM in place of two are the gain over the 40-product form; figures at
 // phis_kernel.
 #include <math.h>
+#include <stddef.h>
 
 #include "accept_reject.cuh"
 #include "angular.cuh"
@@ -136,25 +137,53 @@ struct PhisWarp {
     PhisConsts c;
     double eq[6], mu[4], mv[4];
     double D2, D2s, D2c;      // 2 D, 2 D s, 2 D c
+    // the same in fixed point (rows_fast): eq, mu, mv with max in [1/8, 1/4) at 2^-hexp; c and s
+    // (Q62); rtop: scale of the angular sums' factors at unit weight, below 2^(rtop - 2)
+    int2 fe[6], fu[4], fv[4], fc, fs;
+    int hexp, rtop, fixed, pad_;
 };
+
+static_assert(offsetof(PhisWarp, fs) == offsetof(PhisWarp, fe) + 15 * sizeof(int2), "one run of coefficients");
+
+__device__ __forceinline__ int exponent_field(double x) { return (int)((__double_as_longlong(x) >> 52) & 0x7FF); }
 
 __device__ __forceinline__ void phis_coefficients(PhisWarp& pw, bool cached, int lane) {
     const PhisConsts& c = pw.c;
+    int ex = 0;               // largest exponent field of the coefficients
     if (lane < 10) {
         const int k = lane < 6 ? kEq[lane] : kMix[lane - 6];
         const double sc = 0.25 * c.cs * row_scale(c, k) * (cached ? 1.0 : kBasisScale[k]);
         const double re = kPairIm[k] ? c.bi[k] : c.br[k];
         if (lane < 6) {
             pw.eq[lane] = sc * re;
+            ex = exponent_field(pw.eq[lane]);
         } else {
             const double ej = kEta[kPairJ[k]];
             pw.mu[lane - 6] = sc * (kPairIm[k] ? -ej * c.br[k] : ej * c.bi[k]);
             pw.mv[lane - 6] = sc * re;
+            ex = max(exponent_field(pw.mu[lane - 6]), exponent_field(pw.mv[lane - 6]));
         }
     } else if (lane == 10) {
         pw.D2 = 2.0 * c.D;
         pw.D2s = 2.0 * c.D * c.s;
         pw.D2c = 2.0 * c.D * c.c;
+    }
+    if (cached) return;
+    ex = __reduce_max_sync(0xffffffffu, ex);
+    const int up = 1020 - ex;                             // max|coefficient| 2^up in [1/8, 1/4)
+    const bool ok = up >= -64 && up <= 900 && abs_below(c.c, 1.5) && abs_below(c.s, 1.5);
+    const double sc = __longlong_as_double((long long)((ok ? up : 0) + 1023) << 52);
+    if (lane < 16 && ok) {
+        const double x = lane < 6 ? pw.eq[lane] : (lane < 10 ? pw.mu[lane - 6] : (lane < 14 ? pw.mv[lane - 10] : (lane == 14 ? c.c : c.s)));
+        const Fx v = fx(fx_signed(lane < 14 ? x * sc : x, 1));
+        pw.fe[lane] = make_int2(v.h, v.l);                // fe, fu, fv, fc, fs are contiguous
+    } else if (lane == 16) {
+        // a typical r T is near 1 / max(max|coefficient|, cb / 4)
+        const int ea = ok ? -up - 3 : -1023, eb = exponent_field(c.cb) - 1025;
+        const int e = ea > eb ? ea : eb;
+        pw.rtop = 16 + (e < -900 ? 900 : -e);
+        pw.hexp = 2 - (ok ? up : 0);
+        pw.fixed = ok;
     }
 }
 
@@ -224,6 +253,137 @@ __device__ __forceinline__ void phis_event(const PhisWarp& pw, const MathTables*
     acc[kGc] = fma(gq, FV, acc[kGc]);
     acc[kGd] = fma(gq, X, acc[kGd]);
     acc[kGt1] = fma(gt, Fs, acc[kGt1]);               // (FL + FH) / 2
+    acc[kGt2] = fma(gq * tau, FV, acc[kGt2]);
+}
+
+// ---- the fixed-point form of an event's angular part (NLL + gradient, angles given) ----
+// As in the 4D kernel's fast rows (nll.cu): the ten f'_k (Q62), F+, F-, FU, FV and what is linear
+// in them on the integer pipe, and the 14 angular sums as 64-bit integers: the factors r T+, r T-,
+// r U and r C are converted once per event at a scale that follows the segment's typical r T and
+// the largest weight of the warp's rows (unit 2^-45 of a typical term, 0.41 units rms per
+// event).  The rest is FP64.  The warp's rows are redone by phis_event where some P lies outside
+// the Newton reciprocal's range or some factor outside its scale.  FP64 instructions per
+// event: 92 -> 57; 1e6 events 299 -> 248 us (FP64 unit busy 77 -> 68 %).
+
+// The f'_k in Q62 near |cos| = 1 (rare).
+__device__ __noinline__ void phis_basis_wide(double ck, double cl, double phi, const MathTables* mt, long long F[10]) {
+    double f[10];
+    basis_unscaled(ck, cl, phi, mt, f);
+#pragma unroll
+    for (int k = 0; k < 10; ++k) F[k] = to_q62_nb(f[k]);
+}
+
+// One event: FP64 sums into acc (as phis_event), the angular sums (kE .. kMV + 3) into S.
+template <bool WEIGHTED>
+__device__ __forceinline__ void phis_event_fast(const PhisWarp& pw, const MathTables* mt, const Cols& cols, int64_t e,
+                                                const TagSlow& sl, int top, double* acc, long long* S, double* prod,
+                                                int* esum, bool* bad) {
+    const PhisConsts& c = pw.c;
+    const double t = __ldg(cols.t + e), q = __ldg(cols.q + e);
+    const double ck = __ldg(cols.ck + e), cl = __ldg(cols.cl + e), phi = __ldg(cols.phi + e);
+    const double w = WEIGHTED ? __ldg(cols.w + e) : 1.0;
+    long long F[10];
+    {
+        long long g[10];
+        fx_basis(ck, cl, phi, mt, g);
+        F[0] = g[0] - g[2];
+        F[1] = g[1] - g[3];
+        F[2] = F[1] - g[2] + g[3] + g[3];
+        F[3] = g[4];
+        F[4] = g[5];
+        F[5] = g[6];
+        F[6] = g[0];
+        F[7] = g[7];
+        F[8] = g[8];
+        F[9] = g[9];
+    }
+    if (!fx_angles_ok(ck, cl, phi)) {
+        long long x[10];                                 // (a copy, so that F itself stays in registers)
+        phis_basis_wide(ck, cl, phi, mt, x);
+#pragma unroll
+        for (int k = 0; k < 10; ++k) F[k] = x[k];
+    }
+    const auto K = [](const int2& a) { return Fx{a.x, a.y}; };
+    const long long fp = fx_mad(K(pw.fe[2]), fx(F[4]), fx_mad(K(pw.fe[1]), fx(F[1]), fx_mad(K(pw.fe[0]), fx(F[0]), 0)));
+    const long long fm = fx_mad(K(pw.fe[5]), fx(F[8]), fx_mad(K(pw.fe[4]), fx(F[6]), fx_mad(K(pw.fe[3]), fx(F[2]), 0)));
+    long long fu = 0, fv = 0;                             // Q60, as fp and fm
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        fu = fx_mad(K(pw.fu[i]), fx(F[3 + 2 * i]), fu);
+        fv = fx_mad(K(pw.fv[i]), fx(F[3 + 2 * i]), fv);
+    }
+    const long long fsum = fp + fm, fdif = fp - fm;
+    const Fx D = fx(fdif), U = fx(fu);
+    const long long hd = fx_mad(K(pw.fc), D, fx_mad(K(pw.fs), U, 0)) << 2;
+    const long long xx = (fx_mad(K(pw.fs), D, 0) - fx_mad(K(pw.fc), U, 0)) << 2;
+    const double FL = fx_to_double(fsum + hd, pw.hexp), FH = fx_to_double(fsum - hd, pw.hexp);
+    const double X = fx_to_double(xx, pw.hexp), FV = fx_to_double(fv, pw.hexp);
+    const double FU = fx_to_double(fu, pw.hexp), Fd = fx_to_double(fdif, pw.hexp);
+
+    const double tau = t - c.mu;
+    const TimeValues v = time_values(c, t, tau, mt);
+    const long long bH = __double_as_longlong(sl.xH), bL = __double_as_longlong(sl.xL);
+    const long long bG = __double_as_longlong(sl.gx);
+    const double H = bH < 0 ? -sl.xH : v.H - sl.xH;
+    const double L = bL < 0 ? -sl.xL : v.L - sl.xL;
+    const double Cr = q * (bG < 0 ? sl.wr : fma(v.C, v.cn, -sl.wr));
+    const double Ci = q * (bG < 0 ? sl.wi : fma(v.C, v.sn, -sl.wi));
+    const double Y1 = fma(Cr, FV, Ci * X);
+    const double P = fma(FL, L, fma(FH, H, fma(pw.D2, Y1, c.cb)));
+    *bad |= (unsigned long long)(__double_as_longlong(P) - 0x3820000000000000ll) >= 0x0FB0000000000000ull;
+    if (WEIGHTED) {
+        const bool one = __double_as_longlong(w) == 0x3FF0000000000000ll;
+        acc[kLog] = fma(one ? 0.0 : w, fx_to_double(fx_log(P, mt), 6), acc[kLog]);
+        log_mul_nb(one ? P : 1.0, prod, esum);
+    } else {
+        log_mul_nb(P, prod, esum);
+    }
+    const double r = WEIGHTED ? w * rcp_newton_nb(P) : rcp_newton_nb(P);
+    acc[kQ] += r;
+    const double sG = L + H, dG = L - H;
+    const double m = fma(c.c, dG, pw.D2s * Ci);
+    const double u = fma(c.s, dG, -(pw.D2c * Ci));
+    const double ru = r * u;
+    {
+        const double x[4] = {r * (sG + m), r * (sG - m), ru, r * Cr};
+        Fx A[4];
+        int one[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            *bad |= exponent_field(x[i]) > 1023 - 3 + top;
+            const long long a = fx_odd(x[i], top);
+            one[i] = a != 0;
+            A[i] = fx(a);
+        }
+        S[0] = fx_mad1(A[0], fx(F[0]), S[0], one[0]);
+        S[1] = fx_mad1(A[0], fx(F[1]), S[1], one[0]);
+        S[2] = fx_mad1(A[0], fx(F[4]), S[2], one[0]);
+        S[3] = fx_mad1(A[1], fx(F[2]), S[3], one[1]);
+        S[4] = fx_mad1(A[1], fx(F[6]), S[4], one[1]);
+        S[5] = fx_mad1(A[1], fx(F[8]), S[5], one[1]);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            S[6 + i] = fx_mad1(A[2], fx(F[3 + 2 * i]), S[6 + i], one[2]);
+            S[10 + i] = fx_mad1(A[3], fx(F[3 + 2 * i]), S[10 + i], one[3]);
+        }
+    }
+    acc[kPhi] = fma(r * m, FU, fma(-ru, Fd, acc[kPhi]));
+    const double hL = (r * FL) * L, hH = (r * FH) * H;
+    acc[kL0] += hL;
+    acc[kL1] = fma(hL, tau, acc[kL1]);
+    acc[kH0] += hH;
+    acc[kH1] = fma(hH, tau, acc[kH1]);
+    const double y1 = r * Y1, y2 = r * fma(Ci, FV, -(Cr * X));
+    acc[kY10] += y1;
+    acc[kY11] = fma(y1, tau, acc[kY11]);
+    acc[kY20] += y2;
+    acc[kY21] = fma(y2, tau, acc[kY21]);
+    const double g = r * __longlong_as_double(bG & 0x7FFFFFFFFFFFFFFFll), gq = g * q, gt = g * tau;
+    acc[kGa] = fma(g, FL, acc[kGa]);
+    acc[kGb] = fma(g, FH, acc[kGb]);
+    acc[kGc] = fma(gq, FV, acc[kGc]);
+    acc[kGd] = fma(gq, X, acc[kGd]);
+    acc[kGt1] = fma(gt, fx_to_double(fsum, pw.hexp), acc[kGt1]);              // (FL + FH) / 2
     acc[kGt2] = fma(gq * tau, FV, acc[kGt2]);
 }
 
@@ -425,14 +585,52 @@ phis_kernel(Cols cols, int64_t n, const int64_t* __restrict__ seg_begin, const i
                     sbuf[j] = tag_slow(pw.c, __ldg(cols.t + e) - pw.c.mu, &mt);
                 }
                 __syncwarp();
+const auto slow_of = [&](int k) {
+                    const unsigned m = k == 0 ? m0 : (k == 1 ? m1 : (k == 2 ? m2 : m3));
+                    const int before = k == 0 ? 0 : (k == 1 ? p1 : (k == 2 ? p2 : p3));
+                    TagSlow sl = {0.0, 0.0, 0.0, 0.0, 0.0};
+                    if ((m >> lane) & 1u) sl = sbuf[before + __popc(m & below)];
+                    return sl;
+                };
+                bool plain = true;
+                if (GRAD && !CACHED && pw.fixed) {
+                    int top = pw.rtop;
+                    if (WEIGHTED) {
+                        // the exponent of the rows' largest |w| (0 where all weights are 1)
+                        unsigned hi = 0;
+#pragma unroll
+                        for (int k = 0; k < kSub; ++k) {
+                            const int64_t e = tbase + lane + 32 * (i0 + k);
+                            const double w = e < ev1 ? __ldg(cols.w + e) : 0.0;
+                            hi = max(hi, (unsigned)((unsigned long long)__double_as_longlong(w) >> 32) & 0x7FFFFFFFu);
+                        }
+                        top += (int)(__reduce_max_sync(0xffffffffu, hi) >> 20) - 1023;
+                        top = top < -900 ? -900 : (top > 900 ? 900 : top);
+                    }
+                    long long S[14];
+#pragma unroll
+                    for (int a = 0; a < 14; ++a) S[a] = 0;
+                    bool bad = false;
+#pragma unroll 1
+                    for (int k = 0; k < kSub; ++k) {
+                        const int64_t e = tbase + lane + 32 * (i0 + k);
+                        if (e < ev1) phis_event_fast<WEIGHTED>(pw, &mt, cols, e, slow_of(k), top, acc, S, &prod, &esum, &bad);
+                    }
+                    plain = __any_sync(0xffffffffu, bad);
+#pragma unroll
+                    for (int a = 0; a < NA; ++a) {
+                        if (a >= kE && a < kPhi) acc[a] = fx_to_double(S[a - kE], top + 1);
+                        if (plain) acc[a] = 0.0;
+                    }
+                    if (plain) {
+                        prod = 1.0;
+                        esum = 0;
+                    }
+                }
 #pragma unroll 1
                 for (int k = 0; k < kSub; ++k) {
                     const int64_t e = tbase + lane + 32 * (i0 + k);
-                    if (e < ev1) {
-                        const unsigned m = k == 0 ? m0 : (k == 1 ? m1 : (k == 2 ? m2 : m3));
-                        const int before = k == 0 ? 0 : (k == 1 ? p1 : (k == 2 ? p2 : p3));
-                        TagSlow sl = {0.0, 0.0, 0.0, 0.0, 0.0};
-                        if ((m >> lane) & 1u) sl = sbuf[before + __popc(m & below)];
+                    if (plain && e < ev1) {
                         const double w = WEIGHTED ? __ldg(cols.w + e) : 1.0;
                         double f[10];
                         if (CACHED) {
@@ -441,7 +639,7 @@ phis_kernel(Cols cols, int64_t n, const int64_t* __restrict__ seg_begin, const i
                         } else {
                             phis_basis(__ldg(cols.ck + e), __ldg(cols.cl + e), __ldg(cols.phi + e), &mt, f);
                         }
-                        phis_event<GRAD, WEIGHTED>(pw, &mt, __ldg(cols.t + e), __ldg(cols.q + e), w, f, sl, acc,
+                        phis_event<GRAD, WEIGHTED>(pw, &mt, __ldg(cols.t + e), __ldg(cols.q + e), w, f, slow_of(k), acc,
                                                    &prod, &esum);
                     }
                 }

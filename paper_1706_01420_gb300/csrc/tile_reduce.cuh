@@ -67,6 +67,13 @@ __device__ __forceinline__ void log_mul(double P, double* prod, int* esum) {
     *esum += e;
 }
 
+// log_mul for positive normal P (no branch for zero, subnormal or special P).
+__device__ __forceinline__ void log_mul_nb(double P, double* prod, int* esum) {
+    const long long b = __double_as_longlong(P);
+    *prod *= __longlong_as_double((b & 0x000FFFFFFFFFFFFFll) | 0x3FF0000000000000ll);
+    *esum += (int)(b >> 52) - 1023;
+}
+
 // log(prod) + esum ln 2
 __device__ __forceinline__ double log_of(double prod, int esum, const MathTables* mt) {
     const double ed = (double)esum;

@@ -114,3 +114,31 @@ def test_time_functions_and_their_range(env, kind, ts):
     logl, terms = O.nll_grad_terms(m, ev, th)
     assert abs(got[0] - f) <= 1e-14 * np.abs(logl).sum()
     assert np.all(np.abs(got[1:] - g) <= 5e-13 * np.abs(terms).sum(1)), (got[1:], g)
+
+
+@pytest.mark.parametrize("ws", [None, 1e-30, -3e12])
+@pytest.mark.parametrize("kind", ["tagged", "phis"])
+def test_time_models_weight_scales_and_handover(env, kind, ws):
+    """The tagged and phi_s models' integer sums follow the scale of the weights; a
+    warp's rows with a factor beyond the sums' range (phi_s: all angular products
+    near zero and no background) are redone.  Tolerance as above."""
+    O, G, _ = env
+    import torch
+    from paper_1706_01420_gb300 import api
+    th = np.array({"tagged": [0.66, 0.045, 0.0, 0.1, 0.085, 17.77, 0.8, 0.3],
+                   "phis": list(TH4) + [0.085, 17.77, 0.8, 0.3, 0.8, 0.0]}[kind])
+    th[3] = 0.0
+    ev = {"tagged": synth.events_tagged, "phis": synth.events_phis}[kind](1100, 67, weighted=ws is not None)
+    if ws is not None:
+        ev["w"] = ev["w"] * ws
+        ev["w"][[9, 300]] = 0.0, ws
+    if kind == "phis":
+        ev["ck"][5] = ev["cl"][5] = 1.0 - 2.0 ** -16
+        ev["ck"][600] = 1.0 - 2.0 ** -18                  # the FP64 basis
+    got = api.ipa_nll_grad(getattr(api, "model_" + kind)(0.0, HI), G.to_dev(ev),
+                           torch.tensor(th, device="cuda")).cpu().numpy()
+    m = O.Model("tag" if kind == "tagged" else "phis", 0.0, HI)
+    f, g = O.nll_grad(m, ev, th)
+    logl, terms = O.nll_grad_terms(m, ev, th)
+    assert abs(got[0] - f) <= 1e-14 * np.abs(logl).sum()
+    assert np.all(np.abs(got[1:] - g) <= 5e-13 * np.abs(terms).sum(1)), (got[1:], g)
