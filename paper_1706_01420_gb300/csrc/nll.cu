@@ -343,8 +343,8 @@ __device__ __forceinline__ bool tile_fast(const Consts& c, const MathTables* mt,
             const unsigned h = (unsigned)((unsigned long long)__double_as_longlong(__ldg(cols.w + tbase + lane + 32 * i)) >> 32);
             hi = (h & 0x7FFFFFFFu) > hi ? (h & 0x7FFFFFFFu) : hi;
         }
-        const int top = s.top + (int)(__reduce_max_sync(0xffffffffu, hi) >> 20) - 1023;
-        s.top = top < -900 ? -900 : (top > 900 ? 900 : top);
+        s.top += (int)(__reduce_max_sync(0xffffffffu, hi) >> 20) - 1023;
+        if (s.top < -900 || s.top > 900) return false;
     }
     double tot[5] = {0.0, 0.0, 0.0, 0.0, 0.0}, tprod = 1.0;
 #pragma unroll 1

@@ -145,8 +145,6 @@ struct PhisWarp {
 
 static_assert(offsetof(PhisWarp, fs) == offsetof(PhisWarp, fe) + 15 * sizeof(int2), "one run of coefficients");
 
-__device__ __forceinline__ int exponent_field(double x) { return (int)((__double_as_longlong(x) >> 52) & 0x7FF); }
-
 __device__ __forceinline__ void phis_coefficients(PhisWarp& pw, bool cached, int lane) {
     const PhisConsts& c = pw.c;
     int ex = 0;               // largest exponent field of the coefficients
@@ -593,8 +591,8 @@ const auto slow_of = [&](int k) {
                     return sl;
                 };
                 bool plain = true;
+                int top = pw.rtop;
                 if (GRAD && !CACHED && pw.fixed) {
-                    int top = pw.rtop;
                     if (WEIGHTED) {
                         // the exponent of the rows' largest |w| (0 where all weights are 1)
                         unsigned hi = 0;
@@ -605,8 +603,10 @@ const auto slow_of = [&](int k) {
                             hi = max(hi, (unsigned)((unsigned long long)__double_as_longlong(w) >> 32) & 0x7FFFFFFFu);
                         }
                         top += (int)(__reduce_max_sync(0xffffffffu, hi) >> 20) - 1023;
-                        top = top < -900 ? -900 : (top > 900 ? 900 : top);
                     }
+                    plain = top < -900 || top > 900;
+                }
+                if (!plain) {
                     long long S[14];
 #pragma unroll
                     for (int a = 0; a < 14; ++a) S[a] = 0;

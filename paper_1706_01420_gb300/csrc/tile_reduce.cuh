@@ -44,6 +44,11 @@ __device__ __forceinline__ int nth_set(unsigned m, int n) {
     return pos;
 }
 
+// The exponent field of a double, and its sign-free high word (ordered as |x| is; infinities and
+// NaN largest).
+__device__ __forceinline__ int exponent_field(double x) { return (int)((__double_as_longlong(x) >> 52) & 0x7FF); }
+__device__ __forceinline__ int high_word(double x) { return (int)((unsigned long long)__double_as_longlong(x) >> 32) & 0x7FFFFFFF; }
+
 // P = m 2^e with m in [1, 2): *prod *= m and *esum += e, so that the log of the
 // product of a lane's P values is log(*prod) + *esum ln 2 (bit operations on
 // the integer pipe and one FP64 multiply per event instead of a log).  Zero,
