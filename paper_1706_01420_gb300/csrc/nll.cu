@@ -38,25 +38,23 @@
 // parameter and the angular derivatives cost nothing per event.
 #include <math.h>
 
+#include <type_traits>
+
 #include "fp64_math.cuh"
 #include "int_math.cuh"
 #include "angular.cuh"
 #include "fast_fixed.cuh"
 #include "ipa_internal.cuh"
+#include "team_tile.cuh"
 #include "tile_reduce.cuh"
 
 namespace ipa {
 namespace {
 
 constexpr int kNllBlock = 128;                       // threads per block of the basis kernel
-constexpr int kPerLane = kTile / 32;                 // events per lane per tile
 
 // A warp keeps a copy of its segment's record (Consts, with the factors the event
 // loop multiplies by in its part k: NllCoef) in shared memory.
-// Decay-time events per compaction round of one lane (see nll_kernel).
-constexpr int kSub = 4;
-static_assert(kSub == 4, "a compaction round keeps four ballot masks");
-static_assert((IPA_TILE_EVENTS / 32) % kSub == 0, "events per lane must be a multiple of kSub");
 
 // The part of the decay-time factor that needs the Gaussian and erfcx, for an
 // event with t <= tcut (z >= -6.25 up to rounding): with g = exp(-tau^2 /
@@ -135,237 +133,6 @@ __device__ __forceinline__ void event(const Consts& c, const MathTables* mt, dou
     }
 }
 
-// ---- the fast rows (4D model, fixed point on the integer pipe) ----
-// The rows of 32 events that are complete (lane l: events tbase + l + 32 i of a
-// tile) of the 4D model's NLL + gradient take this path; the last, partial row of
-// a segment and the other variants take the plain loop of tile_plain.
-//
-// On this GPU a warp FP64 instruction occupies the sub-partition's FP64 unit
-// for about 64 cycles (2 FP64 operations per clock per SM), so everything with
-// a known range runs in 64-bit fixed point (fast_fixed.cuh): the decay
-// exponential, the angular basis, A' and the ten angular sums.  What stays FP64:
-// P, 1/P, the log (or the product of the P's) and the four sums with r, tau and
-// the Gaussian.
-//
-// The sums: r T is converted once per event to signed fixed point, in units of
-// 2^(top - 63), each product with a basis function (Q62) is the high part of the
-// 128-bit product (units of 2^(top - 61)), and a lane adds its events exactly in
-// 64-bit integers and converts each sum to a double once per tile (sums of f'_k
-// are differences of sums of basis functions, taken in integers).  top follows
-// the segment's typical r T (NllCoef::rtop) and the largest weight of the tile,
-// so a unit is 2^-46 of a typical term; error of a sum: 0.41 units rms per
-// event, of random sign, below that of the reciprocal r (6e-14 relative), and the
-// mean of the truncation is put back.  Lanes outside the ranges are fixed up in
-// FP64.  A tile in which some P lies outside the Newton reciprocal's range (zero,
-// subnormal, negative, huge, infinite or NaN) or some |r T| >= 2^(top - 3) is redone
-// by the plain loop.  Either way the tile's sums depend only on its events, never
-// on the launch geometry.
-//
-// Measured (one pass of the public call, 512 toys of 20 000 events, then 1e7
-// weighted events): the angular products, A and the exponential in FP64 and
-// 14-instruction 64-bit products, an FP64 multiply-add per angular sum: 1060 and
-// 1073 us; this path: 643 and 685.  About 1150 warp instructions per row now
-// occupy the FP64 unit 60 %, the two 32-bit multiplier and adder pipes 50 % each
-// and the issue slots 50 %; 128 registers leave 16 warps per SM, and launch
-// bounds for 20 or 24 cost more in spills than they hide (728 and 760 us).
-
-// The integer-pipe results of one event that its FP64 work needs.
-struct RowIn {
-    double tau, w, E2, Ap;
-    long long g[10];   // fx_basis
-};
-
-// The FP64 values for a lane outside the fixed-point ranges (rare): the basis, A'
-// (with the f'_k in the plain loop's order) and the exponential.
-__device__ __noinline__ void fix_row(const Consts& c, const MathTables* mt, double t, double ck, double cl, double phi,
-                                     bool ok_exp, RowIn& v) {
-    if (!ok_exp) v.E2 = exp_fast(fma(-c.Gamma, v.tau, c.k.c2), mt);
-    if (!fx_angles_ok(ck, cl, phi)) {
-        double f[10];
-        basis_unscaled(ck, cl, phi, mt, f);
-        v.Ap = amplitude_sum(c.k.hq, f);
-        const double sk2 = fma(-ck, ck, 1.0), G = sk2 * f[6], gcc = sk2 - f[1];
-        const double g[10] = {f[6], sk2, G, gcc, f[3], f[4], f[5], f[7], f[8], f[9]};
-#pragma unroll
-        for (int k = 0; k < 10; ++k) v.g[k] = to_q62_nb(g[k]);
-    }
-}
-
-template <bool WEIGHTED>
-__device__ __forceinline__ void load_row(const Consts& c, const MathTables* mt, const Cols& cols, int64_t e, RowIn& v) {
-    const double t = __ldg(cols.t + e);
-    const double ck = __ldg(cols.ck + e), cl = __ldg(cols.cl + e), phi = __ldg(cols.phi + e);
-    v.w = WEIGHTED ? __ldg(cols.w + e) : 1.0;
-    v.tau = t - c.mu;
-    bool ok_exp = true;
-    v.E2 = fx_exp(fx(fx_signed(t, c.k.ex.top)), c.k.ex, mt, &ok_exp);
-    ok_exp = ok_exp && fx_in_range(t, c.k.ex.top);
-    fx_basis(ck, cl, phi, mt, v.g);
-    long long A = 0;
-#pragma unroll
-    for (int k = 0; k < 10; ++k) A = fx_mad(Fx{c.k.ga[k].x, c.k.ga[k].y}, fx(v.g[k]), A);
-    v.Ap = fx_to_double(A, c.k.hexp);
-    const bool ok = ok_exp && fx_angles_ok(ck, cl, phi);
-    if (__any_sync(0xffffffffu, !ok)) {
-        RowIn x = v;                         // (a copy, so that v itself stays in registers)
-        fix_row(c, mt, t, ck, cl, phi, ok_exp, x);
-        v = x;
-    }
-}
-
-// A lane's sums over rows on the fast path: FP64 (f: sum r, sum r A' tau T2, sum r A'
-// Gx, sum r A' tau Gx, and with weights sum w log P), the log product, and the fixed-
-// point sums of r T g_k.
-struct FastSums {
-    double f[5];
-    double prod;
-    int esum;
-    int n;             // events with r T != 0 (for the mean of the truncation)
-    bool bad;          // P outside [2^-125, 2^126) or |r T| >= 2^(top - 3)
-    int top;           // scale of r T (set once per tile)
-    long long g[10];
-};
-
-template <bool WEIGHTED>
-__device__ __forceinline__ void event_fast(const Consts& c, const MathTables* mt, const RowIn& v, double2 ge, FastSums& s) {
-    const long long gb = __double_as_longlong(ge.y);
-    const double T2 = gb >= 0 ? v.E2 - ge.x : ge.x;
-    const double Gx = __longlong_as_double(gb & 0x7FFFFFFFFFFFFFFFll);
-    const double P = fma(T2, v.Ap, c.cb);
-    const long long pb = __double_as_longlong(P);
-    s.bad |= (unsigned long long)(pb - 0x3820000000000000ll) >= 0x0FB0000000000000ull;
-    if (WEIGHTED) {
-        // weight exactly 1: P joins the lane's product (as in event)
-        const bool one = __double_as_longlong(v.w) == 0x3FF0000000000000ll;
-        s.f[4] = fma(one ? 0.0 : v.w, fx_to_double(fx_log(P, mt), 6), s.f[4]);
-        log_mul_nb(one ? P : 1.0, &s.prod, &s.esum);
-    } else {
-        log_mul_nb(P, &s.prod, &s.esum);
-    }
-    const double r = WEIGHTED ? v.w * rcp_newton_nb(P) : rcp_newton_nb(P);
-    s.f[0] += r;
-    const double rT = r * T2;
-    const int top = WEIGHTED ? s.top : c.k.rtop;
-    s.bad |= (int)((__double_as_longlong(rT) >> 52) & 0x7FF) > 1023 - 4 + top;
-    const long long rq = fx_odd(rT, top);
-    s.n += rq != 0;
-    const Fx R = fx(rq);
-#pragma unroll
-    for (int k = 0; k < 10; ++k) s.g[k] = fx_mad0(R, fx(v.g[k]), s.g[k]);
-    const double rA = r * v.Ap;
-    const double u = rA * v.tau;
-    s.f[1] = fma(u, T2, s.f[1]);
-    s.f[2] = fma(rA, Gx, s.f[2]);
-    s.f[3] = fma(u, Gx, s.f[3]);
-}
-
-// Rows i0 .. i1 - 1 (at most kSub, complete) of a tile of the 4D model: the near-peak
-// events marked by ballot and their Gaussian/erfcx values evaluated packed into
-// sbuf, then the events row by row into s.
-template <bool WEIGHTED>
-__device__ __forceinline__ void rows_fast(const Consts& c, const MathTables* mt, const Cols& cols, int64_t tbase, int i0,
-                                          int i1, double2* sbuf, int lane, FastSums& s) {
-    const unsigned below = (1u << lane) - 1u;
-    unsigned m[kSub];
-    int p[kSub];
-#pragma unroll
-    for (int q = 0; q < kSub; ++q) {
-        const int64_t e = tbase + lane + 32 * (i0 + q);
-        m[q] = __ballot_sync(0xffffffffu, i0 + q < i1 && !greater(__ldg(cols.t + (i0 + q < i1 ? e : tbase)), c.k.tcut));
-    }
-    p[0] = 0;
-    p[1] = __popc(m[0]);
-    p[2] = p[1] + __popc(m[1]);
-    p[3] = p[2] + __popc(m[2]);
-    const int n_slow = p[3] + __popc(m[3]);
-    for (int j = lane; j < n_slow; j += 32) {
-        const int q = (j >= p[1]) + (j >= p[2]) + (j >= p[3]);
-        const unsigned mq = q == 0 ? m[0] : (q == 1 ? m[1] : (q == 2 ? m[2] : m[3]));
-        const int before = q == 0 ? 0 : (q == 1 ? p[1] : (q == 2 ? p[2] : p[3]));
-        const int64_t e = tbase + nth_set(mq, j - before) + 32 * (i0 + q);
-        sbuf[j] = gauss_erfcx(c, __ldg(cols.t + e) - c.mu, mt);
-    }
-    __syncwarp();
-#pragma unroll 1
-    for (int q = 0; q < i1 - i0; ++q) {
-        const unsigned mq = q == 0 ? m[0] : (q == 1 ? m[1] : (q == 2 ? m[2] : m[3]));
-        const int before = q == 0 ? 0 : (q == 1 ? p[1] : (q == 2 ? p[2] : p[3]));
-        const double2 gv = sbuf[(before + __popc(mq & below)) & (kSub * 32 - 1)];
-        const double2 ge = (mq >> lane) & 1u ? gv : make_double2(0.0, 0.0);
-        RowIn v;
-        load_row<WEIGHTED>(c, mt, cols, tbase + lane + 32 * (i0 + q), v);
-        event_fast<WEIGHTED>(c, mt, v, ge, s);
-    }
-    __syncwarp();
-}
-
-__device__ __forceinline__ void clear(FastSums& s) {
-#pragma unroll
-    for (int a = 0; a < 5; ++a) s.f[a] = 0.0;
-    s.prod = 1.0;
-    s.esum = 0;
-    s.n = 0;
-    s.bad = false;
-#pragma unroll
-    for (int k = 0; k < 10; ++k) s.g[k] = 0;
-}
-
-// The lane's sums over a tile's complete rows as the accumulators of the plain
-// loop: each truncated product was a unit low on average.
-__device__ __forceinline__ void fast_accumulators(const FastSums& s, double* acc) {
-    const long long up = s.n;
-    const long long g1 = s.g[1] - s.g[3], g2 = s.g[1] - s.g[2] + s.g[3];
-    const long long S[10] = {s.g[0] - s.g[2], g1, g2 + up, s.g[4] + up, s.g[5] + up,
-                             s.g[6] + up, s.g[0] + up, s.g[7] + up, s.g[8] + up, s.g[9] + up};
-    acc[0] = s.f[4];
-    acc[1] = s.f[0];
-#pragma unroll
-    for (int k = 0; k < 10; ++k) acc[2 + k] = fx_to_double(S[k], s.top + 1);
-    acc[12] = s.f[1];
-    acc[13] = s.f[2];
-    acc[14] = s.f[3];
-}
-
-// The complete rows of one tile of the 4D model's NLL + gradient on the fast
-// path, kSub at a time.  Returns false if the tile must be redone by the plain
-// loop (acc, prod and esum are then meaningless).
-template <bool WEIGHTED>
-__device__ __forceinline__ bool tile_fast(const Consts& c, const MathTables* mt, const Cols& cols, int64_t tbase,
-                                          int rows, double2* sbuf, int lane, double* acc, double* prod, int* esum) {
-    FastSums s;
-    clear(s);
-    s.top = c.k.rtop;
-    if (WEIGHTED) {
-        // the exponent of the tile's largest |w| (0 where all weights are 1, as without weights)
-        unsigned hi = 0;
-#pragma unroll 4
-        for (int i = 0; i < rows; ++i) {
-            const unsigned h = (unsigned)((unsigned long long)__double_as_longlong(__ldg(cols.w + tbase + lane + 32 * i)) >> 32);
-            hi = (h & 0x7FFFFFFFu) > hi ? (h & 0x7FFFFFFFu) : hi;
-        }
-        s.top += (int)(__reduce_max_sync(0xffffffffu, hi) >> 20) - 1023;
-        if (s.top < -900 || s.top > 900) return false;
-    }
-    double tot[5] = {0.0, 0.0, 0.0, 0.0, 0.0}, tprod = 1.0;
-#pragma unroll 1
-    for (int i0 = 0; i0 < rows; i0 += kSub) {
-        rows_fast<WEIGHTED>(c, mt, cols, tbase, i0, i0 + kSub < rows ? i0 + kSub : rows, sbuf, lane, s);
-#pragma unroll
-        for (int a = 0; a < (WEIGHTED ? 5 : 4); ++a) {
-            tot[a] += s.f[a];
-            s.f[a] = 0.0;
-        }
-        tprod *= s.prod;
-        s.prod = 1.0;
-    }
-#pragma unroll
-    for (int a = 0; a < 5; ++a) s.f[a] = tot[a];
-    fast_accumulators(s, acc);
-    *prod = tprod;
-    *esum = s.esum;
-    return !__any_sync(0xffffffffu, s.bad);
-}
-
 // Write NLL (and gradient) of one segment from its reduced accumulators.
 // With S_k = sum r T f_k and SH = sum_k h_k S_k = sum r T A (A = 1 in 1D), and
 // D_j = sum r A dT/dtheta_j where
@@ -415,49 +182,24 @@ __device__ void finalize(const Consts& c, const double* acc, int n_par, double* 
         out[1 + j] = 0.0;
 }
 
-// The plain loop over one tile's rows from `first` on, events below min(tbase +
-// kTile, ev1): lane l adds events l, l + 32, ... in order into acc (and the log product).  Those
-// near the resolution peak are marked by ballot kSub rows at a time and their
-// Gaussian/erfcx values evaluated packed, 32 per pass, into the warp's buffer.
+// The plain loop over rows [i0, i1) of a tile, events below ev1: lane l adds events l, l + 32,
+// ... in order into acc (and the log product).
 template <int KIND, bool GRAD, bool CACHED, bool WEIGHTED>
-__device__ __forceinline__ void tile_plain(const Consts& c, const MathTables* mt, const Cols& cols, int first,
+__device__ __forceinline__ void plain_rows(const Consts& c, const MathTables* mt, const Cols& cols, int i0, int i1,
                                            int64_t tbase, int64_t ev1, double2* sbuf, int lane, double* acc,
                                            double* prod, int* esum) {
     const unsigned below = (1u << lane) - 1u;
 #pragma unroll 1
-    for (int i0 = first; i0 < kPerLane && tbase + 32 * i0 < ev1; i0 += kSub) {
-        unsigned m0, m1, m2, m3;
-        {
-            unsigned mk[kSub];
-#pragma unroll
-            for (int q = 0; q < kSub; ++q) {
-                const int64_t e = tbase + lane + 32 * (i0 + q);
-                const bool slow = e < ev1 && !greater(__ldg(cols.t + e), c.k.tcut);
-                mk[q] = __ballot_sync(0xffffffffu, slow);
-            }
-            m0 = mk[0];
-            m1 = mk[1];
-            m2 = mk[2];
-            m3 = mk[3];
-        }
-        const int p1 = __popc(m0), p2 = p1 + __popc(m1), p3 = p2 + __popc(m2);
-        const int n_slow = p3 + __popc(m3);
-        for (int j = lane; j < n_slow; j += 32) {
-            const int q = (j >= p1) + (j >= p2) + (j >= p3);
-            const unsigned m = q == 0 ? m0 : (q == 1 ? m1 : (q == 2 ? m2 : m3));
-            const int before = q == 0 ? 0 : (q == 1 ? p1 : (q == 2 ? p2 : p3));
-            const int64_t e = tbase + nth_set(m, j - before) + 32 * (i0 + q);
-            sbuf[j] = gauss_erfcx(c, __ldg(cols.t + e) - c.mu, mt);
-        }
-        __syncwarp();
+    for (; i0 < i1; i0 += kSub) {
+        SlowRows r;
+        slow_rows(r, cols, c.k.tcut, tbase, i0, ev1, sbuf, lane,
+                  [&](int64_t e) { return gauss_erfcx(c, __ldg(cols.t + e) - c.mu, mt); });
 #pragma unroll 1
         for (int q = 0; q < kSub; ++q) {
             const int64_t e = tbase + lane + 32 * (i0 + q);
             if (e < ev1) {
-                const unsigned m = q == 0 ? m0 : (q == 1 ? m1 : (q == 2 ? m2 : m3));
-                const int before = q == 0 ? 0 : (q == 1 ? p1 : (q == 2 ? p2 : p3));
-                const double2 ge = (m >> lane) & 1u ? sbuf[before + __popc(m & below)]
-                                                    : make_double2(0.0, 0.0);
+                const int j = r.at(q, below, lane);
+                const double2 ge = j >= 0 ? sbuf[j] : make_double2(0.0, 0.0);
                 const double w = WEIGHTED ? __ldg(cols.w + e) : 1.0;
                 double f[10];
                 double Ap = c.k.aq;
@@ -493,6 +235,246 @@ __device__ __forceinline__ void tile_plain(const Consts& c, const MathTables* mt
         __syncwarp();
     }
 }
+
+// ---- the fixed-point path of NLL + gradient (1D; 4D with the angles given) ----
+// On this GPU a warp FP64 instruction occupies the sub-partition's FP64 unit
+// for about 64 cycles (2 FP64 operations per clock per SM), so everything with
+// a known range runs in 64-bit fixed point (fast_fixed.cuh): the decay
+// exponential, the angular basis, A', the ten angular sums and the 1D model's sums.
+// What stays FP64: P, 1/P, the log (or the product of the P's), and for the 4D model the
+// four sums with r, tau and the Gaussian.
+//
+// The angular sums: r T is converted once per event to signed fixed point, in units of
+// 2^(top - 63), each product with a basis function (Q62) is the high part of the
+// 128-bit product (units of 2^(top - 61)), and a lane adds its events exactly in
+// 64-bit integers and converts each sum to a double once per tile (sums of f'_k
+// are differences of sums of basis functions, taken in integers).  top follows
+// the segment's typical r T (NllCoef::rtop) and the largest weight of the tile,
+// so a unit is 2^-46 of a typical term; error of a sum: 0.41 units rms per
+// event, of random sign, below that of the reciprocal r (6e-14 relative).  The 1D model: sums of r T and r Gx and their products
+// with tau, as in the tagged model (tagged.cu).  Lanes outside the ranges are fixed up in
+// FP64.  A tile in which some P lies outside the Newton reciprocal's range (zero,
+// subnormal, negative, huge, infinite or NaN) or some |r T| >= 2^(top - 3) is redone
+// by the plain loop.  Either way the tile's sums depend only on its events, never
+// on the launch geometry (team_tile.cuh).
+//
+// Measured (one pass of the public call, 512 toys of 20 000 events, then 1e7
+// weighted events): the angular products, A and the exponential in FP64 and
+// 14-instruction 64-bit products, an FP64 multiply-add per angular sum: 1060 and
+// 1073 us; this path: 643 and 685.  About 1150 warp instructions per row now
+// occupy the FP64 unit 60 %, the two 32-bit multiplier and adder pipes 50 % each
+// and the issue slots 50 %; 128 registers leave 16 warps per SM, and launch
+// bounds for 20 or 24 cost more in spills than they hide (728 and 760 us).
+
+// The integer-pipe results of one event that its FP64 work needs.
+struct RowIn {
+    double tau, w, E2, Ap;
+    Fx g[10];   // fx_basis
+};
+
+// The FP64 values for a lane outside the fixed-point ranges (rare): the basis, A'
+// (with the f'_k in the plain loop's order) and the exponential.
+__device__ __noinline__ void fix_row(const Consts& c, const MathTables* mt, double t, double ck, double cl, double phi,
+                                     bool ok_exp, RowIn& v) {
+    if (!ok_exp) v.E2 = exp_fast(fma(-c.Gamma, v.tau, c.k.c2), mt);
+    if (!fx_angles_ok(ck, cl, phi)) {
+        double f[10];
+        basis_unscaled(ck, cl, phi, mt, f);
+        v.Ap = amplitude_sum(c.k.hq, f);
+        const double sk2 = fma(-ck, ck, 1.0), G = sk2 * f[6], gcc = sk2 - f[1];
+        const double g[10] = {f[6], sk2, G, gcc, f[3], f[4], f[5], f[7], f[8], f[9]};
+#pragma unroll
+        for (int k = 0; k < 10; ++k) v.g[k] = fx(to_q62_nb(g[k]));
+    }
+}
+
+// (the same register-saving detour for the exponential)
+__device__ __noinline__ double fix_exp(const Consts& c, const MathTables* mt, double tau) {
+    return exp_fast(fma(-c.Gamma, tau, c.k.c2), mt);
+}
+
+template <bool WEIGHTED>
+__device__ __forceinline__ void load_row(const Consts& c, const MathTables* mt, const Cols& cols, int64_t e, RowIn& v) {
+    const double t = __ldg(cols.t + e);
+    const double ck = __ldg(cols.ck + e), cl = __ldg(cols.cl + e), phi = __ldg(cols.phi + e);
+    v.w = WEIGHTED ? __ldg(cols.w + e) : 1.0;
+    v.tau = t - c.mu;
+    bool ok_exp = fx_in_range(t, c.k.ex.top);
+    v.E2 = fx_exp(fx(fx_signed(t, c.k.ex.top)), c.k.ex, mt, &ok_exp);
+    long long g[10];
+    fx_basis(ck, cl, phi, mt, g);
+    long long A = 0;
+#pragma unroll
+    for (int k = 0; k < 10; ++k) {
+        v.g[k] = fx(g[k]);
+        A = fx_mad(Fx{c.k.ga[k].x, c.k.ga[k].y}, v.g[k], A);
+    }
+    v.Ap = fx_to_double(A, c.k.hexp);
+    if (__any_sync(__activemask(), !(ok_exp && fx_angles_ok(ck, cl, phi)))) {
+        RowIn x = v;                         // (a copy, so that v itself stays in registers)
+        fix_row(c, mt, t, ck, cl, phi, ok_exp, x);
+        v = x;
+    }
+}
+
+// The models of team_tile.cuh.
+struct Angtime {
+    using Record = Consts;
+    using Slow = double2;
+    // FP64: sum r, sum r A' tau T2, sum r A' Gx, sum r A' tau Gx, sum w log P; integers: r T g_k
+    static constexpr int kSums = 5, kInts = 10, NA = n_acc(IPA_MODEL_ANGTIME4D, true);
+    using Sums = FastSums<kSums, kInts>;
+
+    template <bool W>
+    static __device__ __forceinline__ bool usable(const Consts& c, const Cols& cols, int64_t tbase, int64_t ev1, int lane,
+                                                  FastScale* sc) {
+        sc->top = c.k.rtop + (W ? weight_exponent(cols, tbase, ev1, lane) : 0);
+        sc->gtop = 0;
+        return c.k.fixed && ev1 - tbase >= kFewEvents && sc->top >= -900 && sc->top <= 900;
+    }
+    template <bool W>
+    static __device__ __forceinline__ void quarter(const Consts& c, const MathTables* mt, const Cols& cols, int64_t tbase,
+                                                   int i0, int64_t ev1, double2* sbuf, int lane, FastScale sc, Sums& s) {
+        const unsigned below = (1u << lane) - 1u;
+        SlowRows r;
+        slow_rows(r, cols, c.k.tcut, tbase, i0, ev1, sbuf, lane,
+                  [&](int64_t e) { return gauss_erfcx(c, __ldg(cols.t + e) - c.mu, mt); });
+#pragma unroll 1
+        for (int q = 0; q < kSub; ++q) {
+            const int64_t e = tbase + lane + 32 * (i0 + q);
+            if (e < ev1) {
+                const int j = r.at(q, below, lane);
+                const double2 ge = j >= 0 ? sbuf[j] : make_double2(0.0, 0.0);
+                RowIn v;
+                load_row<W>(c, mt, cols, e, v);
+                const long long gb = __double_as_longlong(ge.y);
+                const double T2 = gb >= 0 ? v.E2 - ge.x : ge.x;
+                const double Gx = __longlong_as_double(gb & 0x7FFFFFFFFFFFFFFFll);
+                const double P = fma(T2, v.Ap, c.cb);
+                add_log<W>(P, v.w, mt, &s.f[4], s);
+                const double rr = W ? v.w * rcp_newton_nb(P) : rcp_newton_nb(P);
+                s.f[0] += rr;
+                const double rT = rr * T2;
+                s.most = max(s.most, high_word(rT));
+                const long long rq = fx_odd(rT, W ? sc.top : c.k.rtop);
+                const int one = rq != 0;
+                const Fx R = fx(rq);
+#pragma unroll
+                for (int k = 0; k < 10; ++k) s.g[k] = fx_mad1(R, v.g[k], s.g[k], one);
+                const double rA = rr * v.Ap;
+                const double u = rA * v.tau;
+                s.f[1] = fma(u, T2, s.f[1]);
+                s.f[2] = fma(rA, Gx, s.f[2]);
+                s.f[3] = fma(u, Gx, s.f[3]);
+            }
+        }
+        __syncwarp();
+    }
+    static __device__ __forceinline__ bool bad(const Consts&, FastScale sc, const Sums& s) {
+        return p_out_of_range(s) || (s.most >> 20) > 1023 - 4 + sc.top;
+    }
+    static __device__ __forceinline__ void accumulators(const Consts&, FastScale sc, const Sums& s, double* acc) {
+        const long long S[10] = {s.g[0] - s.g[2], s.g[1] - s.g[3], s.g[1] - s.g[2] + s.g[3], s.g[4], s.g[5],
+                                 s.g[6], s.g[0], s.g[7], s.g[8], s.g[9]};
+        acc[0] = s.f[4];
+        acc[1] = s.f[0];
+#pragma unroll
+        for (int k = 0; k < 10; ++k) acc[2 + k] = fx_to_double(S[k], sc.top + 1);
+        acc[12] = s.f[1];
+        acc[13] = s.f[2];
+        acc[14] = s.f[3];
+    }
+    template <bool W>
+    static __device__ __forceinline__ void plain(const Consts& c, const MathTables* mt, const Cols& cols, int i0, int i1,
+                                                 int64_t tbase, int64_t ev1, double2* sbuf, int lane, double* acc,
+                                                 double* prod, int* esum) {
+        plain_rows<IPA_MODEL_ANGTIME4D, true, false, W>(c, mt, cols, i0, i1, tbase, ev1, sbuf, lane, acc, prod, esum);
+    }
+    static __device__ __forceinline__ void finish(const Consts& c, const double* acc, int n_par, double* out, int lane) {
+        finalize<IPA_MODEL_ANGTIME4D, true, false>(c, acc, n_par, out, lane);
+    }
+};
+
+struct Time1d {
+    using Record = Consts;
+    using Slow = double2;
+    // FP64: sum r, sum w log P; integers: r T, r Gx, r tau T, r tau Gx (the factor A' = cs/2 outside)
+    static constexpr int kSums = 2, kInts = 4, NA = n_acc(IPA_MODEL_TIME1D, true);
+    using Sums = FastSums<kSums, kInts>;
+
+    template <bool W>
+    static __device__ __forceinline__ bool usable(const Consts& c, const Cols& cols, int64_t tbase, int64_t ev1, int lane,
+                                                  FastScale* sc) {
+        // a typical r T is near 1 / max(cs / 2, cb / 2); the Gaussian's tau within 10 sigma (as in tagged.cu)
+        sc->top = 10 + 1023 - max(exponent_field(c.k.aq), exponent_field(c.cb) - 1) +
+                  (W ? weight_exponent(cols, tbase, ev1, lane) : 0);
+        sc->gtop = exponent_field(c.sigma) - 1023 + 5;
+        return c.k.ex.ok && sc->top >= -400 && sc->top <= 400 && sc->gtop >= -400 && sc->gtop <= 400;
+    }
+    template <bool W>
+    static __device__ __forceinline__ void quarter(const Consts& c, const MathTables* mt, const Cols& cols, int64_t tbase,
+                                                   int i0, int64_t ev1, double2* sbuf, int lane, FastScale sc, Sums& s) {
+        const unsigned below = (1u << lane) - 1u;
+        SlowRows r;
+        slow_rows(r, cols, c.k.tcut, tbase, i0, ev1, sbuf, lane,
+                  [&](int64_t e) { return gauss_erfcx(c, __ldg(cols.t + e) - c.mu, mt); });
+#pragma unroll 1
+        for (int q = 0; q < kSub; ++q) {
+            const int64_t e = tbase + lane + 32 * (i0 + q);
+            if (e < ev1) {
+                const int j = r.at(q, below, lane);
+                const double2 ge = j >= 0 ? sbuf[j] : make_double2(0.0, 0.0);
+                const double t = __ldg(cols.t + e), w = W ? __ldg(cols.w + e) : 1.0;
+                const double tau = t - c.mu;
+                bool ok = fx_in_range(t, c.k.ex.top);
+                double E2 = fx_exp(fx(fx_signed(t, c.k.ex.top)), c.k.ex, mt, &ok);
+                if (!ok) E2 = fix_exp(c, mt, tau);
+                const long long gb = __double_as_longlong(ge.y);
+                const double T2 = gb >= 0 ? E2 - ge.x : ge.x;
+                const double Gx = __longlong_as_double(gb & 0x7FFFFFFFFFFFFFFFll);
+                const double P = fma(T2, c.k.aq, c.cb);
+                add_log<W>(P, w, mt, &s.f[1], s);
+                const double rr = W ? w * rcp_newton_nb(P) : rcp_newton_nb(P);
+                s.f[0] += rr;
+                const double x[2] = {rr * T2, rr * Gx};
+                s.tau_most = max(s.tau_most, high_word(tau));
+                const Fx T[2] = {fx(fx_signed(tau, c.k.ex.top)), fx(fx_signed(tau, sc.gtop))};
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    s.most = max(s.most, high_word(x[i]));
+                    const long long a = fx_odd(x[i], sc.top);
+                    s.g[i] += a;
+                    s.g[2 + i] = fx_mad1(fx((long long)((unsigned long long)a << 3)), T[i], s.g[2 + i], a != 0);
+                }
+            }
+        }
+        __syncwarp();
+    }
+    static __device__ __forceinline__ bool bad(const Consts& c, FastScale sc, const Sums& s) {
+        return p_out_of_range(s) || (s.most >> 20) > 1023 - 6 + sc.top ||
+               s.tau_most >= ((1023 - 1 + c.k.ex.top) << 20 | 0xC0000);
+    }
+    static __device__ __forceinline__ void accumulators(const Consts& c, FastScale sc, const Sums& s, double* acc) {
+        acc[0] = s.f[1];
+        acc[1] = s.f[0];
+        acc[2] = fx_to_double(s.g[0], sc.top - 1);
+        acc[3] = c.k.aq * fx_to_double(s.g[2], sc.top + c.k.ex.top - 3);
+        acc[4] = c.k.aq * fx_to_double(s.g[1], sc.top - 1);
+        acc[5] = c.k.aq * fx_to_double(s.g[3], sc.top + sc.gtop - 3);
+    }
+    template <bool W>
+    static __device__ __forceinline__ void plain(const Consts& c, const MathTables* mt, const Cols& cols, int i0, int i1,
+                                                 int64_t tbase, int64_t ev1, double2* sbuf, int lane, double* acc,
+                                                 double* prod, int* esum) {
+        plain_rows<IPA_MODEL_TIME1D, true, false, W>(c, mt, cols, i0, i1, tbase, ev1, sbuf, lane, acc, prod, esum);
+    }
+    static __device__ __forceinline__ void finish(const Consts& c, const double* acc, int n_par, double* out, int lane) {
+        finalize<IPA_MODEL_TIME1D, true, false>(c, acc, n_par, out, lane);
+    }
+};
+
+template <int KIND>
+using Model = std::conditional_t<KIND == IPA_MODEL_TIME1D, Time1d, Angtime>;
 
 // A segment's record into the warp's copy in shared memory (warp-collective).
 __device__ __forceinline__ void load_warp_consts(Consts& c, const Consts* src_consts, int lane) {
@@ -576,27 +558,14 @@ nll_kernel(Cols cols, int64_t n, const int64_t* __restrict__ seg_begin,
             double prod = 1.0;   // unweighted: product of mantissas of P ...
             int esum = 0;        // ... and sum of exponents (log_mul)
 
-            // Events are taken kSub per lane at a time (lane l: l + 32 i).  Those
-            // with t <= tcut need the Gaussian and erfcx (about a fifth of them);
-            // they are listed in a ballot per i and evaluated packed, 32 per pass,
-            // into the warp's buffer, so the FP64 pipe does not spend a full warp
-            // instruction on lanes that would discard the result.
+            // Events are taken kSub rows at a time (lane l: l + 32 i).  Those with t <= tcut
+            // (about a fifth of them) need the Gaussian and erfcx: slow_rows.
             const int64_t tbase = ev0 + (tile - t0) * kTile;
-            int first = 0;               // rows left to the plain loop
-            if (KIND == IPA_MODEL_ANGTIME4D && GRAD && !CACHED) {
-                const int64_t left = ev1 - tbase;
-                const int rows = !wc.k.fixed ? 0 : (left >= kTile ? kPerLane : (int)(left >> 5));
-                if (rows > 0 && tile_fast<WEIGHTED>(wc, &mt, cols, tbase, rows, sbuf, lane, acc, &prod, &esum)) {
-                    first = rows;
-                } else if (rows > 0) {
-#pragma unroll
-                    for (int a = 0; a < NA; ++a) acc[a] = 0.0;
-                    prod = 1.0;
-                    esum = 0;
-                }
-            }
-            if (first < kPerLane)
-                tile_plain<KIND, GRAD, CACHED, WEIGHTED>(wc, &mt, cols, first, tbase, ev1, sbuf, lane, acc, &prod, &esum);
+            if constexpr (GRAD && !CACHED)
+                solo_tile<Model<KIND>, WEIGHTED>(wc, &mt, cols, tbase, ev1, sbuf, lane, acc, &prod, &esum);
+            else
+                plain_rows<KIND, GRAD, CACHED, WEIGHTED>(wc, &mt, cols, 0, tile_rows(tbase, ev1), tbase, ev1, sbuf, lane,
+                                                         acc, &prod, &esum);
             acc[0] += log_of(prod, esum, &mt);
             const double share = warp_butterfly<NA>(acc, lane);
             // the group and segment levels; the warp that completes the
@@ -652,6 +621,11 @@ ipa_status launch_t(const Cols& cols, int64_t n, const int64_t* seg_begin, const
     const bool single = seg_begin == nullptr;
     const int64_t tiles = tile_estimate(n, n_seg);
     const LaunchCfg cfg = force ? *force : launch_cfg(KIND, GRAD, CACHED, n_seg > 1, tiles);
+    if constexpr (GRAD && !CACHED) {
+        if (launch_team_ok(cfg, tiles))
+            return launch_team<Model<KIND>, WEIGHTED>(cols, n, seg_begin, seg_end, seg_tiles, n_seg, consts, sc, out,
+                                                      n_par, tiles, st);
+    }
     const int W = cfg.warps_per_block >= 1 && cfg.warps_per_block <= kMaxWarps ? cfg.warps_per_block : 1;
     const int K = cfg.tiles_per_take >= 1 ? cfg.tiles_per_take : 1;
     const size_t smem = (size_t)W * (sizeof(Consts) + kSub * 32 * sizeof(double2));

@@ -52,15 +52,13 @@
 #include "philox.cuh"
 #include "phis_consts.cuh"
 #include "tagged.cuh"
+#include "team_tile.cuh"
 #include "tile_reduce.cuh"
 
 namespace ipa {
 namespace {
 
-constexpr int kPerLane = kTile / 32;
-constexpr int kSub = 4;
 constexpr int kMaxWarps = 8;
-constexpr int kTeam = kPerLane / kSub;   // warps that share a tile: each takes kSub of a lane's events
 constexpr int kRow = n_acc(IPA_MODEL_PHIS, true);   // doubles per tile or group partial (the width of a shard's rows)
 constexpr int kNA = 31;          // accumulators with the gradient; the row's other entries are zero
 static_assert(kNA <= 32 && kNA <= kRow && kRow <= kMaxAcc, "one accumulator per lane, rows in the scratch");
@@ -592,7 +590,7 @@ const auto slow_of = [&](int k) {
                 };
                 bool plain = true;
                 int top = pw.rtop;
-                if (GRAD && !CACHED && pw.fixed) {
+                if (GRAD && !CACHED && pw.fixed && ev1 - tbase >= kFewEvents) {
                     if (WEIGHTED) {
                         // the exponent of the rows' largest |w| (0 where all weights are 1)
                         unsigned hi = 0;

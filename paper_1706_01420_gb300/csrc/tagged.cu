@@ -26,14 +26,12 @@
 #include "int_math.cuh"
 #include "ipa_internal.cuh"
 #include "tagged.cuh"
+#include "team_tile.cuh"
 #include "tile_reduce.cuh"
 
 namespace ipa {
 namespace {
 
-constexpr int kPerLane = kTile / 32;
-constexpr int kSub = 4;
-static_assert(kPerLane % kSub == 0, "events per lane must be a multiple of kSub");
 constexpr int kMaxWarps = 8;
 
 // One event: w log P into acc[0] (or, for w = 1 exactly, P into the lane's
@@ -73,61 +71,6 @@ __device__ __forceinline__ void tag_event(const TagConsts& c, const MathTables* 
         acc[10] += rG;
         acc[11] = fma(rG, tau, acc[11]);
         acc[12] = fma(rq, gx, acc[12]);
-    }
-}
-
-// A lane's sums of a tile on the fixed-point path (NLL + gradient).  On this GPU a warp FP64
-// instruction occupies its unit for about 64 cycles, so ten of the twelve sums and their
-// products with tau are 64-bit integers: r 2gH, r 2gL, r q 2Re g, r q 2Im g, r Gx and r q Gx
-// are converted once at a scale that follows the segment's typical r g (1 / max(qH, qL, cb / 2))
-// and the tile's largest weight; a unit is 2^-53 of a typical term, 2^-50 in the sums with tau
-// (0.4 units rms per event).  A tile with P outside the Newton reciprocal's range or a factor
-// beyond 2^5 typical ones (near-complete cancellation in P) is redone by tag_event.  FP64 instructions
-// per event: 31 -> 21; 1e6 events 131 -> 124 us (FP64 unit busy 70 -> 58 %; three to four
-// warps a sub-partition then leave its latencies uncovered).
-struct TagSums {
-    double log, Q;
-    long long a[6];        // in the order above
-    long long at[5];       // times tau (not r q Gx)
-    int most, tau_most, p_least, p_most;   // high words: the largest factor, |tau|, the range of P
-};
-
-template <bool WEIGHTED>
-__device__ __forceinline__ void tag_event_fast(const TagConsts& c, const MathTables* mt, double t, double q, double w,
-                                               const TagSlow& sl, int top, int gtop, TagSums& s, double* prod,
-                                               int* esum) {
-    const double tau = t - c.mu;
-    const TimeValues v = time_values(c, t, tau, mt);
-    const long long bH = __double_as_longlong(sl.xH), bL = __double_as_longlong(sl.xL);
-    const long long bG = __double_as_longlong(sl.gx);
-    const double T2H = bH < 0 ? -sl.xH : v.H - sl.xH;
-    const double T2L = bL < 0 ? -sl.xL : v.L - sl.xL;
-    const double Cr = bG < 0 ? sl.wr : fma(v.C, v.cn, -sl.wr);
-    const double Ci = bG < 0 ? sl.wi : fma(v.C, v.sn, -sl.wi);
-    const double gx = __longlong_as_double(bG & 0x7FFFFFFFFFFFFFFFll);
-    const double P = fma(c.qH, T2H, fma(c.qL, T2L, fma(q * c.qD, Ci, c.cb)));
-    const int ph = (int)(__double_as_longlong(P) >> 32);
-    s.p_least = min(s.p_least, ph);                       // (negative for P < 0)
-    s.p_most = max(s.p_most, ph);
-    if (WEIGHTED) {
-        const bool one = __double_as_longlong(w) == 0x3FF0000000000000ll;
-        s.log = fma(one ? 0.0 : w, fx_to_double(fx_log(P, mt), 6), s.log);
-        log_mul_nb(one ? P : 1.0, prod, esum);
-    } else {
-        log_mul_nb(P, prod, esum);
-    }
-    const double r = WEIGHTED ? w * rcp_newton_nb(P) : rcp_newton_nb(P);
-    s.Q += r;
-    const double rq = q * r;
-    const double x[6] = {r * T2H, r * T2L, rq * Cr, rq * Ci, r * gx, rq * gx};
-    s.tau_most = max(s.tau_most, high_word(tau));
-    const Fx T = fx(fx_signed(tau, c.fx[0].top)), TG = fx(fx_signed(tau, gtop));
-#pragma unroll
-    for (int i = 0; i < 6; ++i) {
-        s.most = max(s.most, high_word(x[i]));
-        const long long a = fx_odd(x[i], top);
-        s.a[i] += a;
-        if (i < 5) s.at[i] = fx_mad1(fx((long long)((unsigned long long)a << 3)), i < 4 ? T : TG, s.at[i], a != 0);
     }
 }
 
@@ -175,107 +118,131 @@ __device__ void tag_finalize(const TagConsts& c, const double* acc, int n_par, d
     for (int j = IPA_NPAR_TAGGED + lane; j < n_par; j += 32) out[1 + j] = 0.0;
 }
 
-// Every event of a tile below ev1, lane l taking l, l + 32, ... in order: one(e, slow values).  The
-// events with t <= tcut are listed by ballot kSub rows at a time and their slow values
-// evaluated packed into the warp's buffer.
-template <class F>
-__device__ __forceinline__ void tag_rows(const TagConsts& tc, const MathTables* mt, const Cols& cols, int64_t tbase,
-                                         int64_t ev1, TagSlow* sbuf, int lane, F one) {
+// Rows [i0, i1) of a tile, events below ev1, by tag_event.
+template <bool GRAD, bool WEIGHTED>
+__device__ __forceinline__ void tag_rows(const TagConsts& c, const MathTables* mt, const Cols& cols, int i0, int i1,
+                                         int64_t tbase, int64_t ev1, TagSlow* sbuf, int lane, double* acc, double* prod,
+                                         int* esum) {
     const unsigned below = (1u << lane) - 1u;
 #pragma unroll 1
-    for (int i0 = 0; i0 < kPerLane; i0 += kSub) {
-        unsigned m0, m1, m2, m3;
-        {
-            unsigned mk[kSub];
-#pragma unroll
-            for (int k = 0; k < kSub; ++k) {
-                const int64_t e = tbase + lane + 32 * (i0 + k);
-                const bool slow = e < ev1 && !greater(__ldg(cols.t + e), tc.tcut);
-                mk[k] = __ballot_sync(0xffffffffu, slow);
-            }
-            m0 = mk[0];
-            m1 = mk[1];
-            m2 = mk[2];
-            m3 = mk[3];
-        }
-        const int p1 = __popc(m0), p2 = p1 + __popc(m1), p3 = p2 + __popc(m2);
-        const int n_slow = p3 + __popc(m3);
-        for (int j = lane; j < n_slow; j += 32) {
-            const int k = (j >= p1) + (j >= p2) + (j >= p3);
-            const unsigned m = k == 0 ? m0 : (k == 1 ? m1 : (k == 2 ? m2 : m3));
-            const int before = k == 0 ? 0 : (k == 1 ? p1 : (k == 2 ? p2 : p3));
-            const int64_t e = tbase + nth_set(m, j - before) + 32 * (i0 + k);
-            sbuf[j] = tag_slow(tc, __ldg(cols.t + e) - tc.mu, mt);
-        }
-        __syncwarp();
+    for (; i0 < i1; i0 += kSub) {
+        SlowRows r;
+        slow_rows(r, cols, c.tcut, tbase, i0, ev1, sbuf, lane,
+                  [&](int64_t e) { return tag_slow(c, __ldg(cols.t + e) - c.mu, mt); });
 #pragma unroll 1
         for (int k = 0; k < kSub; ++k) {
             const int64_t e = tbase + lane + 32 * (i0 + k);
             if (e < ev1) {
-                const unsigned m = k == 0 ? m0 : (k == 1 ? m1 : (k == 2 ? m2 : m3));
-                const int before = k == 0 ? 0 : (k == 1 ? p1 : (k == 2 ? p2 : p3));
+                const int j = r.at(k, below, lane);
                 TagSlow sl = {0.0, 0.0, 0.0, 0.0, 0.0};
-                if ((m >> lane) & 1u) sl = sbuf[before + __popc(m & below)];
-                one(e, sl);
+                if (j >= 0) sl = sbuf[j];
+                const double w = WEIGHTED ? __ldg(cols.w + e) : 1.0;
+                tag_event<GRAD, WEIGHTED>(c, mt, __ldg(cols.t + e), __ldg(cols.q + e), w, sl, acc, prod, esum);
             }
         }
         __syncwarp();
     }
 }
 
-// A tile on the fixed-point path into the accumulators of tag_event; false (and nothing
-// changed) if the tile needs tag_event.
-template <bool WEIGHTED>
-__device__ __forceinline__ bool tag_tile_fast(const TagConsts& tc, const MathTables* mt, const Cols& cols,
-                                              int64_t tbase, int64_t ev1, TagSlow* sbuf, int lane, double* acc,
-                                              double* prod, int* esum) {
-    // r g of a typical event: near 2^-e, e the exponent of max(qH, qL, cb / 2)
-    const int e1 = max(exponent_field(tc.qH), exponent_field(tc.qL)), e2 = exponent_field(tc.cb) - 1;
-    int top = 10 + 1023 - max(e1, e2);
-    if (WEIGHTED) {
-        // and the exponent of the tile's largest |w| (0 where all weights are 1)
-        int hi = 0;
-#pragma unroll 4
-        for (int i = 0; i < kPerLane; ++i) {
-            const int64_t e = tbase + lane + 32 * i;
-            hi = max(hi, high_word(e < ev1 ? __ldg(cols.w + e) : 0.0));
+// A lane's sums of a tile on the fixed-point path (NLL + gradient).  On this GPU a warp FP64
+// instruction occupies its unit for about 64 cycles, so ten of the twelve sums and their
+// products with tau are 64-bit integers: r 2gH, r 2gL, r q 2Re g, r q 2Im g, r Gx and r q Gx
+// are converted once at a scale that follows the segment's typical r g (1 / max(qH, qL, cb / 2))
+// and the tile's largest weight; a unit is 2^-53 of a typical term, 2^-50 in the sums with tau
+// (0.4 units rms per event).  A tile with P outside the Newton reciprocal's range or a factor
+// beyond 2^5 typical ones (near-complete cancellation in P) is redone by tag_event.  FP64 instructions
+// per event: 31 -> 21; 1e6 events 131 -> 124 us (FP64 unit busy 70 -> 58 %; three to four
+// warps a sub-partition then leave its latencies uncovered).
+struct Tagged {
+    using Record = TagConsts;
+    using Slow = TagSlow;
+    // FP64: sum r, sum w log P; integers: the six sums in the order above, then times tau (not r q Gx)
+    static constexpr int kSums = 2, kInts = 11, NA = n_acc(IPA_MODEL_TAGGED1D, true);
+    using Sums = FastSums<kSums, kInts>;
+
+    template <bool W>
+    static __device__ __forceinline__ bool usable(const TagConsts& c, const Cols& cols, int64_t tbase, int64_t ev1,
+                                                  int lane, FastScale* sc) {
+        const int e1 = max(exponent_field(c.qH), exponent_field(c.qL)), e2 = exponent_field(c.cb) - 1;
+        sc->top = 10 + 1023 - max(e1, e2) + (W ? weight_exponent(cols, tbase, ev1, lane) : 0);
+        // r Gx counts (its integer is not 0) only for |tau| < 10 sigma, so tau's scale there follows sigma
+        sc->gtop = exponent_field(c.sigma) - 1023 + 5;
+        return c.fx_ok && sc->top >= -400 && sc->top <= 400 && sc->gtop >= -400 && sc->gtop <= 400;
+    }
+    template <bool W>
+    static __device__ __forceinline__ void quarter(const TagConsts& c, const MathTables* mt, const Cols& cols, int64_t tbase,
+                                                   int i0, int64_t ev1, TagSlow* sbuf, int lane, FastScale sc, Sums& s) {
+        const unsigned below = (1u << lane) - 1u;
+        SlowRows r;
+        slow_rows(r, cols, c.tcut, tbase, i0, ev1, sbuf, lane,
+                  [&](int64_t e) { return tag_slow(c, __ldg(cols.t + e) - c.mu, mt); });
+#pragma unroll 1
+        for (int k = 0; k < kSub; ++k) {
+            const int64_t e = tbase + lane + 32 * (i0 + k);
+            if (e < ev1) {
+                const int j = r.at(k, below, lane);
+                TagSlow sl = {0.0, 0.0, 0.0, 0.0, 0.0};
+                if (j >= 0) sl = sbuf[j];
+                event<W>(c, mt, __ldg(cols.t + e), __ldg(cols.q + e), W ? __ldg(cols.w + e) : 1.0, sl, sc, s);
+            }
         }
-        top += (int)(__reduce_max_sync(0xffffffffu, (unsigned)hi) >> 20) - 1023;
+        __syncwarp();
     }
-    // r Gx counts (its integer is not 0) only for |tau| < 10 sigma, so tau's scale there follows sigma
-    const int gtop = exponent_field(tc.sigma) - 1023 + 5;
-    if (!tc.fx_ok || top < -400 || top > 400 || gtop < -400 || gtop > 400) return false;
-    TagSums s;
-    s.log = s.Q = 0.0;
+    template <bool WEIGHTED>
+    static __device__ __forceinline__ void event(const TagConsts& c, const MathTables* mt, double t, double q, double w,
+                                                 const TagSlow& sl, FastScale sc, Sums& s) {
+        const double tau = t - c.mu;
+        const TimeValues v = time_values(c, t, tau, mt);
+        const long long bH = __double_as_longlong(sl.xH), bL = __double_as_longlong(sl.xL);
+        const long long bG = __double_as_longlong(sl.gx);
+        const double T2H = bH < 0 ? -sl.xH : v.H - sl.xH;
+        const double T2L = bL < 0 ? -sl.xL : v.L - sl.xL;
+        const double Cr = bG < 0 ? sl.wr : fma(v.C, v.cn, -sl.wr);
+        const double Ci = bG < 0 ? sl.wi : fma(v.C, v.sn, -sl.wi);
+        const double gx = __longlong_as_double(bG & 0x7FFFFFFFFFFFFFFFll);
+        const double P = fma(c.qH, T2H, fma(c.qL, T2L, fma(q * c.qD, Ci, c.cb)));
+        add_log<WEIGHTED>(P, w, mt, &s.f[1], s);
+        const double r = WEIGHTED ? w * rcp_newton_nb(P) : rcp_newton_nb(P);
+        s.f[0] += r;
+        const double rq = q * r;
+        const double x[6] = {r * T2H, r * T2L, rq * Cr, rq * Ci, r * gx, rq * gx};
+        s.tau_most = max(s.tau_most, high_word(tau));
+        const Fx T = fx(fx_signed(tau, c.fx[0].top)), TG = fx(fx_signed(tau, sc.gtop));
 #pragma unroll
-    for (int i = 0; i < 6; ++i) s.a[i] = 0;
-#pragma unroll
-    for (int i = 0; i < 5; ++i) s.at[i] = 0;
-    s.most = s.tau_most = 0;
-    s.p_least = s.p_most = 0x3FF00000;                    // 1.0
-    double m = 1.0;
-    int x = 0;
-    tag_rows(tc, mt, cols, tbase, ev1, sbuf, lane, [&](int64_t e, const TagSlow& sl) {
-        const double w = WEIGHTED ? __ldg(cols.w + e) : 1.0;
-        tag_event_fast<WEIGHTED>(tc, mt, __ldg(cols.t + e), __ldg(cols.q + e), w, sl, top, gtop, s, &m, &x);
-    });
-    const int tt = tc.fx[0].top;                          // |t| < 2^(tt - 1)
-    // factors below 2^(top - 5): sixteen of them and their products with tau stay in 64 bits
-    const bool bad = s.p_least < 0x38200000 || s.p_most >= 0x47D00000 || (s.most >> 20) > 1023 - 6 + top ||
-                     s.tau_most >= ((1023 - 1 + tt) << 20 | 0xC0000);   // |tau| >= 1.75 2^(tt - 1)
-    if (__any_sync(0xffffffffu, bad)) return false;
-    acc[0] = s.log;
-    acc[1] = s.Q;
-#pragma unroll
-    for (int i = 0; i < 5; ++i) {
-        acc[2 + 2 * i] = fx_to_double(s.a[i], top - 1);
-        acc[3 + 2 * i] = fx_to_double(s.at[i], top + (i < 4 ? tt : gtop) - 3);
+        for (int i = 0; i < 6; ++i) {
+            s.most = max(s.most, high_word(x[i]));
+            const long long a = fx_odd(x[i], sc.top);
+            s.g[i] += a;
+            if (i < 5) s.g[6 + i] = fx_mad1(fx((long long)((unsigned long long)a << 3)), i < 4 ? T : TG, s.g[6 + i], a != 0);
+        }
     }
-    acc[12] = fx_to_double(s.a[5], top - 1);
-    *prod = m;
-    *esum = x;
-    return true;
-}
+    static __device__ __forceinline__ bool bad(const TagConsts& c, FastScale sc, const Sums& s) {
+        // factors below 2^(top - 5): sixteen of them and their products with tau stay in 64 bits;
+        // |tau| below 1.75 2^(fx.top - 1) (|t| < 2^(fx.top - 1))
+        return p_out_of_range(s) || (s.most >> 20) > 1023 - 6 + sc.top ||
+               s.tau_most >= ((1023 - 1 + c.fx[0].top) << 20 | 0xC0000);
+    }
+    static __device__ __forceinline__ void accumulators(const TagConsts& c, FastScale sc, const Sums& s, double* acc) {
+        acc[0] = s.f[1];
+        acc[1] = s.f[0];
+#pragma unroll
+        for (int i = 0; i < 5; ++i) {
+            acc[2 + 2 * i] = fx_to_double(s.g[i], sc.top - 1);
+            acc[3 + 2 * i] = fx_to_double(s.g[6 + i], sc.top + (i < 4 ? c.fx[0].top : sc.gtop) - 3);
+        }
+        acc[12] = fx_to_double(s.g[5], sc.top - 1);
+    }
+    template <bool W>
+    static __device__ __forceinline__ void plain(const TagConsts& c, const MathTables* mt, const Cols& cols, int i0,
+                                                 int i1, int64_t tbase, int64_t ev1, TagSlow* sbuf, int lane,
+                                                 double* acc, double* prod, int* esum) {
+        tag_rows<true, W>(c, mt, cols, i0, i1, tbase, ev1, sbuf, lane, acc, prod, esum);
+    }
+    static __device__ __forceinline__ void finish(const TagConsts& c, const double* acc, int n_par, double* out,
+                                                  int lane) {
+        tag_finalize<true>(c, acc, n_par, out, lane);
+    }
+};
 
 template <bool GRAD, bool WEIGHTED>
 __global__ void __launch_bounds__(32 * kMaxWarps, 2)
@@ -340,12 +307,11 @@ tag_kernel(Cols cols, int64_t n, const int64_t* __restrict__ seg_begin, const in
             double prod = 1.0;
             int esum = 0;
             const int64_t tbase = ev0 + (tile - t0) * kTile;
-            if (!GRAD || !tag_tile_fast<WEIGHTED>(tc, &mt, cols, tbase, ev1, sbuf, lane, acc, &prod, &esum)) {
-                tag_rows(tc, &mt, cols, tbase, ev1, sbuf, lane, [&](int64_t e, const TagSlow& sl) {
-                    const double w = WEIGHTED ? __ldg(cols.w + e) : 1.0;
-                    tag_event<GRAD, WEIGHTED>(tc, &mt, __ldg(cols.t + e), __ldg(cols.q + e), w, sl, acc, &prod, &esum);
-                });
-            }
+            if constexpr (GRAD)
+                solo_tile<Tagged, WEIGHTED>(tc, &mt, cols, tbase, ev1, sbuf, lane, acc, &prod, &esum);
+            else
+                tag_rows<GRAD, WEIGHTED>(tc, &mt, cols, 0, tile_rows(tbase, ev1), tbase, ev1, sbuf, lane, acc, &prod,
+                                         &esum);
             acc[0] += log_of(prod, esum, &mt);
             const double share = warp_butterfly<NA>(acc, lane);
             if (!tile_commit<NA>(share, lane, tile, t0, t1, seg, partials, gcount, counters, acc)) continue;
@@ -363,6 +329,11 @@ ipa_status launch_tag_t(const Cols& cols, int64_t n, const int64_t* seg_begin, c
     const bool single = seg_begin == nullptr;
     const int64_t tiles = tile_estimate(n, n_seg);
     const LaunchCfg cfg = force ? *force : launch_cfg(IPA_MODEL_TAGGED1D, GRAD, false, n_seg > 1, tiles);
+    if constexpr (GRAD) {
+        if (launch_team_ok(cfg, tiles))
+            return launch_team<Tagged, WEIGHTED>(cols, n, seg_begin, seg_end, seg_tiles, n_seg, consts, sc, out, n_par,
+                                                 tiles, st);
+    }
     const int W = cfg.warps_per_block >= 1 && cfg.warps_per_block <= kMaxWarps ? cfg.warps_per_block : 1;
     const int K = cfg.tiles_per_take >= 1 ? cfg.tiles_per_take : 1;
     const size_t smem = (size_t)W * (sizeof(TagConsts) + kSub * 32 * sizeof(TagSlow));

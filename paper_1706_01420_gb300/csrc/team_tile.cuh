@@ -1,0 +1,397 @@
+// A tile's fixed-point sums, by one warp or by a team of four (nll.cu, tagged.cu).
+//
+// Rows of 32 events are taken kSub at a time (a quarter of a tile).  A quarter's
+// FP64 sums start from zero and are added to the tile's in quarter order; the
+// fixed-point ones are exact.  So a tile has the same bits whether one warp takes
+// its four quarters in turn (solo_tile) or the four warps of a block take one each
+// (team_kernel).  If the tile cannot take the fixed-point path, its quarters are
+// redone by the plain loop in the same order.
+//
+// Which one: a team spreads a tile over the SM's four sub-partitions, each with its
+// own FP64 unit, and a small call over four times as many warps; a warp of its own
+// needs no exchange between warps.  launch_team_ok has the line between them.
+//
+// A model is a struct M with
+//   Record, Slow (a near-peak event's values), kSums: FP64 sums, kInts: integer sums, NA;
+//   usable<W>(c, cols, tbase, ev1, lane, &sc)   the scales of the tile, false: plain loop;
+//   quarter<W>(c, mt, cols, tbase, i0, ev1, sbuf, lane, sc, s);
+//   bad(c, sc, s)                               a value left its range;
+//   accumulators(c, sc, s, acc);
+//   plain<W>(c, mt, cols, i0, i1, tbase, ev1, sbuf, lane, acc, &prod, &esum);
+//   finish(c, acc, n_par, out, lane).
+#pragma once
+
+#include "fast_fixed.cuh"
+#include "ipa_internal.cuh"
+#include "tile_reduce.cuh"
+
+namespace ipa {
+
+constexpr int kSub = 4;                              // rows per quarter
+constexpr int kPerLane = kTile / 32;                 // events per lane per tile
+constexpr int kTeam = kPerLane / kSub;               // warps that share a tile
+static_assert(kSub == 4 && kPerLane % kSub == 0, "a quarter keeps four ballot masks");
+
+// The angular sums' unit is 2^-46 of a typical term, which a handful of events with small
+// angular products would show: a tile of fewer events takes the plain loop.
+constexpr int kFewEvents = 64;
+
+// The scales of a tile's integers: its factors, and tau in the Gaussian's sums.
+struct FastScale {
+    int top, gtop;
+};
+
+// A lane's sums over rows on the fixed-point path: FP64 ones, the product of the P's of
+// events without weight (mantissas, exponents), integers, and the high words of the
+// largest factor, of the largest |tau| and of the least and largest P.
+template <int NF, int NG>
+struct FastSums {
+    double f[NF];
+    double prod;
+    long long g[NG];
+    int esum;
+    int most, tau_most, p_least, p_most;
+};
+
+template <int NF, int NG>
+__device__ __forceinline__ void clear(FastSums<NF, NG>& s) {
+#pragma unroll
+    for (int i = 0; i < NF; ++i) s.f[i] = 0.0;
+    s.prod = 1.0;
+#pragma unroll
+    for (int i = 0; i < NG; ++i) s.g[i] = 0;
+    s.esum = 0;
+    s.most = s.tau_most = 0;
+    s.p_least = s.p_most = 0x3FF00000;               // 1.0
+}
+
+// P outside [2^-125, 2^126) (the Newton reciprocal's range) or not a number in some event.
+template <int NF, int NG>
+__device__ __forceinline__ bool p_out_of_range(const FastSums<NF, NG>& s) {
+    return s.p_least < 0x38200000 || s.p_most >= 0x47D00000;
+}
+template <int NF, int NG>
+__device__ __forceinline__ void note_p(double P, FastSums<NF, NG>& s) {
+    const int h = (int)(__double_as_longlong(P) >> 32);   // negative for P < 0
+    s.p_least = min(s.p_least, h);
+    s.p_most = max(s.p_most, h);
+}
+
+// The log term of an event: w log P, or P into the lane's product for weight 1.
+template <bool WEIGHTED, class S>
+__device__ __forceinline__ void add_log(double P, double w, const MathTables* mt, double* sum, S& s) {
+    note_p(P, s);
+    if (WEIGHTED) {
+        const bool one = __double_as_longlong(w) == 0x3FF0000000000000ll;
+        *sum = fma(one ? 0.0 : w, fx_to_double(fx_log(P, mt), 6), *sum);
+        log_mul_nb(one ? P : 1.0, &s.prod, &s.esum);
+    } else {
+        log_mul_nb(P, &s.prod, &s.esum);
+    }
+}
+
+// The exponent of the largest |w| of a tile (0 where all weights are 1, as without weights).
+__device__ __forceinline__ int weight_exponent(const Cols& cols, int64_t tbase, int64_t ev1, int lane) {
+    int hi = 0;
+#pragma unroll 4
+    for (int i = 0; i < kPerLane; ++i) {
+        const int64_t e = tbase + lane + 32 * i;
+        hi = max(hi, high_word(e < ev1 ? __ldg(cols.w + e) : 0.0));
+    }
+    return (int)(__reduce_max_sync(0xffffffffu, (unsigned)hi) >> 20) - 1023;
+}
+
+// Rows of a tile with events below ev1, up to a whole quarter.
+__device__ __forceinline__ int tile_rows(int64_t tbase, int64_t ev1) {
+    const int64_t rows = (ev1 - tbase + 31) >> 5;
+    return rows >= kPerLane ? kPerLane : (int)((rows + kSub - 1) / kSub) * kSub;
+}
+
+// The near-peak events (t <= tcut) of a quarter: listed by a ballot per row and evaluated
+// packed, 32 per pass, into sbuf, so the FP64 pipe does not run the long branch for lanes
+// that discard it.  slow(i): event i's values.
+struct SlowRows {
+    unsigned m[kSub];
+    int p[kSub];
+    // position of row q's event of this lane in sbuf, or -1
+    __device__ __forceinline__ int at(int q, unsigned below, int lane) const {
+        const unsigned mq = q == 0 ? m[0] : (q == 1 ? m[1] : (q == 2 ? m[2] : m[3]));
+        const int before = q == 0 ? 0 : (q == 1 ? p[1] : (q == 2 ? p[2] : p[3]));
+        return (mq >> lane) & 1u ? before + __popc(mq & below) : -1;
+    }
+};
+template <class Slow, class F>
+__device__ __forceinline__ void slow_rows(SlowRows& r, const Cols& cols, double tcut, int64_t tbase, int i0, int64_t ev1,
+                                          Slow* sbuf, int lane, F slow) {
+#pragma unroll
+    for (int q = 0; q < kSub; ++q) {
+        const int64_t e = tbase + lane + 32 * (i0 + q);
+        r.m[q] = __ballot_sync(0xffffffffu, e < ev1 && !greater(__ldg(cols.t + e), tcut));
+    }
+    r.p[0] = 0;
+    r.p[1] = __popc(r.m[0]);
+    r.p[2] = r.p[1] + __popc(r.m[1]);
+    r.p[3] = r.p[2] + __popc(r.m[2]);
+    const int n_slow = r.p[3] + __popc(r.m[3]);
+    for (int j = lane; j < n_slow; j += 32) {
+        const int q = (j >= r.p[1]) + (j >= r.p[2]) + (j >= r.p[3]);
+        const unsigned mq = q == 0 ? r.m[0] : (q == 1 ? r.m[1] : (q == 2 ? r.m[2] : r.m[3]));
+        const int before = q == 0 ? 0 : (q == 1 ? r.p[1] : (q == 2 ? r.p[2] : r.p[3]));
+        sbuf[j] = slow(tbase + nth_set(mq, j - before) + 32 * (i0 + q));
+    }
+    __syncwarp();
+}
+
+// Quarters [i0, i1) by the plain loop (rare): the lane's sums, product and exponent sum in
+// the first NA, next and last word of `out`.
+template <class M, bool W>
+__device__ __noinline__ void plain_quarters(const typename M::Record& c, const MathTables* mt, const Cols& cols, int i0,
+                                            int i1, int64_t tbase, int64_t ev1, typename M::Slow* sbuf, int lane,
+                                            double* out) {
+    double prod = 1.0;
+    int esum = 0;
+#pragma unroll
+    for (int a = 0; a < M::NA; ++a) out[a] = 0.0;
+#pragma unroll 1
+    for (; i0 < i1 && tbase + 32 * i0 < ev1; i0 += kSub) {
+        double q[M::NA], qp = 1.0;
+#pragma unroll
+        for (int a = 0; a < M::NA; ++a) q[a] = 0.0;
+        M::template plain<W>(c, mt, cols, i0, i0 + kSub, tbase, ev1, sbuf, lane, q, &qp, &esum);
+#pragma unroll
+        for (int a = 0; a < M::NA; ++a) out[a] += q[a];
+        prod *= qp;
+    }
+    out[M::NA] = prod;
+    out[M::NA + 1] = __longlong_as_double((long long)(unsigned)esum);
+}
+
+// A whole tile by one warp: acc, prod and esum of the lane.
+template <class M, bool W>
+__device__ __forceinline__ void solo_tile(const typename M::Record& c, const MathTables* mt, const Cols& cols,
+                                          int64_t tbase, int64_t ev1, typename M::Slow* sbuf, int lane, double* acc,
+                                          double* prod, int* esum) {
+    FastScale sc;
+    bool plain = !M::template usable<W>(c, cols, tbase, ev1, lane, &sc);
+    if (!plain) {
+        FastSums<M::kSums, M::kInts> s;
+        clear(s);
+        double tot[M::kSums], tprod = 1.0;
+#pragma unroll
+        for (int i = 0; i < M::kSums; ++i) tot[i] = 0.0;
+#pragma unroll 1
+        for (int i0 = 0; i0 < kPerLane && tbase + 32 * i0 < ev1; i0 += kSub) {
+            M::template quarter<W>(c, mt, cols, tbase, i0, ev1, sbuf, lane, sc, s);
+#pragma unroll
+            for (int i = 0; i < M::kSums; ++i) {
+                tot[i] += s.f[i];
+                s.f[i] = 0.0;
+            }
+            tprod *= s.prod;
+            s.prod = 1.0;
+        }
+        plain = __any_sync(0xffffffffu, M::bad(c, sc, s));
+#pragma unroll
+        for (int i = 0; i < M::kSums; ++i) s.f[i] = tot[i];
+        M::accumulators(c, sc, s, acc);
+        *prod = tprod;
+        *esum = s.esum;
+    }
+    if (plain) {
+        double q[M::NA + 2];                         // (apart from acc, which stays in registers)
+        plain_quarters<M, W>(c, mt, cols, 0, kPerLane, tbase, ev1, sbuf, lane, q);
+#pragma unroll
+        for (int a = 0; a < M::NA; ++a) acc[a] = q[a];
+        *prod = q[M::NA];
+        *esum = (int)__double_as_longlong(q[M::NA + 1]);
+    }
+}
+
+// Doubles a lane exchanges: the sums of either path, the product and the exponents.
+template <class M>
+constexpr int team_words() {
+    return (M::kSums + M::kInts > M::NA ? M::kSums + M::kInts : M::NA) + 2;
+}
+template <class M>
+constexpr size_t team_smem() {
+    return sizeof(double) * 2 * kTeam * team_words<M>() * 32 + sizeof(typename M::Slow) * kTeam * kSub * 32 +
+           sizeof(typename M::Record);
+}
+
+// One tile per block and take, a quarter per warp.  The next take is fetched while a tile is
+// in work; the exchange buffer is used in turns, so that one barrier per tile orders its
+// writes after the reads of two tiles before, and the warps take turns in adding a tile up.
+template <class M, bool W>
+__global__ void __launch_bounds__(32 * kTeam, 4)
+team_kernel(Cols cols, int64_t n, const int64_t* __restrict__ seg_begin, const int64_t* __restrict__ seg_end,
+            const int64_t* __restrict__ seg_tiles, int n_seg, const Consts* __restrict__ consts,
+            double* __restrict__ partials, unsigned* __restrict__ counters, unsigned* __restrict__ gcount,
+            unsigned* __restrict__ work, double* __restrict__ out, int n_par) {
+    constexpr int kWords = team_words<M>();
+    const int out_stride = 1 + n_par;
+    __shared__ MathTables mt;
+    __shared__ int64_t s_take[2];
+    extern __shared__ __align__(16) unsigned char dyn_smem[];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    double* const xbuf = reinterpret_cast<double*>(dyn_smem);               // [2][kTeam][kWords][32]
+    typename M::Slow* const sbuf =
+        reinterpret_cast<typename M::Slow*>(xbuf + 2 * kTeam * kWords * 32) + wib * (kSub * 32);
+    typename M::Record& c = *reinterpret_cast<typename M::Record*>(
+        reinterpret_cast<typename M::Slow*>(xbuf + 2 * kTeam * kWords * 32) + kTeam * kSub * 32);
+
+    load_math_tables(&mt);
+    // a programmatic dependent of the constants kernel: wait for its results
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+
+    const bool single = seg_begin == nullptr;
+    const int64_t total = single ? (n + kTile - 1) / kTile : __ldg(seg_tiles + n_seg);
+    if (blockIdx.x == 0) {
+        for (int s = threadIdx.x; s < n_seg; s += blockDim.x) {
+            const bool empty = single ? (n == 0) : (__ldg(seg_tiles + s + 1) == __ldg(seg_tiles + s));
+            if (empty)
+                for (int j = 0; j < out_stride; ++j) out[(size_t)s * out_stride + j] = 0.0;
+        }
+    }
+    if (threadIdx.x == 0) s_take[0] = (int64_t)atomicAdd(work, 1u);
+    __syncthreads();
+    int cur = -1;
+    for (int turn = 0;; ++turn) {
+        const int64_t tile = s_take[turn & 1];
+        if (tile >= total) break;
+        int seg = 0;
+        int64_t t0 = 0, t1 = total, ev0 = 0, ev1 = n;
+        if (!single) {
+            seg = find_segment(seg_tiles, n_seg, tile);
+            t0 = __ldg(seg_tiles + seg);
+            t1 = __ldg(seg_tiles + seg + 1);
+            ev0 = clamp_off(__ldg(seg_begin + seg), n);
+            ev1 = clamp_off(__ldg(seg_end + seg), n);
+            if (ev1 < ev0) ev1 = ev0;
+        }
+        if (seg != cur) {                            // (the same for the whole block)
+            __syncthreads();
+            const double* src = reinterpret_cast<const double*>(consts + seg);
+            double* dst = reinterpret_cast<double*>(&c);
+            for (int i = threadIdx.x; i < (int)(sizeof(c) / sizeof(double)); i += blockDim.x) dst[i] = __ldg(src + i);
+            __syncthreads();
+            cur = seg;
+        }
+        const int64_t tbase = ev0 + (tile - t0) * kTile;
+        double* const x = xbuf + (size_t)(turn & 1) * kTeam * kWords * 32 + lane;
+        double* const own = x + wib * kWords * 32;
+        const int i0 = wib * kSub;
+        FastScale sc;
+        bool plain = !M::template usable<W>(c, cols, tbase, ev1, lane, &sc);
+        {
+            FastSums<M::kSums, M::kInts> s;
+            clear(s);
+            if (!plain && tbase + 32 * i0 < ev1) {
+                M::template quarter<W>(c, &mt, cols, tbase, i0, ev1, sbuf, lane, sc, s);
+                plain = M::bad(c, sc, s);
+            }
+#pragma unroll
+            for (int i = 0; i < M::kSums; ++i) own[i * 32] = s.f[i];
+#pragma unroll
+            for (int i = 0; i < M::kInts; ++i) own[(M::kSums + i) * 32] = __longlong_as_double(s.g[i]);
+            own[(kWords - 2) * 32] = s.prod;
+            own[(kWords - 1) * 32] = __longlong_as_double((long long)(unsigned)s.esum);
+        }
+        if (threadIdx.x == 32 * ((turn + 2) & (kTeam - 1))) s_take[(turn + 1) & 1] = (int64_t)atomicAdd(work, 1u);
+        plain = __syncthreads_or(plain);
+        if (plain) {
+            double q[M::NA + 2];
+            plain_quarters<M, W>(c, &mt, cols, i0, i0 + kSub, tbase, ev1, sbuf, lane, q);
+#pragma unroll
+            for (int a = 0; a < M::NA; ++a) own[a * 32] = q[a];
+            own[(kWords - 2) * 32] = q[M::NA];
+            own[(kWords - 1) * 32] = q[M::NA + 1];
+            __syncthreads();
+        }
+        if (wib != (turn & (kTeam - 1))) continue;
+
+        double acc[M::NA], prod = 1.0;
+        int esum = 0;
+        if (!plain) {
+            FastSums<M::kSums, M::kInts> s;
+            clear(s);
+#pragma unroll
+            for (int w = 0; w < kTeam; ++w) {
+                const double* y = x + w * kWords * 32;
+#pragma unroll
+                for (int i = 0; i < M::kSums; ++i) s.f[i] += y[i * 32];
+#pragma unroll
+                for (int i = 0; i < M::kInts; ++i) s.g[i] += __double_as_longlong(y[(M::kSums + i) * 32]);
+                prod *= y[(kWords - 2) * 32];
+                esum += (int)__double_as_longlong(y[(kWords - 1) * 32]);
+            }
+            M::accumulators(c, sc, s, acc);
+        } else {
+#pragma unroll
+            for (int a = 0; a < M::NA; ++a) acc[a] = 0.0;
+#pragma unroll 1
+            for (int w = 0; w < kTeam; ++w) {
+                const double* y = x + w * kWords * 32;
+#pragma unroll
+                for (int a = 0; a < M::NA; ++a) acc[a] += y[a * 32];
+                prod *= y[(kWords - 2) * 32];
+                esum += (int)__double_as_longlong(y[(kWords - 1) * 32]);
+            }
+        }
+        acc[0] += log_of(prod, esum, &mt);
+        const double share = warp_butterfly<M::NA>(acc, lane);
+        if (!tile_commit<M::NA>(share, lane, tile, t0, t1, seg, partials, gcount, counters, acc)) continue;
+        M::finish(c, acc, n_par, out + (size_t)seg * out_stride, lane);
+        if (lane == 0) counters[seg] = 0u;
+    }
+    work_done(work, lane);
+}
+
+// Whether a launch of about `tiles` tiles goes to the teams: the built-in geometry (a tuned or
+// given one is for single warps) and at most eight tiles per SM.  Measured, call by call, single
+// warps / teams in us: 16 to 152 tiles 35 / 24 (1D), 56 / 33 (4D), 78 / 41 (tagged); 608 tiles 38 / 28,
+// 64 / 42, 83 / 69; 1216 tiles (eight per SM) 44 / 40, 75 / 64, 100 / 92; 1520 tiles 45 / 47, 76 / 75,
+// 108 / 115; 2048 tiles 51 / 56, 87 / 90, 125 / 137 (a tile's exchange then costs more than the
+// evener load gains).
+constexpr int kTeamTilesPerSm = 8;
+inline bool launch_team_ok(const LaunchCfg& cfg, int64_t tiles) {
+    return cfg.warps_per_block == 1 && cfg.warps_per_sm == 0 && cfg.tiles_per_take == 1 &&
+           tiles <= (int64_t)kTeamTilesPerSm * sm_count();
+}
+
+template <class M, bool W>
+ipa_status launch_team(const Cols& cols, int64_t n, const int64_t* seg_begin, const int64_t* seg_end,
+                       const int64_t* seg_tiles, int n_seg, const Consts* consts, Scratch* sc, double* out, int n_par,
+                       int64_t tiles, cudaStream_t st) {
+    auto kern = team_kernel<M, W>;
+    constexpr size_t smem = team_smem<M>();
+    static int occ[64] = {};                         // resident blocks per SM, per device
+    int dev = 0;
+    cudaGetDevice(&dev);
+    int& per_sm = occ[dev & 63];
+    if (per_sm == 0) {
+        ipa_status q = cuda_fail(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
+                                 "likelihood kernel attribute");
+        if (q != IPA_OK) return q;
+        int v = 0;
+        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, kern, 32 * kTeam, smem);
+        per_sm = e == cudaSuccess && v >= 1 ? v : 1;
+    }
+    int64_t grid = (int64_t)per_sm * sm_count();
+    if (seg_begin == nullptr && tiles < grid) grid = tiles < 1 ? 1 : tiles;
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3((unsigned)grid);
+    lc.blockDim = dim3(32 * kTeam);
+    lc.dynamicSmemBytes = smem;
+    lc.stream = st;
+    // blocks may start (and load their tables) while the constants kernel is still running
+    cudaLaunchAttribute la[1];
+    la[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    la[0].val.programmaticStreamSerializationAllowed = 1;
+    lc.attrs = la;
+    lc.numAttrs = 1;
+    return cuda_fail(cudaLaunchKernelEx(&lc, kern, cols, n, seg_begin, seg_end, seg_tiles, n_seg, consts, sc->partials,
+                                        sc->counters, sc->gcount, sc->work, out, n_par),
+                     "likelihood kernel launch");
+}
+
+}  // namespace ipa

@@ -142,3 +142,42 @@ def test_time_models_weight_scales_and_handover(env, kind, ws):
     logl, terms = O.nll_grad_terms(m, ev, th)
     assert abs(got[0] - f) <= 1e-14 * np.abs(logl).sum()
     assert np.all(np.abs(got[1:] - g) <= 5e-13 * np.abs(terms).sum(1)), (got[1:], g)
+
+
+@pytest.mark.parametrize("redo", [False, True])
+@pytest.mark.parametrize("weighted", [False, True])
+@pytest.mark.parametrize("kind", ["1d", "4d", "tagged"])
+def test_one_warp_or_a_team_per_tile(env, kind, weighted, redo):
+    """A tile's four quarters taken by one warp or by the four of a team give the
+    same bits, on the fixed-point path and where a tile is redone (P below the Newton
+    reciprocal's range); the values against the oracle (tolerance as above)."""
+    O, G, _ = env
+    import torch
+    from paper_1706_01420_gb300 import api
+    th = np.array({"1d": TH4[:4], "4d": TH4, "tagged": [0.66, 0.045, 0.0, 0.1, 0.085, 17.77, 0.8, 0.3]}[kind])
+    th[3] = 0.0 if redo else th[3]
+    m = getattr(api, "model_" + kind)(-2.0, HI)
+    mo = O.Model("tag" if kind == "tagged" else kind, -2.0, HI)
+    theta = torch.tensor(th, device="cuda")
+    for n in (1, 63, 64, 129, 385, 512, 545, 1537):
+        if kind == "1d":
+            cols = {"t": synth.events_1d(n, 71, t_lo=0.0)}
+            if weighted:
+                cols["w"] = synth.weights(n, 73)
+        else:
+            cols = {"4d": synth.events_4d, "tagged": synth.events_tagged}[kind](n, 71, weighted=weighted)
+        if redo:
+            cols["t"][n // 2] = -1.1                      # 24 sigma before the edge: P near 1e-130
+        ev = G.to_dev(cols)
+        got = {}
+        try:
+            for warps in (1, 2):
+                api.ipa_launch_config_set(m, n, {"warps_per_block": warps, "warps_per_sm": 0, "tiles_per_take": 1})
+                got[warps] = api.ipa_nll_grad(m, ev, theta).cpu().numpy()
+        finally:
+            api.ipa_launch_config_set(m, n, {"warps_per_block": 1, "warps_per_sm": 0, "tiles_per_take": 1})
+        assert np.array_equal(got[1], got[2]), n
+        f, g = O.nll_grad(mo, cols, th)
+        logl, terms = O.nll_grad_terms(mo, cols, th)
+        assert abs(got[1][0] - f) <= 1e-14 * np.abs(logl).sum(), n
+        assert np.all(np.abs(got[1][1:] - g) <= 5e-13 * np.abs(terms).sum(1)), n
