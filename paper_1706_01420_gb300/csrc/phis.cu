@@ -136,7 +136,7 @@ struct PhisWarp {
     double eq[6], mu[4], mv[4];
     double D2, D2s, D2c;      // 2 D, 2 D s, 2 D c
     // the same in fixed point (rows_fast): eq, mu, mv with max in [1/8, 1/4) at 2^-hexp; c and s
-    // (Q62); rtop: scale of the angular sums' factors at unit weight, below 2^(rtop - 2)
+    // (Q62); rtop: scale of the angular sums' factors at unit weight (2^11 typical ones, 2^(rtop - 2))
     int2 fe[6], fu[4], fv[4], fc, fs;
     int hexp, rtop, fixed, pad_;
 };
@@ -177,7 +177,7 @@ __device__ __forceinline__ void phis_coefficients(PhisWarp& pw, bool cached, int
         // a typical r T is near 1 / max(max|coefficient|, cb / 4)
         const int ea = ok ? -up - 3 : -1023, eb = exponent_field(c.cb) - 1025;
         const int e = ea > eb ? ea : eb;
-        pw.rtop = 16 + (e < -900 ? 900 : -e);
+        pw.rtop = 13 + (e < -900 ? 900 : -e);
         pw.hexp = 2 - (ok ? up : 0);
         pw.fixed = ok;
     }
@@ -256,7 +256,7 @@ __device__ __forceinline__ void phis_event(const PhisWarp& pw, const MathTables*
 // As in the 4D kernel's fast rows (nll.cu): the ten f'_k (Q62), F+, F-, FU, FV and what is linear
 // in them on the integer pipe, and the 14 angular sums as 64-bit integers: the factors r T+, r T-,
 // r U and r C are converted once per event at a scale that follows the segment's typical r T and
-// the largest weight of the warp's rows (unit 2^-45 of a typical term, 0.41 units rms per
+// the largest weight of the warp's rows (unit 2^-48 of a typical term, 0.41 units rms per
 // event).  The rest is FP64.  The warp's rows are redone by phis_event where some P lies outside
 // the Newton reciprocal's range or some factor outside its scale.  FP64 instructions per
 // event: 92 -> 57; 1e6 events 299 -> 248 us (FP64 unit busy 77 -> 68 %).
