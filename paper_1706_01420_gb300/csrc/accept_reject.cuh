@@ -28,13 +28,15 @@
 // Before, the angular test of the tenth of the candidates that pass the time
 // test ran in almost every iteration of a warp with three lanes active.
 //
-// Bound: instruction issue (about 75 warp instructions per 32 candidates for
-// Philox and the time test, 20 of them 32 x 32 -> 64-bit products, of 190 in
-// all; a 4D event needs 50 candidates) and the latency of the look-back: 46 %
-// of the issue slots busy.  Measured (one block per toy / blocks with barriers /
-// warps): 4D, one sample of 133 725 events 30.2 ms / 92 us / 84 us; 4D, 512 toys
-// of Poisson(2e4) 11.5 / 4.5 / 3.7 ms; phi_s, 102 toys of 8170 (every candidate in
-// FP64 before) 24.0 / 0.77 / 0.69 ms.
+// Bound: instruction issue (about 155 warp instructions per 32 candidates, 45 of
+// them Philox's and the first test's, 18 of those 32 x 32 -> 64-bit products; a 4D
+// event needs 50 candidates) and, where tickets are small, the latency of the
+// look-back: 67 % of the issue slots busy.  Measured (one block per toy / blocks with
+// barriers / warps / the first test folded into one multiply-add and compare on the
+// words, two candidates at once, and larger tickets where there are many): 4D,
+// one sample of 133 725 events 30.2 ms / 92 us / 84 us / 81 us; 4D, 512 toys of
+// Poisson(2e4) 11.5 / 4.5 / 3.7 / 2.8 ms; phi_s, 102 toys of 8170 (every candidate in
+// FP64 before) 24.0 / 0.77 / 0.68 / 0.69 ms.
 #pragma once
 
 #include <stdint.h>
@@ -55,6 +57,13 @@ constexpr int kBkgChunk = 512;           // background events per ticket
 // stay below 1.3 bytes per event.  A toy of an envelope that accepts less is
 // one ticket.
 constexpr int kGenMinKept = 8;
+// ... and more where there is work enough: while kGenPerWarp tickets per resident
+// warp are left and a ticket's events fit the list (kGenPick) with room to spare.
+// Fewer look-backs: the 512 toys take 3.19 ms at one unit per ticket, 2.88 at two and
+// 2.76 at four; a single sample of 133 725 events, with 1.4 units per warp, 82, 91
+// and 102 us.
+constexpr int kGenMostKept = 160;
+constexpr int kGenPerWarp = 16;
 constexpr int kGenMaxSub = 64;
 
 // What a test says of a candidate.
@@ -137,7 +146,7 @@ __device__ __forceinline__ uint32_t gen_decide(const typename G::Shared& S, cons
     uint32_t word = 0u;
     __syncwarp();
     L.keep[lane] = 0u;
-#pragma unroll 1
+#pragma unroll (G::kUnroll)
     for (int i = 0; i < 32; ++i) {
         const int cand = i * 32 + lane;
         const GenCode c = G::quick(S, A, GenIdx{lo + cand, hi, toy});
@@ -376,21 +385,34 @@ __global__ void __launch_bounds__(kBlock, G::kBlocksPerSm) generate_kernel(const
 // chunk accepts fewer than kGenMinKept, or where the total would exceed
 // max_tickets.
 template <class G>
-__global__ void gen_tickets_kernel(const __grid_constant__ GenArgs A, int64_t max_tickets, int64_t* __restrict__ base) {
+__global__ void gen_tickets_kernel(const __grid_constant__ GenArgs A, int64_t max_tickets, int64_t n_warps,
+                                   int64_t* __restrict__ base) {
     __shared__ int64_t run[1024];
     __shared__ float per_cand;
+    __shared__ unsigned long long events;            // of signal, in all toys
+    if (threadIdx.x == 0) events = 0ull;
+    __syncthreads();
+    const int nt = blockDim.x;
+    const int per = (A.n_toys + nt - 1) / nt;
+    const int b = min(A.n_toys, (int)threadIdx.x * per), e = min(A.n_toys, b + per);
+    {
+        unsigned long long sum = 0;
+        for (int s = b; s < e; ++s) {
+            int64_t ns, nb, off;
+            if (gen_toy(A, s, &ns, &nb, &off)) sum += (unsigned long long)ns;
+        }
+        if (sum) atomicAdd(&events, sum);
+    }
     G::acceptance(A, &per_cand);
     __syncthreads();
     float kept = per_cand * (float)kGenCand;
+    const float many = (float)events / ((float)kGenPerWarp * (float)n_warps);   // kept per ticket that leaves kGenPerWarp
     int sub = 1;
-    while (sub < kGenMaxSub && kept < (float)kGenMinKept) {
+    while (sub < kGenMaxSub && (kept < (float)kGenMinKept || 2.0f * kept <= fminf((float)kGenMostKept, many))) {
         sub *= 2;
         kept *= 2.0f;
     }
     const bool cut = kept >= (float)kGenMinKept && kept <= 2.0f * kGenCand;
-    const int nt = blockDim.x;
-    const int per = (A.n_toys + nt - 1) / nt;
-    const int b = min(A.n_toys, (int)threadIdx.x * per), e = min(A.n_toys, b + per);
     for (int round = 0; round < 2; ++round) {
         const bool split = round == 0 && cut;
         auto tickets = [&](int toy) -> int64_t {
@@ -461,7 +483,7 @@ ipa_status launch_generator(GenArgs A, cudaStream_t s) {
         A.ticket = reinterpret_cast<unsigned long long*>(base + A.n_toys + 2);
         A.status = A.ticket + 1;
         if (st == IPA_OK) {
-            gen_tickets_kernel<G><<<1, 1024, 0, s>>>(A, max_tickets, base);
+            gen_tickets_kernel<G><<<1, 1024, 0, s>>>(A, max_tickets, most * kGenWarps, base);
             const int64_t need = (max_tickets + kGenWarps - 1) / kGenWarps;
             generate_kernel<G><<<(unsigned)(need < most ? need : most), kBlock, smem, s>>>(A);
             st = cuda_fail(cudaGetLastError(), "toygen kernel launch");

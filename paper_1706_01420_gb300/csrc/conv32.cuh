@@ -37,6 +37,13 @@ __device__ __forceinline__ Exp32 exp32_of(double x, double off) {
     return Exp32{(float)(x * kLog2e), (float)(off * kLog2e)};
 }
 
+// 2^x (relative error below 2^-22; 0 below -126)
+__device__ __forceinline__ float ex2_approx(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
 // Bound of the relative error of exp2f(off - x tau), tau off by dtau: the
 // argument is off by |x| dtau and by four roundings of terms no larger than
 // |x tau| + |off|; exp2f adds 2 ulp; a factor 2 and 1e-6 to spare.

@@ -157,6 +157,7 @@ template <bool ANGLES>
 struct TimeGen {
     static constexpr bool kQuickKeeps = !ANGLES, kQuick64 = !ANGLES;
     static constexpr int kBlocksPerSm = 4;
+    static constexpr int kUnroll = ANGLES ? 2 : 1;    // two candidates' Philox chains at once
     struct Shared {
         Consts c;
         Filter32 f;
@@ -164,6 +165,10 @@ struct TimeGen {
         float near;       // tau above it: z <= -4.3
         float dl;         // bound of the error of u M_T
         double t_lo, span;
+        // the test away from the peak on the words themselves (4D): for a first word above
+        // far, g = 2^(word lin + con) and the candidate is dropped if its third word > g per_g + more
+        uint32_t far;
+        float lin, con, per_g, more;
     };
 
     __device__ static void setup(Shared& S, const GenArgs& A) {
@@ -189,6 +194,19 @@ struct TimeGen {
         // (a negative sigma has no such region: every candidate takes the full test)
         S.near = c.k_z > 0.0 ? (float)(c.Gs2 + 4.3 / c.k_z) * 1.000001f + 1.0e-6f * (f.span + fabsf(f.d)) : INFINITY;
         S.dl = f.MT * 1.5e-6f;
+        // tau = (t_lo - mu) + u span with u = word 2^-32 within 2^-31: the exponent's error is
+        // below 2^-24 times 3 |x span| + 2 |con| (the word's, lin's, con's and the sum's roundings),
+        // ex2.approx adds 2^-22; a factor 2 and 1e-6 to spare, and 1.5e-6 M_T for u M_T
+        const double x = c.Gamma * kLog2e, d = A.m.t_lo - c.mu;
+        const double con = c.c_exp * kLog2e - x * d, size = fabs(x) * S.span + fabs(con);
+        const double err = 2.0 * (0.7 * 0x1p-22 * size + 2.5e-7) + 1.0e-6;
+        const double at = ((double)S.near - d) / S.span;       // u at the end of the peak
+        S.far = at < 0.0 ? 0u : (at < 0.999999 ? (uint32_t)((at + 1.0e-6) * 4294967296.0) : 0xFFFFFFFFu);
+        if (!(err <= 1.0e-3) || !(c.MT >= 0x1p-90) || !(at < 1.0)) S.far = 0xFFFFFFFFu;   // no such test
+        S.lin = (float)(-x * S.span * 0x1p-32);
+        S.con = (float)con;
+        S.per_g = (float)(4294967296.0 / c.MT * (1.0 + err) * 1.000001);
+        S.more = 6500.0f;                                      // 1.5e-6 2^32
     }
 
     __device__ static bool usable(const Shared& S) {
@@ -208,14 +226,17 @@ struct TimeGen {
     // The decay-time test away from the resolution peak, where g is the exponential alone.
     __device__ __forceinline__ static GenCode quick(const Shared& S, const GenArgs& A, const GenIdx& j) {
         const U4 a = gen_draw(A, j, 0u);
+        if (ANGLES) {
+            const float g = ex2_approx(fmaf(__uint2float_rn(a.x), S.lin, S.con));
+            return a.x > S.far && __uint2float_rn(a.z) > fmaf(g, S.per_g, S.more) ? kDrop : kTest32;
+        }
         const float tau = fmaf(u32of(a.x), S.f.span, S.f.d);
         const float arg = fmaf(-S.e.x, tau, S.e.off);
         const float g = exp2f(arg);
         const float lhs = u32of(a.z) * S.f.MT;
         const float err = exp32_err(fabsf(S.e.x), fabsf(S.e.off), tau, tau32_err(tau, S.f.d, S.f.span));
         if (!(tau > S.near) || !(fabsf(arg) <= kMaxArg) || !(err <= 1.0e-3f)) return kTest32;
-        const GenCode c = decide32(lhs, S.dl, g, g * err);
-        return ANGLES ? (c == kDrop ? kDrop : kTest32) : c;
+        return decide32(lhs, S.dl, g, g * err);
     }
 
     __device__ __forceinline__ static GenCode test32(const Shared& S, const GenArgs& A, const GenIdx& j) {
@@ -282,7 +303,7 @@ struct TimeGen {
 // oscillation, near the peak with FP32 erfc and Faddeeva functions.
 struct TagGen {
     static constexpr bool kQuickKeeps = false, kQuick64 = false;
-    static constexpr int kBlocksPerSm = 3;
+    static constexpr int kBlocksPerSm = 3, kUnroll = 1;
     struct Shared {
         TagConsts c;
         Conv32 v;

@@ -75,6 +75,16 @@ def test_chunks_equal_the_oracle(model):
             at += n
 
 
+def test_tickets_of_several_units():
+    """Enough work for larger tickets (four units of candidates each)."""
+    rng = np.random.default_rng(5)
+    n_sig = rng.integers(15000, 35000, 320)
+    n_sig[[3, 100]] = 0, 1
+    n_bkg = rng.integers(0, 1500, 320)
+    _generate("4d", THETA["4d"], 3, [1], [0])
+    assert _same(_generate("4d", THETA["4d"], 21, n_sig, n_bkg), _alone("4d", THETA["4d"], 21, n_sig, n_bkg))
+
+
 def test_low_acceptance_and_bad_parameters():
     _generate("4d", THETA["4d"], 3, [1], [0])
     steep = np.array(THETA["4d"])
