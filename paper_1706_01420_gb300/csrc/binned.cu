@@ -22,13 +22,16 @@
 // chains; the data take the same order.
 //
 // A lane draws one toy's bins: the 32 toys of a warp meet a bin together, so its
-// thresholds and weight come as one broadcast from shared memory and the
-// Philox counter's bin half is computed once.  Before, a block walked one toy
+// thresholds (their high words: a tie goes by the whole table) and weight come as one
+// broadcast from shared memory, and the first two of Philox's ten rounds are
+// computed once per bin and once per toy.  Before, a block walked one toy
 // with a bin per thread: every draw fetched its own 40-byte record and two or
 // three doubles of the CDF from L2 (2.4 MB of tables), and converted and
 // compared in FP64, four FP64 instructions per draw on a pipe of 2 per clock and
-// SM.  Now one (the FMA into X).  10 000 bins, 10 000 toys: 3.7 -> 0.81 ms; the tables
-// (a serial chain per bin, run twice and to its end before) 305 -> 21 us for both.
+// SM.  Now one (the FMA into X).  Bound by the 32 x 32 -> 64-bit products (15 per draw) and
+// issue.  10 000 bins, 10 000 toys: 3.7 ms before, 0.81 with the ten rounds per draw and
+// 64-bit thresholds, 0.72 now; the tables (a serial chain per bin, run twice and to its
+// end before) 305 -> 21 us for both.
 #include <math.h>
 
 #include "ipa_internal.cuh"
@@ -43,7 +46,7 @@ constexpr int kTabBlock = 64;           // bins per block of the table kernels: 
 constexpr int kTabFixed = 32;           // thresholds per bin in the fixed part of the table
 constexpr int kSlice = 64;              // bins summed by one thread of the CLs kernel
 constexpr int kToyBlock = 128;          // toys per block of the CLs kernel
-constexpr int kFirst = 4;               // thresholds compared without a search
+constexpr int kFirst = 5;               // thresholds compared without a search (4: 732 us, 5: 720, 6: 731, 8: 772)
 constexpr uint32_t kBinnedCall = 8u;
 
 __device__ __forceinline__ uint32_t binned_call(int hyp, int m) {
@@ -234,13 +237,16 @@ __global__ void cls_weights_kernel(const double* __restrict__ s, const double* _
         w[i] = log1p(__ldg(s + i) / __ldg(b + i));
 }
 
-// One bin of a slice in shared memory.
-struct SliceBin {
-    unsigned long long thr[kFirst];   // its first thresholds, ~0 beyond the table
+// One bin of a slice in shared memory: the high words of its first thresholds (~0 beyond the
+// table) behind a zero, its part of the draw's first rounds, its weight.
+struct __align__(16) SliceBin {
+    uint32_t hi[1 + kFirst];
+    PhiloxRow row;
     double w;
-    int one;          // 1: one piece (the draw starts at thr), 0: the general path
     int first;        // min(kFirst, len): a word that passes this many needs the whole table
+    int one;          // 1: one piece, 0: the general path
 };
+static_assert(sizeof(SliceBin) % 16 == 0, "16-byte loads");
 
 // Slice sums of X: part[s * stride + c] = sum over the slice's bins of n_i w_i
 // for column c of the batch: toy toy0 + c of hypothesis 0 (c < n) or toy toy0 +
@@ -277,8 +283,10 @@ cls_slices_kernel(const BinTable* __restrict__ tab, const unsigned long long* __
         const BinTable t = tab[b];
         SliceBin r;
         const unsigned long long* F = t.off >= 0 ? T + t.off : L + (-1 - t.off);
+        r.hi[0] = 0u;
 #pragma unroll
-        for (int q = 0; q < kFirst; ++q) r.thr[q] = q < t.len ? __ldg(F + q) : ~0ull;
+        for (int q = 0; q < kFirst; ++q) r.hi[1 + q] = q < t.len ? (uint32_t)(__ldg(F + q) >> 32) : ~0u;
+        r.row = philox_row(keys, (uint32_t)(i0 + b), binned_call(hyp, 0));
         r.w = __ldg(w + i0 + b);
         r.one = t.M == 1;
         r.first = t.len < kFirst ? t.len : kFirst;
@@ -287,23 +295,24 @@ cls_slices_kernel(const BinTable* __restrict__ tab, const unsigned long long* __
     __syncthreads();
     if (c >= n) return;
     const uint32_t toy = (uint32_t)(toy0 + c);
+    const PhiloxCol col = philox_col(keys, (uint32_t)(i0 >> 32), toy);       // (a slice has one high word)
     double acc = 0.0;
 #pragma unroll 2
     for (int b = 0; b < nb; ++b) {
         const SliceBin& r = bins[b];
-        const uint64_t i = (uint64_t)(i0 + b);
         if (r.one) {
-            const U4 x = keyed(keys, (uint32_t)i, (uint32_t)(i >> 32), toy, binned_call(hyp, 0));
-            const unsigned long long word = word64(x.x, x.y);
+            const U4 x = keyed_from<2>(keys, U4{r.row.a ^ col.y, r.row.b, r.row.c ^ col.h, col.w});
+            // thresholds passed by the high word; a tie with the last one (2^-32) and a word past
+            // them all go by the whole table
             int k = 0;
 #pragma unroll
-            for (int q = 0; q < kFirst; ++q) k += word >= r.thr[q];
+            for (int q = 1; q <= kFirst; ++q) k += x.x >= r.hi[q];
             double m = num[k];
-            if (k >= r.first) {
+            if (k >= r.first || x.x == r.hi[k]) {
                 BinTable t = tab[b];
                 const unsigned long long* F = t.off >= 0 ? T : L;
                 if (t.off < 0) t.off = -1 - t.off;
-                k = bin_draw(t, F, word, r.first);
+                k = bin_draw(t, F, word64(x.x, x.y), 0);
                 m = (double)k;
             }
             if (k) acc = fma(m, r.w, acc);           // (an infinite w counts only where there are events)
@@ -311,7 +320,7 @@ cls_slices_kernel(const BinTable* __restrict__ tab, const unsigned long long* __
             BinTable t = tab[b];
             const unsigned long long* F = t.off >= 0 ? T : L;
             if (t.off < 0) t.off = -1 - t.off;
-            const int k = poisson_bin(t, F, i, toy, hyp, keys.k[0], keys.k[1]);
+            const int k = poisson_bin(t, F, (uint64_t)(i0 + b), toy, hyp, keys.k[0], keys.k[1]);
             if (k) acc = fma((double)k, r.w, acc);
         }
     }
@@ -322,6 +331,13 @@ cls_slices_kernel(const BinTable* __restrict__ tab, const unsigned long long* __
 __device__ __forceinline__ double sum_slices(const double* __restrict__ part, int64_t n_slices, int64_t stride) {
     double a[4] = {0.0, 0.0, 0.0, 0.0};
     int64_t s = 0;
+    for (; s + 16 <= n_slices; s += 16) {            // sixteen loads in flight
+        double x[16];
+#pragma unroll
+        for (int q = 0; q < 16; ++q) x[q] = __ldg(part + (s + q) * stride);
+#pragma unroll
+        for (int q = 0; q < 16; ++q) a[q & 3] += x[q];
+    }
     for (; s + 4 <= n_slices; s += 4) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) a[q] += __ldg(part + (s + q) * stride);

@@ -47,15 +47,39 @@ struct PhiloxKeys {
         }
     }
 };
-__device__ __forceinline__ U4 keyed(const PhiloxKeys& keys, uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3) {
-    U4 c{c0, c1, c2, c3};
+// Rounds R to 9.
+template <int R>
+__device__ __forceinline__ U4 keyed_from(const PhiloxKeys& keys, U4 c) {
 #pragma unroll
-    for (int r = 0; r < 10; ++r) {
+    for (int r = R; r < 10; ++r) {
         const unsigned long long p0 = (unsigned long long)kPhiloxM0 * c.x, p1 = (unsigned long long)kPhiloxM1 * c.z;
         c = U4{(uint32_t)(p1 >> 32) ^ c.y ^ keys.k[2 * r], (uint32_t)p1,
                (uint32_t)(p0 >> 32) ^ c.w ^ keys.k[2 * r + 1], (uint32_t)p0};
     }
     return c;
+}
+__device__ __forceinline__ U4 keyed(const PhiloxKeys& keys, uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3) {
+    return keyed_from<0>(keys, U4{c0, c1, c2, c3});
+}
+
+// The first two rounds apart, for draws of all pairs of some (c0, c3) with some (c1, c2):
+// after them the counter is (a ^ y, b, c ^ h, w), with (a, b, c) from c0 and c3 alone
+// and (y, h, w) from c1 and c2 alone; four of the twenty products less per draw.
+struct PhiloxRow {       // of (c0, c3)
+    uint32_t a, b, c;
+};
+struct PhiloxCol {       // of (c1, c2)
+    uint32_t y, h, w;
+};
+__device__ __forceinline__ PhiloxRow philox_row(const PhiloxKeys& keys, uint32_t c0, uint32_t c3) {
+    const unsigned long long p = (unsigned long long)kPhiloxM0 * c0;
+    const unsigned long long q = (unsigned long long)kPhiloxM1 * ((uint32_t)(p >> 32) ^ c3 ^ keys.k[1]);
+    return PhiloxRow{(uint32_t)(q >> 32) ^ keys.k[2], (uint32_t)q, (uint32_t)p ^ keys.k[3]};
+}
+__device__ __forceinline__ PhiloxCol philox_col(const PhiloxKeys& keys, uint32_t c1, uint32_t c2) {
+    const unsigned long long p = (unsigned long long)kPhiloxM1 * c2;
+    const unsigned long long q = (unsigned long long)kPhiloxM0 * ((uint32_t)(p >> 32) ^ c1 ^ keys.k[0]);
+    return PhiloxCol{(uint32_t)p, (uint32_t)(q >> 32), (uint32_t)q};
 }
 
 // u = ((((a << 32) | b) >> 11) + 1) 2^-53, in (0, 1] (exact).
