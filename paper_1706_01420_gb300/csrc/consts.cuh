@@ -399,9 +399,11 @@ __device__ inline FxExp coef_exp(const ModelDev& m, const Consts& c) {
     const double a = abs_bits(m.t_lo), b = abs_bits(m.t_hi);
     return fx_exp_setup(c.Gamma, c.mu, c.c_exp, a > b ? a : b);
 }
-__device__ inline void coef_flags(Consts* c, int sc) {
+__device__ inline void coef_flags(Consts* c, int sc, int scc) {
     c->k.hexp = 2 - (sc == 9999 ? 0 : sc);
     c->k.fixed = sc != 9999 && abs_below(c->cs, 1e300) && c->k.ex.ok;
+    c->k.cexp = 2 - (scc == 9999 ? 0 : scc);
+    c->k.cached = c->k.fixed && scc != 9999;
     // A typical r T = T2 / (A' T2 + cb) is near 1 / max(max|g| / 4, cb / 2): the scale follows
     // it, so that the sums' relative precision depends neither on the unit of time
     // nor on f_b, with 2^12 of headroom for events where A' is small.
@@ -409,7 +411,7 @@ __device__ inline void coef_flags(Consts* c, int sc) {
     const int eb = (int)((__double_as_longlong(c->cb) >> 52) & 0x7FF) - 1024;
     const int e = ea > eb ? ea : eb;
     c->k.rtop = 15 + (e < -900 ? 900 : -e);
-    c->k.pad[0] = c->k.pad[1] = c->k.pad[2] = 0;
+    c->k.pad = 0;
 }
 
 // The fixed-point parameters of the tagged and phi_s models' time functions: exponential i of
@@ -488,22 +490,27 @@ __device__ inline void compute_consts_thread(const ModelDev& m, const double* th
         for (int i = 0; i < kRowEntries; ++i) hd[i] = i == 0 ? 1.0 : 0.0;
         c->MO = 1.0;
     }
-    long long amax = 0;
+    long long amax = 0, cmax = 0;
     for (int k = 0; k < 10; ++k) {
         c->k.hq[k] = coef_hq(*c, k);
         c->k.hc[k] = coef_hc(*c, k);
     }
     for (int k = 0; k < 10; ++k) {
         const long long a = __double_as_longlong(abs_bits(coef_g(c->k.hq, k)));
+        const long long b = __double_as_longlong(abs_bits(c->k.hc[k]));
         amax = a > amax ? a : amax;
+        cmax = b > cmax ? b : cmax;
     }
-    const int sc = coef_scale(amax);
-    for (int k = 0; k < 10; ++k) c->k.ga[k] = coef_ga(coef_g(c->k.hq, k), sc);
+    const int sc = coef_scale(amax), scc = coef_scale(cmax);
+    for (int k = 0; k < 10; ++k) {
+        c->k.ga[k] = coef_ga(coef_g(c->k.hq, k), sc);
+        c->k.gc[k] = coef_ga(c->k.hc[k], scc);
+    }
     c->k.aq = 0.5 * c->cs;
     c->k.c2 = c->c_exp + fp64tab::kLn2Hi;
     c->k.tcut = coef_tcut(*c);
     c->k.ex = coef_exp(m, *c);
-    coef_flags(c, sc);
+    coef_flags(c, sc, scc);
 }
 
 // Exchange buffer of compute_consts_block.
@@ -515,7 +522,7 @@ struct ConstsBlockScratch {
     double rG;
     double F[2], dF[2][3];
     int ok;                        // theta in the domain
-    int sc;                        // scale of the fixed-point coefficients
+    int sc, scc;                   // scales of the fixed-point coefficients
     Consts c;                      // the record, copied out at the end
 };
 constexpr int kConstsBlock = 192;
@@ -634,16 +641,19 @@ __device__ inline void compute_consts_block(const ModelDev& m, const double* th,
         if (lane < 10) S->c.k.hq[lane] = coef_hq(S->c, lane);
         else if (lane < 20) S->c.k.hc[lane - 10] = coef_hc(S->c, lane - 10);
         __syncwarp();
-        const double g = lane < 10 ? coef_g(S->c.k.hq, lane) : 0.0;
+        // lanes 0-9: the coefficients of fx_basis's products; 16-25: of the cached basis
+        const double g = lane < 10 ? coef_g(S->c.k.hq, lane) : (lane >= 16 && lane < 26 ? S->c.k.hc[lane - 16] : 0.0);
         long long amax = __double_as_longlong(abs_bits(g));
-        for (int o = 16; o > 0; o >>= 1) {
+        for (int o = 8; o > 0; o >>= 1) {
             const long long v = __shfl_xor_sync(0xffffffffu, amax, o);
             amax = v > amax ? v : amax;
         }
         const int sc = coef_scale(amax);
         if (lane < 10) S->c.k.ga[lane] = coef_ga(g, sc);
+        else if (lane >= 16 && lane < 26) S->c.k.gc[lane - 16] = coef_ga(g, sc);
         if (lane == 10) S->c.k.aq = 0.5 * S->c.cs;
         if (lane == 0) S->sc = sc;
+        else if (lane == 16) S->scc = sc;
     } else if (w == 2) {
         if (lane == 0) S->c.k.ex = coef_exp(m, S->c);
         else if (lane == 1) S->c.k.tcut = coef_tcut(S->c);
@@ -658,7 +668,7 @@ __device__ inline void compute_consts_block(const ModelDev& m, const double* th,
         if (lane == 0) S->c.MO = four ? q + a4 : 1.0;
     }
     __syncthreads();
-    if (threadIdx.x == 0) coef_flags(&S->c, S->sc);
+    if (threadIdx.x == 0) coef_flags(&S->c, S->sc, S->scc);
     __syncthreads();
     const double* src = reinterpret_cast<const double*>(&S->c);
     double* dst = reinterpret_cast<double*>(c);

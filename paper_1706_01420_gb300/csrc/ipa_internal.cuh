@@ -67,8 +67,11 @@ struct NllCoef {
     int2 ga[10];
     int hexp;        // A' = (sum_k ga_k g_k in Q60) 2^(hexp - 2)
     int fixed;       // coefficients and exponential in range: the fixed-point path may be used
-    int rtop;        // scale of r T at unit weight in fixed point (tile_fast): below 2^(rtop - 3)
-    int pad[3];
+    int rtop;        // scale of r T at unit weight in fixed point (nll.cu): below 2^(rtop - 3)
+    // the same for the cached basis: A' = (sum_k gc_k f_k in Q60) 2^(cexp - 2)
+    int cexp, cached;
+    int pad;
+    int2 gc[10];
     FxExp ex;
 };
 

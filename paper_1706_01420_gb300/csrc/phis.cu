@@ -164,7 +164,6 @@ __device__ __forceinline__ void phis_coefficients(PhisWarp& pw, bool cached, int
         pw.D2s = 2.0 * c.D * c.s;
         pw.D2c = 2.0 * c.D * c.c;
     }
-    if (cached) return;
     ex = __reduce_max_sync(0xffffffffu, ex);
     const int up = 1020 - ex;                             // max|coefficient| 2^up in [1/8, 1/4)
     const bool ok = up >= -64 && up <= 900 && abs_below(c.c, 1.5) && abs_below(c.s, 1.5);
@@ -252,7 +251,7 @@ __device__ __forceinline__ void phis_event(const PhisWarp& pw, const MathTables*
     acc[kGt2] = fma(gq * tau, FV, acc[kGt2]);
 }
 
-// ---- the fixed-point form of an event's angular part (NLL + gradient, angles given) ----
+// ---- the fixed-point form of an event's angular part (NLL + gradient) ----
 // As in the 4D kernel's fast rows (nll.cu): the ten f'_k (Q62), F+, F-, FU, FV and what is linear
 // in them on the integer pipe, and the 14 angular sums as 64-bit integers: the factors r T+, r T-,
 // r U and r C are converted once per event at a scale that follows the segment's typical r T and
@@ -270,16 +269,23 @@ __device__ __noinline__ void phis_basis_wide(double ck, double cl, double phi, c
 }
 
 // One event: FP64 sums into acc (as phis_event), the angular sums (kE .. kMV + 3) into S.
-template <bool WEIGHTED>
+template <bool WEIGHTED, bool CACHED>
 __device__ __forceinline__ void phis_event_fast(const PhisWarp& pw, const MathTables* mt, const Cols& cols, int64_t e,
                                                 const TagSlow& sl, int top, double* acc, long long* S, double* prod,
                                                 int* esum, bool* bad) {
     const PhisConsts& c = pw.c;
     const double t = __ldg(cols.t + e), q = __ldg(cols.q + e);
-    const double ck = __ldg(cols.ck + e), cl = __ldg(cols.cl + e), phi = __ldg(cols.phi + e);
     const double w = WEIGHTED ? __ldg(cols.w + e) : 1.0;
     long long F[10];
-    {
+    if (CACHED) {
+#pragma unroll
+        for (int k = 0; k < 10; ++k) {
+            const double f = __ldg(cols.fk + k * cols.fk_stride + e);
+            *bad |= high_word(f) >= 0x3FFC0000;           // |f_k| < 1.75
+            F[k] = fx_signed(f, 1);
+        }
+    } else {
+        const double ck = __ldg(cols.ck + e), cl = __ldg(cols.cl + e), phi = __ldg(cols.phi + e);
         long long g[10];
         fx_basis(ck, cl, phi, mt, g);
         F[0] = g[0] - g[2];
@@ -292,12 +298,12 @@ __device__ __forceinline__ void phis_event_fast(const PhisWarp& pw, const MathTa
         F[7] = g[7];
         F[8] = g[8];
         F[9] = g[9];
-    }
-    if (!fx_angles_ok(ck, cl, phi)) {
-        long long x[10];                                 // (a copy, so that F itself stays in registers)
-        phis_basis_wide(ck, cl, phi, mt, x);
+        if (!fx_angles_ok(ck, cl, phi)) {
+            long long x[10];                             // (a copy, so that F itself stays in registers)
+            phis_basis_wide(ck, cl, phi, mt, x);
 #pragma unroll
-        for (int k = 0; k < 10; ++k) F[k] = x[k];
+            for (int k = 0; k < 10; ++k) F[k] = x[k];
+        }
     }
     const auto K = [](const int2& a) { return Fx{a.x, a.y}; };
     const long long fp = fx_mad(K(pw.fe[2]), fx(F[4]), fx_mad(K(pw.fe[1]), fx(F[1]), fx_mad(K(pw.fe[0]), fx(F[0]), 0)));
@@ -590,7 +596,7 @@ const auto slow_of = [&](int k) {
                 };
                 bool plain = true;
                 int top = pw.rtop;
-                if (GRAD && !CACHED && pw.fixed && ev1 - tbase >= kFewEvents) {
+                if (GRAD && pw.fixed && ev1 - tbase >= kFewEvents) {
                     if (WEIGHTED) {
                         // the exponent of the rows' largest |w| (0 where all weights are 1)
                         unsigned hi = 0;
@@ -612,7 +618,7 @@ const auto slow_of = [&](int k) {
 #pragma unroll 1
                     for (int k = 0; k < kSub; ++k) {
                         const int64_t e = tbase + lane + 32 * (i0 + k);
-                        if (e < ev1) phis_event_fast<WEIGHTED>(pw, &mt, cols, e, slow_of(k), top, acc, S, &prod, &esum, &bad);
+                        if (e < ev1) phis_event_fast<WEIGHTED, CACHED>(pw, &mt, cols, e, slow_of(k), top, acc, S, &prod, &esum, &bad);
                     }
                     plain = __any_sync(0xffffffffu, bad);
 #pragma unroll

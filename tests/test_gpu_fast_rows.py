@@ -181,3 +181,49 @@ def test_one_warp_or_a_team_per_tile(env, kind, weighted, redo):
         logl, terms = O.nll_grad_terms(mo, cols, th)
         assert abs(got[1][0] - f) <= 1e-14 * np.abs(logl).sum(), n
         assert np.all(np.abs(got[1][1:] - g) <= 5e-13 * np.abs(terms).sum(1)), n
+
+
+@pytest.mark.parametrize("weighted", [False, True])
+@pytest.mark.parametrize("kind", ["4d", "phis"])
+def test_cached_basis_rows(env, kind, weighted):
+    """The cached basis on the fixed-point path: one warp or a team per tile give the
+    same bits, the values are the oracle's (tolerance as above), and basis values
+    beyond the path's range (1.75) go by the plain loop, as they are."""
+    O, G, _ = env
+    import torch
+    from paper_1706_01420_gb300 import api
+    th = np.array({"4d": TH4, "phis": list(TH4) + [0.085, 17.77, 0.8, 0.3, 0.8, 0.0]}[kind])
+    m = getattr(api, "model_" + kind)(0.0, HI)
+    theta = torch.tensor(th, device="cuda")
+    mo = O.Model(kind, 0.0, HI)
+    for n in (63, 64, 545, 1537):
+        cols = {"4d": synth.events_4d, "phis": synth.events_phis}[kind](n, 79, weighted=weighted)
+        ev = G.to_dev(cols)
+        ev["fk"] = api.ipa_angular_basis(m, ev)
+        got = {}
+        try:
+            for warps in (1, 2):
+                api.ipa_launch_config_set(m, n, {"warps_per_block": warps, "warps_per_sm": 0, "tiles_per_take": 1},
+                                          cached=True)
+                got[warps] = api.ipa_nll_grad(m, ev, theta).cpu().numpy()
+        finally:
+            api.ipa_launch_config_set(m, n, {"warps_per_block": 1, "warps_per_sm": 0, "tiles_per_take": 1}, cached=True)
+        assert np.array_equal(got[1], got[2]), n
+        f, g = O.nll_grad(mo, cols, th)
+        logl, terms = O.nll_grad_terms(mo, cols, th)
+        assert abs(got[1][0] - f) <= 1e-14 * np.abs(logl).sum(), n
+        assert np.all(np.abs(got[1][1:] - g) <= 5e-13 * np.abs(terms).sum(1)), n
+        # without background P is proportional to the basis: scaling it by 8 shifts the NLL by
+        # -sum w ln 8 and leaves the gradient as it is
+        th0 = th.copy()
+        th0[3] = 0.0
+        t0 = torch.tensor(th0, device="cuda")
+        ref = api.ipa_nll_grad(m, ev, t0).cpu().numpy()
+        ev["fk"] = ev["fk"] * 8.0
+        big = api.ipa_nll_grad(m, ev, t0).cpu().numpy()
+        _, terms = O.nll_grad_terms(mo, cols, th0)
+        w = cols["w"] if weighted else np.ones(n)
+        labs = np.abs(O.nll_grad_terms(mo, cols, th0)[0]).sum() + np.abs(w).sum() * np.log(8.0)
+        assert abs(big[0] - (ref[0] - w.sum() * np.log(8.0))) <= 2e-14 * labs, n
+        keep = np.arange(len(th0)) != 3                   # (the derivative in f_b scales with the basis)
+        assert np.all(np.abs(big[1:] - ref[1:])[keep] <= 5e-13 * np.abs(terms).sum(1)[keep]), n
