@@ -61,28 +61,28 @@ WORKLOAD = "4D angular+time unbinned NLL+grad, 1e6 FP64 SoA events, 10 params"
 # FP64 operations of the fused 4D NLL+gradient kernel, counted from the formula
 # as nll.cu evaluates it on whole tiles (FMA = 2 flops; each FP64 function call
 # counts its cost in DFMA issue slots measured live by ipa_calibrate_fp64, times
-# 2 flops).  The angular basis (sin/cos, the ten products, the square root,
-# the amplitude sum A'), the Gaussian's exp, the ten angular adjoint sums S_k
-# (64-bit fixed point) and the lane's product of the P mantissas run on the
-# integer pipe and count no FP64 operation; only their arguments and results do:
-#   every event: tau, the exponent of 2E and 2E itself (the table-driven FP64
-#     exp, its measured slots), T2 = 2E - X (computed for every
-#     event, selected for the near-peak ones), P, 1/P (an FP32 seed and one
-#     FP64 Newton step: 2 FMA), sum r, r T2 (then fixed point), r A', u = r A'
-#     tau and the three sums u T2, r A' Gx, u Gx (Gx = 0 away from the peak);
+# 2 flops).  The decay exponential, the angular basis (sin/cos, the ten products, the
+# square root, the amplitude sum A'), the Gaussian's exp, erfcx, the ten angular
+# adjoint sums S_k (64-bit fixed point) and the weighted log run on the integer
+# pipe and count no FP64 operation; only what joins them does:
+#   every event: tau, T2 = 2E - X (computed for every event, selected for the
+#     near-peak ones), P, 1/P (an FP32 seed and one FP64 Newton step: 2 FMA),
+#     sum r, r T2 (then fixed point), r A', u = r A' tau and the three sums u T2,
+#     r A' Gx, u Gx (Gx = 0 away from the peak), and a quarter of the four sums'
+#     additions per four rows;
 #   unweighted: the lane's product of the P mantissas (one multiply);
 #     weighted: w log P, w / P and the product (by 1 or P);
 #   events near the resolution peak (t <= mu + Gamma sigma^2 + 6.25 sqrt2 sigma,
 #     packed 32 to a warp pass): tau, the Gaussian's exponent (tau^2 k_g), the
-#     erfcx argument ((Gs2 - tau) k_z), erfcx (FP64 polynomial) and g X;
+#     erfcx argument ((Gs2 - tau) k_z) and g X;
 #   once per lane and 512-event tile (16 events): the log of the product and
 #     its exponent term.
 # (Angles within 2^-17 of |cos| = 1, about 1.5e-5 of the events, take the FP64
 # basis instead; they are not counted.)
-OPS_EVENT_4D = {"fma": 7, "mul": 3, "add": 3, "exp_fast": 1}
+OPS_EVENT_4D = {"fma": 6, "mul": 3, "add": 4}
 OPS_UNWEIGHTED = {"mul": 1}
-OPS_WEIGHTED = {"fma": 1, "mul": 2, "log_fast": 1}
-OPS_NEAR_PEAK = {"mul": 4, "add": 2, "erfcx_poly": 1}
+OPS_WEIGHTED = {"fma": 1, "mul": 2}
+OPS_NEAR_PEAK = {"mul": 4, "add": 2}
 OPS_LANE_TILE = {"fma": 2, "log_fast": 1}
 
 
@@ -94,16 +94,16 @@ OPS_LIBRARY_4D = {"fma": 32, "mul": 30, "add": 6, "exp": 2, "erfc": 1, "log": 1,
 
 
 # The flavour-tagged model (IPA_MODEL_TAGGED1D, tagged.cu), counted the same way:
-#   every event: tau, three exponents (integer-pipe exp), the oscillation phase
-#     (its sine and cosine on the integer pipe), 2 gH, 2 gL, 2 g (complex),
-#     q qD and P, 1/P, and the 12 adjoint sums;
+#   every event: tau, 2 gH, 2 gL, 2 g (complex), q qD and P, 1/P, sum r and the six
+#     factors of the sums (the exponentials, the phase's sine and cosine, the
+#     sums and their products with tau run on the integer pipe);
 #   events with t <= tcut (mu + max(Gamma_H, Gamma_L, Gamma) sigma^2 +
 #     sqrt(39.1 + (Dm sigma)^2 / 2) sqrt2 sigma): the Gaussian's exponent, three
-#     erfc arguments, the Faddeeva function's division, Z and final
+#     erfc arguments, the Faddeeva function's reciprocal, Z and final
 #     combination, and the five products stored for the event (two erfcx and
-#     the Faddeeva function's 39 complex Horner steps run on the integer pipe).
-OPS_TAG_EVENT = {"fma": 17, "mul": 8, "add": 9}
-OPS_TAG_SLOW = {"fma": 8, "mul": 19, "add": 5, "rcp": 1}
+#     the Faddeeva function's recurrence run on the integer pipe).
+OPS_TAG_EVENT = {"fma": 7, "mul": 8, "add": 4.5}
+OPS_TAG_SLOW = {"fma": 12, "mul": 19, "add": 6}
 TH_TAG = np.array([0.66, 0.045, 0.0, 0.1, 0.085, 17.77, 0.8, 0.3])
 
 
@@ -192,12 +192,12 @@ COUNT_COMMON = ["tile_reduce.cuh", "fp64_math.cuh", "fp64_tables.cuh", "int_math
                 "ipa_internal.cuh"]
 COUNT_CAPTURES = {
     "nll_kernel<4D, grad>": ("counts_4d.csv", "bench.py --profile-case", 8_000_000,
-                             ["nll.cu", "angular.cuh"] + COUNT_COMMON),
+                             ["nll.cu", "angular.cuh", "team_tile.cuh"] + COUNT_COMMON),
     "phis_kernel<grad>": ("counts_phis.csv", "bench.py --profile-case-phis", 8_000_000,
                           ["phis.cu", "phis_consts.cuh", "angular.cuh", "tagged.cuh", "faddeeva.cuh", "consts.cuh",
-                           "philox.cuh"] + COUNT_COMMON),
+                           "philox.cuh", "team_tile.cuh"] + COUNT_COMMON),
     "tag_kernel<grad>": ("counts_tag.csv", "bench.py --profile-case-tagged", 8_000_000,
-                         ["tagged.cu", "tagged.cuh", "faddeeva.cuh", "consts.cuh"] + COUNT_COMMON),
+                         ["tagged.cu", "tagged.cuh", "faddeeva.cuh", "consts.cuh", "team_tile.cuh"] + COUNT_COMMON),
 }
 
 

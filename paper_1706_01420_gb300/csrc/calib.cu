@@ -21,9 +21,10 @@ template <int OP>
 __global__ void __launch_bounds__(kCalThreads)
 calib_kernel(const double* __restrict__ in, double* __restrict__ out, int iters,
              long long* __restrict__ cycles) {
-    __shared__ MathTables mt;
+    __shared__ FullTables mt;
     if (OP >= 7) {
         load_math_tables(&mt);
+    load_fp64_tables(&mt);
         __syncthreads();
     }
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -174,8 +175,9 @@ namespace {
 
 // The library's own FP64 functions, one element per thread.
 __global__ void math_eval_kernel(int fn, const double* __restrict__ x, double* __restrict__ y, int64_t n) {
-    __shared__ MathTables mt;
+    __shared__ FullTables mt;
     load_math_tables(&mt);
+    load_fp64_tables(&mt);
     __syncthreads();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const double v = x[i];

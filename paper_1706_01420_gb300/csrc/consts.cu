@@ -31,18 +31,18 @@ __global__ void __launch_bounds__(kConstsBlock) consts_block_kernel(ModelDev m, 
 // One thread per fit (many fits: throughput).
 __global__ void consts_thread_kernel(ModelDev m, const double* __restrict__ theta, int n_seg,
                                      Consts* __restrict__ out) {
-    __shared__ MathTables mt;
+    __shared__ FullTables mt;
     asm volatile("griddepcontrol.launch_dependents;");
-    cdetail::load_consts_tables(&mt);
+    load_fp64_tables(&mt);
     __syncthreads();
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s < n_seg) compute_consts_thread(m, theta + (size_t)s * m.n_par, &mt, out + s);
 }
 // The tagged model's record: one thread per segment.
 __global__ void tag_consts_kernel(ModelDev m, const double* __restrict__ theta, int n_seg, Consts* __restrict__ out) {
-    __shared__ MathTables mt;
+    __shared__ FullTables mt;
     asm volatile("griddepcontrol.launch_dependents;");
-    cdetail::load_consts_tables(&mt);
+    load_fp64_tables(&mt);
     __syncthreads();
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s < n_seg) tag_consts_thread(m, theta + (size_t)s * m.n_par, &mt, reinterpret_cast<TagConsts*>(out + s));
@@ -57,9 +57,9 @@ __global__ void __launch_bounds__(kTagConstsBlock) tag_consts_block_kernel(Model
 }
 // The phi_s model's record: one thread per segment.
 __global__ void phis_consts_kernel(ModelDev m, const double* __restrict__ theta, int n_seg, Consts* __restrict__ out) {
-    __shared__ MathTables mt;
+    __shared__ FullTables mt;
     asm volatile("griddepcontrol.launch_dependents;");
-    cdetail::load_consts_tables(&mt);
+    load_fp64_tables(&mt);
     __syncthreads();
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s < n_seg) phis_consts_thread(m, theta + (size_t)s * m.n_par, &mt, reinterpret_cast<PhisConsts*>(out + s));

@@ -199,7 +199,7 @@ __device__ inline double decay_exponent(const TimeScalars& s, double tau) { retu
 // erfcx(w) for w >= 0 and 2 - e^{-w^2} erfcx(-w) for w < 0.  For w < -6.25
 // the erfcx term is below 1e-18 of the term beside it (E for g, 1 for Phi)
 // and leaves the sum unchanged in double precision: 0 without evaluating it.
-__device__ inline double edge_erfcx(double w, const MathTables* t) {
+__device__ inline double edge_erfcx(double w, const FullTables* t) {
     return below_neg(w, -6.25) ? 0.0 : erfcx_fast(abs_bits(w), t);
 }
 
@@ -406,11 +406,11 @@ __device__ inline void coef_flags(Consts* c, int sc, int scc) {
     c->k.cached = c->k.fixed && scc != 9999;
     // A typical r T = T2 / (A' T2 + cb) is near 1 / max(max|g| / 4, cb / 2): the scale follows
     // it, so that the sums' relative precision depends neither on the unit of time
-    // nor on f_b, with 2^12 of headroom for events where A' is small.
+    // nor on f_b, with 2^10 of headroom for events where A' is small.
     const int ea = sc == 9999 ? -1023 : -sc - 3;
     const int eb = (int)((__double_as_longlong(c->cb) >> 52) & 0x7FF) - 1024;
     const int e = ea > eb ? ea : eb;
-    c->k.rtop = 15 + (e < -900 ? 900 : -e);
+    c->k.rtop = 13 + (e < -900 ? 900 : -e);
     c->k.pad = 0;
 }
 
@@ -425,25 +425,13 @@ __device__ inline FxExp fx_field(const ModelDev& m, double GH, double GL, double
     return fx_exp_setup(x, mu, 0.5 * (x - d) * (x + d) * sigma * sigma, tm);
 }
 
-// The tables of exp_fast, sincos_fast and erfcx_fast into shared memory
-// (block-cooperative; the caller syncs).
-__device__ inline void load_consts_tables(MathTables* t) {
-    using namespace fp64tab;
-    for (int i = threadIdx.x; i < 64; i += blockDim.x) {
-        t->exp2[i] = kExp2Tab[i];
-        t->sn[i] = kSinTab[i];
-        t->cs[i] = kCosTab[i];
-    }
-    for (int i = threadIdx.x; i < kErfcxPieces * kErfcxCoeffs; i += blockDim.x) t->ex[i] = kErfcxTab[i];
-}
-
 }  // namespace cdetail
 
 // One thread computes one Consts record: used when many fits are evaluated at
 // once (batched fits, the server), where lanes of a warp hold different fits
 // and every FP64 instruction does useful work in all of them.  mt holds the
-// tables of load_consts_tables.
-__device__ inline void compute_consts_thread(const ModelDev& m, const double* th, const MathTables* mt, Consts* c) {
+// tables of load_fp64_tables.
+__device__ inline void compute_consts_thread(const ModelDev& m, const double* th, const FullTables* mt, Consts* c) {
     using namespace cdetail;
     const bool four = m.kind == IPA_MODEL_ANGTIME4D;
     const bool ok = in_domain(th, four);
@@ -515,7 +503,7 @@ __device__ inline void compute_consts_thread(const ModelDev& m, const double* th
 
 // Exchange buffer of compute_consts_block.
 struct ConstsBlockScratch {
-    MathTables mt;
+    FullTables mt;
     double th[IPA_NPAR_4D];        // theta
     double f[32];                  // angular factors
     double X1[2], X2[2], gq[2], E[2];   // edge 0: t_hi, edge 1: t_lo
@@ -554,7 +542,7 @@ __device__ inline void compute_consts_block(const ModelDev& m, const double* th,
     // theta and the tables come from memory together; everything after the
     // barrier reads them from shared memory
     if (threadIdx.x < (four ? IPA_NPAR_4D : IPA_NPAR_1D)) S->th[threadIdx.x] = th[threadIdx.x];
-    load_consts_tables(&S->mt);
+    load_fp64_tables(&S->mt);
     __syncthreads();
     th = S->th;
 

@@ -31,40 +31,59 @@
 namespace ipa {
 
 struct MathTables {
-    double exp2[64];
     double linv[128];
     double ltab[128];
-    double sn[64];
-    double cs[64];
-    double ex[fp64tab::kErfcxPieces * fp64tab::kErfcxCoeffs];
-    long long exq[fp64tab::kErfcxPieces * fp64tab::kErfcxCoeffs];   // the same pieces in Q62 (int_math.cuh)
+    long long exq[fp64tab::kErfcxPieces * fp64tab::kErfcxCoeffs];   // erfcx's pieces in Q62
     long long sq[65], cq[65];   // sin, cos (j pi/32) in Q62 (int_math.cuh)
     long long eq[64];           // 2^(j/64) in Q62 (int_math.cuh)
     long long lq[128];          // -log(c_j) in Q56 (fast_fixed.cuh)
 };
 
+// With the tables of the FP64 exp_fast, sincos_fast and erfcx_fast, for the parameter
+// records.  The event kernels need those functions only for the rare event outside the
+// fixed-point ranges, where they read the tables from constant memory: 3 KB of shared
+// memory per block more left the 16 blocks of an SM too little L1 cache to hold the
+// columns between their two reads (events read in place over the host link: 1e6 events
+// 208 -> 224 us when the blocks had grown).
+struct FullTables : MathTables {
+    double exp2[64];
+    double sn[64];
+    double cs[64];
+    double ex[fp64tab::kErfcxPieces * fp64tab::kErfcxCoeffs];
+};
+__device__ __forceinline__ double exp2_entry(const MathTables*, int j) { return fp64tab::kExp2Tab[j]; }
+__device__ __forceinline__ double exp2_entry(const FullTables* t, int j) { return t->exp2[j]; }
+__device__ __forceinline__ double sin_entry(const MathTables*, int j) { return fp64tab::kSinTab[j]; }
+__device__ __forceinline__ double sin_entry(const FullTables* t, int j) { return t->sn[j]; }
+__device__ __forceinline__ double cos_entry(const MathTables*, int j) { return fp64tab::kCosTab[j]; }
+__device__ __forceinline__ double cos_entry(const FullTables* t, int j) { return t->cs[j]; }
+__device__ __forceinline__ const double* erfcx_piece(const MathTables*, int k) { return fp64tab::kErfcxTab + k * fp64tab::kErfcxCoeffs; }
+__device__ __forceinline__ const double* erfcx_piece(const FullTables* t, int k) { return t->ex + k * fp64tab::kErfcxCoeffs; }
+
 // Block-cooperative copy of the tables into shared memory (caller syncs).
 __device__ __forceinline__ void load_math_tables(MathTables* t) {
+    using namespace fp64tab;
+    for (int i = threadIdx.x; i < 128; i += blockDim.x) {
+        t->linv[i] = kLogInv[i];
+        t->ltab[i] = kLogTab[i];
+        t->lq[i] = kLogQ56[i];
+    }
+    for (int i = threadIdx.x; i < kErfcxPieces * kErfcxCoeffs; i += blockDim.x) t->exq[i] = kErfcxQ62[i];
+    for (int i = threadIdx.x; i < 65; i += blockDim.x) {
+        t->sq[i] = kSinQ62[i];
+        t->cq[i] = kCosQ62[i];
+    }
+    for (int i = threadIdx.x; i < 64; i += blockDim.x) t->eq[i] = kExp2Q62[i];
+}
+// The FP64 functions' tables alone.
+__device__ __forceinline__ void load_fp64_tables(FullTables* t) {
     using namespace fp64tab;
     for (int i = threadIdx.x; i < 64; i += blockDim.x) {
         t->exp2[i] = kExp2Tab[i];
         t->sn[i] = kSinTab[i];
         t->cs[i] = kCosTab[i];
     }
-    for (int i = threadIdx.x; i < 128; i += blockDim.x) {
-        t->linv[i] = kLogInv[i];
-        t->ltab[i] = kLogTab[i];
-        t->lq[i] = kLogQ56[i];
-    }
-    for (int i = threadIdx.x; i < kErfcxPieces * kErfcxCoeffs; i += blockDim.x) {
-        t->ex[i] = kErfcxTab[i];
-        t->exq[i] = kErfcxQ62[i];
-    }
-    for (int i = threadIdx.x; i < 65; i += blockDim.x) {
-        t->sq[i] = kSinQ62[i];
-        t->cq[i] = kCosQ62[i];
-    }
-    for (int i = threadIdx.x; i < 64; i += blockDim.x) t->eq[i] = kExp2Q62[i];
+    for (int i = threadIdx.x; i < kErfcxPieces * kErfcxCoeffs; i += blockDim.x) t->ex[i] = kErfcxTab[i];
 }
 
 // 1.5 * 2^52: adding it rounds a double of magnitude < 2^51 to an integer held
@@ -92,7 +111,8 @@ __device__ __forceinline__ double neg_bits(double x) {
     return __longlong_as_double(__double_as_longlong(x) ^ (long long)0x8000000000000000ull);
 }
 
-__device__ __forceinline__ double exp_fast(double x, const MathTables* t) {
+template <class T>
+__device__ __forceinline__ double exp_fast(double x, const T* t) {
     using namespace fp64tab;
     const double kd = fma(x, kInvLn2x64, kRoundShift);
     const int k = (int)(uint32_t)__double_as_longlong(kd);
@@ -104,7 +124,7 @@ __device__ __forceinline__ double exp_fast(double x, const MathTables* t) {
     q = fma(q, r, 0.5);
     q = fma(q, r, 1.0);
     const double p = r * q;                       // e^r - 1
-    const double tj = t->exp2[k & 63];
+    const double tj = exp2_entry(t, (int)(k & 63));
     const double v = fma(tj, p, tj);
     const long long scaled = __double_as_longlong(v) + (long long)(k >> 6) * (1ll << 52);
     if (above(x, 709.0)) return exp(x);           // overflow range: library exp
@@ -132,7 +152,8 @@ __device__ __forceinline__ double log_fast(double x, const MathTables* t) {
     return fma(ed, kLn2Hi, fma(ed, kLn2Lo, t->ltab[j] + l));
 }
 
-__device__ __forceinline__ void sincos_fast(double p, const MathTables* t, double* s, double* c) {
+template <class T>
+__device__ __forceinline__ void sincos_fast(double p, const T* t, double* s, double* c) {
     using namespace fp64tab;
     if (!abs_below(p, 1e5)) {
         sincos(p, s, c);
@@ -153,7 +174,7 @@ __device__ __forceinline__ void sincos_fast(double p, const MathTables* t, doubl
     cp = fma(cp, r2, -0.5);
     const double cr = fma(cp, r2, 1.0);           // cos r
     const int j = k & 63;                          // angle j pi/32 on the circle
-    const double sj = t->sn[j], cj = t->cs[j];
+    const double sj = sin_entry(t, j), cj = cos_entry(t, j);
     *s = fma(sj, cr, cj * sr);
     *c = fma(cj, cr, -(sj * sr));
 }
@@ -192,20 +213,22 @@ __device__ __forceinline__ double rcp_newton_nb(double x) {
 
 // Piecewise polynomial of erfcx on [0, 6.25]; outside, the piece index is
 // clamped and the value is meaningless (callers select it away).
-__device__ __forceinline__ double erfcx_poly(double x, const MathTables* t) {
+template <class T>
+__device__ __forceinline__ double erfcx_poly(double x, const T* t) {
     using namespace fp64tab;
     const double kd = fma(x, 2.0, kRoundShift);    // nearest piece centre k/2
     int k = (int)(uint32_t)__double_as_longlong(kd);
     k = k < 0 ? 0 : (k > kErfcxPieces - 1 ? kErfcxPieces - 1 : k);
     const double u = fma((double)k, -0.5, x);
-    const double* c = t->ex + k * kErfcxCoeffs;
+    const double* c = erfcx_piece(t, k);
     double v = c[kErfcxCoeffs - 1];
 #pragma unroll
     for (int i = kErfcxCoeffs - 2; i >= 0; --i) v = fma(v, u, c[i]);
     return v;
 }
 
-__device__ __forceinline__ double erfcx_fast(double x, const MathTables* t) {
+template <class T>
+__device__ __forceinline__ double erfcx_fast(double x, const T* t) {
     return above(x, 6.25) ? erfcx(x) : erfcx_poly(x, t);
 }
 

@@ -250,7 +250,7 @@ __device__ __forceinline__ void plain_rows(const Consts& c, const MathTables* mt
 // 64-bit integers and converts each sum to a double once per tile (sums of f'_k
 // are differences of sums of basis functions, taken in integers).  top follows
 // the segment's typical r T (NllCoef::rtop) and the largest weight of the tile,
-// so a unit is 2^-46 of a typical term; error of a sum: 0.41 units rms per
+// so a unit is 2^-48 of a typical term; error of a sum: 0.41 units rms per
 // event, of random sign, below that of the reciprocal r (6e-14 relative).  The 1D model: sums of r T and r Gx and their products
 // with tau, as in the tagged model (tagged.cu).  Lanes outside the ranges are fixed up in
 // FP64.  A tile in which some P lies outside the Newton reciprocal's range (zero,
@@ -297,11 +297,9 @@ __device__ __noinline__ double fix_exp(const Consts& c, const MathTables* mt, do
 }
 
 // (and the largest |f_k| of the cached basis, by its high word)
-template <bool WEIGHTED>
 __device__ __forceinline__ void load_cached_row(const Consts& c, const MathTables* mt, const Cols& cols, int64_t e,
                                                 RowIn& v, int* f_most) {
     const double t = __ldg(cols.t + e);
-    v.w = WEIGHTED ? __ldg(cols.w + e) : 1.0;
     v.tau = t - c.mu;
     long long A = 0;
 #pragma unroll
@@ -317,11 +315,9 @@ __device__ __forceinline__ void load_cached_row(const Consts& c, const MathTable
     if (!ok) v.E2 = fix_exp(c, mt, v.tau);
 }
 
-template <bool WEIGHTED>
 __device__ __forceinline__ void load_row(const Consts& c, const MathTables* mt, const Cols& cols, int64_t e, RowIn& v) {
     const double t = __ldg(cols.t + e);
     const double ck = __ldg(cols.ck + e), cl = __ldg(cols.cl + e), phi = __ldg(cols.phi + e);
-    v.w = WEIGHTED ? __ldg(cols.w + e) : 1.0;
     v.tau = t - c.mu;
     bool ok_exp = fx_in_range(t, c.k.ex.top);
     v.E2 = fx_exp(fx(fx_signed(t, c.k.ex.top)), c.k.ex, mt, &ok_exp);
@@ -347,19 +343,18 @@ struct Angtime {
     using Record = Consts;
     using Slow = double2;
     // FP64: sum r, sum r A' tau T2, sum r A' Gx, sum r A' tau Gx, sum w log P; integers: r T g_k
-    static constexpr int kSums = 5, kInts = 10, NA = n_acc(IPA_MODEL_ANGTIME4D, true);
+    static constexpr int kTopRange = 900, kSums = 5, kInts = 10, NA = n_acc(IPA_MODEL_ANGTIME4D, true);
     using Sums = FastSums<kSums, kInts>;
 
-    template <bool W>
-    static __device__ __forceinline__ bool usable(const Consts& c, const Cols& cols, int64_t tbase, int64_t ev1, int lane,
-                                                  FastScale* sc) {
-        sc->top = c.k.rtop + (W ? weight_exponent(cols, tbase, ev1, lane) : 0);
+    static __device__ __forceinline__ bool usable(const Consts& c, int64_t events, FastScale* sc) {
+        sc->top = c.k.rtop;
         sc->gtop = 0;
-        return (CACHED ? c.k.cached : c.k.fixed) && ev1 - tbase >= kFewEvents && sc->top >= -900 && sc->top <= 900;
+        return (CACHED ? c.k.cached : c.k.fixed) && events >= kFewEvents;
     }
     template <bool W>
     static __device__ __forceinline__ void quarter(const Consts& c, const MathTables* mt, const Cols& cols, int64_t tbase,
-                                                   int i0, int64_t ev1, double2* sbuf, int lane, FastScale sc, Sums& s) {
+                                                   int i0, int64_t ev1, double2* sbuf, double* wbuf, int lane,
+                                                   FastScale sc, Sums& s) {
         const unsigned below = (1u << lane) - 1u;
         SlowRows r;
         slow_rows(r, cols, c.k.tcut, tbase, i0, ev1, sbuf, lane,
@@ -371,8 +366,9 @@ struct Angtime {
                 const int j = r.at(q, below, lane);
                 const double2 ge = j >= 0 ? sbuf[j] : make_double2(0.0, 0.0);
                 RowIn v;
-                if (CACHED) load_cached_row<W>(c, mt, cols, e, v, &s.tau_most);
-                else load_row<W>(c, mt, cols, e, v);
+                if (CACHED) load_cached_row(c, mt, cols, e, v, &s.tau_most);
+                else load_row(c, mt, cols, e, v);
+                v.w = W ? wbuf[q * 32 + lane] : 1.0;
                 const long long gb = __double_as_longlong(ge.y);
                 const double T2 = gb >= 0 ? v.E2 - ge.x : ge.x;
                 const double Gx = __longlong_as_double(gb & 0x7FFFFFFFFFFFFFFFll);
@@ -431,21 +427,19 @@ struct Time1d {
     using Record = Consts;
     using Slow = double2;
     // FP64: sum r, sum w log P; integers: r T, r Gx, r tau T, r tau Gx (the factor A' = cs/2 outside)
-    static constexpr int kSums = 2, kInts = 4, NA = n_acc(IPA_MODEL_TIME1D, true);
+    static constexpr int kTopRange = 400, kSums = 2, kInts = 4, NA = n_acc(IPA_MODEL_TIME1D, true);
     using Sums = FastSums<kSums, kInts>;
 
-    template <bool W>
-    static __device__ __forceinline__ bool usable(const Consts& c, const Cols& cols, int64_t tbase, int64_t ev1, int lane,
-                                                  FastScale* sc) {
+    static __device__ __forceinline__ bool usable(const Consts& c, int64_t events, FastScale* sc) {
         // a typical r T is near 1 / max(cs / 2, cb / 2); the Gaussian's tau within 10 sigma (as in tagged.cu)
-        sc->top = 10 + 1023 - max(exponent_field(c.k.aq), exponent_field(c.cb) - 1) +
-                  (W ? weight_exponent(cols, tbase, ev1, lane) : 0);
+        sc->top = 10 + 1023 - max(exponent_field(c.k.aq), exponent_field(c.cb) - 1);
         sc->gtop = exponent_field(c.sigma) - 1023 + 5;
-        return c.k.ex.ok && sc->top >= -400 && sc->top <= 400 && sc->gtop >= -400 && sc->gtop <= 400;
+        return c.k.ex.ok && sc->gtop >= -400 && sc->gtop <= 400;
     }
     template <bool W>
     static __device__ __forceinline__ void quarter(const Consts& c, const MathTables* mt, const Cols& cols, int64_t tbase,
-                                                   int i0, int64_t ev1, double2* sbuf, int lane, FastScale sc, Sums& s) {
+                                                   int i0, int64_t ev1, double2* sbuf, double* wbuf, int lane,
+                                                   FastScale sc, Sums& s) {
         const unsigned below = (1u << lane) - 1u;
         SlowRows r;
         slow_rows(r, cols, c.k.tcut, tbase, i0, ev1, sbuf, lane,
@@ -456,7 +450,7 @@ struct Time1d {
             if (e < ev1) {
                 const int j = r.at(q, below, lane);
                 const double2 ge = j >= 0 ? sbuf[j] : make_double2(0.0, 0.0);
-                const double t = __ldg(cols.t + e), w = W ? __ldg(cols.w + e) : 1.0;
+                const double t = __ldg(cols.t + e), w = W ? wbuf[q * 32 + lane] : 1.0;
                 const double tau = t - c.mu;
                 bool ok = fx_in_range(t, c.k.ex.top);
                 double E2 = fx_exp(fx(fx_signed(t, c.k.ex.top)), c.k.ex, mt, &ok);
@@ -537,6 +531,8 @@ nll_kernel(Cols cols, int64_t n, const int64_t* __restrict__ seg_begin,
     const int n_wib = blockDim.x >> 5;
     double2* const sbuf = reinterpret_cast<double2*>(dyn_smem) + wib * (kSub * 32);
     Consts& wc = reinterpret_cast<Consts*>(dyn_smem + (size_t)n_wib * kSub * 32 * sizeof(double2))[wib];
+    double* const wbuf = reinterpret_cast<double*>(dyn_smem + (size_t)n_wib * (kSub * 32 * sizeof(double2) + sizeof(Consts))) +
+                         wib * (kSub * 32);      // with weights and gradient only
 
     load_math_tables(&mt);
     __syncthreads();
@@ -594,7 +590,7 @@ nll_kernel(Cols cols, int64_t n, const int64_t* __restrict__ seg_begin,
             // (about a fifth of them) need the Gaussian and erfcx: slow_rows.
             const int64_t tbase = ev0 + (tile - t0) * kTile;
             if constexpr (GRAD)
-                solo_tile<Model<KIND, CACHED>, WEIGHTED>(wc, &mt, cols, tbase, ev1, sbuf, lane, acc, &prod, &esum);
+                solo_tile<Model<KIND, CACHED>, WEIGHTED>(wc, &mt, cols, tbase, ev1, sbuf, wbuf, lane, acc, &prod, &esum);
             else
                 plain_rows<KIND, GRAD, CACHED, WEIGHTED>(wc, &mt, cols, 0, tile_rows(tbase, ev1), tbase, ev1, sbuf, lane,
                                                          acc, &prod, &esum);
@@ -660,7 +656,7 @@ ipa_status launch_t(const Cols& cols, int64_t n, const int64_t* seg_begin, const
     }
     const int W = cfg.warps_per_block >= 1 && cfg.warps_per_block <= kMaxWarps ? cfg.warps_per_block : 1;
     const int K = cfg.tiles_per_take >= 1 ? cfg.tiles_per_take : 1;
-    const size_t smem = (size_t)W * (sizeof(Consts) + kSub * 32 * sizeof(double2));
+    const size_t smem = (size_t)W * (sizeof(Consts) + kSub * 32 * (sizeof(double2) + (GRAD && WEIGHTED ? sizeof(double) : 0)));
     // resident blocks per SM for each block size (cached per device and variant)
     static int occ[64][kMaxWarps + 1] = {};
     int dev = 0;

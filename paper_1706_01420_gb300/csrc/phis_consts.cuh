@@ -64,7 +64,7 @@ __device__ inline cdetail::TimeScalars rate_scalars(const double* th, int r) {
 
 // Piece k of the real edges: erfcx at the argument of g at edge k (k < 4) or
 // of Phi at edge k - 4 (k = 4, 5); rs = 1 / sigma.
-__device__ inline double edge_X(const ModelDev& m, const double* th, int k, double rs, const MathTables* mt) {
+__device__ inline double edge_X(const ModelDev& m, const double* th, int k, double rs, const FullTables* mt) {
     using namespace cdetail;
     const double x = edge_tau(m, th[IPA_MU], k & 1) * rs;
     const double z = edge_z(rate_scalars(th, (k >> 1) & 1), x);
@@ -73,7 +73,7 @@ __device__ inline double edge_X(const ModelDev& m, const double* th, int k, doub
 
 // Piece k of the real edges: E = exp(-Gamma_r tau + Gamma_r^2 sigma^2 / 2) at
 // edge k (k < 4) or the Gaussian factor exp(-x^2/2) at edge k - 4 (k = 4, 5).
-__device__ inline double edge_exp(const ModelDev& m, const double* th, int k, double rs, const MathTables* mt) {
+__device__ inline double edge_exp(const ModelDev& m, const double* th, int k, double rs, const FullTables* mt) {
     using namespace cdetail;
     const double tau = edge_tau(m, th[IPA_MU], k & 1);
     const double x = tau * rs;
@@ -247,7 +247,7 @@ __device__ inline CEdgeArg cedge_arg(const ModelDev& m, const double* th, int e,
 }
 
 // (Re w, Im w, gx): w at x + i y (y >= 0) or at -x - i y (y < 0).
-__device__ inline void cedge_fad(const ModelDev& m, const double* th, int e, double rs, const MathTables* mt,
+__device__ inline void cedge_fad(const ModelDev& m, const double* th, int e, double rs, const FullTables* mt,
                                  double* out) {
     const CEdgeArg a = cedge_arg(m, th, e, rs);
     const bool up = a.y >= 0.0;
@@ -256,7 +256,7 @@ __device__ inline void cedge_fad(const ModelDev& m, const double* th, int e, dou
 }
 
 // (erfcx for Phi, e^{Re(-z tau + z^2 s^2 / 2)}, sin and cos of its imaginary part).
-__device__ inline void cedge_exp(const ModelDev& m, const double* th, int e, double rs, const MathTables* mt,
+__device__ inline void cedge_exp(const ModelDev& m, const double* th, int e, double rs, const FullTables* mt,
                                  double* out) {
     using namespace cdetail;
     const CEdgeArg a = cedge_arg(m, th, e, rs);
@@ -377,7 +377,7 @@ __device__ inline double norm_dN(int j, const double* th, const double* F, const
 }  // namespace pdetail
 
 // One thread computes the record (many segments: lanes hold different fits).
-__device__ inline void phis_consts_thread(const ModelDev& m, const double* th, const MathTables* mt, PhisConsts* c) {
+__device__ inline void phis_consts_thread(const ModelDev& m, const double* th, const FullTables* mt, PhisConsts* c) {
     using namespace pdetail;
     double rc[4], X[6], Ex[6], r[6], sw[7], cw[7], F[4], dF[4][3], ec[16];
     for (int i = 0; i < 4; ++i) rc[i] = cdetail::recip(recip_arg(m, th, i));
@@ -417,7 +417,7 @@ __device__ inline void phis_consts_thread(const ModelDev& m, const double* th, c
 
 // Exchange buffer of phis_consts_block.
 struct PhisBlockScratch {
-    MathTables mt;
+    FullTables mt;
     double th[IPA_NPAR_PHIS];
     double rc[4];                 // 1/sigma, 1/Gamma_L, 1/Gamma_H, 1/V
     double X[6], Ex[6];           // real-edge pieces (edge_X, edge_exp)
@@ -447,7 +447,7 @@ __device__ inline void phis_consts_block(const ModelDev& m, const double* th, Ph
     using namespace pdetail;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x < IPA_NPAR_PHIS) S->th[threadIdx.x] = th[threadIdx.x];
-    cdetail::load_consts_tables(&S->mt);
+    load_fp64_tables(&S->mt);
     __syncthreads();
     th = S->th;
 

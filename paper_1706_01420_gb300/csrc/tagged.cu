@@ -157,21 +157,20 @@ struct Tagged {
     using Record = TagConsts;
     using Slow = TagSlow;
     // FP64: sum r, sum w log P; integers: the six sums in the order above, then times tau (not r q Gx)
-    static constexpr int kSums = 2, kInts = 11, NA = n_acc(IPA_MODEL_TAGGED1D, true);
+    static constexpr int kTopRange = 400, kSums = 2, kInts = 11, NA = n_acc(IPA_MODEL_TAGGED1D, true);
     using Sums = FastSums<kSums, kInts>;
 
-    template <bool W>
-    static __device__ __forceinline__ bool usable(const TagConsts& c, const Cols& cols, int64_t tbase, int64_t ev1,
-                                                  int lane, FastScale* sc) {
+    static __device__ __forceinline__ bool usable(const TagConsts& c, int64_t events, FastScale* sc) {
         const int e1 = max(exponent_field(c.qH), exponent_field(c.qL)), e2 = exponent_field(c.cb) - 1;
-        sc->top = 10 + 1023 - max(e1, e2) + (W ? weight_exponent(cols, tbase, ev1, lane) : 0);
+        sc->top = 10 + 1023 - max(e1, e2);
         // r Gx counts (its integer is not 0) only for |tau| < 10 sigma, so tau's scale there follows sigma
         sc->gtop = exponent_field(c.sigma) - 1023 + 5;
-        return c.fx_ok && sc->top >= -400 && sc->top <= 400 && sc->gtop >= -400 && sc->gtop <= 400;
+        return c.fx_ok && sc->gtop >= -400 && sc->gtop <= 400;
     }
     template <bool W>
     static __device__ __forceinline__ void quarter(const TagConsts& c, const MathTables* mt, const Cols& cols, int64_t tbase,
-                                                   int i0, int64_t ev1, TagSlow* sbuf, int lane, FastScale sc, Sums& s) {
+                                                   int i0, int64_t ev1, TagSlow* sbuf, double* wbuf, int lane,
+                                                   FastScale sc, Sums& s) {
         const unsigned below = (1u << lane) - 1u;
         SlowRows r;
         slow_rows(r, cols, c.tcut, tbase, i0, ev1, sbuf, lane,
@@ -183,7 +182,7 @@ struct Tagged {
                 const int j = r.at(k, below, lane);
                 TagSlow sl = {0.0, 0.0, 0.0, 0.0, 0.0};
                 if (j >= 0) sl = sbuf[j];
-                event<W>(c, mt, __ldg(cols.t + e), __ldg(cols.q + e), W ? __ldg(cols.w + e) : 1.0, sl, sc, s);
+                event<W>(c, mt, __ldg(cols.t + e), __ldg(cols.q + e), W ? wbuf[k * 32 + lane] : 1.0, sl, sc, s);
             }
         }
         __syncwarp();
@@ -258,6 +257,8 @@ tag_kernel(Cols cols, int64_t n, const int64_t* __restrict__ seg_begin, const in
     const int n_wib = blockDim.x >> 5;
     TagSlow* const sbuf = reinterpret_cast<TagSlow*>(dyn_smem) + wib * (kSub * 32);
     TagConsts& tc = reinterpret_cast<TagConsts*>(dyn_smem + (size_t)n_wib * kSub * 32 * sizeof(TagSlow))[wib];
+    double* const wbuf = reinterpret_cast<double*>(dyn_smem + (size_t)n_wib * (kSub * 32 * sizeof(TagSlow) + sizeof(TagConsts))) +
+                         wib * (kSub * 32);      // with weights and gradient only
 
     load_math_tables(&mt);
     __syncthreads();
@@ -308,7 +309,7 @@ tag_kernel(Cols cols, int64_t n, const int64_t* __restrict__ seg_begin, const in
             int esum = 0;
             const int64_t tbase = ev0 + (tile - t0) * kTile;
             if constexpr (GRAD)
-                solo_tile<Tagged, WEIGHTED>(tc, &mt, cols, tbase, ev1, sbuf, lane, acc, &prod, &esum);
+                solo_tile<Tagged, WEIGHTED>(tc, &mt, cols, tbase, ev1, sbuf, wbuf, lane, acc, &prod, &esum);
             else
                 tag_rows<GRAD, WEIGHTED>(tc, &mt, cols, 0, tile_rows(tbase, ev1), tbase, ev1, sbuf, lane, acc, &prod,
                                          &esum);
@@ -336,7 +337,7 @@ ipa_status launch_tag_t(const Cols& cols, int64_t n, const int64_t* seg_begin, c
     }
     const int W = cfg.warps_per_block >= 1 && cfg.warps_per_block <= kMaxWarps ? cfg.warps_per_block : 1;
     const int K = cfg.tiles_per_take >= 1 ? cfg.tiles_per_take : 1;
-    const size_t smem = (size_t)W * (sizeof(TagConsts) + kSub * 32 * sizeof(TagSlow));
+    const size_t smem = (size_t)W * (sizeof(TagConsts) + kSub * 32 * (sizeof(TagSlow) + (GRAD && WEIGHTED ? sizeof(double) : 0)));
     auto kern = tag_kernel<GRAD, WEIGHTED>;
     // dynamic shared memory above the default limit (8 warps: 44 KB besides
     // the static tables) needs the opt-in, once per device
@@ -346,7 +347,7 @@ ipa_status launch_tag_t(const Cols& cols, int64_t n, const int64_t* seg_begin, c
     cudaGetDevice(&dev);
     if (!attr[dev & 63]) {
         ipa_status q = cuda_fail(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                      (int)(kMaxWarps * (sizeof(TagConsts) + kSub * 32 * sizeof(TagSlow)))),
+                                                      (int)(kMaxWarps * (sizeof(TagConsts) + kSub * 32 * (sizeof(TagSlow) + (GRAD && WEIGHTED ? sizeof(double) : 0))))),
                                  "tagged kernel attribute");
         if (q != IPA_OK) return q;
         attr[dev & 63] = true;

@@ -95,7 +95,7 @@ __device__ inline cdetail::TimeScalars rate_scalars(const double* th, int r) {
 
 // Piece k of the edges: erfcx at the argument of g at edge k (k < 4) or of
 // Phi at edge k - 4 (k = 4, 5); rs = 1 / sigma.
-__device__ inline double edge_X(const ModelDev& m, const double* th, int k, double rs, const MathTables* mt) {
+__device__ inline double edge_X(const ModelDev& m, const double* th, int k, double rs, const FullTables* mt) {
     using namespace cdetail;
     const double x = edge_tau(m, th[IPA_MU], k & 1) * rs;
     const double z = edge_z(rate_scalars(th, (k >> 1) & 1), x);
@@ -104,7 +104,7 @@ __device__ inline double edge_X(const ModelDev& m, const double* th, int k, doub
 
 // Piece k of the edges: E = exp(-Gamma_r tau + Gamma_r^2 sigma^2 / 2) at edge
 // k (k < 4) or the Gaussian factor exp(-x^2/2) at edge k - 4 (k = 4, 5).
-__device__ inline double edge_exp(const ModelDev& m, const double* th, int k, double rs, const MathTables* mt) {
+__device__ inline double edge_exp(const ModelDev& m, const double* th, int k, double rs, const FullTables* mt) {
     using namespace cdetail;
     const double tau = edge_tau(m, th[IPA_MU], k & 1);
     const double x = tau * rs;
@@ -235,7 +235,7 @@ __device__ inline void norm_fields(const double* th, double N, double inv_N, dou
 }  // namespace tdetail
 
 // One thread computes the record (many segments: lanes hold different fits).
-__device__ inline void tag_consts_thread(const ModelDev& m, const double* th, const MathTables* mt, TagConsts* c) {
+__device__ inline void tag_consts_thread(const ModelDev& m, const double* th, const FullTables* mt, TagConsts* c) {
     using namespace tdetail;
     double r[4], X[6], Ex[6], M[3], F[4], dF[4][3];
     for (int i = 0; i < 4; ++i) r[i] = cdetail::recip(recip_arg(m, th, i));
@@ -261,7 +261,7 @@ __device__ inline void tag_consts_thread(const ModelDev& m, const double* th, co
 
 // Exchange buffer of tag_consts_block.
 struct TagBlockScratch {
-    MathTables mt;
+    FullTables mt;
     double th[IPA_NPAR_TAGGED];
     double r[4];                  // 1/sigma, 1/Gamma_H, 1/Gamma_L, 1/(2 (t_hi - t_lo))
     double X[6], Ex[6];           // edge pieces (edge_X, edge_exp)
@@ -287,7 +287,7 @@ __device__ inline void tag_consts_block(const ModelDev& m, const double* th, Tag
     using namespace tdetail;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x < IPA_NPAR_TAGGED) S->th[threadIdx.x] = th[threadIdx.x];
-    cdetail::load_consts_tables(&S->mt);
+    load_fp64_tables(&S->mt);
     __syncthreads();
     th = S->th;
 

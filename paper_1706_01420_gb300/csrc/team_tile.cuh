@@ -13,8 +13,9 @@
 //
 // A model is a struct M with
 //   Record, Slow (a near-peak event's values), kSums: FP64 sums, kInts: integer sums, NA;
-//   usable<W>(c, cols, tbase, ev1, lane, &sc)   the scales of the tile, false: plain loop;
-//   quarter<W>(c, mt, cols, tbase, i0, ev1, sbuf, lane, sc, s);
+//   usable(c, events, &sc)                      the scales at unit weight, false: plain loop;
+//   kTopRange                                   |sc.top| beyond it: plain loop;
+//   quarter<W>(c, mt, cols, tbase, i0, ev1, sbuf, wbuf, lane, sc, s);   (wbuf: the lane's weights)
 //   bad(c, sc, s)                               a value left its range;
 //   accumulators(c, sc, s, acc);
 //   plain<W>(c, mt, cols, i0, i1, tbase, ev1, sbuf, lane, acc, &prod, &esum);
@@ -32,7 +33,7 @@ constexpr int kPerLane = kTile / 32;                 // events per lane per tile
 constexpr int kTeam = kPerLane / kSub;               // warps that share a tile
 static_assert(kSub == 4 && kPerLane % kSub == 0, "a quarter keeps four ballot masks");
 
-// The angular sums' unit is 2^-46 of a typical term, which a handful of events with small
+// The angular sums' unit is 2^-48 of a typical term, which a handful of events with small
 // angular products would show: a tile of fewer events takes the plain loop.
 constexpr int kFewEvents = 64;
 
@@ -90,15 +91,39 @@ __device__ __forceinline__ void add_log(double P, double w, const MathTables* mt
     }
 }
 
-// The exponent of the largest |w| of a tile (0 where all weights are 1, as without weights).
-__device__ __forceinline__ int weight_exponent(const Cols& cols, int64_t tbase, int64_t ev1, int lane) {
+// The exponent of the largest |w| of a quarter (0 where all weights are 1, as without
+// weights), or kNoWeight where all are zero.  The lane keeps its weights in wbuf for the
+// quarter: a second read of the column would go over the host link again where it lies in
+// host memory (8e6 weighted 4D events there: read twice per tile 2.14 ms, twice per
+// quarter 1.95, once 1.74).
+constexpr int kNoWeight = -5000;
+__device__ __forceinline__ int weight_exponent(const Cols& cols, int64_t tbase, int i0, int64_t ev1, double* wbuf,
+                                               int lane) {
     int hi = 0;
-#pragma unroll 4
-    for (int i = 0; i < kPerLane; ++i) {
-        const int64_t e = tbase + lane + 32 * i;
-        hi = max(hi, high_word(e < ev1 ? __ldg(cols.w + e) : 0.0));
+#pragma unroll
+    for (int i = 0; i < kSub; ++i) {
+        const int64_t e = tbase + lane + 32 * (i0 + i);
+        const double w = e < ev1 ? __ldg(cols.w + e) : 0.0;
+        wbuf[i * 32 + lane] = w;
+        hi = max(hi, high_word(w));
     }
-    return (int)(__reduce_max_sync(0xffffffffu, (unsigned)hi) >> 20) - 1023;
+    const int ex = (int)(__reduce_max_sync(0xffffffffu, (unsigned)hi) >> 20);
+    return ex ? ex - 1023 : kNoWeight;
+}
+
+// A weighted quarter's scale follows the largest |w| of its tile up to it (run); the sums
+// of the quarters before, at a lower scale, are shifted to it.
+template <int NF, int NG>
+__device__ __forceinline__ void raise_scale(FastSums<NF, NG>& s, int run, int next) {
+    if (run == kNoWeight || next <= run) return;
+    const int d = next - run > 63 ? 63 : next - run;
+#pragma unroll
+    for (int i = 0; i < NG; ++i) s.g[i] >>= d;
+}
+template <class M>
+__device__ __forceinline__ bool scale_to(FastScale* sc, int base, int run) {
+    sc->top = base + (run == kNoWeight ? 0 : run);
+    return sc->top >= -M::kTopRange && sc->top <= M::kTopRange;
 }
 
 // Rows of a tile with events below ev1, up to a whole quarter.
@@ -169,19 +194,32 @@ __device__ __noinline__ void plain_quarters(const typename M::Record& c, const M
 // A whole tile by one warp: acc, prod and esum of the lane.
 template <class M, bool W>
 __device__ __forceinline__ void solo_tile(const typename M::Record& c, const MathTables* mt, const Cols& cols,
-                                          int64_t tbase, int64_t ev1, typename M::Slow* sbuf, int lane, double* acc,
-                                          double* prod, int* esum) {
+                                          int64_t tbase, int64_t ev1, typename M::Slow* sbuf, double* wbuf, int lane,
+                                          double* acc, double* prod, int* esum) {
     FastScale sc;
-    bool plain = !M::template usable<W>(c, cols, tbase, ev1, lane, &sc);
+    bool plain = !M::usable(c, ev1 - tbase, &sc);
     if (!plain) {
+        const int base = sc.top;
+        int run = W ? kNoWeight : 0;
+        plain = !scale_to<M>(&sc, base, run);
         FastSums<M::kSums, M::kInts> s;
         clear(s);
         double tot[M::kSums], tprod = 1.0;
 #pragma unroll
         for (int i = 0; i < M::kSums; ++i) tot[i] = 0.0;
 #pragma unroll 1
-        for (int i0 = 0; i0 < kPerLane && tbase + 32 * i0 < ev1; i0 += kSub) {
-            M::template quarter<W>(c, mt, cols, tbase, i0, ev1, sbuf, lane, sc, s);
+        for (int i0 = 0; !plain && i0 < kPerLane && tbase + 32 * i0 < ev1; i0 += kSub) {
+            if (W) {
+                const int next = max(run, weight_exponent(cols, tbase, i0, ev1, wbuf, lane));
+                raise_scale(s, run, next);
+                run = next;
+                if (!scale_to<M>(&sc, base, run)) {
+                    plain = true;
+                    break;
+                }
+            }
+            M::template quarter<W>(c, mt, cols, tbase, i0, ev1, sbuf, wbuf, lane, sc, s);
+            if (W) plain = __any_sync(0xffffffffu, M::bad(c, sc, s));
 #pragma unroll
             for (int i = 0; i < M::kSums; ++i) {
                 tot[i] += s.f[i];
@@ -190,7 +228,7 @@ __device__ __forceinline__ void solo_tile(const typename M::Record& c, const Mat
             tprod *= s.prod;
             s.prod = 1.0;
         }
-        plain = __any_sync(0xffffffffu, M::bad(c, sc, s));
+        if (!W) plain = __any_sync(0xffffffffu, M::bad(c, sc, s));
 #pragma unroll
         for (int i = 0; i < M::kSums; ++i) s.f[i] = tot[i];
         M::accumulators(c, sc, s, acc);
@@ -212,10 +250,10 @@ template <class M>
 constexpr int team_words() {
     return (M::kSums + M::kInts > M::NA ? M::kSums + M::kInts : M::NA) + 2;
 }
-template <class M>
+template <class M, bool W>
 constexpr size_t team_smem() {
     return sizeof(double) * 2 * kTeam * team_words<M>() * 32 + sizeof(typename M::Slow) * kTeam * kSub * 32 +
-           sizeof(typename M::Record);
+           sizeof(typename M::Record) + (W ? sizeof(double) * kTeam * kSub * 32 : 0);
 }
 
 // One tile per block and take, a quarter per warp.  The next take is fetched while a tile is
@@ -238,6 +276,8 @@ team_kernel(Cols cols, int64_t n, const int64_t* __restrict__ seg_begin, const i
         reinterpret_cast<typename M::Slow*>(xbuf + 2 * kTeam * kWords * 32) + wib * (kSub * 32);
     typename M::Record& c = *reinterpret_cast<typename M::Record*>(
         reinterpret_cast<typename M::Slow*>(xbuf + 2 * kTeam * kWords * 32) + kTeam * kSub * 32);
+
+    double* const wbuf = reinterpret_cast<double*>(&c + 1) + wib * (kSub * 32);
 
     load_math_tables(&mt);
     // a programmatic dependent of the constants kernel: wait for its results
@@ -281,12 +321,19 @@ team_kernel(Cols cols, int64_t n, const int64_t* __restrict__ seg_begin, const i
         double* const own = x + wib * kWords * 32;
         const int i0 = wib * kSub;
         FastScale sc;
-        bool plain = !M::template usable<W>(c, cols, tbase, ev1, lane, &sc);
+        bool plain = !M::usable(c, ev1 - tbase, &sc);
+        const int base = sc.top;
+        int run = 0;
+        if (W) {
+            run = kNoWeight;
+            for (int j = 0; j <= i0; j += kSub) run = max(run, weight_exponent(cols, tbase, j, ev1, wbuf, lane));
+        }
+        plain = !scale_to<M>(&sc, base, run) || plain;
         {
             FastSums<M::kSums, M::kInts> s;
             clear(s);
             if (!plain && tbase + 32 * i0 < ev1) {
-                M::template quarter<W>(c, &mt, cols, tbase, i0, ev1, sbuf, lane, sc, s);
+                M::template quarter<W>(c, &mt, cols, tbase, i0, ev1, sbuf, wbuf, lane, sc, s);
                 plain = M::bad(c, sc, s);
             }
 #pragma unroll
@@ -294,7 +341,7 @@ team_kernel(Cols cols, int64_t n, const int64_t* __restrict__ seg_begin, const i
 #pragma unroll
             for (int i = 0; i < M::kInts; ++i) own[(M::kSums + i) * 32] = __longlong_as_double(s.g[i]);
             own[(kWords - 2) * 32] = s.prod;
-            own[(kWords - 1) * 32] = __longlong_as_double((long long)(unsigned)s.esum);
+            own[(kWords - 1) * 32] = __longlong_as_double((long long)run << 32 | (unsigned)s.esum);
         }
         if (threadIdx.x == 32 * ((turn + 2) & (kTeam - 1))) s_take[(turn + 1) & 1] = (int64_t)atomicAdd(work, 1u);
         plain = __syncthreads_or(plain);
@@ -317,13 +364,19 @@ team_kernel(Cols cols, int64_t n, const int64_t* __restrict__ seg_begin, const i
 #pragma unroll
             for (int w = 0; w < kTeam; ++w) {
                 const double* y = x + w * kWords * 32;
+                const long long k = __double_as_longlong(y[(kWords - 1) * 32]);
+                if (W) {
+                    if (w) raise_scale(s, run, (int)(k >> 32));
+                    run = (int)(k >> 32);
+                }
+                esum += (int)k;
 #pragma unroll
                 for (int i = 0; i < M::kSums; ++i) s.f[i] += y[i * 32];
 #pragma unroll
                 for (int i = 0; i < M::kInts; ++i) s.g[i] += __double_as_longlong(y[(M::kSums + i) * 32]);
                 prod *= y[(kWords - 2) * 32];
-                esum += (int)__double_as_longlong(y[(kWords - 1) * 32]);
             }
+            scale_to<M>(&sc, base, run);
             M::accumulators(c, sc, s, acc);
         } else {
 #pragma unroll
@@ -363,7 +416,7 @@ ipa_status launch_team(const Cols& cols, int64_t n, const int64_t* seg_begin, co
                        const int64_t* seg_tiles, int n_seg, const Consts* consts, Scratch* sc, double* out, int n_par,
                        int64_t tiles, cudaStream_t st) {
     auto kern = team_kernel<M, W>;
-    constexpr size_t smem = team_smem<M>();
+    constexpr size_t smem = team_smem<M, W>();
     static int occ[64] = {};                         // resident blocks per SM, per device
     int dev = 0;
     cudaGetDevice(&dev);

@@ -12,7 +12,7 @@ tile) and their hand-over to the plain loop, against the oracle:
 
 Tolerance: each gradient component within 2e-13 of the sum of the absolute
 values of the pieces it is built from (the reciprocal's 6e-14, E2's |argument|
-2^-53 with arguments up to 50, and the fixed-point units of 2^-46 of a typical
+2^-53 with arguments up to 50, and the fixed-point units of 2^-48 of a typical
 term), the NLL within 1e-14 of sum |w log P|.
 """
 import numpy as np
@@ -227,3 +227,38 @@ def test_cached_basis_rows(env, kind, weighted):
         assert abs(big[0] - (ref[0] - w.sum() * np.log(8.0))) <= 2e-14 * labs, n
         keep = np.arange(len(th0)) != 3                   # (the derivative in f_b scales with the basis)
         assert np.all(np.abs(big[1:] - ref[1:])[keep] <= 5e-13 * np.abs(terms).sum(1)[keep]), n
+
+
+@pytest.mark.parametrize("kind", ["1d", "4d", "tagged", "phis"])
+def test_weights_of_changing_scale_over_a_tile(env, kind):
+    """The integer sums' scale follows the largest weight so far: weights that are zero
+    for a quarter of a tile, then grow by 2^40 over it, then fall again.  One warp
+    and a team per tile give the same bits; values as above."""
+    O, G, _ = env
+    import torch
+    from paper_1706_01420_gb300 import api
+    th = np.array({"1d": TH4[:4], "4d": TH4, "tagged": [0.66, 0.045, 0.0, 0.1, 0.085, 17.77, 0.8, 0.3],
+                   "phis": list(TH4) + [0.085, 17.77, 0.8, 0.3, 0.8, 0.0]}[kind])
+    m = getattr(api, "model_" + kind)(0.0, HI)
+    mo = O.Model("tag" if kind == "tagged" else kind, 0.0, HI)
+    theta = torch.tensor(th, device="cuda")
+    n = 1100
+    if kind == "1d":
+        cols = {"t": synth.events_1d(n, 83, t_lo=0.0)}
+    else:
+        cols = {"4d": synth.events_4d, "tagged": synth.events_tagged, "phis": synth.events_phis}[kind](n, 83)
+    i = np.arange(n)
+    cols["w"] = np.where(i < 128, 0.0, np.where(i < 512, 2.0 ** ((i - 512) / 10.0), 2.0 ** (-(i - 512) / 20.0)))
+    ev = G.to_dev(cols)
+    got = {}
+    try:
+        for warps in (1, 2):
+            api.ipa_launch_config_set(m, n, {"warps_per_block": warps, "warps_per_sm": 0, "tiles_per_take": 1})
+            got[warps] = api.ipa_nll_grad(m, ev, theta).cpu().numpy()
+    finally:
+        api.ipa_launch_config_set(m, n, {"warps_per_block": 1, "warps_per_sm": 0, "tiles_per_take": 1})
+    assert np.array_equal(got[1], got[2])
+    f, g = O.nll_grad(mo, cols, th)
+    logl, terms = O.nll_grad_terms(mo, cols, th)
+    assert abs(got[1][0] - f) <= 1e-14 * np.abs(logl).sum()
+    assert np.all(np.abs(got[1][1:] - g) <= 5e-13 * np.abs(terms).sum(1))
