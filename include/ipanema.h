@@ -523,8 +523,8 @@ ipa_status ipa_binned_smear(const double* hist_dev, int64_t n_bins, double bin_w
  * Outputs (device): cl_out_dev[3] = (CL_b, CL_s+b, CL_s); counts_out_dev[2]
  * the toy counts behind them (may be NULL); x_out_dev (2 n_toys + 1: X of the
  * b toys, of the s+b toys, X_obs; may be NULL).  Toys are drawn on the fly,
- * one block per toy: nothing of size n_toys x n_bins is stored.  Synchronises
- * `stream` twice (to size the CDF tables), then runs asynchronously on it. */
+ * a lane per toy: nothing of size n_toys x n_bins is stored.  Synchronises
+ * `stream` once (to size the CDF tables), then runs asynchronously on it. */
 ipa_status ipa_cls(const double* s_dev, const double* b_dev, int64_t n_bins, const int32_t* data_dev, int32_t n_toys,
                    uint64_t seed, double* cl_out_dev, int64_t* counts_out_dev, double* x_out_dev, void* stream);
 

@@ -23,7 +23,7 @@
 //   * sin/cos, the whole angular basis, A and the ten angular sums, the decay
 //     exponential, the Gaussian and erfcx run on the integer pipe in 64-bit
 //     fixed point at four to six instructions per product (fast_fixed.cuh); the
-//     rows that allow it (rows_fast) leave about 15 FP64 instructions per event;
+//     rows that allow it (Angtime, Time1d below) leave about 15 FP64 instructions per event;
 //   * sin(theta_K) sin(theta_mu) is one square root; the constant factors of
 //     the ten angular functions are folded into the amplitude coefficients.
 //
@@ -251,9 +251,9 @@ __device__ __forceinline__ void plain_rows(const Consts& c, const MathTables* mt
 // are differences of sums of basis functions, taken in integers).  top follows
 // the segment's typical r T (NllCoef::rtop) and the largest weight of the tile,
 // so a unit is 2^-48 of a typical term; error of a sum: 0.41 units rms per
-// event, of random sign, below that of the reciprocal r (6e-14 relative).  The 1D model: sums of r T and r Gx and their products
-// with tau, as in the tagged model (tagged.cu).  Lanes outside the ranges are fixed up in
-// FP64.  A tile in which some P lies outside the Newton reciprocal's range (zero,
+// event, of random sign, below that of the reciprocal r (6e-14 relative).  The 1D
+// model: sums of r T and r Gx and their products with tau, as in the tagged model
+// (tagged.cu).  Lanes outside the ranges are fixed up in FP64.  A tile in which some P lies outside the Newton reciprocal's range (zero,
 // subnormal, negative, huge, infinite or NaN) or some |r T| >= 2^(top - 3) is redone
 // by the plain loop.  Either way the tile's sums depend only on its events, never
 // on the launch geometry (team_tile.cuh).
@@ -264,10 +264,11 @@ __device__ __forceinline__ void plain_rows(const Consts& c, const MathTables* mt
 // Measured (one pass of the public call, 512 toys of 20 000 events, then 1e7
 // weighted events): the angular products, A and the exponential in FP64 and
 // 14-instruction 64-bit products, an FP64 multiply-add per angular sum: 1060 and
-// 1073 us; this path: 643 and 685.  About 1150 warp instructions per row now
-// occupy the FP64 unit 60 %, the two 32-bit multiplier and adder pipes 50 % each
-// and the issue slots 50 %; 128 registers leave 16 warps per SM, and launch
-// bounds for 20 or 24 cost more in spills than they hide (728 and 760 us).
+// 1073 us; this path: 643 and 685 (now 608, with the records by block, and 689).
+// About 1060 warp instructions per row occupy the FP64 unit 60 %, the two 32-bit
+// multiplier and adder pipes 50 % each and the issue slots 50 %; 128 registers
+// leave 16 warps per SM, and launch bounds for 20 or 24 cost more in spills than
+// they hide (728 and 760 us).
 
 // The integer-pipe results of one event that its FP64 work needs.
 struct RowIn {

@@ -135,7 +135,7 @@ struct PhisWarp {
     PhisConsts c;
     double eq[6], mu[4], mv[4];
     double D2, D2s, D2c;      // 2 D, 2 D s, 2 D c
-    // the same in fixed point (rows_fast): eq, mu, mv with max in [1/8, 1/4) at 2^-hexp; c and s
+    // the same in fixed point (phis_event_fast): eq, mu, mv with max in [1/8, 1/4) at 2^-hexp; c and s
     // (Q62); rtop: scale of the angular sums' factors at unit weight (2^11 typical ones, 2^(rtop - 2))
     int2 fe[6], fu[4], fv[4], fc, fs;
     int hexp, rtop, fixed, pad_;

@@ -2,9 +2,9 @@
 // FP64 reduction of per-tile accumulators, the tile-to-segment lookup, the
 // per-lane log product and two bit-level helpers.
 //
-// Reduction order.  A tile of kTile events is owned by one warp; lane l adds
-// events l, l+32, ... in order; the warp reduces its lanes with the butterfly
-// below into one partial per tile.  The warp that completes the last tile of a
+// Reduction order.  In a tile of kTile events lane l adds events l, l+32, ... in
+// order (with the gradient quarter by quarter, by one warp or four: team_tile.cuh);
+// a warp reduces the lanes with the butterfly below into one partial per tile.  The warp that completes the last tile of a
 // group of kGroupTiles tiles reduces the group (lane l holding tile l), and the
 // warp that completes a segment's last group adds the group partials in fixed
 // order.  The order depends only on the segment's events, never on the launch
