@@ -174,6 +174,11 @@ __device__ __forceinline__ bool fx_angles_ok(double ck, double cl, double phi) {
     return abs_below(ck, kMaxCos) && abs_below(cl, kMaxCos) && abs_below(phi, 4.0);
 }
 
+// |x| < 1.75: a basis value (or product) that Q62 holds, with room; false for NaN.
+__device__ __forceinline__ bool fits_q62(double x) {
+    return ((int)((unsigned long long)__double_as_longlong(x) >> 32) & 0x7FFFFFFF) < 0x3FFC0000;
+}
+
 // Ten products of the helicity angles in Q62 (absolute error a few 2^-60), a basis
 // of the f'_k (angular.cuh) that takes one product less each:
 //   g = {sl2, sk2, G, G cp^2, G sp cp, f'_4, f'_5, f'_7, f'_8, f'_9},  G = sk2 sl2 (sk2 =

@@ -277,7 +277,9 @@ struct RowIn {
 };
 
 // The FP64 values for a lane outside the fixed-point ranges (rare): the basis, A'
-// (with the f'_k in the plain loop's order) and the exponential.
+// (with the f'_k in the plain loop's order) and the exponential.  Basis values beyond
+// the fixed-point range (|cos| > 1, angles that are NaN or infinite) make A' a NaN, so
+// that the tile is redone by the plain loop.
 __device__ __noinline__ void fix_row(const Consts& c, const MathTables* mt, double t, double ck, double cl, double phi,
                                      bool ok_exp, RowIn& v) {
     if (!ok_exp) v.E2 = exp_fast(fma(-c.Gamma, v.tau, c.k.c2), mt);
@@ -288,7 +290,10 @@ __device__ __noinline__ void fix_row(const Consts& c, const MathTables* mt, doub
         const double sk2 = fma(-ck, ck, 1.0), G = sk2 * f[6], gcc = sk2 - f[1];
         const double g[10] = {f[6], sk2, G, gcc, f[3], f[4], f[5], f[7], f[8], f[9]};
 #pragma unroll
-        for (int k = 0; k < 10; ++k) v.g[k] = fx(to_q62_nb(g[k]));
+        for (int k = 0; k < 10; ++k) {
+            if (!fits_q62(g[k])) v.Ap = __longlong_as_double(0x7ff8000000000000ll);
+            v.g[k] = fx(to_q62_nb(g[k]));
+        }
     }
 }
 

@@ -260,12 +260,18 @@ __device__ __forceinline__ void phis_event(const PhisWarp& pw, const MathTables*
 // the Newton reciprocal's range or some factor outside its scale.  FP64 instructions per
 // event: 92 -> 57; 1e6 events 299 -> 248 us (FP64 unit busy 77 -> 68 %).
 
-// The f'_k in Q62 near |cos| = 1 (rare).
-__device__ __noinline__ void phis_basis_wide(double ck, double cl, double phi, const MathTables* mt, long long F[10]) {
+// The f'_k in Q62 near |cos| = 1 (rare).  False where one of them does not fit (angles that
+// are NaN or infinite, |cos| > 1): the rows are left to phis_event.
+__device__ __noinline__ bool phis_basis_wide(double ck, double cl, double phi, const MathTables* mt, long long F[10]) {
     double f[10];
     basis_unscaled(ck, cl, phi, mt, f);
+    bool ok = true;
 #pragma unroll
-    for (int k = 0; k < 10; ++k) F[k] = to_q62_nb(f[k]);
+    for (int k = 0; k < 10; ++k) {
+        ok = ok && fits_q62(f[k]);
+        F[k] = to_q62_nb(f[k]);
+    }
+    return ok;
 }
 
 // One event: FP64 sums into acc (as phis_event), the angular sums (kE .. kMV + 3) into S.
@@ -281,7 +287,7 @@ __device__ __forceinline__ void phis_event_fast(const PhisWarp& pw, const MathTa
 #pragma unroll
         for (int k = 0; k < 10; ++k) {
             const double f = __ldg(cols.fk + k * cols.fk_stride + e);
-            *bad |= high_word(f) >= 0x3FFC0000;           // |f_k| < 1.75
+            *bad |= !fits_q62(f);
             F[k] = fx_signed(f, 1);
         }
     } else {
@@ -300,7 +306,7 @@ __device__ __forceinline__ void phis_event_fast(const PhisWarp& pw, const MathTa
         F[9] = g[9];
         if (!fx_angles_ok(ck, cl, phi)) {
             long long x[10];                             // (a copy, so that F itself stays in registers)
-            phis_basis_wide(ck, cl, phi, mt, x);
+            *bad |= !phis_basis_wide(ck, cl, phi, mt, x);
 #pragma unroll
             for (int k = 0; k < 10; ++k) F[k] = x[k];
         }

@@ -262,3 +262,35 @@ def test_weights_of_changing_scale_over_a_tile(env, kind):
     logl, terms = O.nll_grad_terms(mo, cols, th)
     assert abs(got[1][0] - f) <= 1e-14 * np.abs(logl).sum()
     assert np.all(np.abs(got[1][1:] - g) <= 5e-13 * np.abs(terms).sum(1))
+
+
+@pytest.mark.parametrize("weighted", [False, True])
+@pytest.mark.parametrize("kind", ["4d", "phis"])
+@pytest.mark.parametrize("bad", [(1.5, 0.2, 0.1), (0.1, -1.5, 0.1), (0.2, 0.1, np.nan), (np.nan, 0.1, 0.2),
+                                 (0.2, np.inf, 0.1), (3.0, 3.0, 0.4), (-3.0, 2.0, 1.4)])
+def test_angles_outside_their_domain(env, kind, weighted, bad):
+    """One event whose angles lie outside the domain (|cos| > 1, not a number): the values
+    are those of the plain loop, which takes a call of fewer than 64 events, NaN or not.
+    With both |cos| > 1 the basis values are finite and up to 72; at late t with background
+    P stays positive.  Tolerance: 5e-13 of the sum of |terms| for each of the three calls."""
+    O, G, _ = env
+    import torch
+    from paper_1706_01420_gb300 import api
+    th = np.array({"4d": TH4, "phis": list(TH4) + [0.085, 17.77, 0.8, 0.3, 0.8, 0.0]}[kind])
+    th[3] = 0.5
+    m = getattr(api, "model_" + kind)(0.0, HI)
+    cols = {"4d": synth.events_4d, "phis": synth.events_phis}[kind](200, 89, weighted=weighted)
+    cols["t"][170] = 14.5
+    cols["ck"][170], cols["cl"][170], cols["phi"][170] = bad
+
+    def grad(a, b):
+        ev = G.to_dev({k: np.ascontiguousarray(v[a:b]) for k, v in cols.items()})
+        return api.ipa_nll_grad(m, ev, torch.tensor(th, device="cuda")).cpu().numpy()
+    whole, most, few = grad(0, 200), grad(0, 160), grad(160, 200)
+    assert np.isfinite(most).all()
+    assert np.array_equal(np.isnan(whole), np.isnan(few)), (whole, few)
+    assert np.isnan(few[0]) == (max(abs(bad[0]), abs(bad[1])) != 3.0)
+    logl, terms = O.nll_grad_terms(O.Model(kind, 0.0, HI), {k: v[:160] for k, v in cols.items()}, th)
+    scale = 2.0 * np.append(np.abs(logl).sum(), np.abs(terms).sum(1)) + np.abs(few)
+    ok = ~np.isnan(few)
+    assert np.all(np.abs(whole - most - few)[ok] <= 1e-12 * scale[ok]), (whole, most + few)
