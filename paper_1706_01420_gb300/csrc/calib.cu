@@ -24,7 +24,7 @@ calib_kernel(const double* __restrict__ in, double* __restrict__ out, int iters,
     __shared__ FullTables mt;
     if (OP >= 7) {
         load_math_tables(&mt);
-    load_fp64_tables(&mt);
+        load_fp64_tables(&mt);
         __syncthreads();
     }
     const int i = blockIdx.x * blockDim.x + threadIdx.x;

@@ -239,6 +239,7 @@ ipa_status scratch_get(int64_t tiles, int64_t segs, Scratch** out) {
         s.partials_cap = cap;
     }
     if (!s.work) {
+        pool_of_device();                            // created here: a capturing stream could not
         if ((st = device_alloc((void**)&s.work, 2 * sizeof(unsigned), "scratch work counters")) != IPA_OK) return st;
         if ((st = cuda_fail(cudaMemset(s.work, 0, 2 * sizeof(unsigned)), "scratch memset")) != IPA_OK) return st;
         if ((st = cuda_fail(cudaDeviceSynchronize(), "scratch init")) != IPA_OK) return st;

@@ -125,3 +125,43 @@ def test_under_stream_capture():
         g.replay()
         torch.cuda.synchronize()
         assert all(torch.equal(out[k], ref[k]) for k in out)
+
+
+FIRST_CAPTURED = """
+import sys
+sys.path.insert(0, sys.argv[1])
+import torch
+from paper_1706_01420_gb300 import api, synth
+dev = torch.device("cuda")
+th = torch.tensor([0.66, 0.045, 0.0, 0.1, 0.52, 0.25, 3.2, 3.1, 0.04, 0.3], dtype=torch.float64, device=dev)
+m = api.model_4d(0.0, 15.0)
+ev = {k: torch.tensor(v, device=dev) for k, v in synth.events_4d(1000, 1).items()}
+api.ipa_nll_grad(m, ev, th)
+n = 30000
+out = {k: torch.zeros(n, dtype=torch.float64, device=dev) for k in ("t", "ck", "cl", "phi")}
+i64 = lambda v: torch.tensor([v], dtype=torch.int64, device=dev)
+ns, nb, off = i64(n - 100), i64(100), i64(0)
+torch.cuda.synchronize()
+g = torch.cuda.CUDAGraph()
+s = torch.cuda.Stream()
+with torch.cuda.stream(s):
+    with torch.cuda.graph(g, stream=s):
+        api.ipa_toygen(m, th, 5, ns, nb, off, out, stream=s)
+g.replay()
+torch.cuda.synchronize()
+a = {k: v.clone() for k, v in out.items()}
+api.ipa_toygen(m, th, 5, ns, nb, off, out)
+torch.cuda.synchronize()
+assert all(torch.equal(a[k], out[k]) for k in out) and a["t"].min() > 0
+print("captured first")
+"""
+
+
+def test_first_call_of_a_process_under_stream_capture():
+    """After a likelihood call (which sizes the scratch) the generator's first call may be captured."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", FIRST_CAPTURED, root], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "captured first" in r.stdout, r.stderr[-2000:]
