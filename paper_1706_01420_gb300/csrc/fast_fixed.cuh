@@ -24,6 +24,7 @@ namespace ipa {
 struct Fx {
     int h, l;
 };
+// x < 2^63 - 2^31 (from there on h would be 2^31): a magnitude that fills 63 bits goes in negated.
 __device__ __forceinline__ Fx fx(long long x) {
     return Fx{(int)(x >> 32) + (int)((unsigned)x >> 31), (int)x};
 }
@@ -288,15 +289,15 @@ __device__ __forceinline__ void fx_phase(Fx T, const FxExp& s, const MathTables*
 }
 
 // e^a for -705 <= a <= 0: |a| in units of ln2/64, its fixed point following its
-// exponent (relative error below 2^-55 for |a| < 32, below |a|'s own rounding beyond).
+// exponent (error before the last rounding below 2^-54 for |a| < 32, |a| 2^-59 beyond).
 __device__ __forceinline__ double fx_exp_neg(double a, const MathTables* mt) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(a);
     const int E = (int)((b >> 52) & 0x7FFull) - 1023;
     const int top = E + 1 > 2 ? E + 1 : 2;
-    const long long T = (long long)fx_magnitude(b, top);
+    const long long T = (long long)fx_magnitude(b, top);   // up to 2^63 - 1
     constexpr Fx kInv = {774541002, 1460010031};        // 64 / ln2 in 2^55
     int x;
-    return fx_exp2(-fx_mad(fx(T), kInv, 0), (54 - top) & 63, mt, &x);
+    return fx_exp2(fx_mad(fx(-T), kInv, 0), (54 - top) & 63, mt, &x);
 }
 
 // erfcx(x) = exp(x^2) erfc(x) for 0 <= x <= 6.25 (the pieces of erfcx_poly); larger x,

@@ -1,0 +1,86 @@
+"""Inputs at the edges of the event loops' fixed-point formats and scales, against the
+oracle, for all models that share them.
+
+Tolerances: the NLL within 1e-14 of sum |w log P| and each gradient component within
+5e-13 of the sum of |terms| (the reciprocal's 6e-14 and the fixed-point units, with
+cancellation among the terms of a component by a factor of a few), unless a test says
+otherwise."""
+import numpy as np
+import pytest
+
+from paper_1706_01420_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+TH4 = [0.66, 0.045, 0.0, 0.1, 0.52, 0.25, 3.2, 3.1, 0.04, 0.3]
+TRUTH = {"1d": TH4[:4], "4d": TH4, "tagged": [0.66, 0.045, 0.0, 0.1, 0.085, 17.77, 0.8, 0.3],
+         "phis": TH4 + [0.085, 17.77, 0.8, 0.3, 0.8, 0.0]}
+KINDS = list(TRUTH)
+
+
+@pytest.fixture(scope="module")
+def env(oracle):
+    from tests import gpu_common as G
+    G.need_gpu()
+    import torch
+    from paper_1706_01420_gb300 import api
+    return oracle, G, torch, api
+
+
+def columns(kind, n, seed, weighted=False):
+    if kind == "1d":
+        cols = {"t": synth.events_1d(n, seed, t_lo=0.0)}
+        if weighted:
+            cols["w"] = synth.weights(n, seed + 1)
+        return cols
+    return {"4d": synth.events_4d, "tagged": synth.events_tagged,
+            "phis": synth.events_phis}[kind](n, seed, weighted=weighted)
+
+
+def oracle_model(O, kind, lo, hi):
+    return O.Model("tag" if kind == "tagged" else kind, lo, hi)
+
+
+def gradients(env, kind, lo, hi, cols, th, cached=False):
+    """The call with one warp per tile and with a team per tile: the same bits."""
+    _, G, torch, api = env
+    m = getattr(api, "model_" + kind)(lo, hi)
+    n = len(cols["t"])
+    ev = G.to_dev(cols)
+    if cached:
+        ev["fk"] = cached if isinstance(cached, torch.Tensor) else api.ipa_angular_basis(m, ev)
+    theta = torch.tensor(np.asarray(th), device="cuda")
+    got = {}
+    try:
+        for warps in (1, 2):
+            api.ipa_launch_config_set(m, n, {"warps_per_block": warps, "warps_per_sm": 0, "tiles_per_take": 1},
+                                      cached=bool(ev.get("fk") is not None))
+            got[warps] = api.ipa_nll_grad(m, ev, theta).cpu().numpy()
+    finally:
+        api.ipa_launch_config_set(m, n, {"warps_per_block": 1, "warps_per_sm": 0, "tiles_per_take": 1},
+                                  cached=bool(ev.get("fk") is not None))
+    assert np.array_equal(got[1], got[2], equal_nan=True), (got[1], got[2])
+    return got[1]
+
+
+def check(env, kind, lo, hi, cols, th, rtol_f=1e-14, rtol_g=5e-13):
+    O = env[0]
+    got = gradients(env, kind, lo, hi, cols, th)
+    m = oracle_model(O, kind, lo, hi)
+    f, g = O.nll_grad(m, cols, th)
+    logl, terms = O.nll_grad_terms(m, cols, th)
+    assert abs(got[0] - f) <= rtol_f * np.abs(logl).sum(), (got[0], f)
+    assert np.all(np.abs(got[1:] - g) <= rtol_g * np.abs(terms).sum(1)), (got[1:], g)
+
+
+@pytest.mark.parametrize("weighted", [False, True])
+@pytest.mark.parametrize("kind", KINDS)
+def test_gaussian_just_below_a_power_of_two(env, kind, weighted):
+    """tau^2 / (2 sigma^2) within a few last places of 1, 2, .., 32, on both sides of the peak
+    (times on a grid meet these: 0.18 is 4 sigma)."""
+    x = np.sqrt(2.0 * 2.0 ** np.arange(6.0)) * TRUTH[kind][1]
+    steps = np.arange(-24, 25)
+    t = (x[:, None] + steps * np.spacing(x)[:, None]).ravel()
+    cols = columns(kind, 2 * t.size, 5, weighted)
+    cols["t"] = np.concatenate([t, -t])
+    check(env, kind, -0.5, 15.0, cols, TRUTH[kind])
