@@ -317,9 +317,10 @@ __device__ __forceinline__ double fx_erfcx(double x, const MathTables* t) {
     return fx_to_double(v, 0);
 }
 
-// log x for 2^-126 <= x < 2^127 (positive and normal, the caller checks) in Q56, error
-// below 2^-55: x = 2^e m, r = m c_j - 1 with the table's c_j (log_fast), |r| <= 2^-8,
-// log1p's series to r^7, its terms from r^4 on in 32 bits.
+// log x for 2^-126 <= x < 2^127 (positive and normal, the caller checks) in Q56: x = 2^e m,
+// r = m c_j - 1 with the table's c_j (log_fast), |r| <= 2^-8, log1p's series to r^7, its
+// terms from r^4 on in 32 bits.  Error below (2 + |e| / 3) 2^-56, the second part ln 2's
+// rounding: 2^-55 at e = 0, 2^-50.5 at |e| = 126, and always below 2^-55 of |log x| + 1.
 __device__ __forceinline__ long long fx_log(double x, const MathTables* t) {
     const long long b = __double_as_longlong(x);
     const int e = (int)(b >> 52) - 1023;
@@ -327,7 +328,7 @@ __device__ __forceinline__ long long fx_log(double x, const MathTables* t) {
     const long long m = (long long)(((unsigned long long)b << 10 & 0x3FFFFFFFFFFFFFFFull) | 0x4000000000000000ull);  // Q62
     const long long cb = __double_as_longlong(t->linv[j]);                    // in [1/2, 1)
     const long long c = (long long)(((unsigned long long)cb << 9 & 0x1FFFFFFFFFFFFFFFull) | 0x2000000000000000ull);  // Q62
-    const long long r = fx_mad(fx(m), fx(c), 0) - (1ll << 60);                // Q60
+    const long long r = -fx_mad(fx(-m), fx(c), 1ll << 60);                    // Q60 (m < 2^63: negated for fx)
     const Fx R = fx(r << 10);                                                 // Q70
     const int r32 = R.h;                                                      // Q38, |r32| <= 2^30
     const int i6 = 357913941 - (__mulhi(r32, 306783378) >> 6);                // 1/6 - r/7 in 2^31

@@ -67,3 +67,14 @@ def test_gaussian_exponential(lib):
         ref = mp.exp(mp.mpf(float(x)))
         bound = mp.mpf(2) ** -53 + max(mp.mpf(2) ** -54, -mp.mpf(float(x)) * mp.mpf(2) ** -59)
         assert abs(mp.mpf(float(v)) - ref) <= bound * ref, (x, v)
+
+
+def test_log(lib):
+    rng = np.random.default_rng(12)
+    x = np.concatenate([2.0 ** rng.uniform(-126.0, 126.9, 4000), rng.uniform(0.5, 2.0, 4000), [1.0],
+                        1.0 + np.arange(128) / 128.0, np.nextafter(1.0 + np.arange(1, 129) / 128.0, 0.0), FULL,
+                        FULL * 2.0 ** -110, FULL * 2.0 ** 110])
+    y = call(lib, lib.log_q56, x, np.int64)
+    for v, a in zip(y, x):
+        e = abs(int(np.frexp(a)[1]) - 1)
+        assert abs(int(v) - mp.log(mp.mpf(float(a))) * 2 ** 56) <= 2 + e / 3.0, (a, v)

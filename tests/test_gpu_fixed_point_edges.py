@@ -84,3 +84,33 @@ def test_gaussian_just_below_a_power_of_two(env, kind, weighted):
     cols = columns(kind, 2 * t.size, 5, weighted)
     cols["t"] = np.concatenate([t, -t])
     check(env, kind, -0.5, 15.0, cols, TRUTH[kind])
+
+
+@pytest.mark.parametrize("kind", KINDS)
+def test_weighted_log_just_below_a_power_of_two(env, kind):
+    """Weighted events with P = 2^e (1 - 2^-k), k = 32 .. 40, placed by bisection in t."""
+    O = env[0]
+    th = np.array(TRUTH[kind])
+    m = oracle_model(O, kind, 0.0, 15.0)
+    cols = columns(kind, 400, 7, weighted=True)
+    one = {k: v[200:201].copy() for k, v in cols.items()}
+
+    def density(t):
+        one["t"][0] = t
+        return float(O.pdf(m, one, th)[0])
+    p = np.array([density(t) for t in np.linspace(0.35, 4.0, 400)])
+    e = np.floor(np.log2(p))
+    for i in np.nonzero(e[1:] != e[:-1])[0][:3]:
+        edge = 2.0 ** max(e[i], e[i + 1])
+        for k in (32, 33, 36, 40):
+            goal = edge * (1.0 - 2.0 ** -k)
+            lo, hi = np.linspace(0.35, 4.0, 400)[i:i + 2]
+            for _ in range(80):
+                mid = 0.5 * (lo + hi)
+                if (density(mid) < goal) == (p[i] < goal):
+                    lo = mid
+                else:
+                    hi = mid
+            assert abs(density(lo) / edge - (1.0 - 2.0 ** -k)) < 2.0 ** -45
+            cols["t"][200], cols["w"][200] = lo, 1.7
+            check(env, kind, 0.0, 15.0, cols, th)
