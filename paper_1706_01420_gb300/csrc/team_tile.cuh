@@ -228,7 +228,7 @@ __device__ __forceinline__ void solo_tile(const typename M::Record& c, const Mat
             tprod *= s.prod;
             s.prod = 1.0;
         }
-        if (!W) plain = __any_sync(0xffffffffu, M::bad(c, sc, s));
+        if (!W && !plain) plain = __any_sync(0xffffffffu, M::bad(c, sc, s));
 #pragma unroll
         for (int i = 0; i < M::kSums; ++i) s.f[i] = tot[i];
         M::accumulators(c, sc, s, acc);

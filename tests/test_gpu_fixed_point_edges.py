@@ -114,3 +114,51 @@ def test_weighted_log_just_below_a_power_of_two(env, kind):
             assert abs(density(lo) / edge - (1.0 - 2.0 ** -k)) < 2.0 ** -45
             cols["t"][200], cols["w"][200] = lo, 1.7
             check(env, kind, 0.0, 15.0, cols, th)
+
+
+OUTSIDE = [("1d", 3, 1.5), ("1d", 3, -0.1), ("1d", 1, -0.045), ("1d", 0, -0.1), ("1d", 0, np.nan),
+           ("tagged", 3, np.nan), ("tagged", 6, np.nan), ("tagged", 0, np.nan)]
+
+
+@pytest.mark.parametrize("kind, index, value", OUTSIDE)
+@pytest.mark.parametrize("n", [3000, 700_000])
+def test_no_scale_outside_the_domain(env, kind, index, value, n):
+    """Parameters for which the integers' scale is out of range leave the tile to the plain
+    loop in either form: NaN throughout, as from the NLL alone (the larger call takes single
+    warps in the built-in geometry, and has NaN in every component too)."""
+    _, G, torch, api = env
+    th = np.array(TRUTH[kind])
+    th[index] = value
+    cols = columns(kind, n, 9)
+    if n == 3000:
+        got = gradients(env, kind, 0.0, 15.0, cols, th)
+    else:
+        m = getattr(api, "model_" + kind)(0.0, 15.0)
+        got = api.ipa_nll_grad(m, G.to_dev(cols), torch.tensor(th, device="cuda")).cpu().numpy()
+    assert np.isnan(got).all(), got
+
+
+def test_fit_of_one_parameter_from_outside_the_domain(env):
+    _, G, torch, api = env
+    n = 700_000
+    start = np.array(TRUTH["1d"])
+    start[3] = 1.5
+    params = [api.Param(float(v), fixed=True) for v in start[:3]] + [api.Param(1.5, -1.0, 2.0, 0.01)]
+    off = torch.tensor([0, n], dtype=torch.int64, device="cuda")
+    r = api.ipa_fit_batch(api.model_1d(0.0, 15.0), G.to_dev(columns("1d", n, 9)), off, params,
+                          torch.tensor(start[None, :], device="cuda"), max_iter=50, tol=1e-8)
+    assert int(r["status"].cpu()[0]) == 3                 # IPA_FIT_BAD_PDF
+
+
+@pytest.mark.parametrize("kind", ["1d", "tagged"])
+@pytest.mark.parametrize("sigmas", [24.0, 26.0, 30.0])
+def test_no_scale_far_below_the_peak(env, kind, sigmas):
+    """A range that ends 24 sigma and more below mu: cs is beyond the integers' scale.  The
+    normalisation cancels to |x| / (Gamma sigma) = 1e3 times FP64's rounding and its
+    derivative in sigma once more: 1e-7 of the sum of |terms| (a tile that was left out
+    gave nothing)."""
+    th = np.array(TRUTH[kind])
+    cols = columns(kind, 3000, 13)
+    hi = -sigmas * th[1]
+    cols["t"] = np.random.default_rng(3).uniform(hi - 3.0 * th[1], hi, 3000)
+    check(env, kind, hi - 3.0 * th[1], hi, cols, th, rtol_f=1e-9, rtol_g=1e-7)
