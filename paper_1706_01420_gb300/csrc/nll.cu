@@ -437,7 +437,9 @@ struct Time1d {
     using Sums = FastSums<kSums, kInts>;
 
     static __device__ __forceinline__ bool usable(const Consts& c, int64_t events, FastScale* sc) {
-        // a typical r T is near 1 / max(cs / 2, cb / 2); the Gaussian's tau within 10 sigma (as in tagged.cu)
+        // a typical r T is near 1 / max(cs / 2, cb / 2); the Gaussian's tau is taken within 14 to 28 sigma:
+        // r Gx is above the sums' unit within 8.6 sigma only, except where P itself falls with the
+        // Gaussian (bad)
         sc->top = 10 + 1023 - max(exponent_field(c.k.aq), exponent_field(c.cb) - 1);
         sc->gtop = exponent_field(c.sigma) - 1023 + 5;
         return c.k.ex.ok && sc->gtop >= -400 && sc->gtop <= 400;
@@ -477,14 +479,15 @@ struct Time1d {
                     const long long a = fx_odd(x[i], sc.top);
                     s.g[i] += a;
                     s.g[2 + i] = fx_mad1(fx((long long)((unsigned long long)a << 3)), T[i], s.g[2 + i], a != 0);
+                    if (i == 1) s.gtau_most = max(s.gtau_most, a != 0 ? high_word(tau) : 0);
                 }
             }
         }
         __syncwarp();
     }
     static __device__ __forceinline__ bool bad(const Consts& c, FastScale sc, const Sums& s) {
-        return p_out_of_range(s) || (s.most >> 20) > 1023 - 6 + sc.top ||
-               s.tau_most >= ((1023 - 1 + c.k.ex.top) << 20 | 0xC0000);
+        return p_out_of_range(s) || beyond_factor(s.most, sc.top) || beyond_tau(s.tau_most, c.k.ex.top) ||
+               beyond_tau(s.gtau_most, sc.gtop);
     }
     static __device__ __forceinline__ void accumulators(const Consts& c, FastScale sc, const Sums& s, double* acc) {
         acc[0] = s.f[1];

@@ -150,7 +150,7 @@ __device__ __forceinline__ void tag_rows(const TagConsts& c, const MathTables* m
 // are converted once at a scale that follows the segment's typical r g (1 / max(qH, qL, cb / 2))
 // and the tile's largest weight; a unit is 2^-53 of a typical term, 2^-50 in the sums with tau
 // (0.4 units rms per event).  A tile with P outside the Newton reciprocal's range or a factor
-// beyond 2^5 typical ones (near-complete cancellation in P) is redone by tag_event.  FP64 instructions
+// beyond 2^4 typical ones (near-complete cancellation in P) is redone by tag_event.  FP64 instructions
 // per event: 31 -> 21; 1e6 events 131 -> 124 us (FP64 unit busy 70 -> 58 %; three to four
 // warps a sub-partition then leave its latencies uncovered).
 struct Tagged {
@@ -163,7 +163,9 @@ struct Tagged {
     static __device__ __forceinline__ bool usable(const TagConsts& c, int64_t events, FastScale* sc) {
         const int e1 = max(exponent_field(c.qH), exponent_field(c.qL)), e2 = exponent_field(c.cb) - 1;
         sc->top = 10 + 1023 - max(e1, e2);
-        // r Gx counts (its integer is not 0) only for |tau| < 10 sigma, so tau's scale there follows sigma
+        // tau's scale in the Gaussian's sums follows sigma, within 14 to 28 of it: r Gx is above the sums'
+        // unit (its integer is not 0) within 8.6 sigma only, except where P itself falls with the
+        // Gaussian (bad)
         sc->gtop = exponent_field(c.sigma) - 1023 + 5;
         return c.fx_ok && sc->gtop >= -400 && sc->gtop <= 400;
     }
@@ -212,14 +214,13 @@ struct Tagged {
             s.most = max(s.most, high_word(x[i]));
             const long long a = fx_odd(x[i], sc.top);
             s.g[i] += a;
+            if (i == 4) s.gtau_most = max(s.gtau_most, a != 0 ? high_word(tau) : 0);
             if (i < 5) s.g[6 + i] = fx_mad1(fx((long long)((unsigned long long)a << 3)), i < 4 ? T : TG, s.g[6 + i], a != 0);
         }
     }
     static __device__ __forceinline__ bool bad(const TagConsts& c, FastScale sc, const Sums& s) {
-        // factors below 2^(top - 5): sixteen of them and their products with tau stay in 64 bits;
-        // |tau| below 1.75 2^(fx.top - 1) (|t| < 2^(fx.top - 1))
-        return p_out_of_range(s) || (s.most >> 20) > 1023 - 6 + sc.top ||
-               s.tau_most >= ((1023 - 1 + c.fx[0].top) << 20 | 0xC0000);
+        return p_out_of_range(s) || beyond_factor(s.most, sc.top) || beyond_tau(s.tau_most, c.fx[0].top) ||
+               beyond_tau(s.gtau_most, sc.gtop);
     }
     static __device__ __forceinline__ void accumulators(const TagConsts& c, FastScale sc, const Sums& s, double* acc) {
         acc[0] = s.f[1];

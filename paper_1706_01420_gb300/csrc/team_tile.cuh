@@ -44,14 +44,15 @@ struct FastScale {
 
 // A lane's sums over rows on the fixed-point path: FP64 ones, the product of the P's of
 // events without weight (mantissas, exponents), integers, and the high words of the
-// largest factor, of the largest |tau| and of the least and largest P.
+// largest factor, of the largest |tau| (gtau_most: of those that enter the Gaussian's sums)
+// and of the least and largest P.
 template <int NF, int NG>
 struct FastSums {
     double f[NF];
     double prod;
     long long g[NG];
     int esum;
-    int most, tau_most, p_least, p_most;
+    int most, tau_most, gtau_most, p_least, p_most;
 };
 
 template <int NF, int NG>
@@ -62,9 +63,15 @@ __device__ __forceinline__ void clear(FastSums<NF, NG>& s) {
 #pragma unroll
     for (int i = 0; i < NG; ++i) s.g[i] = 0;
     s.esum = 0;
-    s.most = s.tau_most = 0;
+    s.most = s.tau_most = s.gtau_most = 0;
     s.p_least = s.p_most = 0x3FF00000;               // 1.0
 }
+
+// Sums over a lane's 16 events of factors below 2^(top - 6), in units of 2^(top - 63), and of
+// their products with tau at `ttop`, |tau| < 1.75 2^(ttop - 1): a product (the factor shifted up
+// by 3) is below 1.75 2^58, the sum below 1.75 2^62.  `most` and `tau` are high words.
+__device__ __forceinline__ bool beyond_factor(int most, int top) { return (most >> 20) > 1023 - 7 + top; }
+__device__ __forceinline__ bool beyond_tau(int tau, int ttop) { return tau >= ((1022 + ttop) << 20 | 0xC0000); }
 
 // P outside [2^-125, 2^126) (the Newton reciprocal's range) or not a number in some event.
 template <int NF, int NG>

@@ -162,3 +162,26 @@ def test_no_scale_far_below_the_peak(env, kind, sigmas):
     hi = -sigmas * th[1]
     cols["t"] = np.random.default_rng(3).uniform(hi - 3.0 * th[1], hi, 3000)
     check(env, kind, hi - 3.0 * th[1], hi, cols, th, rtol_f=1e-9, rtol_g=1e-7)
+
+
+@pytest.mark.parametrize("kind", ["1d", "tagged"])
+@pytest.mark.parametrize("sigma", [0.0313, 0.045, 0.0624])
+@pytest.mark.parametrize("f_b", [0.0, 0.1, 0.99])
+@pytest.mark.parametrize("below", [6.0, 8.0, 10.0, 14.0, 16.0, 18.0, 20.0, 22.0])
+def test_gaussian_sums_below_the_peak(env, kind, sigma, f_b, below):
+    """Ranges of 3.5 sigma that end `below` sigma under mu.  A weight of 2^-500 takes the tile
+    to the plain loop and scales every sum exactly, so that loop's gradient is at hand.  The
+    integers' unit against the pieces of a component, which cancel to sigma / (|tau| Gamma sigma)
+    of themselves, and again in sigma: 1e3 times (|tau| / sigma)^2 units of 2^-49, below 1e-9 of
+    the sum of |terms| for |tau| = 26 sigma.  Against the oracle 1e-7, as above."""
+    _, G, torch, api = env
+    th = np.array(TRUTH[kind])
+    th[1], th[3] = sigma, f_b
+    hi, lo = -below * sigma, -(below + 3.5) * sigma
+    cols = columns(kind, 1500, 17)
+    cols["t"] = np.random.default_rng(5).uniform(lo, hi, 1500)
+    check(env, kind, lo, hi, cols, th, rtol_f=1e-9, rtol_g=1e-7)
+    fast = gradients(env, kind, lo, hi, cols, th)
+    plain = gradients(env, kind, lo, hi, {**cols, "w": np.full(1500, 2.0 ** -500)}, th)
+    _, terms = env[0].nll_grad_terms(oracle_model(env[0], kind, lo, hi), cols, th)
+    assert np.all(np.abs(fast[1:] - plain[1:] * 2.0 ** 500) <= 1e-9 * np.abs(terms).sum(1)), (fast, plain)
