@@ -257,7 +257,7 @@ __device__ __forceinline__ void phis_event(const PhisWarp& pw, const MathTables*
 // r U and r C are converted once per event at a scale that follows the segment's typical r T and
 // the largest weight of the warp's rows (unit 2^-48 of a typical term, 0.41 units rms per
 // event).  The rest is FP64.  The warp's rows are redone by phis_event where some P lies outside
-// the Newton reciprocal's range or some factor outside its scale.  FP64 instructions per
+// the Newton reciprocal's range, some factor above its scale or all of them far below it.  FP64 instructions per
 // event: 92 -> 57; 1e6 events 299 -> 248 us (FP64 unit busy 77 -> 68 %).
 
 // The f'_k in Q62 near |cos| = 1 (rare).  False where one of them does not fit (angles that
@@ -626,7 +626,12 @@ const auto slow_of = [&](int k) {
                         const int64_t e = tbase + lane + 32 * (i0 + k);
                         if (e < ev1) phis_event_fast<WEIGHTED, CACHED>(pw, &mt, cols, e, slow_of(k), top, acc, S, &prod, &esum, &bad);
                     }
-                    plain = __any_sync(0xffffffffu, bad);
+                    // (none of the sums reaches 2^-6 of a typical term's 2^48 units: few of their bits would be
+                    // left, as far from the peak with f_b near 1)
+                    unsigned long long mag = 0;
+#pragma unroll
+                    for (int a = 0; a < 14; ++a) mag |= (unsigned long long)(S[a] ^ (S[a] >> 63));
+                    plain = __any_sync(0xffffffffu, bad) || !__any_sync(0xffffffffu, (mag >> 42) != 0ull);
 #pragma unroll
                     for (int a = 0; a < NA; ++a) {
                         if (a >= kE && a < kPhi) acc[a] = fx_to_double(S[a - kE], top + 1);

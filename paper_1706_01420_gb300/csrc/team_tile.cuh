@@ -15,6 +15,7 @@
 //   Record, Slow (a near-peak event's values), kSums: FP64 sums, kInts: integer sums, NA;
 //   usable(c, events, &sc)                      the scales at unit weight, false: plain loop;
 //   kTopRange                                   |sc.top| beyond it: plain loop;
+//   kLeast                                      no factor of the tile reaches 2^(top - kLeast): plain loop;
 //   quarter<W>(c, mt, cols, tbase, i0, ev1, sbuf, wbuf, lane, sc, s);   (wbuf: the lane's weights)
 //   bad(c, sc, s)                               a value left its range;
 //   accumulators(c, sc, s, acc);
@@ -133,6 +134,15 @@ __device__ __forceinline__ bool scale_to(FastScale* sc, int base, int run) {
     return sc->top >= -M::kTopRange && sc->top <= M::kTopRange;
 }
 
+// The integers' unit is set for typical factors.  A tile whose largest factor lies far below
+// (every signal term small beside the background, as far from the peak with f_b near 1) would
+// keep few of its bits.  `most`: the tile's largest factor (high word); not asked where all
+// weights are zero, which the integers hold exactly.
+template <class M>
+__device__ __forceinline__ bool too_small(int most, FastScale sc, int run) {
+    return run != kNoWeight && most < (1023 + sc.top - M::kLeast) << 20;
+}
+
 // Rows of a tile with events below ev1, up to a whole quarter.
 __device__ __forceinline__ int tile_rows(int64_t tbase, int64_t ev1) {
     const int64_t rows = (ev1 - tbase + 31) >> 5;
@@ -235,7 +245,10 @@ __device__ __forceinline__ void solo_tile(const typename M::Record& c, const Mat
             tprod *= s.prod;
             s.prod = 1.0;
         }
-        if (!W && !plain) plain = __any_sync(0xffffffffu, M::bad(c, sc, s));
+        if (!plain) {
+            if (!W) plain = __any_sync(0xffffffffu, M::bad(c, sc, s));
+            plain = plain || too_small<M>((int)__reduce_max_sync(0xffffffffu, (unsigned)s.most), sc, run);
+        }
 #pragma unroll
         for (int i = 0; i < M::kSums; ++i) s.f[i] = tot[i];
         M::accumulators(c, sc, s, acc);
@@ -276,6 +289,8 @@ team_kernel(Cols cols, int64_t n, const int64_t* __restrict__ seg_begin, const i
     const int out_stride = 1 + n_par;
     __shared__ MathTables mt;
     __shared__ int64_t s_take[2];
+    __shared__ int2 s_state[2][kTeam];               // of a quarter: its largest factor (kBad: redo the tile), run
+    constexpr int kBad = 0x7FFFFFFF;
     extern __shared__ __align__(16) unsigned char dyn_smem[];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     double* const xbuf = reinterpret_cast<double*>(dyn_smem);               // [2][kTeam][kWords][32]
@@ -343,6 +358,8 @@ team_kernel(Cols cols, int64_t n, const int64_t* __restrict__ seg_begin, const i
                 M::template quarter<W>(c, &mt, cols, tbase, i0, ev1, sbuf, wbuf, lane, sc, s);
                 plain = M::bad(c, sc, s);
             }
+            const int most = (int)__reduce_max_sync(0xffffffffu, (unsigned)(plain ? kBad : s.most));
+            if (lane == 0) s_state[turn & 1][wib] = make_int2(most, run);
 #pragma unroll
             for (int i = 0; i < M::kSums; ++i) own[i * 32] = s.f[i];
 #pragma unroll
@@ -351,7 +368,16 @@ team_kernel(Cols cols, int64_t n, const int64_t* __restrict__ seg_begin, const i
             own[(kWords - 1) * 32] = __longlong_as_double((long long)run << 32 | (unsigned)s.esum);
         }
         if (threadIdx.x == 32 * ((turn + 2) & (kTeam - 1))) s_take[(turn + 1) & 1] = (int64_t)atomicAdd(work, 1u);
-        plain = __syncthreads_or(plain);
+        __syncthreads();
+        {
+            int most = 0;
+#pragma unroll
+            for (int w = 0; w < kTeam; ++w) most = max(most, s_state[turn & 1][w].x);
+            run = s_state[turn & 1][kTeam - 1].y;    // the tile's largest weight
+            FastScale t;
+            scale_to<M>(&t, base, run);
+            plain = most == kBad || too_small<M>(most, t, run);
+        }
         if (plain) {
             double q[M::NA + 2];
             plain_quarters<M, W>(c, &mt, cols, i0, i0 + kSub, tbase, ev1, sbuf, lane, q);

@@ -185,3 +185,19 @@ def test_gaussian_sums_below_the_peak(env, kind, sigma, f_b, below):
     plain = gradients(env, kind, lo, hi, {**cols, "w": np.full(1500, 2.0 ** -500)}, th)
     _, terms = env[0].nll_grad_terms(oracle_model(env[0], kind, lo, hi), cols, th)
     assert np.all(np.abs(fast[1:] - plain[1:] * 2.0 ** 500) <= 1e-9 * np.abs(terms).sum(1)), (fast, plain)
+
+
+@pytest.mark.parametrize("weighted", [False, True])
+@pytest.mark.parametrize("miss", [0.0, 1e-13, 1e-4])
+@pytest.mark.parametrize("kind", KINDS)
+def test_signal_terms_all_small(env, kind, miss, weighted):
+    """f_b = 1 - miss and a range 9 to 14 sigma under the peak: P is all background, every
+    signal term is 1e-4 and less of what the sums' unit is set for, and the derivative in f_b is
+    made of them.  Against the oracle 1e-7 (the normalisation, as above)."""
+    th = np.array(TRUTH[kind])
+    th[3] = 1.0 - miss
+    cols = columns(kind, 700, 19, weighted)
+    for lo, hi in ((-12.0, -9.0), (-14.0, -11.0)):
+        lo, hi = lo * th[1], hi * th[1]
+        cols["t"] = np.random.default_rng(9).uniform(lo, hi, 700)
+        check(env, kind, lo, hi, cols, th, rtol_f=1e-9, rtol_g=1e-7)
