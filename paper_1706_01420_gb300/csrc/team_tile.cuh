@@ -100,7 +100,7 @@ __device__ __forceinline__ void add_log(double P, double w, const MathTables* mt
 }
 
 // The exponent of the largest |w| of a quarter (0 where all weights are 1, as without
-// weights), or kNoWeight where all are zero.  The lane keeps its weights in wbuf for the
+// weights; -1023 for subnormal ones), or kNoWeight where all are zero.  The lane keeps its weights in wbuf for the
 // quarter: a second read of the column would go over the host link again where it lies in
 // host memory (8e6 weighted 4D events there: read twice per tile 2.14 ms, twice per
 // quarter 1.95, once 1.74).
@@ -113,10 +113,10 @@ __device__ __forceinline__ int weight_exponent(const Cols& cols, int64_t tbase, 
         const int64_t e = tbase + lane + 32 * (i0 + i);
         const double w = e < ev1 ? __ldg(cols.w + e) : 0.0;
         wbuf[i * 32 + lane] = w;
-        hi = max(hi, high_word(w));
+        hi = max(hi, high_word(w) | (int)((unsigned)__double_as_longlong(w) != 0u));   // not 0 for any w but 0
     }
-    const int ex = (int)(__reduce_max_sync(0xffffffffu, (unsigned)hi) >> 20);
-    return ex ? ex - 1023 : kNoWeight;
+    const unsigned most = __reduce_max_sync(0xffffffffu, (unsigned)hi);
+    return most ? (int)(most >> 20) - 1023 : kNoWeight;
 }
 
 // A weighted quarter's scale follows the largest |w| of its tile up to it (run); the sums

@@ -201,3 +201,18 @@ def test_signal_terms_all_small(env, kind, miss, weighted):
         lo, hi = lo * th[1], hi * th[1]
         cols["t"] = np.random.default_rng(9).uniform(lo, hi, 700)
         check(env, kind, lo, hi, cols, th, rtol_f=1e-9, rtol_g=1e-7)
+
+
+@pytest.mark.parametrize("kind", KINDS)
+def test_subnormal_weights(env, kind):
+    """Weights of 2^-1030: the terms and partial sums are subnormal and keep 44 bits at unit size;
+    the constants that multiply them take up to 2^14 of that: 1e-8 of the sum of |terms|."""
+    O, G, torch, api = env
+    th = np.array(TRUTH[kind])
+    cols = columns(kind, 512, 23)
+    unit = gradients(env, kind, 0.0, 15.0, cols, th)
+    cols["w"] = np.full(512, 2.0 ** -1030)
+    tiny = gradients(env, kind, 0.0, 15.0, cols, th)
+    _, terms = O.nll_grad_terms(oracle_model(O, kind, 0.0, 15.0), {k: v for k, v in cols.items() if k != "w"}, th)
+    scale = np.abs(terms).sum(1)
+    assert np.all(np.abs(np.ldexp(np.ldexp(tiny[1:], 1000), 30) - unit[1:]) <= 1e-8 * scale), (tiny, unit)
