@@ -387,6 +387,13 @@ __device__ inline int coef_scale(long long amax) {
     const int sc = 1022 - (int)(amax >> 52);
     return amax < 0x7FF0000000000000ll && sc >= -64 && sc <= 900 ? sc : 9999;
 }
+// The cached basis' coefficients are a bit lower, in [1/4, 1/2): ten of them with |f_k| < 1.5 (nll.cu)
+// stay below 8, which A' in Q60 holds.  (The basis of angles within their domain is below 1.2, but
+// the columns are the caller's.)
+__device__ inline int coef_scale_cached(long long cmax) {
+    const int sc = coef_scale(cmax);
+    return sc == 9999 ? sc : sc - 1;
+}
 __device__ inline int2 coef_ga(double g, int sc) {
     const Fx v = fx(sc == 9999 ? 0 : to_q62(g * __longlong_as_double((long long)(sc + 1023) << 52)));
     return make_int2(v.h, v.l);
@@ -489,7 +496,7 @@ __device__ inline void compute_consts_thread(const ModelDev& m, const double* th
         amax = a > amax ? a : amax;
         cmax = b > cmax ? b : cmax;
     }
-    const int sc = coef_scale(amax), scc = coef_scale(cmax);
+    const int sc = coef_scale(amax), scc = coef_scale_cached(cmax);
     for (int k = 0; k < 10; ++k) {
         c->k.ga[k] = coef_ga(coef_g(c->k.hq, k), sc);
         c->k.gc[k] = coef_ga(c->k.hc[k], scc);
@@ -636,7 +643,7 @@ __device__ inline void compute_consts_block(const ModelDev& m, const double* th,
             const long long v = __shfl_xor_sync(0xffffffffu, amax, o);
             amax = v > amax ? v : amax;
         }
-        const int sc = coef_scale(amax);
+        const int sc = lane < 16 ? coef_scale(amax) : coef_scale_cached(amax);
         if (lane < 10) S->c.k.ga[lane] = coef_ga(g, sc);
         else if (lane >= 16 && lane < 26) S->c.k.gc[lane - 16] = coef_ga(g, sc);
         if (lane == 10) S->c.k.aq = 0.5 * S->c.cs;

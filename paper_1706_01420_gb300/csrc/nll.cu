@@ -258,7 +258,7 @@ __device__ __forceinline__ void plain_rows(const Consts& c, const MathTables* mt
 // by the plain loop.  Either way the tile's sums depend only on its events, never
 // on the launch geometry (team_tile.cuh).
 //
-// The cached basis takes the same path (its f_k converted to Q62, |f_k| < 1.75): 4.2e6 events
+// The cached basis takes the same path (its f_k converted to Q62, |f_k| < 1.5): 4.2e6 events
 // 327 us by the plain loop, 239 here, weighted 431 and 267; 1000 events 58 and 32 (teams).
 //
 // Measured (one pass of the public call, 512 toys of 20 000 events, then 1e7
@@ -400,7 +400,7 @@ struct Angtime {
     }
     static __device__ __forceinline__ bool bad(const Consts&, FastScale sc, const Sums& s) {
         return p_out_of_range(s) || (s.most >> 20) > 1023 - 4 + sc.top ||
-               (CACHED && s.tau_most >= 0x3FFC0000);      // |f_k| < 1.75
+               (CACHED && s.tau_most >= 0x3FF80000);      // |f_k| < 1.5 (coef_scale_cached)
     }
     static __device__ __forceinline__ void accumulators(const Consts&, FastScale sc, const Sums& s, double* acc) {
         const long long S[10] = {s.g[0] - s.g[2], s.g[1] - s.g[3], s.g[1] - s.g[2] + s.g[3], s.g[4], s.g[5],

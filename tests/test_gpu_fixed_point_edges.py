@@ -216,3 +216,36 @@ def test_subnormal_weights(env, kind):
     _, terms = O.nll_grad_terms(oracle_model(O, kind, 0.0, 15.0), {k: v for k, v in cols.items() if k != "w"}, th)
     scale = np.abs(terms).sum(1)
     assert np.all(np.abs(np.ldexp(np.ldexp(tiny[1:], 1000), 30) - unit[1:]) <= 1e-8 * scale), (tiny, unit)
+
+
+def test_cached_columns_add_up_within_their_range(env):
+    """Columns of one sign with the coefficients, up to 1.7 each: A' is up to twice eight times its
+    largest coefficient.  Late events with background, where P stays positive whatever A' is.
+    The whole call, without the odd events, and those alone (fewer than 64: the plain loop)."""
+    O, G, torch, api = env
+    th = np.array([0.66, 0.045, 0.0, 0.5, 0.3045, 0.3433, 0.439, 1.896, 0.2397, 0.1279])
+    h = O.amplitude_coeffs(th)
+    IT = O.time_norm(*th[:3], 0.0, 15.0)
+    largest = np.abs(h).max() * (1.0 - th[3]) / (IT * O.I_OMEGA) / 2.0
+    th[3] = 1.0 - (1.0 - th[3]) * 2.0 ** np.ceil(np.log2(largest)) * 0.98 / largest / 2.0
+    m = api.model_4d(0.0, 15.0)
+    cols = columns("4d", 200, 29)
+    cols["t"][160:] = 14.5
+    ev = G.to_dev(cols)
+    fk = api.ipa_angular_basis(m, ev)
+    for size in (1.2, 1.45, 1.55, 1.7):
+        fk[:, 160:] = torch.tensor(size * np.sign(h), device="cuda")[:, None]
+
+        def part(a, b):
+            return gradients(env, "4d", 0.0, 15.0, {k: np.ascontiguousarray(v[a:b]) for k, v in cols.items()}, th,
+                             cached=fk[:, a:b].contiguous())
+        whole, most, few = part(0, 200), part(0, 160), part(160, 200)
+        P = (1.0 - th[3]) * O.time_conv(14.5, *th[:2]) / IT * size * np.abs(h).sum() / O.I_OMEGA + th[3] / m_volume(O)
+        assert abs(few[0] + 40.0 * np.log(P)) <= 1e-12 * 40.0 * abs(np.log(P))
+        logl, terms = O.nll_grad_terms(O.Model("4d", 0.0, 15.0), {k: v[:160] for k, v in cols.items()}, th)
+        scale = 2.0 * np.append(np.abs(logl).sum(), np.abs(terms).sum(1)) + np.abs(few)
+        assert np.all(np.abs(whole - most - few) <= 1e-12 * scale), (size, whole, most + few)
+
+
+def m_volume(O):
+    return O.Model("4d", 0.0, 15.0).volume
