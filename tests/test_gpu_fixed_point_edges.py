@@ -41,36 +41,63 @@ def oracle_model(O, kind, lo, hi):
     return O.Model("tag" if kind == "tagged" else kind, lo, hi)
 
 
-def gradients(env, kind, lo, hi, cols, th, cached=False):
+def gradients(env, kind, lo, hi, cols, th, cached=None):
     """The call with one warp per tile and with a team per tile: the same bits."""
     _, G, torch, api = env
     m = getattr(api, "model_" + kind)(lo, hi)
     n = len(cols["t"])
     ev = G.to_dev(cols)
-    if cached:
-        ev["fk"] = cached if isinstance(cached, torch.Tensor) else api.ipa_angular_basis(m, ev)
+    if cached is not None:
+        ev["fk"] = cached
     theta = torch.tensor(np.asarray(th), device="cuda")
     got = {}
     try:
         for warps in (1, 2):
             api.ipa_launch_config_set(m, n, {"warps_per_block": warps, "warps_per_sm": 0, "tiles_per_take": 1},
-                                      cached=bool(ev.get("fk") is not None))
+                                      cached=cached is not None)
             got[warps] = api.ipa_nll_grad(m, ev, theta).cpu().numpy()
     finally:
         api.ipa_launch_config_set(m, n, {"warps_per_block": 1, "warps_per_sm": 0, "tiles_per_take": 1},
-                                  cached=bool(ev.get("fk") is not None))
+                                  cached=cached is not None)
     assert np.array_equal(got[1], got[2], equal_nan=True), (got[1], got[2])
     return got[1]
 
 
-def check(env, kind, lo, hi, cols, th, rtol_f=1e-14, rtol_g=5e-13):
+def check(env, kind, lo, hi, cols, th):
     O = env[0]
     got = gradients(env, kind, lo, hi, cols, th)
     m = oracle_model(O, kind, lo, hi)
     f, g = O.nll_grad(m, cols, th)
     logl, terms = O.nll_grad_terms(m, cols, th)
-    assert abs(got[0] - f) <= rtol_f * np.abs(logl).sum(), (got[0], f)
-    assert np.all(np.abs(got[1:] - g) <= rtol_g * np.abs(terms).sum(1)), (got[1:], g)
+    assert abs(got[0] - f) <= 1e-14 * np.abs(logl).sum(), (got[0], f)
+    assert np.all(np.abs(got[1:] - g) <= 5e-13 * np.abs(terms).sum(1)), (got[1:], g)
+
+
+def by_the_plain_loop(env, kind, lo, hi, cols, th):
+    """The same gradient from the FP64 loop, which the oracle tests cover elsewhere (a range
+    under the peak has a normalisation that cancels in FP64, the oracle's and the library's
+    differently, so there the two paths of the library are compared).  4D and phi_s: as fits
+    of fewer than 64 events, which take it; 1D and tagged: with weights of 2^-500, whose scale
+    is out of the integers' range and which multiply every sum exactly."""
+    _, G, torch, api = env
+    m = getattr(api, "model_" + kind)(lo, hi)
+    n = len(cols["t"])
+    if kind in ("1d", "tagged"):
+        w = cols.get("w", np.ones(n))
+        return np.ldexp(gradients(env, kind, lo, hi, {**cols, "w": np.ldexp(w, -500)}, th), 500)
+    off = np.append(np.arange(0, n, 60), n)
+    out = api.ipa_nll_grad_segmented(m, G.to_dev(cols), torch.tensor(off, device="cuda"),
+                                     torch.tensor(np.tile(th, (len(off) - 1, 1)), device="cuda"))
+    return out.cpu().numpy().sum(0)
+
+
+def check_paths(env, kind, lo, hi, cols, th, rtol):
+    fast, plain = gradients(env, kind, lo, hi, cols, th), by_the_plain_loop(env, kind, lo, hi, cols, th)
+    logl, terms = env[0].nll_grad_terms(oracle_model(env[0], kind, lo, hi), cols, th)
+    scale = np.abs(terms).sum(1)
+    assert np.isfinite(plain).all() and np.isfinite(scale).all()
+    assert abs(fast[0] - plain[0]) <= 1e-13 * np.abs(logl).sum(), (fast, plain)
+    assert np.all(np.abs(fast[1:] - plain[1:]) <= rtol * scale), (fast, plain)
 
 
 @pytest.mark.parametrize("weighted", [False, True])
@@ -151,17 +178,16 @@ def test_fit_of_one_parameter_from_outside_the_domain(env):
 
 
 @pytest.mark.parametrize("kind", ["1d", "tagged"])
-@pytest.mark.parametrize("sigmas", [24.0, 26.0, 30.0])
+@pytest.mark.parametrize("sigmas", [20.0, 24.0, 26.0, 28.0])
 def test_no_scale_far_below_the_peak(env, kind, sigmas):
-    """A range that ends 24 sigma and more below mu: cs is beyond the integers' scale.  The
-    normalisation cancels to |x| / (Gamma sigma) = 1e3 times FP64's rounding and its
-    derivative in sigma once more: 1e-7 of the sum of |terms| (a tile that was left out
-    gave nothing)."""
+    """A range that ends 24 sigma and more below mu: cs is beyond the integers' scale, and both
+    calls take the plain loop (a tile that was left out gave nothing): 5e-13 of the sum of |terms|;
+    20 sigma is within it, at the next test's tolerance."""
     th = np.array(TRUTH[kind])
     cols = columns(kind, 3000, 13)
     hi = -sigmas * th[1]
     cols["t"] = np.random.default_rng(3).uniform(hi - 3.0 * th[1], hi, 3000)
-    check(env, kind, hi - 3.0 * th[1], hi, cols, th, rtol_f=1e-9, rtol_g=1e-7)
+    check_paths(env, kind, hi - 3.0 * th[1], hi, cols, th, 1e-9 if sigmas == 20.0 else 5e-13)
 
 
 @pytest.mark.parametrize("kind", ["1d", "tagged"])
@@ -169,22 +195,16 @@ def test_no_scale_far_below_the_peak(env, kind, sigmas):
 @pytest.mark.parametrize("f_b", [0.0, 0.1, 0.99])
 @pytest.mark.parametrize("below", [6.0, 8.0, 10.0, 14.0, 16.0, 18.0, 20.0, 22.0])
 def test_gaussian_sums_below_the_peak(env, kind, sigma, f_b, below):
-    """Ranges of 3.5 sigma that end `below` sigma under mu.  A weight of 2^-500 takes the tile
-    to the plain loop and scales every sum exactly, so that loop's gradient is at hand.  The
-    integers' unit against the pieces of a component, which cancel to sigma / (|tau| Gamma sigma)
-    of themselves, and again in sigma: 1e3 times (|tau| / sigma)^2 units of 2^-49, below 1e-9 of
-    the sum of |terms| for |tau| = 26 sigma.  Against the oracle 1e-7, as above."""
-    _, G, torch, api = env
+    """Ranges of 3.5 sigma that end `below` sigma under mu.  The integers' unit against the
+    pieces of a component, which cancel to sigma / (|tau| Gamma sigma) of themselves, and again
+    in sigma: 1e3 times (|tau| / sigma)^2 units of 2^-49, below 1e-9 of the sum of |terms| for
+    |tau| = 26 sigma."""
     th = np.array(TRUTH[kind])
     th[1], th[3] = sigma, f_b
     hi, lo = -below * sigma, -(below + 3.5) * sigma
     cols = columns(kind, 1500, 17)
     cols["t"] = np.random.default_rng(5).uniform(lo, hi, 1500)
-    check(env, kind, lo, hi, cols, th, rtol_f=1e-9, rtol_g=1e-7)
-    fast = gradients(env, kind, lo, hi, cols, th)
-    plain = gradients(env, kind, lo, hi, {**cols, "w": np.full(1500, 2.0 ** -500)}, th)
-    _, terms = env[0].nll_grad_terms(oracle_model(env[0], kind, lo, hi), cols, th)
-    assert np.all(np.abs(fast[1:] - plain[1:] * 2.0 ** 500) <= 1e-9 * np.abs(terms).sum(1)), (fast, plain)
+    check_paths(env, kind, lo, hi, cols, th, 1e-9)
 
 
 @pytest.mark.parametrize("weighted", [False, True])
@@ -193,14 +213,14 @@ def test_gaussian_sums_below_the_peak(env, kind, sigma, f_b, below):
 def test_signal_terms_all_small(env, kind, miss, weighted):
     """f_b = 1 - miss and a range 9 to 14 sigma under the peak: P is all background, every
     signal term is 1e-4 and less of what the sums' unit is set for, and the derivative in f_b is
-    made of them.  Against the oracle 1e-7 (the normalisation, as above)."""
+    made of them.  1e-9 of the sum of |terms|, as above."""
     th = np.array(TRUTH[kind])
     th[3] = 1.0 - miss
     cols = columns(kind, 700, 19, weighted)
     for lo, hi in ((-12.0, -9.0), (-14.0, -11.0)):
         lo, hi = lo * th[1], hi * th[1]
         cols["t"] = np.random.default_rng(9).uniform(lo, hi, 700)
-        check(env, kind, lo, hi, cols, th, rtol_f=1e-9, rtol_g=1e-7)
+        check_paths(env, kind, lo, hi, cols, th, 1e-9)
 
 
 @pytest.mark.parametrize("kind", KINDS)
