@@ -432,16 +432,21 @@ team_kernel(Cols cols, int64_t n, const int64_t* __restrict__ seg_begin, const i
     work_done(work, lane);
 }
 
-// Whether a launch of about `tiles` tiles goes to the teams: the built-in geometry (a tuned or
-// given one is for single warps) and at most eight tiles per SM.  Measured, call by call, single
-// warps / teams in us: 16 to 152 tiles 35 / 24 (1D), 56 / 33 (4D), 78 / 41 (tagged); 608 tiles 38 / 28,
-// 64 / 42, 83 / 69; 1216 tiles (eight per SM) 44 / 40, 75 / 64, 100 / 92; 1520 tiles 45 / 47, 76 / 75,
-// 108 / 115; 2048 tiles 51 / 56, 87 / 90, 125 / 137 (a tile's exchange then costs more than the
-// evener load gains).
-constexpr int kTeamTilesPerSm = 8;
-inline bool launch_team_ok(const LaunchCfg& cfg, int64_t tiles) {
-    return cfg.warps_per_block == 1 && cfg.warps_per_sm == 0 && cfg.tiles_per_take == 1 &&
-           tiles <= (int64_t)kTeamTilesPerSm * sm_count();
+// Whether a launch over n events in n_seg segments goes to the teams: the built-in geometry (a
+// tuned or given one is for single warps) and at most eight tiles per SM.  Measured, call by call,
+// single warps / teams in us: 16 to 152 tiles 35 / 24 (1D), 56 / 33 (4D), 78 / 41 (tagged); 608 tiles
+// 38 / 28, 64 / 42, 83 / 69; 1216 tiles (eight per SM) 44 / 40, 75 / 64, 100 / 92; 1520 tiles 45 / 47,
+// 76 / 75, 108 / 115; 2048 tiles 51 / 56, 87 / 90, 125 / 137 (a tile's exchange then costs more than
+// the evener load gains).  Segments of up to a quarter tile (128 events) leave three of a team's warps
+// idle: four tiles per SM there (segments of 20 events: 600 of them 42 / 35, 61 / 50, 67 / 66; 1000
+// 52 / 55, 73 / 83, 76 / 92).
+constexpr int kTeamTilesPerSm = 8, kTeamShortPerSm = 4;
+inline bool launch_team_ok(const LaunchCfg& cfg, int64_t n, int n_seg) {
+    if (cfg.warps_per_block != 1 || cfg.warps_per_sm != 0 || cfg.tiles_per_take != 1) return false;
+    // a tile at least per segment
+    const int64_t tiles = n_seg > 1 && tile_estimate(n, n_seg) < n_seg ? n_seg : tile_estimate(n, n_seg);
+    const bool few = n_seg > 1 && n <= (int64_t)n_seg * (32 * kSub);
+    return tiles <= (int64_t)(few ? kTeamShortPerSm : kTeamTilesPerSm) * sm_count();
 }
 
 template <class M, bool W>
