@@ -55,7 +55,8 @@ constexpr int kBkgChunk = 512;           // background events per ticket
 // A ticket is 1, 2, 4, ... kGenMaxSub times kGenCand candidates, as many as
 // accept kGenMinKept events on average: the look-back's status words then
 // stay below 1.3 bytes per event.  A toy of an envelope that accepts less is
-// one ticket.
+// one ticket: a warp alone (with tickets of at most 64 units, a range of 2e4
+// lifetimes was one: 300 1D events 624 ms, 142 at a block per toy).
 constexpr int kGenMinKept = 8;
 // ... and more where there is work enough: while kGenPerWarp tickets per resident
 // warp are left and a ticket's events fit the list (kGenPick) with room to spare.
@@ -64,7 +65,7 @@ constexpr int kGenMinKept = 8;
 // and 102 us.
 constexpr int kGenMostKept = 160;
 constexpr int kGenPerWarp = 16;
-constexpr int kGenMaxSub = 64;
+constexpr int kGenMaxSub = 1 << 12;      // a tenth of a second of one warp; acceptances down to 2e-6 are cut
 
 // What a test says of a candidate.
 enum GenCode { kDrop = 0, kKeep = 1, kTest32 = 2, kTest64 = 3 };
@@ -125,7 +126,7 @@ __device__ __forceinline__ GenCode decide32(float lhs, float dl, float v, float 
 struct GenLists {
     uint16_t l32[kGenCand];
     uint16_t l64[kGenCand];
-    uint16_t pick[kGenPick];
+    uint32_t pick[kGenPick];
     uint32_t keep[32];
     int64_t ns, off, got;          // the toy's signal, its first event, events accepted before unit u
     int64_t tk, local, n_chunks;   // ticket, its chunk of the toy, the toy's chunks
@@ -207,7 +208,7 @@ __device__ __forceinline__ void gen_pick(GenLists& L, uint32_t word, int pre, in
     for (int r = pre - r0; word && r < kGenPick; ++r) {
         const int bit = __ffs((int)word) - 1;
         word &= word - 1u;
-        if (r >= 0) L.pick[r] = (uint16_t)(off + lane * 32 + bit);
+        if (r >= 0) L.pick[r] = (uint32_t)(off + lane * 32 + bit);
     }
 }
 
