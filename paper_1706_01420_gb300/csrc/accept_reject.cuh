@@ -472,10 +472,17 @@ ipa_status launch_generator(GenArgs A, cudaStream_t s) {
         cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, generate_kernel<G>, kBlock, smem);
         per_sm = e == cudaSuccess && v >= 1 ? v : 1;
     }
-    // (n_sig + 3 sqrt(n_sig) + 8) / kGenMinKept + 2 <= n_sig / 5 + 4, and one per kBkgChunk background events
-    const int64_t max_tickets = A.capacity / 5 + 5 * (int64_t)A.n_toys + A.capacity / kBkgChunk + 1;
-    const size_t words = (size_t)A.n_toys + 3 + (size_t)max_tickets;
     const int64_t most = (int64_t)sm_count() * per_sm;
+    // Tickets at most, one per kBkgChunk background events among them.  A ticket accepts kept >=
+    // kGenMinKept = 8 of a toy's n + 3 sqrt(n) + 8 events on average: n / 5 + 4 tickets.  With many
+    // events it is larger: kept > kGenMostKept / 2, n / 40 + 2 tickets, or kept > events / (2
+    // kGenPerWarp warps), 2 kGenPerWarp per warp, n / 128 and 7 a toy (3 sqrt(n) <= n / 16 + 36).  The
+    // workspace follows what the events in work can need, not the buffers alone: 1000 events
+    // into buffers of 2e8 took 90 us with n / 5 words to reset.
+    const int64_t few = A.capacity / 5 + 4 * (int64_t)A.n_toys;
+    const int64_t many = A.capacity / 40 + 2 * kGenPerWarp * kGenWarps * most + 7 * (int64_t)A.n_toys;
+    const int64_t max_tickets = (few < many ? few : many) + A.capacity / kBkgChunk + A.n_toys + 1;
+    const size_t words = (size_t)A.n_toys + 3 + (size_t)max_tickets;
     void* ws = nullptr;
     if (pool_alloc(&ws, words * 8, s, "generator workspace") == IPA_OK) {
         ipa_status st = cuda_fail(cudaMemsetAsync(ws, 0, words * 8, s), "generator workspace reset");

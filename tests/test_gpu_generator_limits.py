@@ -55,3 +55,17 @@ def test_tickets_of_many_units(api, kind, hi):
     a = generate(api, kind, hi, 41, n_sig, n_bkg)
     assert all(np.isfinite(v).all() for v in a.values())
     assert same(a, without_workspace(api, kind, hi, 41, n_sig, n_bkg))
+
+
+@pytest.mark.parametrize("kind", list(COLS))
+def test_buffers_larger_than_the_events(api, kind):
+    """The workspace follows the events, not the buffers alone: the same events in 3e7 of room,
+    and a batch of many toys in buffers of its own size."""
+    generate(api, kind, 15.0, 3, [1], [0])
+    n_sig, n_bkg = [900, 0, 20000], [5, 1000, 0]
+    a = generate(api, kind, 15.0, 43, n_sig, n_bkg, room=30_000_000)
+    assert same(a, generate(api, kind, 15.0, 43, n_sig, n_bkg))
+    rng = np.random.default_rng(3)
+    n_sig = rng.integers(0, 4000, 3000)
+    n_bkg = rng.integers(0, 40, 3000)
+    assert same(generate(api, kind, 15.0, 47, n_sig, n_bkg), without_workspace(api, kind, 15.0, 47, n_sig, n_bkg))
