@@ -136,8 +136,9 @@ __device__ __forceinline__ bool scale_to(FastScale* sc, int base, int run) {
 
 // The integers' unit is set for typical factors.  A tile whose largest factor lies far below
 // (every signal term small beside the background, as far from the peak with f_b near 1) would
-// keep few of its bits.  `most`: the tile's largest factor (high word); not asked where all
-// weights are zero, which the integers hold exactly.
+// keep few of its bits: below 2^-3 to 2^-4 of a typical one the FP64 loop adds it.  `most`: the
+// tile's largest factor (high word); not asked where all weights are zero, which the integers
+// hold exactly.
 template <class M>
 __device__ __forceinline__ bool too_small(int most, FastScale sc, int run) {
     return run != kNoWeight && most < (1023 + sc.top - M::kLeast) << 20;

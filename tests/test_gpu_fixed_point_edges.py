@@ -178,7 +178,7 @@ def test_fit_of_one_parameter_from_outside_the_domain(env):
 
 
 @pytest.mark.parametrize("kind", ["1d", "tagged"])
-@pytest.mark.parametrize("sigmas", [20.0, 24.0, 26.0, 28.0])
+@pytest.mark.parametrize("sigmas", [20.0, 24.0, 26.0])
 def test_no_scale_far_below_the_peak(env, kind, sigmas):
     """A range that ends 24 sigma and more below mu: cs is beyond the integers' scale, and both
     calls take the plain loop (a tile that was left out gave nothing): 5e-13 of the sum of |terms|;

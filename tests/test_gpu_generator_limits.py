@@ -28,7 +28,7 @@ def generate(api, kind, hi, seed, n_sig, n_bkg, room=0):
     off = np.concatenate([[0], np.cumsum(n_sig + n_bkg)]).astype(np.int64)
     out = {k: torch.full((int(off[-1]) + room,), -7.0, dtype=torch.float64, device="cuda") for k in COLS[kind]}
     dev = [torch.tensor(a, device="cuda") for a in (n_sig, n_bkg, off[:-1].copy())]
-    api.ipa_toygen(m, torch.tensor(THETA[kind], device="cuda"), seed, *dev, out)
+    api.ipa_toygen(m, torch.tensor(THETA[kind], dtype=torch.float64, device="cuda"), seed, *dev, out)
     torch.cuda.synchronize()
     assert all(bool((v[int(off[-1]):] == -7.0).all()) for v in out.values())
     return {k: v[:int(off[-1])].cpu().numpy() for k, v in out.items()}
