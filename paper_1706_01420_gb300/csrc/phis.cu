@@ -626,12 +626,12 @@ const auto slow_of = [&](int k) {
                         const int64_t e = tbase + lane + 32 * (i0 + k);
                         if (e < ev1) phis_event_fast<WEIGHTED, CACHED>(pw, &mt, cols, e, slow_of(k), top, acc, S, &prod, &esum, &bad);
                     }
-                    // (none of the sums reaches 2^-6 of a typical term's 2^48 units: few of their bits would be
+                    // (none of the sums reaches 2^-4 of a typical term's 2^48 units: few of their bits would be
                     // left, as far from the peak with f_b near 1)
                     unsigned long long mag = 0;
 #pragma unroll
                     for (int a = 0; a < 14; ++a) mag |= (unsigned long long)(S[a] ^ (S[a] >> 63));
-                    plain = __any_sync(0xffffffffu, bad) || !__any_sync(0xffffffffu, (mag >> 42) != 0ull);
+                    plain = __any_sync(0xffffffffu, bad) || !__any_sync(0xffffffffu, (mag >> 44) != 0ull);
 #pragma unroll
                     for (int a = 0; a < NA; ++a) {
                         if (a >= kE && a < kPhi) acc[a] = fx_to_double(S[a - kE], top + 1);
