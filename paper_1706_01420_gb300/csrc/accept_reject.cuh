@@ -380,6 +380,64 @@ __global__ void __launch_bounds__(kBlock, G::kBlocksPerSm) generate_kernel(const
     }
 }
 
+// A block per toy, its warps 128 candidates each at a time: for the few events of G::kBlockEvents
+// and fewer per toy, where a warp's 1024 candidates at once are most of the toy's and the
+// tickets cost two launches.  1D, one toy of 100 / 500 / 1000 events: 37 us by tickets, 26 / 63 / 110
+// by one warp, 19 / 27 / 35 so.
+template <class G>
+__global__ void __launch_bounds__(kBlock) generate_block_kernel(const __grid_constant__ GenArgs A) {
+    constexpr int kRows = 4;
+    __shared__ typename G::Shared S;
+    __shared__ int s_kept[2][kGenWarps];
+    G::setup(S, A);
+    __syncthreads();
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const unsigned below = (1u << lane) - 1u;
+    const bool usable = G::usable(S);
+    int turn = 0;
+    for (int toy = blockIdx.x; toy < A.n_toys; toy += gridDim.x) {
+        int64_t ns, nb, off;
+        if (!gen_toy(A, toy, &ns, &nb, &off)) continue;
+        for (int64_t i = threadIdx.x; i < nb; i += kBlock)
+            G::background(S, A, GenIdx{(uint32_t)i, (uint32_t)((uint64_t)i >> 32), (uint32_t)toy}, off + ns + i);
+        const uint64_t budget = usable ? (uint64_t)ns * 65536ull + (1ull << 22) : 0ull;    // as generate_kernel
+        int64_t got = 0;
+        for (uint64_t j0 = 0; got < ns && j0 < budget; j0 += kRows * kBlock, turn ^= 1) {
+            const uint64_t j1 = j0 + (uint64_t)(wib * kRows * 32 + lane);
+            unsigned kept[kRows];
+            int n = 0;
+#pragma unroll
+            for (int r = 0; r < kRows; ++r) {
+                const uint64_t jr = j1 + 32u * r;
+                const GenIdx j = {(uint32_t)jr, (uint32_t)(jr >> 32), (uint32_t)toy};
+                GenCode c = G::quick(S, A, j);
+                if (c == kTest32) c = G::test32(S, A, j);
+                if (c == kTest64) c = G::test64(S, A, j) ? kKeep : kDrop;
+                kept[r] = __ballot_sync(0xffffffffu, c == kKeep);
+                n += __popc(kept[r]);
+            }
+            if (lane == 0) s_kept[turn][wib] = n;
+            __syncthreads();                         // (the next round writes the other half)
+            int64_t pos = got;
+#pragma unroll
+            for (int w = 0; w < kGenWarps; ++w) {
+                const int v = s_kept[turn][w];
+                pos += w < wib ? v : 0;
+                got += v;
+            }
+#pragma unroll
+            for (int r = 0; r < kRows; ++r) {
+                const int64_t at = pos + __popc(kept[r] & below);
+                const uint64_t jr = j1 + 32u * r;
+                if ((kept[r] >> lane & 1u) && at < ns)
+                    G::signal(S, A, GenIdx{(uint32_t)jr, (uint32_t)(jr >> 32), (uint32_t)toy}, off + at);
+                pos += __popc(kept[r]);
+            }
+        }
+        for (int64_t pos = got + threadIdx.x; pos < ns; pos += kBlock) G::fill_nan(A, off + pos);
+    }
+}
+
 // Tickets per toy, their prefix and the candidates per ticket (one block).
 // Signal chunks: enough for n_sig + 3 sqrt(n_sig) + 8 accepted candidates at the
 // model's acceptance; one (whose warp goes on alone) where even the largest
@@ -454,8 +512,8 @@ __global__ void gen_tickets_kernel(const __grid_constant__ GenArgs A, int64_t ma
 
 // consts.cu's record is in place on the stream.  The workspace (ticket prefix,
 // counter, status words) is allocated in stream order and given back after the
-// kernel; without it (no memory) a warp generates a toy alone, with the same
-// events.
+// kernel; without it (no memory, or many toys of few events) a warp generates a
+// toy alone, with the same events.
 template <class G>
 ipa_status launch_generator(GenArgs A, cudaStream_t s) {
     int dev = 0;
@@ -483,8 +541,18 @@ ipa_status launch_generator(GenArgs A, cudaStream_t s) {
     const int64_t many = A.capacity / 40 + 2 * kGenPerWarp * kGenWarps * most + 7 * (int64_t)A.n_toys;
     const int64_t max_tickets = (few < many ? few : many) + A.capacity / kBkgChunk + A.n_toys + 1;
     const size_t words = (size_t)A.n_toys + 3 + (size_t)max_tickets;
+    // Few events per toy, by the buffers' room: a block per toy while all are resident at once, a warp
+    // per toy beyond (1D, 2000 toys of 10 / 100 and 5000 of 300: 34 / 45 / 138 us, by tickets 92 / 100 / 197)
+    bool tickets = true;
+    if constexpr (G::kBlockEvents > 0) {
+        if (A.n_toys <= 4 * sm_count() && A.capacity <= (int64_t)G::kBlockEvents * A.n_toys) {
+            generate_block_kernel<G><<<A.n_toys, kBlock, 0, s>>>(A);
+            return cuda_fail(cudaGetLastError(), "toygen kernel launch");
+        }
+        tickets = A.n_toys <= 4 * sm_count() || A.capacity > (int64_t)G::kBlockEvents / 2 * A.n_toys;
+    }
     void* ws = nullptr;
-    if (pool_alloc(&ws, words * 8, s, "generator workspace") == IPA_OK) {
+    if (tickets && pool_alloc(&ws, words * 8, s, "generator workspace") == IPA_OK) {
         ipa_status st = cuda_fail(cudaMemsetAsync(ws, 0, words * 8, s), "generator workspace reset");
         int64_t* base = static_cast<int64_t*>(ws);
         A.base = base;

@@ -811,7 +811,7 @@ __device__ double phis_rate_exact(const PhisConsts& c, const MathTables* mt, dou
 // (gL + gH + 2 C) (rel + 3 ef), doubled to spare.
 struct PhisGen {
     static constexpr bool kQuickKeeps = true, kQuick64 = true;
-    static constexpr int kBlocksPerSm = 3, kUnroll = 1;
+    static constexpr int kBlocksPerSm = 3, kUnroll = 1, kBlockEvents = 0;
     struct Shared {
         PhisConsts c;
         MathTables mt;

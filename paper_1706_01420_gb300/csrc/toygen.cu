@@ -158,6 +158,7 @@ struct TimeGen {
     static constexpr bool kQuickKeeps = !ANGLES, kQuick64 = !ANGLES;
     static constexpr int kBlocksPerSm = 4;
     static constexpr int kUnroll = ANGLES ? 2 : 1;    // two candidates' Philox chains at once
+    static constexpr int kBlockEvents = ANGLES ? 0 : 1000;
     struct Shared {
         Consts c;
         Filter32 f;
@@ -303,7 +304,7 @@ struct TimeGen {
 // oscillation, near the peak with FP32 erfc and Faddeeva functions.
 struct TagGen {
     static constexpr bool kQuickKeeps = false, kQuick64 = false;
-    static constexpr int kBlocksPerSm = 3, kUnroll = 1;
+    static constexpr int kBlocksPerSm = 3, kUnroll = 1, kBlockEvents = 0;
     struct Shared {
         TagConsts c;
         Conv32 v;

@@ -69,3 +69,33 @@ def test_buffers_larger_than_the_events(api, kind):
     n_sig = rng.integers(0, 4000, 3000)
     n_bkg = rng.integers(0, 40, 3000)
     assert same(generate(api, kind, 15.0, 47, n_sig, n_bkg), without_workspace(api, kind, 15.0, 47, n_sig, n_bkg))
+
+
+@pytest.mark.parametrize("toys, most", [(1, 1), (1, 130), (1, 1000), (3, 900), (600, 90), (700, 3), (2000, 60)])
+def test_few_events_per_toy(api, toys, most):
+    """1D calls of few events: a block per toy, or a warp per toy where there are many, by
+    the room of the buffers; the events are those of the tickets, which the same call takes in
+    buffers of ample room, and the oracle's."""
+    from oracle import ipa_oracle as O
+    rng = np.random.default_rng(toys + most)
+    n_sig, n_bkg = rng.integers(0, most + 1, toys), rng.integers(0, most // 8 + 1, toys)
+    n_sig[0], n_bkg[0] = most, most // 9
+    generate(api, "1d", 15.0, 3, [1], [0])
+    a = generate(api, "1d", 15.0, (3 << 34) + 5, n_sig, n_bkg)
+    assert same(a, generate(api, "1d", 15.0, (3 << 34) + 5, n_sig, n_bkg, room=1000 * toys + 1))
+    ref = O.toy_one(O.Model("1d", 0.0, 15.0), np.array(THETA["1d"]), (3 << 34) + 5, 0, most, most // 9)
+    assert np.array_equal(a["t"][:most + most // 9], ref["t"])
+
+
+@pytest.mark.parametrize("sigma", [np.nan, -1.0])
+def test_few_events_and_bad_parameters(api, sigma):
+    m = api.model_1d(0.0, 15.0)
+    th = torch.tensor([0.66, sigma, 0.0, 0.1], dtype=torch.float64, device="cuda")
+    got = {}
+    i64 = lambda v: torch.tensor([v], dtype=torch.int64, device="cuda")
+    for room in (70, 5000):
+        t = torch.full((room,), -7.0, dtype=torch.float64, device="cuda")
+        api.ipa_toygen(m, th, 9, i64(60), i64(10), i64(0), {"t": t})
+        got[room] = t.cpu().numpy()
+    assert np.array_equal(got[70], got[5000][:70], equal_nan=True)
+    assert np.all(got[5000][70:] == -7.0) and np.isfinite(got[70][60:]).all()
