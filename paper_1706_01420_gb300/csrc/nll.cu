@@ -349,7 +349,7 @@ struct Angtime {
     using Record = Consts;
     using Slow = double2;
     // FP64: sum r, sum r A' tau T2, sum r A' Gx, sum r A' tau Gx, sum w log P; integers: r T g_k
-    static constexpr int kTopRange = 900, kLeast = 16, kSums = 5, kInts = 10, NA = n_acc(IPA_MODEL_ANGTIME4D, true);
+    static constexpr int kTopRange = 900, kLeast = 16, kPlainBelow = kFewEvents, kSums = 5, kInts = 10, NA = n_acc(IPA_MODEL_ANGTIME4D, true);
     using Sums = FastSums<kSums, kInts>;
 
     static __device__ __forceinline__ bool usable(const Consts& c, int64_t events, FastScale* sc) {
@@ -433,7 +433,7 @@ struct Time1d {
     using Record = Consts;
     using Slow = double2;
     // FP64: sum r, sum w log P; integers: r T, r Gx, r tau T, r tau Gx (the factor A' = cs/2 outside)
-    static constexpr int kTopRange = 400, kLeast = 14, kSums = 2, kInts = 4, NA = n_acc(IPA_MODEL_TIME1D, true);
+    static constexpr int kTopRange = 400, kLeast = 14, kPlainBelow = 0, kSums = 2, kInts = 4, NA = n_acc(IPA_MODEL_TIME1D, true);
     using Sums = FastSums<kSums, kInts>;
 
     static __device__ __forceinline__ bool usable(const Consts& c, int64_t events, FastScale* sc) {
@@ -659,7 +659,7 @@ ipa_status launch_t(const Cols& cols, int64_t n, const int64_t* seg_begin, const
     const int64_t tiles = tile_estimate(n, n_seg);
     const LaunchCfg cfg = force ? *force : launch_cfg(KIND, GRAD, CACHED, n_seg > 1, tiles);
     if constexpr (GRAD) {
-        if (launch_team_ok(cfg, n, n_seg))
+        if (launch_team_ok(cfg, n, n_seg, Model<KIND, CACHED>::kPlainBelow))
             return launch_team<Model<KIND, CACHED>, WEIGHTED>(cols, n, seg_begin, seg_end, seg_tiles, n_seg, consts, sc, out,
                                                       n_par, tiles, st);
     }

@@ -157,7 +157,7 @@ struct Tagged {
     using Record = TagConsts;
     using Slow = TagSlow;
     // FP64: sum r, sum w log P; integers: the six sums in the order above, then times tau (not r q Gx)
-    static constexpr int kTopRange = 400, kLeast = 14, kSums = 2, kInts = 11, NA = n_acc(IPA_MODEL_TAGGED1D, true);
+    static constexpr int kTopRange = 400, kLeast = 14, kPlainBelow = 0, kSums = 2, kInts = 11, NA = n_acc(IPA_MODEL_TAGGED1D, true);
     using Sums = FastSums<kSums, kInts>;
 
     static __device__ __forceinline__ bool usable(const TagConsts& c, int64_t events, FastScale* sc) {
@@ -332,7 +332,7 @@ ipa_status launch_tag_t(const Cols& cols, int64_t n, const int64_t* seg_begin, c
     const int64_t tiles = tile_estimate(n, n_seg);
     const LaunchCfg cfg = force ? *force : launch_cfg(IPA_MODEL_TAGGED1D, GRAD, false, n_seg > 1, tiles);
     if constexpr (GRAD) {
-        if (launch_team_ok(cfg, n, n_seg))
+        if (launch_team_ok(cfg, n, n_seg, Tagged::kPlainBelow))
             return launch_team<Tagged, WEIGHTED>(cols, n, seg_begin, seg_end, seg_tiles, n_seg, consts, sc, out, n_par,
                                                  tiles, st);
     }

@@ -15,6 +15,7 @@
 //   Record, Slow (a near-peak event's values), kSums: FP64 sums, kInts: integer sums, NA;
 //   usable(c, events, &sc)                      the scales at unit weight, false: plain loop;
 //   kTopRange                                   |sc.top| beyond it: plain loop;
+//   kPlainBelow                                 segments of fewer events never use the integers;
 //   kLeast                                      no factor of the tile reaches 2^(top - kLeast): plain loop;
 //   quarter<W>(c, mt, cols, tbase, i0, ev1, sbuf, wbuf, lane, sc, s);   (wbuf: the lane's weights)
 //   bad(c, sc, s)                               a value left its range;
@@ -440,13 +441,16 @@ team_kernel(Cols cols, int64_t n, const int64_t* __restrict__ seg_begin, const i
 // 76 / 75, 108 / 115; 2048 tiles 51 / 56, 87 / 90, 125 / 137 (a tile's exchange then costs more than
 // the evener load gains).  Segments of up to a quarter tile (128 events) leave three of a team's warps
 // idle: four tiles per SM there (segments of 20 events: 600 of them 42 / 35, 61 / 50, 67 / 66; 1000
-// 52 / 55, 73 / 83, 76 / 92).
+// 52 / 55, 73 / 83, 76 / 92).  Segments below `plain_below` events take the plain loop in either form:
+// a warp each while there are at most as many as SMs (4D, 1, 30 and 100 segments of 20 events: 31 / 35,
+// 37 / 41, 38 / 42; 200, two to an SM, 55 / 44).
 constexpr int kTeamTilesPerSm = 8, kTeamShortPerSm = 4;
-inline bool launch_team_ok(const LaunchCfg& cfg, int64_t n, int n_seg) {
+inline bool launch_team_ok(const LaunchCfg& cfg, int64_t n, int n_seg, int plain_below) {
     if (cfg.warps_per_block != 1 || cfg.warps_per_sm != 0 || cfg.tiles_per_take != 1) return false;
     // a tile at least per segment
     const int64_t tiles = n_seg > 1 && tile_estimate(n, n_seg) < n_seg ? n_seg : tile_estimate(n, n_seg);
     const bool few = n_seg > 1 && n <= (int64_t)n_seg * (32 * kSub);
+    if (n < (int64_t)n_seg * plain_below && tiles <= sm_count()) return false;
     return tiles <= (int64_t)(few ? kTeamShortPerSm : kTeamTilesPerSm) * sm_count();
 }
 
