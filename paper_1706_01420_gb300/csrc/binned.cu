@@ -152,19 +152,19 @@ __device__ __forceinline__ int poisson_bin(const BinTable& t, const unsigned lon
 }
 
 // Tables of n_tab histograms over the same bins (table h: means lam, plus add
-// for h = 1).  Bin x = h n_bins + i has kTabFixed entries at x kTabFixed; a
-// longer table goes to the part behind them, whose entries *more counts.
+// for h = 1).  Bin x = h n_bins + i has `fixed` entries at x fixed; a longer
+// table goes to the part behind them, whose entries *more counts.
 __global__ void __launch_bounds__(kTabBlock)
-table_kernel(const double* __restrict__ lam, const double* __restrict__ add, int64_t n_bins, int n_tab,
+table_kernel(const double* __restrict__ lam, const double* __restrict__ add, int64_t n_bins, int n_tab, int fixed,
              BinTable* __restrict__ tab, unsigned long long* __restrict__ T, unsigned long long* __restrict__ more) {
     const int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (x >= n_bins * n_tab) return;
     const int64_t i = x < n_bins ? x : x - n_bins;
     const double l = x < n_bins ? __ldg(lam + i) : __ldg(lam + i) + __ldg(add + i);
     BinTable t;
-    bin_table(l, &t, T + x * kTabFixed, kTabFixed);
-    t.off = x * kTabFixed;
-    if (t.len > kTabFixed) t.off = -1 - (int64_t)atomicAdd(more, (unsigned long long)t.len);
+    bin_table(l, &t, T + x * fixed, fixed);
+    t.off = x * fixed;
+    if (t.len > fixed) t.off = -1 - (int64_t)atomicAdd(more, (unsigned long long)t.len);
     tab[x] = t;
 }
 
@@ -392,27 +392,39 @@ int grid_for(int64_t work) {
 
 // The tables of one histogram (add == nullptr) or of lam and lam + add, in
 // stream-ordered memory.  Synchronises the stream once (the size of the second
-// part; nothing of it is needed where every table fits kTabFixed entries).
+// part; nothing of it is needed where every table fits kTabFixed entries), twice where memory is short.
 struct Tables {
     BinTable* tab = nullptr;
     unsigned long long *T = nullptr, *L = nullptr, *more = nullptr;
     cudaStream_t s;
     explicit Tables(cudaStream_t s_) : s(s_) {}
-    ~Tables() {
+    ~Tables() { release(); }
+    void release() {
         pool_free(tab, s);
         pool_free(T, s);
         pool_free(L, s);
+        tab = nullptr;
+        T = L = more = nullptr;
     }
+    // Memory for n x kTabFixed entries (256 bytes a bin) may be refused where the tables themselves
+    // would fit: then every table goes to the second part, of just their size.
     ipa_status build(const double* lam, const double* add, int64_t n_bins) {
+        ipa_status st = build_with(kTabFixed, lam, add, n_bins);
+        if (st != IPA_ERR_OOM) return st;
+        cudaGetLastError();
+        release();
+        return build_with(0, lam, add, n_bins);
+    }
+    ipa_status build_with(int fixed, const double* lam, const double* add, int64_t n_bins) {
         const int n_tab = add ? 2 : 1;
         const size_t n = (size_t)n_bins * n_tab;
         ipa_status st = pool_alloc((void**)&tab, sizeof(BinTable) * n, s, "binned tables");
-        if (st == IPA_OK) st = pool_alloc((void**)&T, 8 * (n * kTabFixed + 1), s, "binned tables");
+        if (st == IPA_OK) st = pool_alloc((void**)&T, 8 * (n * fixed + 1), s, "binned tables");
         if (st != IPA_OK) return st;
-        more = T + n * kTabFixed;
+        more = T + n * fixed;
         if ((st = cuda_fail(cudaMemsetAsync(more, 0, 8, s), "binned table size")) != IPA_OK) return st;
         const unsigned grid = (unsigned)((n + kTabBlock - 1) / kTabBlock);
-        table_kernel<<<grid, kTabBlock, 0, s>>>(lam, add, n_bins, n_tab, tab, T, more);
+        table_kernel<<<grid, kTabBlock, 0, s>>>(lam, add, n_bins, n_tab, fixed, tab, T, more);
         unsigned long long h = 0;
         if ((st = cuda_fail(cudaMemcpyAsync(&h, more, 8, cudaMemcpyDeviceToHost, s), "binned table size")) != IPA_OK)
             return st;

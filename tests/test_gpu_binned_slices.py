@@ -45,3 +45,24 @@ def test_bin_without_background_counts_only_its_events():
     for k in range(200):
         n = B.generate_binned_fast(s + b, 4, k, 1)
         assert np.isfinite(x_sb[k]) == (n[0] == 0 and n[65] == 0)
+
+
+def test_tables_where_memory_is_short():
+    """Tables of 256 bytes a bin do not fit, those of the entries alone do: the same counts."""
+    from tests import gpu_common as G
+    G.need_gpu()
+    import torch
+    from paper_1706_01420_gb300 import api
+    n = 30_000_000
+    lam = torch.rand(n, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(3)) * 0.6
+    ref = api.ipa_binned_generate(lam, 11, 1)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    free = torch.cuda.mem_get_info()[0]
+    ballast = torch.empty(free - (6 << 30), dtype=torch.uint8, device="cuda")
+    try:
+        got = api.ipa_binned_generate(lam, 11, 1)
+        assert torch.equal(got, ref)
+    finally:
+        del ballast
+        torch.cuda.empty_cache()
