@@ -659,7 +659,7 @@ ipa_status launch_t(const Cols& cols, int64_t n, const int64_t* seg_begin, const
     const int64_t tiles = tile_estimate(n, n_seg);
     const LaunchCfg cfg = force ? *force : launch_cfg(KIND, GRAD, CACHED, n_seg > 1, tiles);
     if constexpr (GRAD) {
-        if (launch_team_ok(cfg, n, n_seg, Model<KIND, CACHED>::kPlainBelow))
+        if (launch_team_ok<Model<KIND, CACHED>, WEIGHTED>(cfg, n, n_seg))
             return launch_team<Model<KIND, CACHED>, WEIGHTED>(cols, n, seg_begin, seg_end, seg_tiles, n_seg, consts, sc, out,
                                                       n_par, tiles, st);
     }

@@ -332,7 +332,7 @@ ipa_status launch_tag_t(const Cols& cols, int64_t n, const int64_t* seg_begin, c
     const int64_t tiles = tile_estimate(n, n_seg);
     const LaunchCfg cfg = force ? *force : launch_cfg(IPA_MODEL_TAGGED1D, GRAD, false, n_seg > 1, tiles);
     if constexpr (GRAD) {
-        if (launch_team_ok(cfg, n, n_seg, Tagged::kPlainBelow))
+        if (launch_team_ok<Tagged, WEIGHTED>(cfg, n, n_seg))
             return launch_team<Tagged, WEIGHTED>(cols, n, seg_begin, seg_end, seg_tiles, n_seg, consts, sc, out, n_par,
                                                  tiles, st);
     }

@@ -434,24 +434,47 @@ team_kernel(Cols cols, int64_t n, const int64_t* __restrict__ seg_begin, const i
     work_done(work, lane);
 }
 
+// Resident blocks per SM of a team kernel (0: not to be launched), per device.
+template <class M, bool W>
+int team_blocks_per_sm() {
+    static int occ[64] = {};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    int& per_sm = occ[dev & 63];
+    if (per_sm == 0) {
+        auto kern = team_kernel<M, W>;
+        int v = 0;
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)team_smem<M, W>()) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, kern, 32 * kTeam, team_smem<M, W>()) != cudaSuccess) {
+            cudaGetLastError();
+            return 0;
+        }
+        per_sm = v;
+    }
+    return per_sm;
+}
+
 // Whether a launch over n events in n_seg segments goes to the teams: the built-in geometry (a
-// tuned or given one is for single warps) and at most eight tiles per SM.  Measured, call by call,
-// single warps / teams in us: 16 to 152 tiles 35 / 24 (1D), 56 / 33 (4D), 78 / 41 (tagged); 608 tiles
-// 38 / 28, 64 / 42, 83 / 69; 1216 tiles (eight per SM) 44 / 40, 75 / 64, 100 / 92; 1520 tiles 45 / 47,
-// 76 / 75, 108 / 115; 2048 tiles 51 / 56, 87 / 90, 125 / 137 (a tile's exchange then costs more than
-// the evener load gains).  Segments of up to a quarter tile (128 events) leave three of a team's warps
-// idle: four tiles per SM there (segments of 20 events: 600 of them 42 / 35, 61 / 50, 67 / 66; 1000
-// 52 / 55, 73 / 83, 76 / 92).  Segments below `plain_below` events take the plain loop in either form:
-// a warp each while there are at most as many as SMs (4D, 1, 30 and 100 segments of 20 events: 31 / 35,
-// 37 / 41, 38 / 42; 200, two to an SM, 55 / 44).
-constexpr int kTeamTilesPerSm = 8, kTeamShortPerSm = 4;
-inline bool launch_team_ok(const LaunchCfg& cfg, int64_t n, int n_seg, int plain_below) {
+// tuned or given one is for single warps), and
+//   * the tiles are resident at once (a team takes a quarter of a single warp's time), or
+//   * at most eight per SM and two thirds full on average: a second wave of teams costs as much as
+//     the first whatever its tiles hold, and short segments leave warps of a team idle.
+// Measured, single warps / teams in us for 1D, 4D, tagged.  Full tiles: 300 35 / 25, 61 / 37, 81 / 47;
+// 608 37 / 29, 62 / 42, 84 / 70; 1000 40 / 38, 66 / 58, 94 / 88; 1216 43 / 41, 74 / 65, 100 / 98; 1520 45 / 47,
+// 76 / 75, 108 / 115.  Segments of 300 events: 608 of them 46 / 39, 66 / 52, 86 / 87; 900 51 / 57, 74 / 80,
+// 95 / 97.  Of 20 events: 600 42 / 35, 61 / 50, 67 / 66; 1000 52 / 55, 73 / 83, 76 / 92.
+// Segments below M::kPlainBelow events take the plain loop in either form: a warp each while there
+// are at most as many as SMs (4D, 1, 30 and 100 segments of 20 events: 31 / 35, 37 / 41, 38 / 42; 200 of
+// them, two to an SM, 55 / 44).
+constexpr int kTeamTilesPerSm = 8;
+template <class M, bool W>
+bool launch_team_ok(const LaunchCfg& cfg, int64_t n, int n_seg) {
     if (cfg.warps_per_block != 1 || cfg.warps_per_sm != 0 || cfg.tiles_per_take != 1) return false;
-    // a tile at least per segment
-    const int64_t tiles = n_seg > 1 && tile_estimate(n, n_seg) < n_seg ? n_seg : tile_estimate(n, n_seg);
-    const bool few = n_seg > 1 && n <= (int64_t)n_seg * (32 * kSub);
-    if (n < (int64_t)n_seg * plain_below && tiles <= sm_count()) return false;
-    return tiles <= (int64_t)(few ? kTeamShortPerSm : kTeamTilesPerSm) * sm_count();
+    const int64_t sms = sm_count(), guess = tile_estimate(n, n_seg);
+    const int64_t tiles = n_seg > 1 && guess < n_seg ? n_seg : guess;      // a segment has one at least
+    if (n < (int64_t)n_seg * M::kPlainBelow && tiles <= sms) return false;
+    const int64_t per_sm = team_blocks_per_sm<M, W>();
+    return per_sm > 0 && (tiles <= per_sm * sms || (tiles <= kTeamTilesPerSm * sms && 3 * n >= 2 * kTile * tiles));
 }
 
 template <class M, bool W>
@@ -460,18 +483,7 @@ ipa_status launch_team(const Cols& cols, int64_t n, const int64_t* seg_begin, co
                        int64_t tiles, cudaStream_t st) {
     auto kern = team_kernel<M, W>;
     constexpr size_t smem = team_smem<M, W>();
-    static int occ[64] = {};                         // resident blocks per SM, per device
-    int dev = 0;
-    cudaGetDevice(&dev);
-    int& per_sm = occ[dev & 63];
-    if (per_sm == 0) {
-        ipa_status q = cuda_fail(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
-                                 "likelihood kernel attribute");
-        if (q != IPA_OK) return q;
-        int v = 0;
-        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, kern, 32 * kTeam, smem);
-        per_sm = e == cudaSuccess && v >= 1 ? v : 1;
-    }
+    const int per_sm = team_blocks_per_sm<M, W>();
     int64_t grid = (int64_t)per_sm * sm_count();
     if (seg_begin == nullptr && tiles < grid) grid = tiles < 1 ? 1 : tiles;
     cudaLaunchConfig_t lc = {};

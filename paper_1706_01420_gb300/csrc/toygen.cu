@@ -158,7 +158,7 @@ struct TimeGen {
     static constexpr bool kQuickKeeps = !ANGLES, kQuick64 = !ANGLES;
     static constexpr int kBlocksPerSm = 4;
     static constexpr int kUnroll = ANGLES ? 2 : 1;    // two candidates' Philox chains at once
-    static constexpr int kBlockEvents = ANGLES ? 0 : 1000;
+    static constexpr int kBlockEvents = ANGLES ? 0 : 512;
     struct Shared {
         Consts c;
         Filter32 f;
