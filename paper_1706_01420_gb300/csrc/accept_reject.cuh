@@ -384,7 +384,9 @@ __global__ void __launch_bounds__(kBlock, G::kBlocksPerSm) generate_kernel(const
 // and fewer per toy, where a warp's 1024 candidates at once are most of the toy's and the
 // tickets cost two launches.  1D, one toy of 100 / 500 / 1000 events: 37 us by tickets, 26 / 63 / 110
 // by one warp, 20 / 32 / 47 so (the line is where the tickets win; an envelope that accepts little
-// is walked by a block whatever it costs, as the host does not know).
+// is walked by a block whatever it costs, as the host does not know).  2000 toys of 10 / 100: 93 / 100 us
+// by tickets, 41 / 52 so; more toys than warps take a warp each (5000 of 300 and 20 000 of 500:
+// 197 / 866 by tickets, 200 / 1130 by blocks, 138 / 657).
 template <class G>
 __global__ void __launch_bounds__(kBlock) generate_block_kernel(const __grid_constant__ GenArgs A) {
     constexpr int kRows = 4;
@@ -513,8 +515,8 @@ __global__ void gen_tickets_kernel(const __grid_constant__ GenArgs A, int64_t ma
 
 // consts.cu's record is in place on the stream.  The workspace (ticket prefix,
 // counter, status words) is allocated in stream order and given back after the
-// kernel; without it (no memory) a warp generates a toy alone, with the same
-// events.
+// kernel; without it (no memory, or more toys of few events than resident warps) a
+// warp generates a toy alone, with the same events.
 template <class G>
 ipa_status launch_generator(GenArgs A, cudaStream_t s) {
     int dev = 0;
@@ -542,15 +544,17 @@ ipa_status launch_generator(GenArgs A, cudaStream_t s) {
     const int64_t many = A.capacity / 40 + 2 * kGenPerWarp * kGenWarps * most + 7 * (int64_t)A.n_toys;
     const int64_t max_tickets = (few < many ? few : many) + A.capacity / kBkgChunk + A.n_toys + 1;
     const size_t words = (size_t)A.n_toys + 3 + (size_t)max_tickets;
+    bool tickets = true;
     if constexpr (G::kBlockEvents > 0) {             // few events per toy, by the buffers' room
-        if (A.capacity <= (int64_t)G::kBlockEvents * A.n_toys) {
+        tickets = A.capacity > (int64_t)G::kBlockEvents * A.n_toys;
+        if (!tickets && A.n_toys <= most * kGenWarps) {
             const int64_t blocks = 8 * (int64_t)sm_count();
             generate_block_kernel<G><<<(unsigned)(A.n_toys < blocks ? A.n_toys : blocks), kBlock, 0, s>>>(A);
             return cuda_fail(cudaGetLastError(), "toygen kernel launch");
         }
     }
     void* ws = nullptr;
-    if (pool_alloc(&ws, words * 8, s, "generator workspace") == IPA_OK) {
+    if (tickets && pool_alloc(&ws, words * 8, s, "generator workspace") == IPA_OK) {
         ipa_status st = cuda_fail(cudaMemsetAsync(ws, 0, words * 8, s), "generator workspace reset");
         int64_t* base = static_cast<int64_t*>(ws);
         A.base = base;

@@ -104,15 +104,25 @@ __device__ __forceinline__ void add_log(double P, double w, const MathTables* mt
 // weights; -1023 for subnormal ones), or kNoWeight where all are zero.  The lane keeps its weights in wbuf for the
 // quarter: a second read of the column would go over the host link again where it lies in
 // host memory (8e6 weighted 4D events there: read twice per tile 2.14 ms, twice per
-// quarter 1.95, once 1.74).
+// quarter 1.95, once 1.74).  ONCE: nothing reads these weights again, so they leave the L1 cache
+// to the times, which are read twice (1e6 1D events in host memory 119 -> 115 us; a team's warps
+// read the quarters before their own as well).
 constexpr int kNoWeight = -5000;
+template <bool ONCE>
+__device__ __forceinline__ double load_weight(const double* p) {
+    if (!ONCE) return __ldg(p);
+    double w;
+    asm volatile("ld.global.nc.L1::no_allocate.f64 %0, [%1];" : "=d"(w) : "l"(p));
+    return w;
+}
+template <bool ONCE>
 __device__ __forceinline__ int weight_exponent(const Cols& cols, int64_t tbase, int i0, int64_t ev1, double* wbuf,
                                                int lane) {
     int hi = 0;
 #pragma unroll
     for (int i = 0; i < kSub; ++i) {
         const int64_t e = tbase + lane + 32 * (i0 + i);
-        const double w = e < ev1 ? __ldg(cols.w + e) : 0.0;
+        const double w = e < ev1 ? load_weight<ONCE>(cols.w + e) : 0.0;
         wbuf[i * 32 + lane] = w;
         hi = max(hi, high_word(w) | (int)((unsigned)__double_as_longlong(w) != 0u));   // not 0 for any w but 0
     }
@@ -229,7 +239,7 @@ __device__ __forceinline__ void solo_tile(const typename M::Record& c, const Mat
 #pragma unroll 1
         for (int i0 = 0; !plain && i0 < kPerLane && tbase + 32 * i0 < ev1; i0 += kSub) {
             if (W) {
-                const int next = max(run, weight_exponent(cols, tbase, i0, ev1, wbuf, lane));
+                const int next = max(run, weight_exponent<true>(cols, tbase, i0, ev1, wbuf, lane));
                 raise_scale(s, run, next);
                 run = next;
                 if (!scale_to<M>(&sc, base, run)) {
@@ -291,8 +301,10 @@ team_kernel(Cols cols, int64_t n, const int64_t* __restrict__ seg_begin, const i
     const int out_stride = 1 + n_par;
     __shared__ MathTables mt;
     __shared__ int64_t s_take[2];
-    __shared__ int2 s_state[2][kTeam];               // of a quarter: its largest factor (kBad: redo the tile), run
+    __shared__ __align__(16) int s_most[2][kTeam];   // a quarter's largest factor, or kBad: redo the tile
+    __shared__ int s_run[2];                         // the tile's largest weight
     constexpr int kBad = 0x7FFFFFFF;
+    static_assert(kTeam == 4, "the quarters' largest factors are read as one word");
     extern __shared__ __align__(16) unsigned char dyn_smem[];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     double* const xbuf = reinterpret_cast<double*>(dyn_smem);               // [2][kTeam][kWords][32]
@@ -350,7 +362,7 @@ team_kernel(Cols cols, int64_t n, const int64_t* __restrict__ seg_begin, const i
         int run = 0;
         if (W) {
             run = kNoWeight;
-            for (int j = 0; j <= i0; j += kSub) run = max(run, weight_exponent(cols, tbase, j, ev1, wbuf, lane));
+            for (int j = 0; j <= i0; j += kSub) run = max(run, weight_exponent<false>(cols, tbase, j, ev1, wbuf, lane));
         }
         plain = !scale_to<M>(&sc, base, run) || plain;
         {
@@ -361,7 +373,8 @@ team_kernel(Cols cols, int64_t n, const int64_t* __restrict__ seg_begin, const i
                 plain = M::bad(c, sc, s);
             }
             const int most = (int)__reduce_max_sync(0xffffffffu, (unsigned)(plain ? kBad : s.most));
-            if (lane == 0) s_state[turn & 1][wib] = make_int2(most, run);
+            if (lane == 0) s_most[turn & 1][wib] = most;
+            if (W && threadIdx.x == 32 * (kTeam - 1)) s_run[turn & 1] = run;
 #pragma unroll
             for (int i = 0; i < M::kSums; ++i) own[i * 32] = s.f[i];
 #pragma unroll
@@ -372,10 +385,9 @@ team_kernel(Cols cols, int64_t n, const int64_t* __restrict__ seg_begin, const i
         if (threadIdx.x == 32 * ((turn + 2) & (kTeam - 1))) s_take[(turn + 1) & 1] = (int64_t)atomicAdd(work, 1u);
         __syncthreads();
         {
-            int most = 0;
-#pragma unroll
-            for (int w = 0; w < kTeam; ++w) most = max(most, s_state[turn & 1][w].x);
-            run = s_state[turn & 1][kTeam - 1].y;    // the tile's largest weight
+            const int4 q = *reinterpret_cast<const int4*>(s_most[turn & 1]);
+            const int most = max(max(q.x, q.y), max(q.z, q.w));
+            if (W) run = s_run[turn & 1];
             FastScale t;
             scale_to<M>(&t, base, run);
             plain = most == kBad || too_small<M>(most, t, run);

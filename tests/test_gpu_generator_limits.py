@@ -71,10 +71,11 @@ def test_buffers_larger_than_the_events(api, kind):
     assert same(generate(api, kind, 15.0, 47, n_sig, n_bkg), without_workspace(api, kind, 15.0, 47, n_sig, n_bkg))
 
 
-@pytest.mark.parametrize("toys, most", [(1, 1), (1, 130), (1, 450), (3, 460), (600, 90), (700, 3), (3000, 60)])
+@pytest.mark.parametrize("toys, most", [(1, 1), (1, 130), (1, 450), (3, 460), (600, 90), (700, 3), (3000, 60), (6000, 40)])
 def test_few_events_per_toy(api, toys, most):
-    """1D calls of few events: a block per toy, by the room of the buffers; the events are those of
-    the tickets, which the same call takes in buffers of ample room, and the oracle's."""
+    """1D calls of few events: a block per toy, by the room of the buffers, a warp where there are
+    more toys than warps; the events are those of the tickets, which the same call takes in
+    buffers of ample room, and the oracle's."""
     from oracle import ipa_oracle as O
     rng = np.random.default_rng(toys + most)
     n_sig, n_bkg = rng.integers(0, most + 1, toys), rng.integers(0, most // 8 + 1, toys)
