@@ -662,8 +662,9 @@ ipa_status ipa_launch_config_set(const ipa_model* model, int64_t n_events, int32
 ipa_status ipa_calibrate_fp64(double* results, void* stream);
 
 /* The library's own FP64 elementary functions, evaluated elementwise: test
- * support with no counterpart in the paper (the likelihood kernel calls these
- * functions; their accuracy is tested against the CPU's libm).
+ * support with no counterpart in the paper.  The parameter records call them, and
+ * the likelihood kernels where an event leaves the ranges of their fixed-point
+ * functions; their accuracy is tested against the CPU's libm.
  *   IPA_MATH_EXP    table-driven exp (library exp above 709)
  *   IPA_MATH_LOG    table-driven log (library log for zero, negative,
  *                   subnormal, infinite and NaN arguments)

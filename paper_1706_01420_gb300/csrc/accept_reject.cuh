@@ -96,7 +96,7 @@ __device__ __forceinline__ U4 gen_draw(const GenArgs& A, const GenIdx& j, uint32
 }
 
 // (v + 1) 2^-53 and 2 (v + 1) 2^-53 - 1 for the 53-bit v of two words, exactly,
-// by integer operations (u01 and 2 u01 - 1 cost two and four FP64 instructions).
+// by integer operations (a conversion, a product and a sum would be two and four FP64 instructions).
 __device__ __forceinline__ unsigned long long u53(uint32_t a, uint32_t b) {
     return (((((unsigned long long)a) << 32) | b) >> 11) + 1ull;
 }

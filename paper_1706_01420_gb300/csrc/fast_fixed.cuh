@@ -180,8 +180,9 @@ __device__ __forceinline__ bool fits_q62(double x) {
     return ((int)((unsigned long long)__double_as_longlong(x) >> 32) & 0x7FFFFFFF) < 0x3FFC0000;
 }
 
-// Ten products of the helicity angles in Q62 (absolute error a few 2^-60), a basis
-// of the f'_k (angular.cuh) that takes one product less each:
+// Ten products of the helicity angles in Q62, a basis of the f'_k (angular.cuh) that takes
+// one product less each.  Absolute error a few 2^-60; in the four with the square root q of
+// sk2 sl2 also those factors' last places times (sk2 + sl2) / (2 q), up to 2^-55 near |cos| = 1:
 //   g = {sl2, sk2, G, G cp^2, G sp cp, f'_4, f'_5, f'_7, f'_8, f'_9},  G = sk2 sl2 (sk2 =
 //   sin^2 thK, sl2 = sin^2 thmu, cp = cos phi, sp = sin phi);
 //   f'_0 = sl2 - G, f'_1 = sk2 - G cp^2, f'_2 = sk2 - G + G cp^2, f'_3 = G sp cp, f'_6 = sl2.
@@ -267,8 +268,10 @@ __device__ __forceinline__ double fx_exp2(long long y, int ysh, const MathTables
                                             ((unsigned long long)(unsigned)(*x + 1023) << 52)));
 }
 
-// 2 e^{-Gamma tau + Gamma^2 sigma^2 / 2} (fx_exp_setup) at t, T = fx(fx_signed(t, s.top)); relative
-// error below 2^-54, most of it from y's last place.  *ok is cleared where the result lies
+// 2 e^{-Gamma tau + Gamma^2 sigma^2 / 2} (fx_exp_setup) at t, T = fx(fx_signed(t, s.top)).  Relative
+// error before the last rounding: ln2 / 64 times the error of y, two units of 2^-ysh (ysh = 54
+// where |y| < 64 throughout the range, 44 at 65000) and the rounding of c as a double (2^-47 for
+// |c| < 128, as with mu near 0): 2^-53.5 for the usual ranges, 2^-50 at the widest.  *ok is cleared where the result lies
 // outside its range (the caller checks fx_in_range).
 __device__ __forceinline__ double fx_exp(Fx T, const FxExp& s, const MathTables* mt, bool* ok) {
     int x;

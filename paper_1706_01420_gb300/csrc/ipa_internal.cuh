@@ -33,7 +33,8 @@ __host__ __device__ constexpr int npar_of(int kind) {
 //   NLL only:      L = sum w log P
 //   1D + grad:     L, Q = sum w/P, S = sum (w/P) T, D_Gamma, D_sigma, D_mu
 //   4D + grad:     L, Q, S_1..S_10 = sum (w/P) T f_k, D_Gamma, D_sigma, D_mu
-//   tagged + grad: 13 (tagged.cu);  phi_s + grad: 47 (phis.cu)
+//   tagged + grad: 13 (tagged.cu)
+//   phi_s + grad:  31 sums in rows of 47, the rest zero (phis.cu; a shard's rows are that wide)
 __host__ __device__ constexpr int n_acc(int kind, bool grad) {
     return !grad ? 1
                  : (kind == IPA_MODEL_TIME1D ? 6

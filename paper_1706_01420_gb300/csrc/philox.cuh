@@ -1,6 +1,5 @@
 // Philox-4x32-10 (Salmon, Moraes, Dror and Shaw, "Parallel random numbers: as
-// easy as 1, 2, 3", SC'11), written out here, and the 53-bit uniform built from
-// two of its words.  Every draw is a pure function of (counter, key), so the
+// easy as 1, 2, 3", SC'11), written out here.  Every draw is a pure function of (counter, key), so the
 // generators address their random numbers by (index, toy, call) and the
 // result of a draw does not depend on which thread makes it.
 #pragma once
@@ -80,12 +79,6 @@ __device__ __forceinline__ PhiloxCol philox_col(const PhiloxKeys& keys, uint32_t
     const unsigned long long p = (unsigned long long)kPhiloxM1 * c2;
     const unsigned long long q = (unsigned long long)kPhiloxM0 * ((uint32_t)(p >> 32) ^ c1 ^ keys.k[0]);
     return PhiloxCol{(uint32_t)p, (uint32_t)(q >> 32), (uint32_t)q};
-}
-
-// u = ((((a << 32) | b) >> 11) + 1) 2^-53, in (0, 1] (exact).
-__device__ __forceinline__ double u01(uint32_t a, uint32_t b) {
-    const unsigned long long v = ((((unsigned long long)a) << 32) | b) >> 11;
-    return __dmul_rn(__ull2double_rn(v + 1ull), 0x1p-53);
 }
 
 // Counter (idx lo32, idx hi32, toy, call) with key (k0, k1).

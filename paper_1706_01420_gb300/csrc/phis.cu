@@ -593,7 +593,7 @@ phis_kernel(Cols cols, int64_t n, const int64_t* __restrict__ seg_begin, const i
                     sbuf[j] = tag_slow(pw.c, __ldg(cols.t + e) - pw.c.mu, &mt);
                 }
                 __syncwarp();
-const auto slow_of = [&](int k) {
+                const auto slow_of = [&](int k) {
                     const unsigned m = k == 0 ? m0 : (k == 1 ? m1 : (k == 2 ? m2 : m3));
                     const int before = k == 0 ? 0 : (k == 1 ? p1 : (k == 2 ? p2 : p3));
                     TagSlow sl = {0.0, 0.0, 0.0, 0.0, 0.0};
@@ -604,7 +604,7 @@ const auto slow_of = [&](int k) {
                 int top = pw.rtop;
                 if (GRAD && pw.fixed && ev1 - tbase >= kFewEvents) {
                     if (WEIGHTED) {
-                        // the exponent of the rows' largest |w| (0 where all weights are 1)
+                        // the exponent of the rows' largest |w| (0 where all weights are 1); the rows read them again
                         unsigned hi = 0;
 #pragma unroll
                         for (int k = 0; k < kSub; ++k) {
