@@ -46,7 +46,10 @@ constexpr int kTabBlock = 64;           // bins per block of the table kernels: 
 constexpr int kTabFixed = 32;           // thresholds per bin in the fixed part of the table
 constexpr int kSlice = 64;              // bins summed by one thread of the CLs kernel
 constexpr int kToyBlock = 128;          // toys per block of the CLs kernel
-constexpr int kFirst = 5;               // thresholds compared without a search (4: 732 us, 5: 720, 6: 731, 8: 772)
+// Thresholds compared without a search.  10 000 bins and toys, means 0.1 / 0.5 / 2 / 5 / 20 in us: 3 of them
+// 681 / 892 / 1328 / 1477 / 1698, 5 711 / 724 / 1160 / 1511 / 1731, 8 765 / 772 / 835 / 1403 / 1774, 12 843 / 852 / 863 /
+// 1098 / 1827: 5 for means around one half (Example 4's), where a draw passes few.
+constexpr int kFirst = 5;
 constexpr uint32_t kBinnedCall = 8u;
 
 __device__ __forceinline__ uint32_t binned_call(int hyp, int m) {

@@ -13,8 +13,8 @@
 //   w(z) = 1 / (sqrt(pi) (L - i z)) + 2 sum_{n>=1} a_n Z^{n-1} / (L - i z)^2,
 //   Z = (L + i z) / (L - i z),
 // truncated at n = N = 40 with L = 2^(-1/4) sqrt(N).  The coefficients are
-// generated in 60-digit arithmetic (gen_fp64_tables.py).  |Z| <= 1 in the closed upper half plane, and |L - i z| >= L keeps
-// every division away from zero.
+// generated in 60-digit arithmetic (gen_fp64_tables.py).  |Z| <= 1 in the closed
+// upper half plane, and |L - i z| >= L keeps every division away from zero.
 //
 // The coefficients are real, so p(Z) = sum a_k Z^k takes two real products per
 // step instead of four:

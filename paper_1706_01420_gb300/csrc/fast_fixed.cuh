@@ -268,11 +268,11 @@ __device__ __forceinline__ double fx_exp2(long long y, int ysh, const MathTables
                                             ((unsigned long long)(unsigned)(*x + 1023) << 52)));
 }
 
-// 2 e^{-Gamma tau + Gamma^2 sigma^2 / 2} (fx_exp_setup) at t, T = fx(fx_signed(t, s.top)).  Relative
-// error before the last rounding: ln2 / 64 times the error of y, two units of 2^-ysh (ysh = 54
-// where |y| < 64 throughout the range, 44 at 65000) and the rounding of c as a double (2^-47 for
-// |c| < 128, as with mu near 0): 2^-53.5 for the usual ranges, 2^-50 at the widest.  *ok is cleared where the result lies
-// outside its range (the caller checks fx_in_range).
+// 2 e^{-Gamma tau + Gamma^2 sigma^2 / 2} (fx_exp_setup) at t, T = fx(fx_signed(t, s.top)).
+// Relative error before the last rounding: ln2 / 64 times the error of y, two units of 2^-ysh
+// (ysh = 54 where |y| < 64 throughout the range, 44 at 65000) and the rounding of c as a double
+// (2^-47 for |c| < 128, as with mu near 0): 2^-53.5 for the usual ranges, 2^-50 at the widest.
+// *ok is cleared where the result lies outside its range (the caller checks fx_in_range).
 __device__ __forceinline__ double fx_exp(Fx T, const FxExp& s, const MathTables* mt, bool* ok) {
     int x;
     const double v = fx_exp2(s.c - fx_mad(T, Fx{s.gh, s.gl}, 0), s.ysh, mt, &x);

@@ -349,7 +349,8 @@ struct Angtime {
     using Record = Consts;
     using Slow = double2;
     // FP64: sum r, sum r A' tau T2, sum r A' Gx, sum r A' tau Gx, sum w log P; integers: r T g_k
-    static constexpr int kTopRange = 900, kLeast = 16, kPlainBelow = kFewEvents, kSums = 5, kInts = 10, NA = n_acc(IPA_MODEL_ANGTIME4D, true);
+    static constexpr int kTopRange = 900, kLeast = 16, kPlainBelow = kFewEvents;
+    static constexpr int kSums = 5, kInts = 10, NA = n_acc(IPA_MODEL_ANGTIME4D, true);
     using Sums = FastSums<kSums, kInts>;
 
     static __device__ __forceinline__ bool usable(const Consts& c, int64_t events, FastScale* sc) {
@@ -433,7 +434,8 @@ struct Time1d {
     using Record = Consts;
     using Slow = double2;
     // FP64: sum r, sum w log P; integers: r T, r Gx, r tau T, r tau Gx (the factor A' = cs/2 outside)
-    static constexpr int kTopRange = 400, kLeast = 14, kPlainBelow = 0, kSums = 2, kInts = 4, NA = n_acc(IPA_MODEL_TIME1D, true);
+    static constexpr int kTopRange = 400, kLeast = 14, kPlainBelow = 0;
+    static constexpr int kSums = 2, kInts = 4, NA = n_acc(IPA_MODEL_TIME1D, true);
     using Sums = FastSums<kSums, kInts>;
 
     static __device__ __forceinline__ bool usable(const Consts& c, int64_t events, FastScale* sc) {

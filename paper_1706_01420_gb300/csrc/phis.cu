@@ -257,8 +257,8 @@ __device__ __forceinline__ void phis_event(const PhisWarp& pw, const MathTables*
 // r U and r C are converted once per event at a scale that follows the segment's typical r T and
 // the largest weight of the warp's rows (unit 2^-48 of a typical term, 0.41 units rms per
 // event).  The rest is FP64.  The warp's rows are redone by phis_event where some P lies outside
-// the Newton reciprocal's range, some factor above its scale or all of them far below it.  FP64 instructions per
-// event: 92 -> 57; 1e6 events 299 -> 248 us (FP64 unit busy 77 -> 68 %).
+// the Newton reciprocal's range, some factor above its scale or all of them far below it.
+// FP64 instructions per event: 92 -> 57; 1e6 events 299 -> 248 us (FP64 unit busy 77 -> 68 %).
 
 // The f'_k in Q62 near |cos| = 1 (rare).  False where one of them does not fit (angles that
 // are NaN or infinite, |cos| > 1): the rows are left to phis_event.
@@ -604,7 +604,7 @@ phis_kernel(Cols cols, int64_t n, const int64_t* __restrict__ seg_begin, const i
                 int top = pw.rtop;
                 if (GRAD && pw.fixed && ev1 - tbase >= kFewEvents) {
                     if (WEIGHTED) {
-                        // the exponent of the rows' largest |w| (0 where all weights are 1); the rows read them again
+                        // the exponent of the rows' largest |w| (0 where all weights are 1; the rows read them again)
                         unsigned hi = 0;
 #pragma unroll
                         for (int k = 0; k < kSub; ++k) {

@@ -157,7 +157,8 @@ struct Tagged {
     using Record = TagConsts;
     using Slow = TagSlow;
     // FP64: sum r, sum w log P; integers: the six sums in the order above, then times tau (not r q Gx)
-    static constexpr int kTopRange = 400, kLeast = 14, kPlainBelow = 0, kSums = 2, kInts = 11, NA = n_acc(IPA_MODEL_TAGGED1D, true);
+    static constexpr int kTopRange = 400, kLeast = 14, kPlainBelow = 0;
+    static constexpr int kSums = 2, kInts = 11, NA = n_acc(IPA_MODEL_TAGGED1D, true);
     using Sums = FastSums<kSums, kInts>;
 
     static __device__ __forceinline__ bool usable(const TagConsts& c, int64_t events, FastScale* sc) {

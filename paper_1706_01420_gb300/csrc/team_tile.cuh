@@ -101,12 +101,12 @@ __device__ __forceinline__ void add_log(double P, double w, const MathTables* mt
 }
 
 // The exponent of the largest |w| of a quarter (0 where all weights are 1, as without
-// weights; -1023 for subnormal ones), or kNoWeight where all are zero.  The lane keeps its weights in wbuf for the
-// quarter: a second read of the column would go over the host link again where it lies in
-// host memory (8e6 weighted 4D events there: read twice per tile 2.14 ms, twice per
-// quarter 1.95, once 1.74).  ONCE: nothing reads these weights again, so they leave the L1 cache
-// to the times, which are read twice (1e6 1D events in host memory 119 -> 115 us; a team's warps
-// read the quarters before their own as well).
+// weights; -1023 for subnormal ones), or kNoWeight where all are zero.  The lane keeps its
+// weights in wbuf for the quarter: a second read of the column would go over the host link again
+// where it lies in host memory (8e6 weighted 4D events there: read twice per tile 2.14 ms, twice
+// per quarter 1.95, once 1.74).  ONCE: nothing reads these weights again, so they leave the L1
+// cache to the times, which are read twice (1e6 1D events in host memory 119 -> 115 us; a team's
+// warps read the quarters before their own as well).
 constexpr int kNoWeight = -5000;
 template <bool ONCE>
 __device__ __forceinline__ double load_weight(const double* p) {
