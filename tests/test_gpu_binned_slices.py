@@ -59,7 +59,10 @@ def test_tables_where_memory_is_short():
     torch.cuda.synchronize()
     torch.cuda.empty_cache()
     free = torch.cuda.mem_get_info()[0]
-    ballast = torch.empty(free - (6 << 30), dtype=torch.uint8, device="cuda")
+    try:
+        ballast = torch.empty(free - (6 << 30), dtype=torch.uint8, device="cuda")
+    except torch.cuda.OutOfMemoryError:
+        pytest.skip("the card's free memory cannot be held")
     try:
         got = api.ipa_binned_generate(lam, 11, 1)
         assert torch.equal(got, ref)
